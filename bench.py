@@ -245,8 +245,8 @@ def extra_workload(idx, torch, stairs, local_rank, peak, tflops_peak):
         res["prefill"] = {"ms_per_request": float(np.mean(pre_ms)), "tokens_per_s": prefix / (float(np.mean(pre_ms)) * 1e-3),
                           "useful_tflops": fl / (sum(pre_ms) * 1e-3) / 1e12,
                           "frac_of_bf16_sustained_peak": fl / (sum(pre_ms) * 1e-3) / 1e12 / tflops_peak if tflops_peak else None,
-                          "note": "target and assistant, 64 positions per pass of the persistent kernel (weights re-streamed every pass; "
-                                  "operands are bf16 hi+lo pairs, so the tensor pipe does twice the useful work)"}
+                          "note": "target and assistant, up to 2048 positions per pass (operands are bf16 hi+lo pairs, so the tensor pipe "
+                                  "does twice the useful work)"}
         # validate latency per k (uniform random drafts: the time does not depend on the accept length)
         rng = np.random.default_rng(6)
         per_k = {}

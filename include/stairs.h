@@ -94,7 +94,8 @@ typedef struct stairs_config {
   int32_t kv_page_tokens; /* tokens per KV page: 16, 32, 64 or 128                   */
   int32_t kv_pages;       /* pages in the pool; 0 = enough for every slot to reach
                              max_seq_len                                             */
-  int32_t prefill_chunk;  /* rows per prefill pass; 0 = 256                          */
+  int32_t prefill_chunk;  /* most rows per prefill pass; 0 = up to 2048 where the
+                             many-row tensor-core passes apply, else 256             */
   int32_t device;         /* CUDA device ordinal                                     */
   int32_t gemm_impl;      /* 0 = best available (bf16: one persistent kernel per pass
                              of <= 64 rows, tensor-core GEMMs otherwise), 1 = force

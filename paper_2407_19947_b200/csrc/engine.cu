@@ -19,6 +19,7 @@
 #include "gemm_tc.cuh"
 #include "kernels_basic.cuh"
 #include "megakernel.cuh"
+#include "wide.cuh"
 
 using namespace stairs;
 
@@ -63,6 +64,7 @@ struct DevModel {
 struct Layout {
   size_t status, seq, n_seq, page_table, tok, pos, req, val_req, val_k, val_off, keys, x, h, qkv, q,
       o, ff, logits, draft_buf, tt_buf, al_buf, gemm_partial, gemm_counters, mk_partial, mk_partial_bytes, mk_bar, attn_part, prog_t, prog_d, mk_trace, mk_stats, rope_t, rope_d, aux_t, aux_d, w13_t, w13_d, kv_t_k, kv_t_v, kv_d_k, kv_d_v, total;
+  size_t kv_row, wide_rope, wide_stats;
   int max_rows, logit_rows, max_pages, n_pages, t_box_max, attn_units, stat_tiles;
   size_t prog_slot_t, prog_slot_d, prog_maps_off_t, prog_maps_off_d;
   size_t kv_t_layer, kv_d_layer;
@@ -95,6 +97,7 @@ struct stairs_ctx {
   int sm_count = 0;
   EncodeTiledFn encode = nullptr;
   std::map<std::tuple<const void*, int, int>, CUtensorMap> act_maps;
+  std::map<std::tuple<const void*, int, int>, CUtensorMap> wide_maps;   // many-row passes: (matrix or buffer, K, box rows)
   unsigned int* status_host = nullptr;  // pinned, device-visible status words
   unsigned int* status_dev = nullptr;
   // pinned, device-visible block of the host-buffer entry points: drafts in (staged for one
@@ -110,6 +113,7 @@ struct stairs_ctx {
   int att_nbuf_force = 0;            // tuning: K/V chunk buffers of the attention phases (0 = chosen from the context length)
   int att_tc_force = 0;              // tuning: 1 = tcgen05 attention for every call it can serve
   int att_tc_off = 0;                // tuning: 1 = attention contractions on mma.sync even where the tcgen05 path applies
+  int wide_cg_force = 0, wide_split_force = 0;   // tuning: CTAs per tile and K ranges of the many-row GEMMs (0 = planned)
   int att_tma_off = 0;               // tuning: 1 = stage K/V with 16-byte copies from the compute warps even where bulk copies apply
 };
 
@@ -149,6 +153,21 @@ const char* check_model(const stairs_model& m) {
   return nullptr;
 }
 
+// Models the persistent kernel and the many-row passes take (the epilogues' vector stores want every GEMM
+// width but the vocabulary to be a multiple of 64).
+bool shape_fits_tc(const stairs_model& m) {
+  return m.wdtype == 1 && m.n_layers >= 1 && m.head_dim % 16 == 0 && m.head_dim <= 128 && m.d_model % 64 == 0 && m.d_ff % 64 == 0 &&
+         (m.n_heads * m.head_dim) % 64 == 0 && m.d_model <= 8192;
+}
+
+// Rows of one prefill pass.  The many-row passes read all weights once per pass and fill the chip from
+// about a thousand rows on; the other paths keep their activations small.
+int prefill_rows(const stairs_config& c) {
+  if (c.prefill_chunk > 0) return c.prefill_chunk;
+  const bool wide = c.gemm_impl == 0 && shape_fits_tc(c.target);
+  return wide ? std::max(64, std::min(2048, c.max_seq_len)) : 256;
+}
+
 // Upper bound of the attention units of one request with `rows` rows in the persistent kernel: the
 // kernel picks chunks per unit so that kv heads x position ranges fit the grid (or, for contexts
 // too long for that, at most twice the grid: stairs_init checks this); the rows of the call can
@@ -179,7 +198,7 @@ bool compute_layout(const stairs_config& c, Layout* L, const char** why) {
   if (pt != 16 && pt != 32 && pt != 64 && pt != 128) { *why = "kv_page_tokens must be 16, 32, 64 or 128"; return false; }
   if (c.target.pos == 0 && c.max_seq_len > c.target.max_pos) { *why = "max_seq_len exceeds max_pos of the learned positions"; return false; }
   if (c.kv_pages < 0 || c.prefill_chunk < 0) { *why = "kv_pages and prefill_chunk must not be negative"; return false; }
-  const int chunk = c.prefill_chunk > 0 ? c.prefill_chunk : 256;
+  const int chunk = prefill_rows(c);
   L->max_rows = (std::max(std::max(chunk, c.max_requests * (c.k_max + 1)), 2) + 15) / 16 * 16;
   if (c.target.wdtype == 1) L->max_rows = std::max(L->max_rows, MK_MAX_ROWS);   // prefill passes of the persistent kernel
   L->t_box_max = std::min(256, L->max_rows);
@@ -222,7 +241,7 @@ bool compute_layout(const stairs_config& c, Layout* L, const char** why) {
   L->gemm_counters = take(t.wdtype == 1 ? (size_t)TC_COUNTERS * 4 : 0);
   // split-tile partial sums of the persistent kernel: two sets (alternate GEMM phases) of one slot per CTA;
   // every element holds the "empty" pattern between uses
-  L->mk_partial_bytes = t.wdtype == 1 ? (size_t)2 * TC_GRID_MAX * L->t_box_max * tc::BM * 4 : 0;
+  L->mk_partial_bytes = t.wdtype == 1 ? (size_t)2 * TC_GRID_MAX * MK_MAX_ROWS * tc::BM * 4 : 0;
   L->mk_partial = take(L->mk_partial_bytes);
   {
     // persistent-kernel scratch: attention unit states and the per-(model, row box) programs
@@ -251,6 +270,10 @@ bool compute_layout(const stairs_config& c, Layout* L, const char** why) {
     L->mk_stats = take(t.wdtype == 1 ? (size_t)MK_MAX_ROWS * L->stat_tiles * 16 : 0);
     L->rope_t = take(t.wdtype == 1 ? (size_t)t.head_dim * 2 * (1 + 2 * 64) : 0);   // inverse frequencies, then cos and sin of 64 rows
     L->rope_d = take((t.wdtype == 1 && has_draft) ? (size_t)d.head_dim * 2 * (1 + 2 * 64) : 0);
+    // many-row passes: cache row and rotation table of every row, statistics per row and column tile of x
+    L->kv_row = take(t.wdtype == 1 ? R * 4 : 0);
+    L->wide_rope = take(t.wdtype == 1 ? R * (size_t)mx(t.head_dim, d.head_dim) * 4 : 0);
+    L->wide_stats = take(t.wdtype == 1 ? R * ((dm + 63) / 64) * 16 : 0);
     // LayerNorm models: u = W.gain and c = W.bias per normalised GEMM (fp32)
     auto aux = [&](const stairs_model& m) {
       if (m.norm != 0) return (size_t)0;
@@ -723,9 +746,7 @@ struct MkCall {
 };
 
 bool mk_eligible(const stairs_ctx* ctx, const DevModel& M, int T) {
-  // (the epilogue's vector stores want every GEMM width but the vocabulary to be a multiple of 4)
-  return ctx->use_mk && M.m.n_layers >= 1 && T >= 1 && T <= MK_MAX_ROWS && M.m.head_dim % 16 == 0 && M.m.head_dim <= 128 &&
-         M.m.d_model % 64 == 0 && M.m.d_ff % 64 == 0 && (M.m.n_heads * M.m.head_dim) % 64 == 0 && M.m.d_model <= 8192;
+  return ctx->use_mk && T >= 1 && T <= MK_MAX_ROWS && shape_fits_tc(M.m);
 }
 
 int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, int n_logit_rows, const MkCall& c) {
@@ -739,14 +760,14 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
     // attention scratch: refuse a call whose units might not fit rather than compute part of it
     const int hkv = m.n_kv_heads, gq = m.n_heads / m.n_kv_heads;
     long long need = 0;
-    // The tcgen05 attention path pays where a unit walks many chunks (long contexts) or a request has
-    // many query rows (prefill passes: 128 queries share a chunk instead of 48); short units are
+    // The tcgen05 attention path pays where a unit walks many chunks (long contexts); short units are
     // quicker on the register path, whose per-unit set-up is smaller.
     int r_max0 = 0; long long len_max = 0;
     if (c.mode == mk::CALL_VALIDATE) for (int i = 0; i < c.n_req; ++i) { r_max0 = std::max(r_max0, c.k_host[i] + 1); len_max = std::max<long long>(len_max, ctx->n_seq_ub[c.req_host[i]]); }
     else { r_max0 = T; len_max = c.mode == mk::CALL_PREFILL ? c.draft_step + T : ctx->n_seq_ub[c.slot]; }
     const long long chunks_per_unit = (len_max / mk::ATT_CHUNK + 1) * hkv / std::max(ctx->sm_count, 1);
-    // (with many query rows its tiles take shared memory from the GEMM ring: only past a few thousand positions)
+    // (a draft of many query rows shares a chunk between 128 queries instead of 48, but its tiles take shared
+    // memory from the GEMM ring: only past a few thousand positions)
     tc_call = (ctx->att_tc_force > 0 || chunks_per_unit >= 6 || (r_max0 * gq >= 96 && len_max >= 4096)) ? 1 : 0;
     const MkPlan pl0 = mk_plan(ctx, m, t_box, 0, tc_call);
     int r_max = 0;
@@ -809,6 +830,221 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
   ctx->bar_base += (unsigned long long)n_run * grid;
   ctx->launches++;
   return STAIRS_OK;
+}
+
+// ---------------------------------------------------------------------------------------------
+// Many-row passes (wide.cuh): tile plan per GEMM, launches chained with programmatic dependent launch.
+// ---------------------------------------------------------------------------------------------
+struct WidePlan { int cg, tn, splits; };
+
+// Tile shape of one GEMM over T rows: pairs of CTAs (256 rows) or single CTAs (128 rows), tile width a
+// multiple of `gran` (whole heads for the QKV projection, whole gate/up blocks), K cut in up to 8 ranges
+// where few tiles would leave the chip idle.  The estimate: a k-block costs the slower of its MMAs
+// (hi and lo part, TN / 2 cycles each at full rate, never less than their issue time) and the L2 traffic
+// of its tiles at about 45 bytes per cycle and SM; whole waves of units; weights from HBM once; the
+// last tile's epilogue is exposed, and split tiles add the round trip of their parked sums.
+WidePlan wide_plan(const stairs_ctx* ctx, int T, int K, const int* rows, int n_src, int gran, int max_splits, size_t partial_bytes) {
+  const int sms = std::min(ctx->sm_count, TC_GRID_MAX);
+  const int kblocks = (K + tc::BK - 1) / tc::BK;
+  double w_bytes = 0;
+  for (int s = 0; s < n_src; ++s) w_bytes += 2.0 * rows[s] * K;
+  WidePlan best{1, gran, 1};
+  double best_us = 1e30;
+  for (int cg = 1; cg <= 2; ++cg) {
+    if (cg == 2 && T <= wide::WM) continue;
+    if (ctx->wide_cg_force && cg != ctx->wide_cg_force && T > wide::WM) continue;
+    const int m_tiles = (T + wide::WM * cg - 1) / (wide::WM * cg);
+    const int x_box = m_tiles == 1 && cg == 1 ? (T + 15) / 16 * 16 : wide::WM;
+    for (int tn = gran; tn <= 256; tn += gran) {
+      if (cg == 2 && (tn % 32 || tn < 64)) continue;   // (either CTA holds half of the weight tile)
+      int n_tiles = 0;
+      for (int s = 0; s < n_src; ++s) n_tiles += (rows[s] + tn - 1) / tn;
+      for (int sp = 1; sp <= max_splits; sp *= 2) {
+        if (ctx->wide_split_force && cg == 1 && sp != std::min(ctx->wide_split_force, max_splits)) continue;
+        const long long units = (long long)n_tiles * m_tiles * sp;
+        if (sp > 1 && (cg == 2 || units > sms || kblocks < sp || (size_t)units * tn * wide::WM * 4 > partial_bytes)) continue;
+        const double waves = std::ceil((double)units / (sms / cg));
+        const double mma = 8.0 * std::max(tn / 2.0, 52.0), load = (2.0 * x_box + tn / cg) * 128.0 / 45.0;
+        const double kb = std::ceil((double)kblocks / sp);
+        const double stream = std::max(waves * kb * std::max(mma, load) / 1.75e3, w_bytes / 6.5e6);
+        const double us = stream + (1500.0 + tn * 25.0 + (sp > 1 ? 3500.0 + sp * tn * 6.0 : 0.0)) / 1.75e3;
+        if (us < best_us - 1e-9) { best_us = us; best = {cg, tn, sp}; }
+      }
+    }
+  }
+  return best;
+}
+
+template <typename... A>
+cudaError_t launch_chained(cudaStream_t st, void (*kern)(A...), dim3 grid, int threads, size_t smem, dim3 cluster, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension; at[1].val.clusterDim.x = cluster.x; at[1].val.clusterDim.y = cluster.y; at[1].val.clusterDim.z = cluster.z;
+  cfg.attrs = at; cfg.numAttrs = cluster.x * cluster.y * cluster.z > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// Weight matrices of one many-row GEMM: up to three sources that share the operand.
+struct WideW { const void* ptr[3]; int rows[3]; int n_src; };
+
+const CUtensorMap* wide_map(stairs_ctx* ctx, const void* ptr, long long rows, int K, int box) {
+  auto key = std::make_tuple(ptr, K, box);
+  auto it = ctx->wide_maps.find(key);
+  if (it == ctx->wide_maps.end()) {
+    CUtensorMap mp;
+    if (!encode_map(ctx, &mp, ptr, rows, K, box)) return nullptr;
+    it = ctx->wide_maps.emplace(key, mp).first;
+  }
+  return &it->second;
+}
+
+int launch_wide_gemm(stairs_ctx* ctx, wide::WideJob& job, const void* x, int K, const WideW& w, int gran, int max_splits) {
+  const Layout& L = ctx->lay;
+  const WidePlan pl = wide_plan(ctx, job.T, K, w.rows, w.n_src, gran, max_splits, L.gemm_counters - L.gemm_partial);
+  job.TN = pl.tn; job.splits = pl.splits;
+  job.kblocks = (K + tc::BK - 1) / tc::BK;
+  job.m_tiles = (job.T + wide::WM * pl.cg - 1) / (wide::WM * pl.cg);
+  job.x_box = job.m_tiles == 1 && pl.cg == 1 ? (job.T + 15) / 16 * 16 : wide::WM;
+  job.n_src = w.n_src; job.n_tiles = 0;
+  const bool half_block = job.epi == wide::W_SWIGLU && pl.tn == 64;
+  job.b_boxes = half_block ? 2 : 1;
+  job.b_box = half_block ? 32 : pl.tn / pl.cg;
+  job.gsz = pl.tn == 64 ? 32 : 64;
+  for (int s = 0; s < 3; ++s) {
+    const int i = s < w.n_src ? s : 0;
+    const CUtensorMap* m = wide_map(ctx, w.ptr[i], w.rows[i], K, job.b_box);
+    if (!m) return fail(ctx, STAIRS_ECUDA, "cuTensorMapEncodeTiled failed for a weight matrix");
+    job.w_map[s] = *m;
+    job.src_tiles[s] = (w.rows[i] + pl.tn - 1) / pl.tn; job.src_rows[s] = w.rows[i];
+    if (s < w.n_src) job.n_tiles += job.src_tiles[s];
+  }
+  const CUtensorMap* xm = wide_map(ctx, x, 2 * (long long)L.max_rows, K, job.x_box);
+  if (!xm) return fail(ctx, STAIRS_ECUDA, "cuTensorMapEncodeTiled failed for an activation buffer");
+  job.x_map = *xm;
+  if (job.n_tiles * job.m_tiles > TC_COUNTERS) return fail(ctx, STAIRS_EUNSUPPORTED, "too many tiles for the split bookkeeping");
+  job.stages = wide::gemm_stages(pl.tn, pl.cg);
+  job.lo_row = L.max_rows;
+  job.partial = reinterpret_cast<float*>(ctx->ws + L.gemm_partial);
+  job.counters = reinterpret_cast<int*>(ctx->ws + L.gemm_counters);
+  job.status = ctx->status_dev; job.wait_limit = ctx->wait_limit;
+  const int slots = std::min(ctx->sm_count, TC_GRID_MAX) / pl.cg;
+  const int grid = std::min(slots, job.n_tiles * job.m_tiles * pl.splits) * pl.cg;
+  const size_t smem = wide::gemm_smem(pl.tn, pl.cg, job.stages);
+  ctx->launches++;
+  CK(launch_chained(ctx->stream, pl.cg == 2 ? wide::k_wide_gemm<2> : wide::k_wide_gemm<1>, dim3(grid), wide::WTHREADS, smem, dim3(pl.cg, 1, 1), job));
+  return STAIRS_OK;
+}
+
+template <int KS, bool EXACT>
+int launch_wide_attn_ks(stairs_ctx* ctx, const wide::WideAttn& a, int n_req, int q_max, int chunks) {
+  // prefill chunks and long drafts: 128 queries per block; few query rows: the four warps split the positions
+  auto go = [&](auto nw, auto mtc) -> int {
+    constexpr int NW = decltype(nw)::value, MT = decltype(mtc)::value;
+    wide::WideAttn p = a;
+    p.n_qblk = (q_max + MT * 16 - 1) / (MT * 16);
+    // ranges of the context, one CTA of a cluster each, while blocks are few and ranges hold two chunks at least
+    int ns = 1;
+    const long long blocks = (long long)n_req * p.n_qblk * a.Hkv;
+    while (ns < 8 && blocks * ns * 2 <= 2ll * ctx->sm_count && chunks / (ns * 2) >= 2) ns *= 2;
+    const size_t smem = wide::attn_smem(a.hd, NW, MT);
+    auto kern = wide::k_wide_attn<KS, EXACT, NW, MT>;
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ctx->launches++;
+    CK(launch_chained(ctx->stream, kern, dim3(n_req * p.n_qblk, a.Hkv, ns), NW * 32, smem, dim3(1, 1, ns), p));
+    return STAIRS_OK;
+  };
+  using std::integral_constant;
+  if (q_max <= 16) return go(integral_constant<int, 4>(), integral_constant<int, 1>());
+  if (q_max <= 32) return go(integral_constant<int, 4>(), integral_constant<int, 2>());
+  if (q_max <= 64) return go(integral_constant<int, 4>(), integral_constant<int, 4>());
+  return go(integral_constant<int, 8>(), integral_constant<int, 8>());
+}
+int launch_wide_attn(stairs_ctx* ctx, const wide::WideAttn& a, int n_req, int q_max, int chunks) {
+  if (a.hd == 64) return launch_wide_attn_ks<4, true>(ctx, a, n_req, q_max, chunks);
+  if (a.hd == 80) return launch_wide_attn_ks<5, true>(ctx, a, n_req, q_max, chunks);
+  if (a.hd == 128) return launch_wide_attn_ks<8, true>(ctx, a, n_req, q_max, chunks);
+  return launch_wide_attn_ks<8, false>(ctx, a, n_req, q_max, chunks);
+}
+
+bool wide_eligible(const stairs_ctx* ctx, const DevModel& M) { return ctx->use_mk && shape_fits_tc(M.m); }
+
+// One many-row pass over the T rows in tok/pos/req.  Prefill chunks (n_logit_rows 0) end with the last
+// layer's keys and values: nothing reads more of them.
+int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* logits, const wide::WideAttn& at, int n_req, int r_max, int len_max) {
+  const stairs_model& m = M.m;
+  const Layout& L = ctx->lay;
+  char* ws = ctx->ws;
+  const int d = m.d_model, hd = m.head_dim, nq = m.n_heads * hd, nkv = m.n_kv_heads * hd, nqkv = nq + 2 * nkv, F = m.d_ff, half = hd / 2;
+  float* x = reinterpret_cast<float*>(ws + L.x);
+  bf16* h = reinterpret_cast<bf16*>(ws + L.h);
+  bf16* o = reinterpret_cast<bf16*>(ws + L.o);
+  bf16* ff = reinterpret_cast<bf16*>(ws + L.ff);
+  int* kv_row = reinterpret_cast<int*>(ws + L.kv_row);
+  float* cs = reinterpret_cast<float*>(ws + L.wide_rope);
+  float* sn = cs + (size_t)L.max_rows * half;
+  float4* stats = reinterpret_cast<float4*>(ws + L.wide_stats);
+  const bool ln = m.norm == 0;
+  const size_t f_aux = (size_t)F * (m.act == 1 ? 2 : 1), aux_layer = ((size_t)nqkv + f_aux) * 2;
+  CK(launch_chained(ctx->stream, wide::k_wide_embed, dim3(T), 256, (size_t)0, dim3(1, 1, 1), (const bf16*)M.w.tok_emb, (const bf16*)M.w.pos_emb,
+                    (const int*)(ws + L.tok), (const int*)(ws + L.pos), (const int*)(ws + L.req), (const int*)(ws + L.page_table), (int)ctx->cfg.kv_page_tokens,
+                    L.max_pages, (const float*)M.layers[0].norm1_w, x, h, L.max_rows, d, stats, m.pos == 1 ? (const float*)M.rope_inv : (const float*)nullptr,
+                    half, cs, sn, kv_row));
+  ctx->launches++;
+  int stat_tiles = 1;
+  auto job0 = [&](int epi, bool norm) {
+    wide::WideJob j;
+    memset(&j, 0, sizeof j);
+    j.T = T; j.epi = epi;
+    j.norm_in = norm ? 1 : 0; j.norm_kind = m.norm; j.d = d; j.eps = m.norm_eps; j.stats_in = stats; j.stat_tiles_in = stat_tiles;
+    return j;
+  };
+  auto residual = [&](const void* w, const void* in, int K, const void* g) -> int {
+    wide::WideJob j = job0(wide::W_ADD, false);
+    j.N = d; j.ldo = d; j.out_f32 = x; j.out_act = h; j.next_g = (const float*)g; j.stats_out = stats;
+    const int rc = launch_wide_gemm(ctx, j, in, K, WideW{{w}, {d}, 1}, 64, 8);
+    stat_tiles = j.n_tiles;
+    return rc;
+  };
+  int rc = STAIRS_OK;
+  for (int l = 0; l < m.n_layers && !rc; ++l) {
+    const stairs_layer_w& w = M.layers[l];
+    const bool last_kv = n_logit_rows == 0 && l == m.n_layers - 1;
+    char* kc = M.kpool + (size_t)l * M.kv_layer_bytes;
+    char* vc = M.vpool + (size_t)l * M.kv_layer_bytes;
+    {
+      wide::WideJob j = job0(wide::W_QKV, true);
+      j.hd = hd; j.rope = m.pos; j.qscale = 1.4426950408889634f / sqrtf((float)hd);   // log2(e) / sqrt(hd): base-2 softmax
+      j.rope_cs = cs; j.rope_sn = sn; j.kv_row = kv_row;
+      j.q16 = reinterpret_cast<__half*>(ws + L.q); j.kc = reinterpret_cast<__half*>(kc); j.vc = reinterpret_cast<__half*>(vc);
+      if (ln) { j.u = M.ln_aux + (size_t)l * aux_layer; j.c = j.u + nqkv; }
+      j.src0 = last_kv ? 1 : 0;
+      const WideW all{{w.wq, w.wk, w.wv}, {nq, nkv, nkv}, 3}, kv{{w.wk, w.wv}, {nkv, nkv}, 2};
+      const int off[4] = {0, nq, nq + nkv, 0};
+      for (int s = 0; s < 3; ++s) j.u_off[s] = off[s + j.src0];
+      rc = launch_wide_gemm(ctx, j, h, d, last_kv ? kv : all, hd, 8);
+    }
+    if (rc || last_kv) break;
+    wide::WideAttn a = at;
+    a.q16 = reinterpret_cast<const __half*>(ws + L.q); a.kc = reinterpret_cast<const __half*>(kc); a.vc = reinterpret_cast<const __half*>(vc);
+    a.o = o; a.lo_row = L.max_rows; a.Hq = m.n_heads; a.Hkv = m.n_kv_heads; a.hd = hd;
+    if ((rc = launch_wide_attn(ctx, a, n_req, r_max * (m.n_heads / m.n_kv_heads), (len_max + wide::WCH - 1) / wide::WCH))) break;
+    if ((rc = residual(w.wo, o, nq, w.norm2_w))) break;
+    {
+      wide::WideJob j = job0(m.act == 1 ? wide::W_SWIGLU : wide::W_GELU, true);
+      j.N = F; j.ldo = F; j.out_act = ff;
+      if (ln) { j.u = M.ln_aux + (size_t)l * aux_layer + 2 * (size_t)nqkv; j.c = j.u + f_aux; }
+      rc = m.act == 1 ? launch_wide_gemm(ctx, j, h, d, WideW{{M.w13_ptr[l]}, {(F + 63) / 64 * 128}, 1}, 128, 4)
+                      : launch_wide_gemm(ctx, j, h, d, WideW{{w.w_gate_or_fc1}, {F}, 1}, 64, 4);
+    }
+    if (!rc) rc = residual(w.w_down_or_fc2, ff, F, l + 1 < m.n_layers ? M.layers[l + 1].norm1_w : M.w.final_norm_w);
+  }
+  if (rc || n_logit_rows == 0) return rc;
+  wide::WideJob j = job0(wide::W_LMHEAD, true);
+  j.N = m.vocab; j.ldo = m.vocab; j.out_f32 = logits; j.keys = reinterpret_cast<unsigned long long*>(ws + L.keys);
+  if (ln) { j.u = M.ln_aux + (size_t)m.n_layers * aux_layer; j.c = j.u + m.vocab; }
+  return launch_wide_gemm(ctx, j, h, d, WideW{{M.w.lm_head}, {m.vocab}, 1}, 32, 1);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -984,25 +1220,30 @@ int check_slot(stairs_ctx* ctx, int req, bool must_be_active) {
 }
 
 int prefill_model(stairs_ctx* ctx, DevModel& M, int slot, int n_ctx) {
-  if (mk_eligible(ctx, M, MK_MAX_ROWS)) {
-    // through the persistent kernel, 64 positions per pass: same arithmetic (hi+lo operands,
-    // fp16 attention tiles) as the validation pass, so cached K/V are as accurate as new ones
-    for (int c0 = 0; c0 < n_ctx; c0 += MK_MAX_ROWS) {
-      MkCall c;
-      c.mode = mk::CALL_PREFILL; c.slot = slot; c.draft_step = c0; c.skip_head = true;
-      int rc = launch_forward_mk(ctx, M, std::min(MK_MAX_ROWS, n_ctx - c0), 0, 0, c);
-      if (rc) return rc;
-    }
-    return STAIRS_OK;
+  // Same arithmetic on both bf16 paths (hi+lo operands, fp16 attention tiles) as in the validation pass, so
+  // cached K/V are as accurate as new ones.  Up to 64 positions: one launch of the persistent kernel.
+  if (n_ctx <= MK_MAX_ROWS && mk_eligible(ctx, M, n_ctx)) {
+    MkCall c;
+    c.mode = mk::CALL_PREFILL; c.slot = slot; c.draft_step = 0; c.skip_head = true;
+    return launch_forward_mk(ctx, M, n_ctx, 0, 0, c);
   }
-  const int chunk = ctx->cfg.prefill_chunk > 0 ? ctx->cfg.prefill_chunk : 256;
+  // longer: chunks of equal length
+  const bool wide = wide_eligible(ctx, M);
+  const int most = prefill_rows(ctx->cfg), n_chunks = (n_ctx + most - 1) / most, chunk = (n_ctx + n_chunks - 1) / n_chunks;
   for (int c0 = 0; c0 < n_ctx; c0 += chunk) {
     const int n = std::min(chunk, n_ctx - c0);
     RowParams p = base_rows(ctx);
     p.mode = ROWS_PREFILL; p.slot = slot; p.first = c0; p.n_rows = n;
     int rc = launch_rows(ctx, p, n);
     if (rc) return rc;
-    rc = forward(ctx, M, n, 0, 0, nullptr);
+    if (wide) {
+      wide::WideAttn a{};
+      a.page_table = reinterpret_cast<const int*>(ctx->ws + ctx->lay.page_table); a.page_tokens = ctx->cfg.kv_page_tokens; a.max_pages = ctx->lay.max_pages;
+      a.slot = slot; a.first = c0; a.rows = n;
+      rc = forward_wide(ctx, M, n, 0, nullptr, a, 1, n, c0 + n);
+    } else {
+      rc = forward(ctx, M, n, 0, 0, nullptr);
+    }
     if (rc) return rc;
   }
   return STAIRS_OK;
@@ -1148,6 +1389,8 @@ int stairs_init(const stairs_config* cfg, const stairs_weights* target, const st
       const bool fits = mk::pick_stages(MK_MAX_ROWS, hdm, 1, 1) >= 3 && worst_chunks * hkvm / 64 <= 2 * std::min(ctx->sm_count, TC_GRID_MAX);
       if (coop && fits && cfg->gemm_impl == 0) {
         e = cudaFuncSetAttribute(mk::k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_gemm<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
         if (e == cudaSuccess) {
           ctx->use_mk = true;
           ctx->target.prog_base = ctx->ws + L.prog_t; ctx->target.prog_slot_bytes = L.prog_slot_t; ctx->target.prog_maps_off = L.prog_maps_off_t;
@@ -1289,7 +1532,16 @@ int stairs_validate(stairs_ctx* ctx, int n_req, const int32_t* req_ids_host, con
   RowParams p = base_rows(ctx);
   p.mode = ROWS_VALIDATE; p.n_req = n_req; p.draft = draft_dev;
   int rc = launch_rows(ctx, p, n_req * (ctx->cfg.k_max + 1));
-  if (!rc) rc = forward(ctx, ctx->target, T, 0, T, logits_dev_or_null);
+  if (!rc && wide_eligible(ctx, ctx->target)) {
+    wide::WideAttn a2{};
+    a2.page_table = reinterpret_cast<const int*>(ws + L.page_table); a2.page_tokens = ctx->cfg.kv_page_tokens; a2.max_pages = L.max_pages;
+    a2.val_req = p.val_req; a2.val_k = p.val_k; a2.val_off = p.val_off; a2.n_seq = p.n_seq;
+    int r_max = 0, len_max = 0;
+    for (int i = 0; i < n_req; ++i) { r_max = std::max(r_max, k_host[i] + 1); len_max = std::max(len_max, ctx->n_seq_ub[req_ids_host[i]] + k_host[i]); }
+    rc = forward_wide(ctx, ctx->target, T, T, logits_dev_or_null, a2, n_req, r_max, len_max);
+  } else if (!rc) {
+    rc = forward(ctx, ctx->target, T, 0, T, logits_dev_or_null);
+  }
   ctx->in_validate = false;
   if (rc) return rc;
   AcceptParams a{};
@@ -1545,6 +1797,14 @@ int stairs_debug_tune(stairs_ctx* ctx, int what, long long value) {
       break;
     case 2: ctx->att_tma_off = value ? 1 : 0; break;
     case 3: ctx->att_tc_off = value == 1 ? 1 : 0; ctx->att_tc_force = value == 2 ? 1 : 0; break;
+    case 4:
+      if (value < 0 || value > 2) return fail(ctx, STAIRS_EINVAL, "CTAs per tile must be 0 (planned), 1 or 2");
+      ctx->wide_cg_force = (int)value;
+      return STAIRS_OK;
+    case 5:
+      if (value != 0 && value != 1 && value != 2 && value != 4 && value != 8) return fail(ctx, STAIRS_EINVAL, "K ranges must be 0 (planned), 1, 2, 4 or 8");
+      ctx->wide_split_force = (int)value;
+      return STAIRS_OK;
     default: return fail(ctx, STAIRS_EINVAL, "unknown tuning knob %d", what);
   }
   // programs carry the tensor maps' box depth, which follows from the shared-memory plan

@@ -1,0 +1,78 @@
+"""Passes over many rows (prefill of more than 64 positions, validate calls of more than 64 rows): logits
+against the oracle within the bf16 bar, at the edges of the row tiles, for both tile forms (one CTA, CTA
+pair), whole and split K ranges, all attention forms and head sizes."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import stairs_oracle as so
+from paper_2407_19947_b200 import workloads as wl
+from tests import gpu_util as gu
+from tests.test_gpu_parity import _stairs, small_a, small_b, sources
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = {"gqa_hd64": small_b(8, 2, 64), "mha_hd80": small_b(4, 4, 80, d=320, f=640), "mqa_hd128": small_b(4, 1, 128, d=512, f=832),
+          "hd96": small_b(4, 2, 96, d=384, f=448), "family_a": small_a()}
+
+
+@pytest.mark.parametrize("cg,split", [(1, 1), (1, 4), (2, 0), (0, 0)], ids=["cta", "cta_split4", "pair", "planned"])
+@pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES.keys())
+def test_long_prefill_matches_oracle(shape, cg, split):
+    st = _stairs()
+    tsrc, _ = sources(shape)
+    tgt, _ = gu.oracle_pair(tsrc)
+    eng = st.Stairs(tsrc, None, max_requests=1, max_seq_len=400, k_max=2, kv_page_tokens=16)
+    eng.debug_tune(4, cg)
+    eng.debug_tune(5, split)
+    for n in (66, 129, 258, 333):        # 65 positions, one whole row tile, one whole pair of tiles + 1, ragged
+        prompt = list(wl.zipf_tokens(n, shape.vocab, n))
+        eng.prefill(0, prompt)
+        tt, al, logits = eng.validate([0], [0], None, want_logits=True)
+        eng.sync()
+        ref = np.stack([so.forward_logits(tgt, prompt)])
+        gu.check_rows_against_oracle(logits.cpu().numpy(), tt.cpu().numpy()[0], ref, gu.LOGIT_TOL_BF16)
+    eng.close()
+
+
+@pytest.mark.parametrize("k", [4, 17, 40])
+@pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES.keys())
+def test_calls_of_more_than_64_rows_match_oracle(shape, k):
+    # 75, 90 and 123 rows; 5 to 164 queries per kv head: every way the attention splits its warps, and
+    # contexts short and long enough to be cut over several CTAs
+    st = _stairs()
+    tsrc, _ = sources(shape)
+    tgt, _ = gu.oracle_pair(tsrc)
+    n_req = {4: 15, 17: 5, 40: 3}[k]
+    lens = [300 - 19 * i if i < 5 else 3 + 4 * i for i in range(n_req)]
+    eng = st.Stairs(tsrc, None, max_requests=n_req, max_seq_len=400, k_max=k, kv_page_tokens=32)
+    prompts = [list(wl.zipf_tokens(n, shape.vocab, 60 + i)) for i, n in enumerate(lens)]
+    for i, p in enumerate(prompts):
+        eng.prefill(i, p)
+    drafts = np.random.default_rng(k).integers(0, shape.vocab, size=(n_req, k)).astype(np.int32)
+    ks = [k] * n_req
+    tt, al, logits = eng.validate(list(range(n_req)), ks, torch.from_numpy(drafts).cuda(), want_logits=True)
+    eng.sync()
+    logits, tt, al = logits.cpu().numpy(), tt.cpu().numpy(), al.cpu().numpy()
+    for i in range(n_req):
+        assert int(al[i]) == gu.first_mismatch(drafts[i], tt[i])
+        if i in (0, n_req - 1):
+            ref, _ = gu.oracle_stair_logits(tgt, prompts[i], drafts[i])
+            gu.check_rows_against_oracle(logits[i * (k + 1):(i + 1) * (k + 1)], tt[i], ref, gu.LOGIT_TOL_BF16)
+    eng.close()
+
+
+def test_prefill_in_several_chunks_matches_one_chunk():
+    st = _stairs()
+    shape = small_b(8, 2, 64)
+    tsrc, _ = sources(shape)
+    prompt = list(wl.zipf_tokens(331, shape.vocab, 9))
+    got = []
+    for chunk in (0, 100):
+        eng = st.Stairs(tsrc, None, max_requests=1, max_seq_len=400, k_max=2, kv_page_tokens=64, prefill_chunk=chunk)
+        eng.prefill(0, prompt)
+        _, _, lg = eng.validate([0], [0], None, want_logits=True)
+        eng.sync()
+        got.append(lg.cpu())
+        eng.close()
+    assert float((got[0] - got[1]).abs().max()) < 5e-3
