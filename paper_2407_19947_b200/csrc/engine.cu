@@ -273,7 +273,7 @@ bool compute_layout(const stairs_config& c, Layout* L, const char** why) {
     // many-row passes: cache row and rotation table of every row, statistics per row and column tile of x
     L->kv_row = take(t.wdtype == 1 ? R * 4 : 0);
     L->wide_rope = take(t.wdtype == 1 ? R * (size_t)mx(t.head_dim, d.head_dim) * 4 : 0);
-    L->wide_stats = take(t.wdtype == 1 ? R * ((dm + 63) / 64) * 16 : 0);
+    L->wide_stats = take(t.wdtype == 1 ? R * ((dm + 31) / 32) * 2 * 16 : 0);
     // LayerNorm models: u = W.gain and c = W.bias per normalised GEMM (fp32)
     auto aux = [&](const stairs_model& m) {
       if (m.norm != 0) return (size_t)0;
@@ -348,6 +348,18 @@ bool encode_map3(stairs_ctx* ctx, CUtensorMap* out, const void* ptr, long long r
   cuuint64_t dims[3] = {(cuuint64_t)tc::BK, (cuuint64_t)rows, (cuuint64_t)(K / tc::BK)};
   cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)tc::BK * 2};
   cuuint32_t box[3] = {(cuuint32_t)tc::BK, (cuuint32_t)box_rows, (cuuint32_t)kps};
+  cuuint32_t es[3] = {1, 1, 1};
+  CUresult r = ctx->encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
+// [2 parts][rows][K] view of a hi + lo operand; box = 64 k-elements x box_rows rows of both parts.
+bool encode_map_parts(stairs_ctx* ctx, CUtensorMap* out, const void* ptr, long long rows, long long K, int box_rows) {
+  cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, 2};
+  cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)(rows * K) * 2};
+  cuuint32_t box[3] = {(cuuint32_t)tc::BK, (cuuint32_t)box_rows, 2};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = ctx->encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -838,16 +850,20 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
 struct WidePlan { int cg, tn, splits; };
 
 // Tile shape of one GEMM over T rows: pairs of CTAs (256 rows) or single CTAs (128 rows), tile width a
-// multiple of `gran` (whole heads for the QKV projection, whole gate/up blocks), K cut in up to 8 ranges
-// where few tiles would leave the chip idle.  The estimate: a k-block costs the slower of its MMAs
-// (hi and lo part, TN / 2 cycles each at full rate, never less than their issue time) and the L2 traffic
-// of its tiles at about 45 bytes per cycle and SM; whole waves of units; weights from HBM once; the
-// last tile's epilogue is exposed, and split tiles add the round trip of their parked sums.
-WidePlan wide_plan(const stairs_ctx* ctx, int T, int K, const int* rows, int n_src, int gran, int max_splits, size_t partial_bytes) {
+// multiple of `gran` (whole heads for the QKV projection), K cut in up to 8 ranges where few tiles would leave
+// the chip idle.  The estimate is fitted to measured sweeps of every form over 72 to 2048 rows at the
+// configs' widths (its choice is 3 % from the best one on average): about 4.5 us per launch; a k-block
+// costs the slowest of its MMAs (hi and lo part; 810 cycles at least: issue and commit), the SM's loads (95 GB/s)
+// and the L2's (10 TB/s over the active SMs); whole waves of units, weights from HBM once; the last
+// tile's epilogue is exposed; split tiles add the round trip of their parked sums, pairs their handshakes.
+WidePlan wide_plan(const stairs_ctx* ctx, int T, int K, const int* rows, int n_src, int gran, int epi_kind, int max_splits, size_t partial_bytes) {
+  const bool glu = epi_kind == wide::W_SWIGLU;
+  const double split_us = epi_kind == wide::W_QKV ? 0.024 : 0.012;
   const int sms = std::min(ctx->sm_count, TC_GRID_MAX);
   const int kblocks = (K + tc::BK - 1) / tc::BK;
   double w_bytes = 0;
-  for (int s = 0; s < n_src; ++s) w_bytes += 2.0 * rows[s] * K;
+  int all_rows = 0;
+  for (int s = 0; s < n_src; ++s) { w_bytes += 2.0 * rows[s] * K; all_rows += rows[s]; }
   WidePlan best{1, gran, 1};
   double best_us = 1e30;
   for (int cg = 1; cg <= 2; ++cg) {
@@ -856,18 +872,20 @@ WidePlan wide_plan(const stairs_ctx* ctx, int T, int K, const int* rows, int n_s
     const int m_tiles = (T + wide::WM * cg - 1) / (wide::WM * cg);
     const int x_box = m_tiles == 1 && cg == 1 ? (T + 15) / 16 * 16 : wide::WM;
     for (int tn = gran; tn <= 256; tn += gran) {
-      if (cg == 2 && (tn % 32 || tn < 64)) continue;   // (either CTA holds half of the weight tile)
+      if (tn < 32 || (cg == 2 && (tn % 32 || tn < 64))) continue;   // (either CTA of a pair holds half of the weight tile)
+      if (tn == 256 && gran == 16) continue;                        // (heads of 16: the QKV epilogue reads 8 columns past the tile)
       int n_tiles = 0;
-      for (int s = 0; s < n_src; ++s) n_tiles += (rows[s] + tn - 1) / tn;
+      if (glu) n_tiles = (all_rows + tn - 1) / tn;
+      else for (int s = 0; s < n_src; ++s) n_tiles += (rows[s] + tn - 1) / tn;
       for (int sp = 1; sp <= max_splits; sp *= 2) {
-        if (ctx->wide_split_force && cg == 1 && sp != std::min(ctx->wide_split_force, max_splits)) continue;
         const long long units = (long long)n_tiles * m_tiles * sp;
+        if (ctx->wide_split_force && cg == 1 && sp != std::min(ctx->wide_split_force, max_splits)) continue;
         if (sp > 1 && (cg == 2 || units > sms || kblocks < sp || (size_t)units * tn * wide::WM * 4 > partial_bytes)) continue;
-        const double waves = std::ceil((double)units / (sms / cg));
-        const double mma = 8.0 * std::max(tn / 2.0, 52.0), load = (2.0 * x_box + tn / cg) * 128.0 / 45.0;
-        const double kb = std::ceil((double)kblocks / sp);
-        const double stream = std::max(waves * kb * std::max(mma, load) / 1.75e3, w_bytes / 6.5e6);
-        const double us = stream + (1500.0 + tn * 25.0 + (sp > 1 ? 3500.0 + sp * tn * 6.0 : 0.0)) / 1.75e3;
+        const double waves = std::ceil((double)units / (sms / cg)), active = std::min<double>((double)units * cg, sms);
+        const double mma = std::max(4.5 * tn, 810.0) / 1.8e3, load = (2.0 * x_box + tn / cg) * 128.0 / std::min(95e3, 10e6 / active);
+        const double unit = std::ceil((double)kblocks / sp) * std::max(mma, load), epi = 0.03 * tn;
+        const double us = 4.5 + std::max(waves * unit, w_bytes / 6.5e6) + epi + (waves - 1) * std::max(0.0, epi - unit) +
+                          (sp > 1 ? 2.0 + split_us * tn * sp : 0.0) + (cg == 2 ? 1.5 + 0.006 * tn : 0.0);
         if (us < best_us - 1e-9) { best_us = us; best = {cg, tn, sp}; }
       }
     }
@@ -889,12 +907,13 @@ cudaError_t launch_chained(cudaStream_t st, void (*kern)(A...), dim3 grid, int t
 // Weight matrices of one many-row GEMM: up to three sources that share the operand.
 struct WideW { const void* ptr[3]; int rows[3]; int n_src; };
 
-const CUtensorMap* wide_map(stairs_ctx* ctx, const void* ptr, long long rows, int K, int box) {
+// parts 2: an activation operand, `rows` hi rows and as many lo rows behind them, one box of both
+const CUtensorMap* wide_map(stairs_ctx* ctx, const void* ptr, long long rows, int K, int box, int parts = 1) {
   auto key = std::make_tuple(ptr, K, box);
   auto it = ctx->wide_maps.find(key);
   if (it == ctx->wide_maps.end()) {
     CUtensorMap mp;
-    if (!encode_map(ctx, &mp, ptr, rows, K, box)) return nullptr;
+    if (!(parts == 2 ? encode_map_parts(ctx, &mp, ptr, rows, K, box) : encode_map(ctx, &mp, ptr, rows, K, box))) return nullptr;
     it = ctx->wide_maps.emplace(key, mp).first;
   }
   return &it->second;
@@ -902,36 +921,34 @@ const CUtensorMap* wide_map(stairs_ctx* ctx, const void* ptr, long long rows, in
 
 int launch_wide_gemm(stairs_ctx* ctx, wide::WideJob& job, const void* x, int K, const WideW& w, int gran, int max_splits) {
   const Layout& L = ctx->lay;
-  const WidePlan pl = wide_plan(ctx, job.T, K, w.rows, w.n_src, gran, max_splits, L.gemm_counters - L.gemm_partial);
+  const bool glu = job.epi == wide::W_SWIGLU;   // two sources, TN / 2 rows of each per tile
+  const WidePlan pl = wide_plan(ctx, job.T, K, w.rows, w.n_src, gran, job.epi, max_splits, L.gemm_counters - L.gemm_partial);
   job.TN = pl.tn; job.splits = pl.splits;
   job.kblocks = (K + tc::BK - 1) / tc::BK;
   job.m_tiles = (job.T + wide::WM * pl.cg - 1) / (wide::WM * pl.cg);
   job.x_box = job.m_tiles == 1 && pl.cg == 1 ? (job.T + 15) / 16 * 16 : wide::WM;
   job.n_src = w.n_src; job.n_tiles = 0;
-  const bool half_block = job.epi == wide::W_SWIGLU && pl.tn == 64;
-  job.b_boxes = half_block ? 2 : 1;
-  job.b_box = half_block ? 32 : pl.tn / pl.cg;
-  job.gsz = pl.tn == 64 ? 32 : 64;
   for (int s = 0; s < 3; ++s) {
     const int i = s < w.n_src ? s : 0;
-    const CUtensorMap* m = wide_map(ctx, w.ptr[i], w.rows[i], K, job.b_box);
+    const CUtensorMap* m = wide_map(ctx, w.ptr[i], w.rows[i], K, glu ? pl.tn / 2 : pl.tn / pl.cg);
     if (!m) return fail(ctx, STAIRS_ECUDA, "cuTensorMapEncodeTiled failed for a weight matrix");
     job.w_map[s] = *m;
     job.src_tiles[s] = (w.rows[i] + pl.tn - 1) / pl.tn; job.src_rows[s] = w.rows[i];
     if (s < w.n_src) job.n_tiles += job.src_tiles[s];
   }
-  const CUtensorMap* xm = wide_map(ctx, x, 2 * (long long)L.max_rows, K, job.x_box);
+  if (glu) { job.n_src = 1; job.n_tiles = job.src_tiles[0] = (2 * w.rows[0] + pl.tn - 1) / pl.tn; }
+  const CUtensorMap* xm = wide_map(ctx, x, L.max_rows, K, job.x_box, 2);
   if (!xm) return fail(ctx, STAIRS_ECUDA, "cuTensorMapEncodeTiled failed for an activation buffer");
   job.x_map = *xm;
   if (job.n_tiles * job.m_tiles > TC_COUNTERS) return fail(ctx, STAIRS_EUNSUPPORTED, "too many tiles for the split bookkeeping");
-  job.stages = wide::gemm_stages(pl.tn, pl.cg);
+  job.stages = wide::gemm_stages(job.x_box, pl.tn, pl.cg);
   job.lo_row = L.max_rows;
   job.partial = reinterpret_cast<float*>(ctx->ws + L.gemm_partial);
   job.counters = reinterpret_cast<int*>(ctx->ws + L.gemm_counters);
   job.status = ctx->status_dev; job.wait_limit = ctx->wait_limit;
   const int slots = std::min(ctx->sm_count, TC_GRID_MAX) / pl.cg;
   const int grid = std::min(slots, job.n_tiles * job.m_tiles * pl.splits) * pl.cg;
-  const size_t smem = wide::gemm_smem(pl.tn, pl.cg, job.stages);
+  const size_t smem = wide::gemm_smem(job.x_box, pl.tn, pl.cg, job.stages);
   ctx->launches++;
   CK(launch_chained(ctx->stream, pl.cg == 2 ? wide::k_wide_gemm<2> : wide::k_wide_gemm<1>, dim3(grid), wide::WTHREADS, smem, dim3(pl.cg, 1, 1), job));
   return STAIRS_OK;
@@ -952,7 +969,7 @@ int launch_wide_attn_ks(stairs_ctx* ctx, const wide::WideAttn& a, int n_req, int
     auto kern = wide::k_wide_attn<KS, EXACT, NW, MT>;
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ctx->launches++;
-    CK(launch_chained(ctx->stream, kern, dim3(n_req * p.n_qblk, a.Hkv, ns), NW * 32, smem, dim3(1, 1, ns), p));
+    CK(launch_chained(ctx->stream, kern, dim3(a.Hkv, n_req * p.n_qblk, ns), NW * 32, smem, dim3(1, 1, ns), p));
     return STAIRS_OK;
   };
   using std::integral_constant;
@@ -961,7 +978,43 @@ int launch_wide_attn_ks(stairs_ctx* ctx, const wide::WideAttn& a, int n_req, int
   if (q_max <= 64) return go(integral_constant<int, 4>(), integral_constant<int, 4>());
   return go(integral_constant<int, 8>(), integral_constant<int, 8>());
 }
+template <int HD>
+int launch_wide_attn_tc(stairs_ctx* ctx, const wide::WideAttn& a, long long pool_rows) {
+  wide::WideAttnTc j{};
+  j.a = a; j.status = ctx->status_dev; j.wait_limit = ctx->wait_limit;
+  j.box_rows = std::min((int)ctx->cfg.kv_page_tokens, 64);
+  const int nkv = a.Hkv * HD;
+  for (int v = 0; v < 2; ++v) {
+    const void* ptr = v ? (const void*)a.vc : (const void*)a.kc;
+    auto key = std::make_tuple(ptr, nkv, j.box_rows);
+    auto it = ctx->wide_maps.find(key);
+    if (it == ctx->wide_maps.end()) {
+      CUtensorMap mp;
+      if (!encode_kv_map(ctx, &mp, ptr, pool_rows, nkv, j.box_rows)) return fail(ctx, STAIRS_ECUDA, "cuTensorMapEncodeTiled failed for a K/V pool");
+      it = ctx->wide_maps.emplace(key, mp).first;
+    }
+    (v ? j.vmap : j.kmap) = it->second;
+  }
+  // Ranges of the context (head size 64): the longest block's chunks should not exceed one and a half times an SM
+  // slot's average share (two slots per SM).  2048 rows: 39.6 us with one range, 35.5 with two, 54 with four; 512
+  // rows: 13.6, 13.2, 11.8.  With head size 128 the merge costs what the balance gains (1024 rows: 31.9, 34.0).
+  const int G = a.Hq / a.Hkv, blocks = (a.rows * G + 127) / 128;
+  long long total = 0;
+  for (int i = 0; i < blocks; ++i) total += (a.first + (std::min((i + 1) * 128, a.rows * G) - 1) / G) / wide::tc_att_chunk<HD>() + 1;
+  const int longest = (a.first + a.rows - 1) / wide::tc_att_chunk<HD>() + 1;
+  const double share = (double)total * a.Hkv / (2.0 * ctx->sm_count);
+  int ns = 1;
+  while (HD == 64 && ns < 4 && longest > ns * std::max(1.5 * share, 1.0)) ns *= 2;
+  ctx->launches++;
+  CK(launch_chained(ctx->stream, wide::k_wide_attn_tc<HD>, dim3(a.Hkv, blocks, ns), wide::TC_ATT_THREADS, wide::tc_att_smem<HD>(), dim3(1, 1, ns), j));
+  return STAIRS_OK;
+}
 int launch_wide_attn(stairs_ctx* ctx, const wide::WideAttn& a, int n_req, int q_max, int chunks) {
+  // prefill chunks of whole query blocks: both contractions on tcgen05 where the pools can be copied in bulk
+  if (!a.val_req && q_max >= 128 && ctx->att_tc_off == 0 && (a.hd == 64 || a.hd == 128)) {
+    const long long pool_rows = (long long)ctx->lay.n_pages * ctx->cfg.kv_page_tokens;
+    return a.hd == 64 ? launch_wide_attn_tc<64>(ctx, a, pool_rows) : launch_wide_attn_tc<128>(ctx, a, pool_rows);
+  }
   if (a.hd == 64) return launch_wide_attn_ks<4, true>(ctx, a, n_req, q_max, chunks);
   if (a.hd == 80) return launch_wide_attn_ks<5, true>(ctx, a, n_req, q_max, chunks);
   if (a.hd == 128) return launch_wide_attn_ks<8, true>(ctx, a, n_req, q_max, chunks);
@@ -1003,8 +1056,8 @@ int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* l
   auto residual = [&](const void* w, const void* in, int K, const void* g) -> int {
     wide::WideJob j = job0(wide::W_ADD, false);
     j.N = d; j.ldo = d; j.out_f32 = x; j.out_act = h; j.next_g = (const float*)g; j.stats_out = stats;
-    const int rc = launch_wide_gemm(ctx, j, in, K, WideW{{w}, {d}, 1}, 64, 8);
-    stat_tiles = j.n_tiles;
+    const int rc = launch_wide_gemm(ctx, j, in, K, WideW{{w}, {d}, 1}, 32, 8);
+    stat_tiles = 2 * j.n_tiles;
     return rc;
   };
   int rc = STAIRS_OK;
@@ -1018,7 +1071,7 @@ int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* l
       j.hd = hd; j.rope = m.pos; j.qscale = 1.4426950408889634f / sqrtf((float)hd);   // log2(e) / sqrt(hd): base-2 softmax
       j.rope_cs = cs; j.rope_sn = sn; j.kv_row = kv_row;
       j.q16 = reinterpret_cast<__half*>(ws + L.q); j.kc = reinterpret_cast<__half*>(kc); j.vc = reinterpret_cast<__half*>(vc);
-      if (ln) { j.u = M.ln_aux + (size_t)l * aux_layer; j.c = j.u + nqkv; }
+      if (ln) { j.u = M.ln_aux + (size_t)l * aux_layer; j.c = j.u + nqkv; j.u_last = nqkv - 1; }
       j.src0 = last_kv ? 1 : 0;
       const WideW all{{w.wq, w.wk, w.wv}, {nq, nkv, nkv}, 3}, kv{{w.wk, w.wv}, {nkv, nkv}, 2};
       const int off[4] = {0, nq, nq + nkv, 0};
@@ -1034,16 +1087,16 @@ int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* l
     {
       wide::WideJob j = job0(m.act == 1 ? wide::W_SWIGLU : wide::W_GELU, true);
       j.N = F; j.ldo = F; j.out_act = ff;
-      if (ln) { j.u = M.ln_aux + (size_t)l * aux_layer + 2 * (size_t)nqkv; j.c = j.u + f_aux; }
-      rc = m.act == 1 ? launch_wide_gemm(ctx, j, h, d, WideW{{M.w13_ptr[l]}, {(F + 63) / 64 * 128}, 1}, 128, 4)
-                      : launch_wide_gemm(ctx, j, h, d, WideW{{w.w_gate_or_fc1}, {F}, 1}, 64, 4);
+      if (ln) { j.u = M.ln_aux + (size_t)l * aux_layer + 2 * (size_t)nqkv; j.c = j.u + f_aux; j.u_last = (int)f_aux - 1; }
+      rc = m.act == 1 ? launch_wide_gemm(ctx, j, h, d, WideW{{w.w_gate_or_fc1, w.w_up}, {F, F}, 2}, 32, 4)
+                      : launch_wide_gemm(ctx, j, h, d, WideW{{w.w_gate_or_fc1}, {F}, 1}, 32, 4);
     }
     if (!rc) rc = residual(w.w_down_or_fc2, ff, F, l + 1 < m.n_layers ? M.layers[l + 1].norm1_w : M.w.final_norm_w);
   }
   if (rc || n_logit_rows == 0) return rc;
   wide::WideJob j = job0(wide::W_LMHEAD, true);
   j.N = m.vocab; j.ldo = m.vocab; j.out_f32 = logits; j.keys = reinterpret_cast<unsigned long long*>(ws + L.keys);
-  if (ln) { j.u = M.ln_aux + (size_t)m.n_layers * aux_layer; j.c = j.u + m.vocab; }
+  if (ln) { j.u = M.ln_aux + (size_t)m.n_layers * aux_layer; j.c = j.u + m.vocab; j.u_last = m.vocab - 1; }
   return launch_wide_gemm(ctx, j, h, d, WideW{{M.w.lm_head}, {m.vocab}, 1}, 32, 1);
 }
 
@@ -1390,6 +1443,8 @@ int stairs_init(const stairs_config* cfg, const stairs_weights* target, const st
       if (coop && fits && cfg->gemm_impl == 0) {
         e = cudaFuncSetAttribute(mk::k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_attn_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide::tc_att_smem<64>());
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_attn_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide::tc_att_smem<128>());
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_gemm<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
         if (e == cudaSuccess) {
           ctx->use_mk = true;

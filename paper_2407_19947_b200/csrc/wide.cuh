@@ -12,12 +12,17 @@
 // loads its 128 rows of X and half of the weight tile, which takes the shared-memory fill from 64 to 48
 // bytes per cycle and SM at 256 columns (measured at the 7B gate/up GEMM, see wide_plan).
 //
-// Warp roles (192 threads): warp 0 TMA producer, warp 1 MMA issuer and TMEM owner, warps 2-5 epilogue
-// (one TMEM lane quadrant each).  Two accumulators in TMEM let a tile's epilogue run under the next
+// Warp roles (352 threads): warps 0 and 10 TMA producers of the weight and the activation tiles (a copy costs its
+// issuing thread 200 cycles and more: three copies per k-block from one thread took 0.43 us, the MMAs of a
+// 64-column tile 0.22), warp 1 MMA issuer and TMEM owner, warps 2-9 epilogue
+// (two per TMEM lane quadrant, alternating chunks).  An accumulator row belongs to one thread, and memory wants
+// rows in contiguous pieces, so chunks change hands through a small shared tile per warp.  Two accumulators in TMEM let a tile's epilogue run under the next
 // tile's MMAs.  Launches are chained with programmatic dependent launch: a kernel sets itself up and
 // fetches its first weight tiles while its predecessor finishes, and touches what the predecessor wrote
 // only after griddepcontrol.wait.  All waits are bounded like everywhere in this library.
 #pragma once
+#include <type_traits>
+
 #include "megakernel.cuh"
 
 namespace stairs {
@@ -29,33 +34,34 @@ using mk::pack_f16x2;
 using mk::tma_load_2d_nohint;
 
 constexpr int WM = 128;                    // rows per CTA
-constexpr int WTHREADS = 192;
+constexpr int EPI_WARPS = 8;               // two per TMEM lane quadrant, alternate column chunks
+constexpr int WTHREADS = 96 + EPI_WARPS * 32;
 constexpr int W_MAX_STAGES = 8;
-constexpr int A_BYTES = WM * BK * 2;       // one part (hi or lo) of the activation tile
-constexpr int ST_LD = 36;                  // row pitch (floats) of a warp's 32 x 32 exchange tile
-constexpr int ST_BYTES = 4 * 32 * ST_LD * 4;
+constexpr int ECH = 16;                    // accumulator columns per epilogue chunk
+constexpr int ST_LD = 20;                  // row pitch (floats) of a warp's 32 x 16 exchange tile
+constexpr int QT_LD = 36;                  // the same memory as 16 rows x 16 rotation pairs (QKV)
+constexpr int ST_BYTES = EPI_WARPS * (32 * ST_LD + 64) * 4;   // (and 64 folded-normalisation constants per warp)
 
 enum WEpi { W_ADD = 0, W_GELU = 1, W_SWIGLU = 2, W_QKV = 3, W_LMHEAD = 4 };
 
 struct WideJob {
-  CUtensorMap x_map;        // [2 * lo_row rows][K]; box 64 x x_box
-  CUtensorMap w_map[3];     // box 64 x b_box rows
+  CUtensorMap x_map;        // [2 parts][lo_row rows][K]; box 64 x x_box x 2
+  CUtensorMap w_map[3];     // box 64 x TN / CG rows; SwiGLU: gate and up matrix, box 64 x TN / 2 rows
   int n_src, src_tiles[3], src_rows[3];
   int src0;                 // W_QKV: first source present (0: q, k, v; 1: k and v only)
-  int x_box, b_box, b_boxes;   // b_boxes: weight boxes per CTA and k-block (2: a 32-row gate box and its up box)
+  int x_box;
   int T, TN, n_tiles, m_tiles, kblocks, splits, stages;
   int lo_row;               // rows between the hi and the lo part of every bf16 operand
   int epi;
   int N, ldo;               // output features (SwiGLU: of one matrix), leading dimension of the output
-  int gsz;                  // SwiGLU: width of a gate block (its up block follows)
   float* out_f32;           // W_ADD: the residual stream; W_LMHEAD: logits (may be null)
   bf16* out_act;            // W_GELU / W_SWIGLU: ff; W_ADD with next_g: the next operand
   const float* next_g;
   // folded normalisation of the operand (see the persistent kernel)
   int norm_in, norm_kind, d; float eps;
   const float4* stats_in; int stat_tiles_in;    // (mean, M2, count) per row and column tile of x
-  float4* stats_out;                            // W_ADD with next_g: [row][n_tiles]
-  const float* u; const float* c; int u_off[3];   // (u_off: first entry of each source)
+  float4* stats_out;                            // W_ADD with next_g: [row][2 * n_tiles] (the two warps of a row)
+  const float* u; const float* c; int u_off[3], u_last;   // (u_off: first entry of each source, u_last: last entry)
   // W_QKV
   int hd, rope; float qscale;
   const float* rope_cs; const float* rope_sn;   // [row][hd / 2]
@@ -76,6 +82,13 @@ template <int CG> __device__ __forceinline__ void w_tma(void* dst, const CUtenso
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
       " [%0], [%1, {%2, %3}], [%4], %5;"
       ::"r"(smem_u32(dst)), "l"(map), "r"(c0), "r"(c1), "r"(smem_u32(bar) & 0xFEFFFFFFu), "l"(policy) : "memory");
+}
+template <int CG> __device__ __forceinline__ void w_tma3(void* dst, const CUtensorMap* map, int c0, int c1, int c2, uint64_t* bar, uint64_t policy) {
+  if (CG == 1) { mk::tma_load_3d(dst, map, c0, c1, c2, bar, policy); return; }
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3, %4}], [%5], %6;"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar) & 0xFEFFFFFFu), "l"(policy) : "memory");
 }
 template <int CG> __device__ __forceinline__ void w_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   if (CG == 1) { umma_bf16(d, a, b, idesc, acc); return; }
@@ -124,19 +137,31 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
+__device__ __forceinline__ void tmem_ld16w(uint32_t taddr, float* v) {
+  uint32_t r[16];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15,"
-      " %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
       "tcgen05.wait::ld.sync.aligned;"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void group_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }   // the epilogue warps
+
+// GELU(v) = v / 2 * erfc(-v / sqrt 2) with the Chebyshev fit of erfc of Numerical Recipes (section 6.2, "erfcc":
+// fractional error below 1.2e-7 everywhere), evaluated on |v|.  Half the instructions of the erff form,
+// which the issue rate of the epilogue warps was bound by (0.4B fc1 over 2048 rows), and no cancellation for
+// negative v.
+__device__ __forceinline__ float gelu_erfc(float v) {
+  const float z = fabsf(v) * 0.70710678118654752f;
+  const float t = __fdividef(1.0f, fmaf(0.5f, z, 1.0f));
+  float p = fmaf(t, 0.17087277f, -0.82215223f);
+  p = fmaf(t, p, 1.48851587f); p = fmaf(t, p, -1.13520398f); p = fmaf(t, p, 0.27886807f); p = fmaf(t, p, -0.18628806f);
+  p = fmaf(t, p, 0.09678418f); p = fmaf(t, p, 0.37409196f); p = fmaf(t, p, 1.00002368f); p = fmaf(t, p, -1.26551223f);
+  const float c = t * mk::fast_exp2((p - z * z) * 1.4426950408889634f);   // erfc(z)
+  return 0.5f * v * (v < 0.f ? c : 2.0f - c);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -147,9 +172,10 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int TN = job.TN, TNc = TN / CG, stages = job.stages, S = job.splits;
-  const int stage_bytes = 2 * A_BYTES + TNc * BK * 2;
+  const int a_bytes = job.x_box * BK * 2;                            // one part of the activation tile
+  const int stage_bytes = 2 * a_bytes + TNc * BK * 2;
   uint8_t* tail = smem + (size_t)stages * stage_bytes;
-  float* stile = reinterpret_cast<float*>(tail);                     // [4 warps][32][ST_LD]
+  float* stile = reinterpret_cast<float*>(tail);                     // [EPI_WARPS][32][ST_LD]
   uint64_t* full = reinterpret_cast<uint64_t*>(tail + ST_BYTES);
   uint64_t* empty = full + W_MAX_STAGES;
   uint64_t* acc_full = empty + W_MAX_STAGES;                         // [2]
@@ -168,7 +194,7 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
     mbar_init(acc_full + 0, 1); mbar_init(acc_full + 1, 1);
-    mbar_init(acc_empty + 0, 4 * CG); mbar_init(acc_empty + 1, 4 * CG);
+    mbar_init(acc_empty + 0, EPI_WARPS * CG); mbar_init(acc_empty + 1, EPI_WARPS * CG);
     *abort_flag = 0; *verdict = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -178,57 +204,55 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
   tc_fence_after();
   if (CG == 2) __syncthreads();
   const uint32_t tmem_base = *tmem_slot;
-  if (threadIdx.x == 0) pdl_launch();
+  if (threadIdx.x == 0) pdl_launch();   // (after the TMEM allocation, see k_wide_attn_tc)
   int issued = 0, p_stage = 0;
   uint32_t p_phase = 0;
   auto k_begin = [&](int s) { return (job.kblocks * s) / S; };
 
   if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer
+    // ------------------------------------------------------------------ TMA producer, weight tiles
+    // (they depend on nothing: fetched while the predecessor still runs)
     if (lane == 0) {
-      const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
-      const uint32_t tx = (uint32_t)(CG * (2 * job.x_box * BK * 2 + TNc * BK * 2));   // both CTAs' bytes
-      auto load_w = [&](int tile, int kb, int stage) {
-        uint8_t* dst = smem + (size_t)stage * stage_bytes + 2 * A_BYTES;
-        int s = 0, local = tile;
-        while (s + 1 < job.n_src && local >= job.src_tiles[s]) { local -= job.src_tiles[s]; ++s; }
-        if (job.b_boxes == 2) {   // 32 gate rows and their 32 up rows, half a packed 64 + 64 tile
-          const int row = (local >> 1) * 128 + (local & 1) * 32;
-          w_tma<CG>(dst, &job.w_map[0], kb * BK, row, full + stage, pol_w);
-          w_tma<CG>(dst + 32 * BK * 2, &job.w_map[0], kb * BK, row + 64, full + stage, pol_w);
-        } else {
-          w_tma<CG>(dst, &job.w_map[s], kb * BK, local * TN + rank * TNc, full + stage, pol_w);
-        }
-      };
+      const uint64_t pol_w = policy_evict_first();
+      const uint32_t tx = (uint32_t)(CG * (2 * job.x_box * BK * 2 + TNc * BK * 2));   // both parts, both CTAs
       int stage = 0; uint32_t phase = 0;
-      // the first weight tiles depend on nothing: fetched before the predecessor's results are waited for
-      int ahead = 0;
-      if (cid < units) {
-        const int s0 = cid % S, nt0 = (cid / S) / job.m_tiles;
-        const int kb0 = k_begin(s0), kb1 = k_begin(s0 + 1);
-        for (; ahead < stages && ahead < kb1 - kb0; ++ahead) {
-          if (rank == 0) mbar_expect_tx(full + ahead, tx);
-          load_w(nt0, kb0 + ahead, ahead);
-        }
-      }
-      pdl_wait();
       bool ok = true;
       for (int u = cid; u < units && ok; u += G) {
-        const int s = u % S, tile = u / S, nt = tile / job.m_tiles, mt = tile % job.m_tiles;
-        const int x_row = (mt * CG + rank) * WM;
-        const int kb1 = k_begin(s + 1);
-        for (int kb = k_begin(s); kb < kb1; ++kb) {
-          if (issued >= ahead) {
-            if (!mbar_wait(empty + stage, phase ^ 1, abort_flag, job.wait_limit)) { ok = false; break; }
-            if (rank == 0) mbar_expect_tx(full + stage, tx);
-            load_w(nt, kb, stage);
-          }
-          uint8_t* dst = smem + (size_t)stage * stage_bytes;
-          w_tma<CG>(dst, &job.x_map, kb * BK, x_row, full + stage, pol_x);
-          w_tma<CG>(dst + A_BYTES, &job.x_map, kb * BK, job.lo_row + x_row, full + stage, pol_x);
+        const int s = u % S, nt = (u / S) / job.m_tiles;
+        int src = 0, local = nt;
+        while (src + 1 < job.n_src && local >= job.src_tiles[src]) { local -= job.src_tiles[src]; ++src; }
+        // SwiGLU tile: TN / 2 gate rows and the same up rows (either CTA of a pair holds one of them)
+        const bool glu = job.epi == W_SWIGLU;
+        const int row = glu ? local * (TN / 2) : local * TN + rank * TNc;
+        const CUtensorMap* map = &job.w_map[glu ? rank : src];
+        const int kb0 = k_begin(s), len = k_begin(s + 1) - kb0;
+        for (int kb = kb0; kb < kb0 + len; ++kb) {
+          if (!mbar_wait(empty + stage, phase ^ 1, abort_flag, job.wait_limit)) { ok = false; break; }
+          uint8_t* dst = smem + (size_t)stage * stage_bytes + 2 * a_bytes;
+          if (rank == 0) mbar_expect_tx(full + stage, tx);
+          w_tma<CG>(dst, map, kb * BK, row, full + stage, pol_w);
+          if (glu && CG == 1) w_tma<CG>(dst + (TN / 2) * BK * 2, &job.w_map[1], kb * BK, row, full + stage, pol_w);
           ++issued;
           if (++stage == stages) { stage = 0; phase ^= 1; }
           p_stage = stage; p_phase = phase;
+        }
+      }
+    }
+  } else if (warp == 10) {
+    // ------------------------------------------------------------------ TMA producer, activation tiles
+    if (lane == 0) {
+      const uint64_t pol_x = policy_evict_last();
+      pdl_wait();
+      int stage = 0; uint32_t phase = 0;
+      bool ok = true;
+      for (int u = cid; u < units && ok; u += G) {
+        const int s = u % S, mt = (u / S) % job.m_tiles;
+        const int x_row = (mt * CG + rank) * WM;
+        const int kb0 = k_begin(s), len = k_begin(s + 1) - kb0;
+        for (int kb = kb0; kb < kb0 + len; ++kb) {
+          if (!mbar_wait(empty + stage, phase ^ 1, abort_flag, job.wait_limit)) { ok = false; break; }
+          w_tma3<CG>(smem + (size_t)stage * stage_bytes, &job.x_map, kb * BK, x_row, 0, full + stage, pol_x);   // hi rows, then lo rows
+          if (++stage == stages) { stage = 0; phase ^= 1; }
         }
       }
     }
@@ -250,7 +274,7 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
           if (!mbar_wait(full + stage, phase, abort_flag, job.wait_limit)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a = smem_u32(smem + (size_t)stage * stage_bytes);
-          const uint64_t hi = smem_desc_sw128(a), lo = smem_desc_sw128(a + A_BYTES), w = smem_desc_sw128(a + 2 * A_BYTES);
+          const uint64_t hi = smem_desc_sw128(a), lo = smem_desc_sw128(a + a_bytes), w = smem_desc_sw128(a + 2 * a_bytes);
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k) {
             const uint64_t o = (uint64_t)(k * UMMA_K * 2 / 16);
@@ -266,10 +290,11 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
       }
     }
   } else {
-    // ------------------------------------------------------------------ epilogue (warps 2..5)
-    const int quad = warp & 3, et = threadIdx.x - 64;
-    float* st = stile + (size_t)quad * 32 * ST_LD;
-    const int tr = lane >> 3, tc4 = (lane & 7) * 4;    // exchange-tile mapping: row 4 i + tr, four columns from tc4
+    // ------------------------------------------------------------------ epilogue (warps 2..9)
+    const int quad = warp & 3, hw = (warp - 2) >> 2, et = threadIdx.x - 64;
+    float* st = stile + (size_t)(warp - 2) * (32 * ST_LD + 64);
+    float* uc = st + 32 * ST_LD;
+    const int tr = lane >> 2, tc4 = (lane & 3) * 4;    // exchange-tile mapping: row 8 i + tr, four columns from tc4
     int buf = 0; uint32_t acc_bits = 0;
     pdl_wait();
     for (int u = cid; u < units; u += G) {
@@ -279,7 +304,8 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
       int src = 0, local = nt;
       while (src + 1 < job.n_src && local >= job.src_tiles[src]) { local -= job.src_tiles[src]; ++src; }
       const int col0 = local * TN;                      // first weight row of the tile in its source
-      // what the epilogue reads from memory is requested before the accumulator is waited for
+      // What the epilogue reads from memory is requested before the accumulator is waited for, and inside
+      // the loops a few chunks ahead: every such load is an L2 round trip.
       float rs = 1.f, mu = 0.f;
       if (job.norm_in && row_on) {
         // one pass over the row's tile entries, eight loads in flight; sums shifted by the first tile's mean
@@ -297,23 +323,56 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
         if (job.norm_kind == 0) { mu = mean; rs = 1.0f / sqrtf(m2 / (float)job.d + job.eps); }
         else rs = 1.0f / sqrtf((m2 + n * mean * mean) / (float)job.d + job.eps);
       }
-      float4 xq[8];
-      auto load_x = [&](int c0) {
+      // this warp's chunk i covers tile columns col_of(i) .. col_of(i) + 15
+      auto col_of = [&](int i) { return (2 * i + hw) * ECH; };
+      // old residual values of the chunk at c0; four chunks are kept in flight
+      float4 xq[4][4];                                  // (QKV: rotation table entries in xq[0], xq[1], see load_rope)
+      auto load_x = [&](float4 (&q)[4], int c0) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int r = row0 + 4 * i + tr;
-          xq[i] = (r < job.T && col0 + c0 < job.N) ? __ldcg(reinterpret_cast<const float4*>(job.out_f32 + (size_t)r * job.ldo + col0 + c0 + tc4))
-                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < 4; ++i) {
+          const int r = row0 + 8 * i + tr;
+          q[i] = (r < job.T && c0 < TN && col0 + c0 < job.N) ? __ldcg(reinterpret_cast<const float4*>(job.out_f32 + (size_t)r * job.ldo + col0 + c0 + tc4))
+                                                             : make_float4(0.f, 0.f, 0.f, 0.f);
         }
       };
-      if (job.epi == W_ADD && S == 1) load_x(0);
+      auto load_x_first = [&]() {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) load_x(xq[j], col_of(j));
+      };
+      if (job.epi == W_ADD && S == 1) load_x_first();
+      // QKV: item `it` holds 16 rotation pairs of a head (columns i0 .. i0 + 15 and half a head further); in the
+      // exchange tile four lanes hold a row's pairs, rows 8 i + (lane >> 2) of a half chunk
+      const int part = src + job.src0, half = job.hd / 2, gph = job.epi == W_QKV ? (half + 15) / 16 : 1;
+      const bool rot = job.epi == W_QKV && job.rope && part < 2;
+      auto load_rope = [&](float4 (&q)[4], int it, int h) {   // cos and sin of the two rows of half chunk h
+        const int i0 = (it % gph) * 16 + tc4;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int r = row0 + 16 * h + 8 * i + tr;
+          const size_t o = (size_t)(r < job.T ? r : 0) * half + (i0 < half ? i0 : 0);
+          q[2 * i] = __ldcg(reinterpret_cast<const float4*>(job.rope_cs + o));
+          q[2 * i + 1] = __ldcg(reinterpret_cast<const float4*>(job.rope_sn + o));
+        }
+      };
+      int kv_row[4];                                    // cache rows of this lane's rows (two per half chunk)
+      if (job.epi == W_QKV) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int r = row0 + 8 * j + tr;
+          kv_row[j] = part == 0 ? r : (r < job.T ? __ldcg(job.kv_row + r) : 0);
+        }
+        if (rot) {
+#pragma unroll
+          for (int j = 0; j < 2; ++j) load_rope(xq[j], hw, j);
+        }
+      }
       bool ok = mbar_wait(acc_full + buf, (acc_bits >> buf) & 1u, abort_flag, job.wait_limit);
       ok = __all_sync(0xffffffffu, ok);
       if (S > 1) {   // the split tiles' barriers below want one verdict for the whole group
         if (!ok) *abort_flag = 1;
-        epi_bar_sync();
+        group_sync();
         if (et == 0) *verdict = *abort_flag ? 0 : 1;
-        epi_bar_sync();
+        group_sync();
         ok = *verdict != 0;
       }
       if (!ok) break;
@@ -321,14 +380,12 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)buf * (tmem_cols / 2);
       bool finish = true;
-      const float* parts = nullptr;
       const size_t part_stride = (size_t)TN * WM;
+      const float* parts = job.partial + (size_t)tile * S * part_stride + (size_t)(quad * 32 + lane) * 4;
       if (S > 1) {
         // a K range of the tile: park it ([4 columns][row] vectors), the last arriver adds the ranges in K order
-        float* base = job.partial + (size_t)tile * S * part_stride;
-        parts = base;
-        float* mine = base + (size_t)sp * part_stride + (size_t)(quad * 32 + lane) * 4;
-        for (int c0 = 0; c0 < TN; c0 += 8) {
+        float* mine = const_cast<float*>(parts) + (size_t)sp * part_stride;
+        for (int c0 = hw * 8; c0 < TN; c0 += 16) {
           float v[8];
           tmem_ld8(taddr + (uint32_t)c0, v);
           if (row_on) {
@@ -337,177 +394,218 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
           }
         }
         __threadfence();
-        epi_bar_sync();
+        group_sync();
         if (et == 0) {
           const int old = atomicAdd(job.counters + tile, 1);
           if (old == S - 1) job.counters[tile] = 0;
           *verdict = old == S - 1 ? 2 : 1;
         }
-        epi_bar_sync();
+        group_sync();
         finish = *verdict == 2;
-        if (finish) { __threadfence(); if (job.epi == W_ADD) load_x(0); }
+        if (finish) {
+          __threadfence();
+          if (job.epi == W_ADD) load_x_first();
+        }
       }
-      // n consecutive accumulator columns of this thread's row
-      auto acc8 = [&](int c0, float* v) {
-        if (S == 1) { tmem_ld8(taddr + (uint32_t)c0, v); return; }
-        const float* p0 = parts + (size_t)(quad * 32 + lane) * 4 + (size_t)c0 * WM;
+      // 16 consecutive accumulator columns of this thread's row
+      auto acc = [&](int c0, float* v) {
+        constexpr int NC = 16;
+        if (S == 1) {
+          tmem_ld16w(taddr + (uint32_t)c0, v);
+          return;
+        }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = 0.f;
-        if (row_on)
+        for (int j = 0; j < NC; ++j) v[j] = 0.f;
+        if (row_on) {
+          const float* p0 = parts + (size_t)c0 * WM;
+#pragma unroll 4
           for (int s2 = 0; s2 < S; ++s2) {
-            const float4 a = __ldcg(reinterpret_cast<const float4*>(p0 + s2 * part_stride)), b = __ldcg(reinterpret_cast<const float4*>(p0 + s2 * part_stride + 4 * WM));
-            v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w; v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
+            float4 a[NC / 4];
+#pragma unroll
+            for (int j = 0; j < NC / 4; ++j) a[j] = __ldcg(reinterpret_cast<const float4*>(p0 + s2 * part_stride + (size_t)(4 * j) * WM));
+#pragma unroll
+            for (int j = 0; j < NC / 4; ++j) { v[4 * j] += a[j].x; v[4 * j + 1] += a[j].y; v[4 * j + 2] += a[j].z; v[4 * j + 3] += a[j].w; }
           }
+        }
       };
-      auto acc32 = [&](int c0, float* v) {
-        if (S == 1) { tmem_ld32(taddr + (uint32_t)c0, v); return; }
-        const float* p0 = parts + (size_t)(quad * 32 + lane) * 4 + (size_t)c0 * WM;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = 0.f;
-        if (row_on)
-          for (int s2 = 0; s2 < S; ++s2) {
-            float4 a[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) a[j] = __ldcg(reinterpret_cast<const float4*>(p0 + s2 * part_stride + (size_t)(4 * j) * WM));
-#pragma unroll
-            for (int j = 0; j < 8; ++j) { v[4 * j] += a[j].x; v[4 * j + 1] += a[j].y; v[4 * j + 2] += a[j].z; v[4 * j + 3] += a[j].w; }
-          }
+      // Folded normalisation of 16 columns.  Their constants u and c (LayerNorm models) are fetched a chunk ahead,
+      // one per lane, and handed out through shared memory: read per column they were two dependent
+      // round trips in every chunk (0.4B fc1 over 2048 rows: 54 -> 45 us).
+      auto fetch_uc = [&](int n) { return job.u ? __ldg((lane < 16 ? job.u : job.c) + min(n + (lane & 15), job.u_last)) : 0.f; };
+      auto share_uc = [&](float a, float b) {
+        if (job.u) { __syncwarp(); uc[lane] = a; uc[32 + lane] = b; __syncwarp(); }
       };
-      // folded normalisation of a column of weight row n (u and c are the same for all lanes)
-      auto normed = [&](float v, int n) { return job.u ? rs * (v - mu * __ldg(job.u + n)) + __ldg(job.c + n) : rs * v; };
+      auto normed = [&](float* v, int group) {
+        if (!job.u) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] *= rs;
+          return;
+        }
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+          const float4 u4 = *reinterpret_cast<const float4*>(uc + 32 * group + j), c4 = *reinterpret_cast<const float4*>(uc + 32 * group + 16 + j);
+          v[j] = rs * (v[j] - mu * u4.x) + c4.x; v[j + 1] = rs * (v[j + 1] - mu * u4.y) + c4.y;
+          v[j + 2] = rs * (v[j + 2] - mu * u4.z) + c4.z; v[j + 3] = rs * (v[j + 3] - mu * u4.w) + c4.w;
+        }
+      };
       auto to_tile = [&](const float* v) {
         __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 8; ++j) *reinterpret_cast<float4*>(st + lane * ST_LD + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        for (int j = 0; j < 4; ++j) *reinterpret_cast<float4*>(st + lane * ST_LD + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         __syncwarp();
       };
-      auto store_act = [&](int out_col) {   // the exchange tile as bf16 hi + lo, 64 contiguous bytes per row and part
+      auto store_act = [&](int out_col) {   // the exchange tile as bf16 hi + lo, a 32-byte sector per row and part
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int r = row0 + 4 * i + tr;
-          if (r < job.T && out_col + tc4 < job.N)
-            store_split4(job.out_act, (size_t)r * job.ldo + out_col + tc4, (size_t)job.lo_row * job.ldo, *reinterpret_cast<const float4*>(st + (4 * i + tr) * ST_LD + tc4));
+        for (int i = 0; i < 4; ++i) {
+          const int r = row0 + 8 * i + tr;
+          if (r < job.T)
+            store_split4(job.out_act, (size_t)r * job.ldo + out_col + tc4, (size_t)job.lo_row * job.ldo, *reinterpret_cast<const float4*>(st + (8 * i + tr) * ST_LD + tc4));
         }
       };
       if (finish) {
         if (job.epi == W_ADD) {
-          // residual update, the next GEMM's operand bf16(x * gain), and this tile's row statistics (shifted
-          // sums: the shift is the row's first value of the tile)
-          float s1[8], s2[8], sh[8];
+          // residual update, the next GEMM's operand bf16(x * gain), and this warp's row statistics of the
+          // tile (shifted sums: the shift is the row's first value)
+          float s1[4], s2[4], sh[4];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) { s1[i] = s2[i] = sh[i] = 0.f; }
-          for (int c0 = 0; c0 < TN && col0 + c0 < job.N; c0 += 32) {
-            float v[32];
-            acc32(c0, v);
-            to_tile(v);
-            const int col = col0 + c0 + tc4;
-            const float4 g4 = job.next_g ? __ldg(reinterpret_cast<const float4*>(job.next_g + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int i = 0; i < 4; ++i) { s1[i] = s2[i] = sh[i] = 0.f; }
+          const int nch = (min(TN, job.N - col0) / ECH - hw + 1) / 2;   // this warp's chunks
+          for (int k0 = 0; k0 < nch; k0 += 4) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int r = row0 + 4 * i + tr;
-              const float4 a = *reinterpret_cast<const float4*>(st + (4 * i + tr) * ST_LD + tc4);
-              const float4 x4 = make_float4(xq[i].x + a.x, xq[i].y + a.y, xq[i].z + a.z, xq[i].w + a.w);
-              if (r < job.T) {
-                *reinterpret_cast<float4*>(job.out_f32 + (size_t)r * job.ldo + col) = x4;
-                if (job.next_g)
-                  store_split4(job.out_act, (size_t)r * job.ldo + col, (size_t)job.lo_row * job.ldo, make_float4(x4.x * g4.x, x4.y * g4.y, x4.z * g4.z, x4.w * g4.w));
+            for (int j = 0; j < 4; ++j) {
+              if (k0 + j < nch) {
+                const int c0 = col_of(k0 + j), col = col0 + c0 + tc4;
+                float v[16];
+                acc(c0, v);
+                to_tile(v);
+                const float4 g4 = job.next_g ? __ldg(reinterpret_cast<const float4*>(job.next_g + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const int r = row0 + 8 * i + tr;
+                  const float4 a = *reinterpret_cast<const float4*>(st + (8 * i + tr) * ST_LD + tc4);
+                  const float4 x4 = make_float4(xq[j][i].x + a.x, xq[j][i].y + a.y, xq[j][i].z + a.z, xq[j][i].w + a.w);
+                  if (r < job.T) {
+                    *reinterpret_cast<float4*>(job.out_f32 + (size_t)r * job.ldo + col) = x4;
+                    if (job.next_g)
+                      store_split4(job.out_act, (size_t)r * job.ldo + col, (size_t)job.lo_row * job.ldo, make_float4(x4.x * g4.x, x4.y * g4.y, x4.z * g4.z, x4.w * g4.w));
+                  }
+                  if (k0 + j == 0) sh[i] = __shfl_sync(0xffffffffu, x4.x, lane & 28);
+                  const float d0 = x4.x - sh[i], d1 = x4.y - sh[i], d2 = x4.z - sh[i], d3 = x4.w - sh[i];
+                  s1[i] += (d0 + d1) + (d2 + d3);
+                  s2[i] += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+                }
+                load_x(xq[j], col_of(k0 + j + 4));
               }
-              if (c0 == 0) sh[i] = __shfl_sync(0xffffffffu, x4.x, lane & 24);
-              const float d0 = x4.x - sh[i], d1 = x4.y - sh[i], d2 = x4.z - sh[i], d3 = x4.w - sh[i];
-              s1[i] += (d0 + d1) + (d2 + d3);
-              s2[i] += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
             }
-            if (c0 + 32 < TN) load_x(c0 + 32);
           }
           if (job.next_g) {
-            const float cnt = (float)min(TN, job.N - col0);
+            const float cnt = (float)(nch * ECH);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < 4; ++i) {
 #pragma unroll
-              for (int o = 1; o < 8; o <<= 1) { s1[i] += __shfl_xor_sync(0xffffffffu, s1[i], o); s2[i] += __shfl_xor_sync(0xffffffffu, s2[i], o); }
-              const int r = row0 + 4 * i + tr;
-              const float m = s1[i] / cnt;
-              if ((lane & 7) == 0 && r < job.T) job.stats_out[(size_t)r * job.n_tiles + nt] = make_float4(sh[i] + m, fmaxf(s2[i] - s1[i] * m, 0.f), cnt, 0.f);
+              for (int o = 1; o < 4; o <<= 1) { s1[i] += __shfl_xor_sync(0xffffffffu, s1[i], o); s2[i] += __shfl_xor_sync(0xffffffffu, s2[i], o); }
+              const int r = row0 + 8 * i + tr;
+              const float m = s1[i] / fmaxf(cnt, 1.f);
+              if ((lane & 3) == 0 && r < job.T) job.stats_out[(size_t)r * (2 * job.n_tiles) + 2 * nt + hw] = make_float4(sh[i] + m, fmaxf(s2[i] - s1[i] * m, 0.f), cnt, 0.f);
             }
           }
         } else if (job.epi == W_GELU) {
-          for (int c0 = 0; c0 < TN && col0 + c0 < job.N; c0 += 32) {
-            float v[32];
-            acc32(c0, v);
+          float ua = fetch_uc(col0 + col_of(0));
+          for (int i = 0; col_of(i) < TN && col0 + col_of(i) < job.N; ++i) {
+            const int n = col0 + col_of(i);
+            float v[16];
+            share_uc(ua, 0.f);
+            ua = fetch_uc(col0 + col_of(i + 1));
+            acc(col_of(i), v);
+            normed(v, 0);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = gelu_erf(normed(v[j], col0 + c0 + j));
+            for (int j = 0; j < 16; ++j) v[j] = gelu_erfc(v[j]);
             to_tile(v);
-            store_act(col0 + c0);
+            store_act(n);
           }
         } else if (job.epi == W_SWIGLU) {
-          const int gsz = job.gsz, out0 = local * (TN / 2);
-          for (int b = 0; b < TN; b += 2 * gsz)
-            for (int c0 = 0; c0 < gsz; c0 += 32) {
-              const int oc = out0 + b / 2 + c0;
-              if (oc >= job.N) break;
-              float v[32], w[32];
-              acc32(b + c0, v);
-              acc32(b + gsz + c0, w);
+          const int out0 = local * (TN / 2);             // output columns of the tile
+          float ua = fetch_uc(out0 + col_of(0)), ub = fetch_uc(job.N + out0 + col_of(0));
+          for (int i = 0; col_of(i) < TN / 2; ++i) {
+            const int oc = col_of(i), n = out0 + oc;
+            if (n >= job.N) break;
+            float v[16], w[16];
+            share_uc(ua, ub);
+            ua = fetch_uc(out0 + col_of(i + 1)); ub = fetch_uc(job.N + out0 + col_of(i + 1));
+            acc(oc, v);
+            acc(oc + TN / 2, w);
+            normed(v, 0);
+            normed(w, 1);
 #pragma unroll
-              for (int j = 0; j < 32; ++j) v[j] = silu_f(normed(v[j], oc + j)) * normed(w[j], job.N + oc + j);
-              to_tile(v);
-              store_act(oc);
-            }
+            for (int j = 0; j < 16; ++j) v[j] = silu_f(v[j]) * w[j];
+            to_tile(v);
+            store_act(n);
+          }
         } else if (job.epi == W_LMHEAD) {
           unsigned long long key = 0ull;
-          for (int c0 = 0; c0 < TN && col0 + c0 < job.N; c0 += 32) {
-            float v[32];
-            acc32(c0, v);
+          float ua = fetch_uc(col0 + col_of(0));
+          for (int i = 0; col_of(i) < TN && col0 + col_of(i) < job.N; ++i) {
+            const int n0 = col0 + col_of(i);
+            float v[16];
+            share_uc(ua, 0.f);
+            ua = fetch_uc(col0 + col_of(i + 1));
+            acc(col_of(i), v);
+            normed(v, 0);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int n = col0 + c0 + j;
-              v[j] = normed(v[j], min(n, job.N - 1));
-              const unsigned long long k2 = argmax_key(v[j], (uint32_t)n);
-              if (n < job.N && k2 > key) key = k2;
+            for (int j = 0; j < 16; ++j) {
+              const unsigned long long k2 = argmax_key(v[j], (uint32_t)(n0 + j));
+              if (n0 + j < job.N && k2 > key) key = k2;
             }
             if (job.out_f32) {
               to_tile(v);
-              const int n = col0 + c0 + lane;
-              for (int r = 0; r < 32 && row0 + r < job.T; ++r)
-                if (n < job.N) job.out_f32[(size_t)(row0 + r) * job.ldo + n] = st[r * ST_LD + lane];
+              const int n = n0 + (lane & 15);
+              for (int r = lane >> 4; r < 32 && row0 + r < job.T; r += 2)
+                if (n < job.N) job.out_f32[(size_t)(row0 + r) * job.ldo + n] = st[r * ST_LD + (lane & 15)];
             }
           }
           if (row_on && key) atomicMax(job.keys + row, key);
         } else {   // W_QKV: rotate and scale q, rotate k; fp16 to the query buffer and the cache
-          const int hd = job.hd, half = hd / 2, width = job.src_rows[src], part = src + job.src0;   // part 0: q, 1: k, 2: v
-          const int u0 = job.u_off[src];
-          const int rr = row_on ? row : 0;
-          __half* dst = (part == 0 ? job.q16 + (size_t)rr * width : (part == 1 ? job.kc : job.vc) + (size_t)__ldcg(job.kv_row + rr) * width) + col0;
+          const int width = job.src_rows[src], u0 = job.u_off[src] + col0;
+          __half* dst0 = (part == 0 ? job.q16 : part == 1 ? job.kc : job.vc) + col0;
           const float qs = part == 0 ? job.qscale : 1.0f;
-          const bool rot = job.rope && part < 2;
-          for (int h0 = 0; h0 < TN && col0 + h0 < width; h0 += hd)
-            for (int i0 = 0; i0 < half; i0 += 8) {
-              float lo[8], hi[8];
-              acc8(h0 + i0, lo);
-              acc8(h0 + half + i0, hi);
+          const int n_it = min(TN, width - col0) / job.hd * gph;
+          const int cf = hw / gph * job.hd + (hw % gph) * 16;
+          float ua = fetch_uc(u0 + cf), ub = fetch_uc(u0 + cf + half);
+          for (int it = hw; it < n_it; it += 2) {
+            const int i0 = (it % gph) * 16, c_lo = it / gph * job.hd + i0, c_hi = c_lo + half;
+            float v[32];
+            share_uc(ua, ub);
+            { const int i1 = ((it + 2) % gph) * 16, c1 = (it + 2) / gph * job.hd + i1; ua = fetch_uc(u0 + c1); ub = fetch_uc(u0 + c1 + half); }
+            acc(c_lo, v);
+            acc(c_hi, v + 16);
+            normed(v, 0);
+            normed(v + 16, 1);
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                lo[j] = normed(lo[j], u0 + col0 + h0 + i0 + j);
-                hi[j] = normed(hi[j], u0 + col0 + h0 + half + i0 + j);
+            for (int h = 0; h < 2; ++h) {
+              __syncwarp();
+              if ((lane >> 4) == h) {   // rows 16 h .. 16 h + 15
+#pragma unroll
+                for (int e = 0; e < 8; ++e) *reinterpret_cast<float4*>(st + (lane & 15) * QT_LD + 4 * e) = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
               }
-              if (rot) {
-                const float4* cp = reinterpret_cast<const float4*>(job.rope_cs + (size_t)rr * half + i0);
-                const float4* sp4 = reinterpret_cast<const float4*>(job.rope_sn + (size_t)rr * half + i0);
-                const float4 ca = __ldcg(cp), cb = __ldcg(cp + 1), sa = __ldcg(sp4), sb = __ldcg(sp4 + 1);
-                const float cs[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w}, sn[8] = {sa.x, sa.y, sa.z, sa.w, sb.x, sb.y, sb.z, sb.w};
+              __syncwarp();
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  const float l = lo[j], h = hi[j];
-                  lo[j] = l * cs[j] - h * sn[j]; hi[j] = h * cs[j] + l * sn[j];
+              for (int i = 0; i < 2; ++i) {
+                const int rl = 8 * i + tr, r = row0 + 16 * h + rl;
+                float4 lo = *reinterpret_cast<const float4*>(st + rl * QT_LD + tc4), hi = *reinterpret_cast<const float4*>(st + rl * QT_LD + 16 + tc4);
+                if (rot) {
+                  const float4 cs = xq[h][2 * i], sn = xq[h][2 * i + 1], l = lo, g = hi;
+                  lo = make_float4(l.x * cs.x - g.x * sn.x, l.y * cs.y - g.y * sn.y, l.z * cs.z - g.z * sn.z, l.w * cs.w - g.w * sn.w);
+                  hi = make_float4(g.x * cs.x + l.x * sn.x, g.y * cs.y + l.y * sn.y, g.z * cs.z + l.z * sn.z, g.w * cs.w + l.w * sn.w);
+                }
+                if (r < job.T && i0 + tc4 < half) {
+                  __half* dst = dst0 + (size_t)kv_row[2 * h + i] * width + tc4;
+                  *reinterpret_cast<uint2*>(dst + c_lo) = make_uint2(pack_f16x2(lo.x * qs, lo.y * qs), pack_f16x2(lo.z * qs, lo.w * qs));
+                  *reinterpret_cast<uint2*>(dst + c_hi) = make_uint2(pack_f16x2(hi.x * qs, hi.y * qs), pack_f16x2(hi.z * qs, hi.w * qs));
                 }
               }
-              if (row_on) {
-                *reinterpret_cast<uint4*>(dst + h0 + i0) = make_uint4(pack_f16x2(lo[0] * qs, lo[1] * qs), pack_f16x2(lo[2] * qs, lo[3] * qs),
-                                                                      pack_f16x2(lo[4] * qs, lo[5] * qs), pack_f16x2(lo[6] * qs, lo[7] * qs));
-                *reinterpret_cast<uint4*>(dst + h0 + half + i0) = make_uint4(pack_f16x2(hi[0] * qs, hi[1] * qs), pack_f16x2(hi[2] * qs, hi[3] * qs),
-                                                                             pack_f16x2(hi[4] * qs, hi[5] * qs), pack_f16x2(hi[6] * qs, hi[7] * qs));
-              }
+              if (rot) load_rope(xq[h], it + 2, h);
             }
+          }
         }
       }
       tc_fence_before();
@@ -542,12 +640,15 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
   if (warp == 1) { tc_fence_after(); w_dealloc<CG>(tmem_base, tmem_cols); }
 }
 
-inline size_t gemm_smem(int TN, int CG, int stages) {
-  return 1024 + (size_t)stages * (2 * A_BYTES + (size_t)(TN / CG) * BK * 2) + ST_BYTES + (2 * W_MAX_STAGES + 4) * 8 + 64;
+// x_box: rows of the activation box (a single row tile only fetches its own rows; the MMAs of the last stage
+// still read 128 from the lo part's start, so the tail behind the stages has to be as long)
+inline size_t gemm_smem(int x_box, int TN, int CG, int stages) {
+  const size_t stage = 2 * (size_t)x_box * BK * 2 + (size_t)(TN / CG) * BK * 2;
+  return 1024 + stages * stage + ST_BYTES + (2 * W_MAX_STAGES + 4) * 8 + 64;
 }
-inline int gemm_stages(int TN, int CG) {
+inline int gemm_stages(int x_box, int TN, int CG) {
   int s = W_MAX_STAGES;
-  while (s > 2 && gemm_smem(TN, CG, s) > (size_t)SMEM_LIMIT) --s;
+  while (s > 2 && gemm_smem(x_box, TN, CG, s) > (size_t)SMEM_LIMIT) --s;
   return s;
 }
 
@@ -574,6 +675,12 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t r) {
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ float ld_cluster_f1(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
   return v;
 }
 
@@ -608,8 +715,8 @@ __global__ void __launch_bounds__(NW * 32, (KS <= 5 && NW == 8) ? 2 : 1) k_wide_
   if (tid == 0) pdl_launch();
   pdl_wait();
   int slot, base, R, off;
-  const int i_req = blockIdx.x / P.n_qblk, kvh = blockIdx.y;
-  int qblk = blockIdx.x % P.n_qblk;
+  const int i_req = blockIdx.y / P.n_qblk, kvh = blockIdx.x;
+  int qblk = blockIdx.y % P.n_qblk;
   if (P.val_req) {
     slot = P.val_req[i_req]; R = P.val_k[i_req] + 1; off = P.val_off[i_req]; base = P.n_seq[slot] - 1;
   } else { slot = P.slot; R = P.rows; off = 0; base = P.first; qblk = P.n_qblk - 1 - qblk; }   // (the longest blocks first)
@@ -760,26 +867,8 @@ __global__ void __launch_bounds__(NW * 32, (KS <= 5 && NW == 8) ? 2 : 1) k_wide_
   l_a += __shfl_xor_sync(0xffffffffu, l_a, 1); l_a += __shfl_xor_sync(0xffffffffu, l_a, 2);
   l_b += __shfl_xor_sync(0xffffffffu, l_b, 1); l_b += __shfl_xor_sync(0xffffffffu, l_b, 2);
 
-  if (NP == 1 && NS == 1) {
-#pragma unroll
-    for (int hr = 0; hr < 2; ++hr) {
-      if (hr ? on_b : on_a) {
-        const int q = hr ? qb : qa;
-        const float l = hr ? l_b : l_a, inv = l > 0.f ? 1.0f / l : 0.f;
-        bf16* orow = P.o + (size_t)(off + q / G) * nq + (size_t)(kvh * G + q % G) * hd + t4 * 2;
-#pragma unroll
-        for (int nd = 0; nd < 2 * KS; ++nd)
-          if (EXACT || nd < ntiles) {
-            const float v0 = o[nd][2 * hr] * inv, v1 = o[nd][2 * hr + 1] * inv;
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(v0, v1);
-            *reinterpret_cast<__nv_bfloat162*>(orow + nd * 8) = h2;
-            *reinterpret_cast<uint32_t*>(orow + (size_t)P.lo_row * nq + nd * 8) = mk::pack_bf16x2(v0 - __low2float(h2), v1 - __high2float(h2));
-          }
-      }
-    }
-    return;
-  }
-  // states [part][query][hd + 4] (O, then max and sum) in the staging area, merged over parts and ranges
+  // states [part][query][hd + 4] (O, then max and sum) in the staging area, merged over parts and ranges (also
+  // where there is one of each: stores from the fragments are pieces of 16 bytes)
   float* states = reinterpret_cast<float*>(asm_raw);
   const int ld = hd + 4;
 #pragma unroll
@@ -814,6 +903,371 @@ __global__ void __launch_bounds__(NW * 32, (KS <= 5 && NW == 8) ? 2 : 1) k_wide_
                  make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
   }
   if (NS > 1) cluster_sync();                        // the other CTAs have read this one's states
+}
+
+// ---------------------------------------------------------------------------------------------
+// Prefill attention on tcgen05 (head sizes 64 and 128)
+// ---------------------------------------------------------------------------------------------
+struct WideAttnTc {
+  CUtensorMap kmap, vmap;        // the layer's pools, box = 64 columns x box_rows rows, 128-byte swizzle
+  int box_rows;
+  WideAttn a;
+  unsigned int* status; unsigned long long wait_limit;
+};
+
+// D[tmem] (+)= A[tmem] * B[smem], fp16 inputs (two per 32-bit column of A), fp32 accumulate, M = 128.
+__device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15,"
+      " %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+// the same in two steps, so that several loads are in flight (the wait is tied to the registers it guards)
+__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15,"
+      " %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+}
+template <int N> __device__ __forceinline__ void tmem_ld_wait(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
+}
+__device__ __forceinline__ void tmem_st16u(uint32_t taddr, const uint32_t* v) {   // completed by tmem_wait_st
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+        "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {   // packed fp32 addition
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+constexpr int TC_ATT_SOFT = 256;            // softmax threads: two per query, half of a chunk's positions each
+constexpr int TC_ATT_THREADS = TC_ATT_SOFT + 64;
+constexpr int TC_ATT_STAGES = 2;
+template <int HD> constexpr int tc_att_chunk() { return HD == 64 ? 128 : 64; }   // positions per chunk: 32 KB of K and V either way
+template <int HD> constexpr size_t tc_att_smem() { return 1024 + (size_t)128 * HD * 2 + TC_ATT_STAGES * (size_t)2 * tc_att_chunk<HD>() * HD * 2 + 256 + 2048 + 64 + 2048; }
+
+// One block: 128 queries (query q of the chunk = row q / G, head q % G of the kv head) against every visible
+// position.  S = Q.K^T and O += P.V are M = 128 MMAs, thread (TMEM lane) q owns query q; P goes to TMEM as
+// fp16 and is the second MMA's A operand, so the softmax weights never touch shared memory.  A thread takes its
+// half row of S into registers at once, so that the next chunk's S is computed under this one's softmax.
+// The longest block's chain of chunks is what a pass takes, and most of a chunk is one thread's
+// exponentials: two threads share a query (they agree on the row maximum through shared memory).  Two blocks
+// share an SM (half its shared memory and TMEM each), launched longest first, so that long and short ones
+// meet; where blocks are few, the CTAs of a cluster (grid z) take a range of the context each.  Warps 0-7: softmax, warp 8: K/V bulk copies (one box per page slice and 64-column half, one lane
+// each), warp 9: MMA issue, TMEM.
+// Measured at 0.4B, 2048 rows from position 0 (16 heads of 64): mma.sync form 72 us, with P in S's place 48,
+// one thread per query 38, with rows stored from the accumulator's threads 35, this one 31 us.
+template <int HD>
+__global__ void __launch_bounds__(TC_ATT_THREADS, 2) k_wide_attn_tc(const __grid_constant__ WideAttnTc J) {
+  extern __shared__ __align__(1024) uint8_t atc_raw[];
+  constexpr int CH = tc_att_chunk<HD>(), HALVES = HD / 64, NST = TC_ATT_STAGES;
+  constexpr int KBYTES = CH * HD * 2;
+  const WideAttn& P = J.a;
+  uint8_t* qs = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(atc_raw) + 1023) & ~(uintptr_t)1023);   // HALVES x [128][128 bytes]
+  uint8_t* ring = qs + 128 * HD * 2;
+  // [0], [1]: K buffers, [2], [3]: V buffers, handed back by plain arrivals of threads that have seen the MMAs'
+  // completion anyway (a commit costs the issuing thread about 240 cycles)
+  uint64_t* kv_full = reinterpret_cast<uint64_t*>(ring + NST * 2 * KBYTES);
+  uint64_t* kv_empty = kv_full + 2 * NST;
+  uint64_t* q_full = kv_empty + 2 * NST;
+  uint64_t* s_full = q_full + 1;
+  uint64_t* s_free = s_full + 1;
+  uint64_t* p_full = s_free + 1;
+  uint64_t* o_done = p_full + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_done + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  float* row_x = reinterpret_cast<float*>(tmem_slot + 4);          // [2][2 halves][128] row maxima (alternate chunks), at the end the sums
+  volatile int* vx = reinterpret_cast<volatile int*>(row_x + 512);  // [2][8 warps] verdicts, exchanged with the maxima
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < 2 * NST; ++s) { mbar_init(kv_full + s, 1); mbar_init(kv_empty + s, 1); }
+    mbar_init(q_full, 8); mbar_init(s_full, 1); mbar_init(s_free, 8); mbar_init(p_full, 8); mbar_init(o_done, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 9) tmem_alloc(tmem_slot, 256);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  // (the successor may start only once this block owns its TMEM: it would take the columns and wait for this grid)
+  if (threadIdx.x == 0) pdl_launch();
+  const uint32_t tmem_s = *tmem_slot, tmem_p = tmem_s + CH, tmem_o = tmem_p + CH / 2;   // CH + CH / 2 + HD <= 256 columns
+  const int G = P.Hq / P.Hkv, nq = P.Hq * HD;
+  const int kvh = blockIdx.x, qblk = gridDim.y - 1 - blockIdx.y;
+  const int Q = P.rows * G, q0 = qblk * 128, nQ = min(128, Q - q0);
+  const int all_chunks = (P.first + (q0 + nQ - 1) / G) / CH + 1, NS = gridDim.z, zr = blockIdx.z;
+  const int c_first = (all_chunks * zr) / NS, n_chunks = (all_chunks * (zr + 1)) / NS - c_first;   // this CTA's range of the context
+  const unsigned long long lim = J.wait_limit;
+  int fills = 0;   // chunks fetched (copies in flight are drained after an abort)
+
+  if (warp == 8) {
+    // ------------------------------------------------------------------ K/V loader
+    pdl_wait();
+    const int* pt = P.page_table + (size_t)P.slot * P.max_pages;
+    const int slots = CH / J.box_rows;
+    const int half = lane / slots, sl = lane % slots;
+    bool ok = true;
+    for (int c = 0; c < n_chunks && ok; ++c) {
+      const int pz = min((c_first + c) * CH + sl * J.box_rows, (P.max_pages - 1) * P.page_tokens);   // (slices past the page table: any finite rows, they are masked)
+      const int row = half < HALVES ? __ldcg(pt + pz / P.page_tokens) * P.page_tokens + pz % P.page_tokens : 0;
+      for (int v = 0; v < 2 && ok; ++v) {
+        const int s = v * NST + c % NST;
+        ok = __all_sync(0xffffffffu, mbar_wait(kv_empty + s, ((c / NST) & 1) ^ 1, abort_flag, lim));
+        if (!ok) break;
+        if (lane == 0) mbar_expect_tx(kv_full + s, KBYTES);
+        __syncwarp();
+        if (half < HALVES)
+          tma_load_2d_nohint(ring + (size_t)s * KBYTES + half * (CH * 128) + sl * J.box_rows * 128, v ? &J.vmap : &J.kmap, kvh * HD + half * 64, row, kv_full + s);
+        ++fills;
+      }
+    }
+  } else if (warp == 9) {
+    // ------------------------------------------------------------------ MMA issuer
+    if (lane == 0) {
+      const uint32_t idesc_s = mk::instr_desc_f16(CH, 0), idesc_o = mk::instr_desc_f16(HD, 1);
+      auto issue_s = [&](int c) {
+        if (!mbar_wait(kv_full + c % NST, (c / NST) & 1, abort_flag, lim)) return false;
+        tc_fence_after();
+        const uint32_t kb = smem_u32(ring + (size_t)(c % NST) * KBYTES);
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h)
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            umma_bf16(tmem_s, mk::smem_desc_sw128_ex(smem_u32(qs) + (uint32_t)(h * 128 * 128 + k * 32), 16, 1024),
+                      mk::smem_desc_sw128_ex(kb + (uint32_t)(h * CH * 128 + k * 32), 16, 1024), idesc_s, (h | k) ? 1u : 0u);
+        umma_commit(s_full);
+        return true;
+      };
+      bool ok = mbar_wait(q_full, 0, abort_flag, lim) && n_chunks > 0 && issue_s(0);
+      for (int c = 0; c < n_chunks && ok; ++c) {
+        if (c + 1 < n_chunks) {
+          ok = mbar_wait(s_free, c & 1, abort_flag, lim);
+          if (ok) mbar_arrive(kv_empty + c % NST);               // (S has been read, so its MMAs are done with K)
+          tc_fence_after();
+          ok = ok && issue_s(c + 1);
+        }
+        ok = ok && mbar_wait(kv_full + NST + c % NST, (c / NST) & 1, abort_flag, lim) && mbar_wait(p_full, c & 1, abort_flag, lim);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t vb = smem_u32(ring + (size_t)(NST + c % NST) * KBYTES);
+#pragma unroll
+        for (int k = 0; k < CH / 16; ++k)
+          umma_f16_ts(tmem_o, tmem_p + (uint32_t)(k * 8), mk::smem_desc_sw128_ex(vb + (uint32_t)(k * 2048), (uint32_t)(CH * 128), 1024), idesc_o, (c > 0 || k > 0) ? 1u : 0u);
+        umma_commit(o_done);
+      }
+    }
+  } else {
+    // ------------------------------------------------------------------ softmax (warps 0..7)
+    pdl_wait();
+    const int quad = warp & 3, hf = warp >> 2;                   // TMEM lanes 32 quad .., half hf of a chunk's positions
+    const int ql = quad * 32 + lane;
+    constexpr int CW = CH / 2, HW = HD / 2;                      // positions and head columns of this thread
+    {
+      // the block's queries, swizzled; rows past its queries are zero
+      constexpr int PIECES = HD / 8;
+      for (int it = threadIdx.x; it < 128 * PIECES; it += TC_ATT_SOFT) {
+        const int r = it / PIECES, c = it % PIECES;
+        const bool on = r < nQ;
+        const int q = on ? q0 + r : q0;
+        mk::cp_async16(qs + (size_t)(c >> 3) * (128 * 128) + (size_t)r * 128 + (size_t)(((c & 7) ^ (r & 7)) << 4),
+                       reinterpret_cast<const uint4*>(P.q16 + (size_t)(q / G) * nq + (size_t)(kvh * G + q % G) * HD) + c, on);
+      }
+      mk::cp_async_commit();
+      mk::cp_async_wait_all();
+      mk::fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(q_full);
+    }
+    const bool mine = ql < nQ;
+    const int q = q0 + (mine ? ql : nQ - 1);
+    const int last = P.first + q / G;                           // last visible position of this thread's query
+    const int warp_first = P.first + (q0 + min(quad * 32, nQ - 1)) / G;
+    const uint32_t sel = (uint32_t)(quad * 32) << 16;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {            // one verdict per warp
+      if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+      return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, lim));
+    };
+    auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory"); };   // the two warps of these 32 queries
+    float m_run = -INFINITY, l_run = 0.f;
+    bool ok = true;
+    for (int c = 0; c < n_chunks; ++c) {
+      // (after an expired wait both warps of a pair have to leave together: a warp goes on until the next
+      // exchange, where the pair agrees on one verdict)
+      ok = ok && wait(s_full, c & 1);
+      tc_fence_after();
+      const int p0 = (c_first + c) * CH + hf * CW;
+      uint32_t sr[CW];
+#pragma unroll
+      for (int j0 = 0; j0 < CW; j0 += 32) tmem_ld32_issue(tmem_s + sel + (uint32_t)(hf * CW + j0), sr + j0);
+      tmem_ld_wait<CW>(sr);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(s_free);                        // the next chunk's S may take its place
+      if (p0 + CW - 1 > warp_first) {
+#pragma unroll
+        for (int j = 0; j < CW; ++j) if (p0 + j > last) sr[j] = 0xff800000u;   // -inf
+      }
+      float mxa = __uint_as_float(sr[0]), mxb = __uint_as_float(sr[1]);
+#pragma unroll
+      for (int j = 2; j < CW; j += 4) {                          // (three-operand maxima)
+        mxa = fmaxf(fmaxf(mxa, __uint_as_float(sr[j])), __uint_as_float(sr[j + 1]));
+        if (j + 2 < CW) mxb = fmaxf(fmaxf(mxb, __uint_as_float(sr[j + 2])), __uint_as_float(sr[j + 3]));
+      }
+      float* rx = row_x + (c & 1) * 256;
+      rx[hf * 128 + ql] = fmaxf(mxa, mxb);
+      if (lane == 0) vx[(c & 1) * 8 + warp] = ok ? 1 : 0;
+      pair_sync();
+      const float mx = fmaxf(rx[ql], rx[128 + ql]);
+      ok = vx[(c & 1) * 8 + quad] && vx[(c & 1) * 8 + quad + 4];
+      if (!ok) break;
+      // the reference exponent follows the running maximum only when that has moved by more than 2^8 (see the persistent kernel)
+      const float m_seen = fmaxf(m_run, mx);
+      const float m_new = (m_seen > m_run + 8.0f || m_run == -INFINITY) ? m_seen : m_run;
+      const float off = m_new == -INFINITY ? 0.f : m_new;
+      const float corr = mk::fast_exp2(m_run - off);
+      // (two elements per addition: the loop is bound by instruction issue and fetch)
+      const float2 noff = make_float2(-off, -off);
+      float2 sum2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+      for (int j = 0; j < CW; j += 2) {
+        float2 e = add2(make_float2(__uint_as_float(sr[j]), __uint_as_float(sr[j + 1])), noff);
+        e.x = mk::fast_exp2(e.x); e.y = mk::fast_exp2(e.y);
+        sum2[(j >> 1) & 1] = add2(sum2[(j >> 1) & 1], e);
+        sr[j / 2] = pack_f16x2(e.x, e.y);
+      }
+      sum2[0] = add2(sum2[0], sum2[1]);
+      l_run = l_run * corr + (sum2[0].x + sum2[0].y);
+      m_run = m_new;
+      if (c > 0) {
+        ok = wait(o_done, (c - 1) & 1);
+        if (threadIdx.x == 0) mbar_arrive(kv_empty + NST + (c - 1) % NST);   // the V buffer of that P.V is free
+        tc_fence_after();
+        if (__any_sync(0xffffffffu, corr != 1.0f)) {
+#pragma unroll
+          for (int d0 = 0; d0 < HW; d0 += 32) {
+            float v[32];
+            uint32_t u[32];
+            tmem_ld32(tmem_o + sel + (uint32_t)(hf * HW + d0), v);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) u[j] = __float_as_uint(v[j] * corr);
+            tmem_st16u(tmem_o + sel + (uint32_t)(hf * HW + d0), u);
+            tmem_st16u(tmem_o + sel + (uint32_t)(hf * HW + d0 + 16), u + 16);
+          }
+        }
+      }
+#pragma unroll
+      for (int j0 = 0; j0 < CW / 2; j0 += 16) tmem_st16u(tmem_p + sel + (uint32_t)(hf * (CW / 2) + j0), sr + j0);   // (the previous P.V, waited for above, has read its P)
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_full);
+    }
+    if (ok && n_chunks > 0) ok = wait(o_done, (n_chunks - 1) & 1);
+    if (!ok) *abort_flag = 1;
+    __syncwarp();
+    asm volatile("bar.sync 5, 256;" ::: "memory");               // (every pair is past its last exchange of maxima)
+    row_x[hf * 128 + ql] = l_run;
+    asm volatile("bar.sync 5, 256;" ::: "memory");
+    if (*abort_flag == 0) {
+      tc_fence_after();
+      if (hf == 0) { row_x[256 + ql] = m_run; row_x[384 + ql] = row_x[ql] + row_x[128 + ql]; }
+      float* part = reinterpret_cast<float*>(qs) + (size_t)ql * (HD + 4) + hf * HW;   // (every MMA has completed: the tiles are free)
+#pragma unroll
+      for (int d0 = 0; d0 < HW; d0 += 32) {
+        float v[32];
+        tmem_ld32(tmem_o + sel + (uint32_t)(hf * HW + d0), v);
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+          *reinterpret_cast<float4*>(part + d0 + j) = n_chunks > 0 ? make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      tc_fence_before();
+    }
+  }
+  {
+    // The ranges' states, merged in range order (the cluster's CTAs share the rows), through shared memory in any
+    // case: stores of one row per thread took 8 us of a block with head size 128.
+    __syncwarp();
+    if (NS > 1) cluster_sync(); else __syncthreads();
+    // every range's weight of every row, once (the maxima and sums of the other CTAs are a long way off)
+    float* wgt = row_x + 528;                                    // [4 ranges][128]
+    if (threadIdx.x < 128) {
+      const int r = threadIdx.x;
+      const uint32_t mbase = smem_u32(row_x) + (uint32_t)(256 + r) * 4;
+      float m[4], l[4], M = -INFINITY, L = 0.f;
+#pragma unroll
+      for (int z = 0; z < 4; ++z) {
+        m[z] = -INFINITY; l[z] = 0.f;
+        if (z < NS) { const uint32_t at = map_rank(mbase, z); m[z] = ld_cluster_f1(at); l[z] = ld_cluster_f1(at + 512); }
+        M = fmaxf(M, m[z]);
+      }
+#pragma unroll
+      for (int z = 0; z < 4; ++z) { m[z] = m[z] == -INFINITY ? 0.f : mk::fast_exp2(m[z] - M); L += l[z] * m[z]; }
+      const float inv = L > 0.f ? 1.0f / L : 0.f;
+#pragma unroll
+      for (int z = 0; z < 4; ++z) wgt[z * 128 + r] = m[z] * inv;
+    }
+    __syncthreads();
+    const uint32_t pbase = smem_u32(qs);
+#pragma unroll 4
+    for (int it = zr * TC_ATT_THREADS + threadIdx.x; it < nQ * (HD / 4); it += NS * TC_ATT_THREADS) {
+      const int r = it / (HD / 4), d4 = it % (HD / 4) * 4;
+      const uint32_t at = (uint32_t)(r * (HD + 4) + d4) * 4;
+      const float w0 = wgt[r];
+      float4 acc = NS == 1 ? *reinterpret_cast<const float4*>(qs + at) : ld_cluster_f4(map_rank(pbase + at, 0));
+      acc.x *= w0; acc.y *= w0; acc.z *= w0; acc.w *= w0;
+      for (int z = 1; z < NS; ++z) {
+        const float w = wgt[z * 128 + r];
+        const float4 v = ld_cluster_f4(map_rank(pbase + at, z));
+        acc.x += v.x * w; acc.y += v.y * w; acc.z += v.z * w; acc.w += v.w * w;
+      }
+      const int q = q0 + r;
+      store_split4(P.o + (size_t)(q / G) * nq + (size_t)(kvh * G + q % G) * HD, (size_t)d4, (size_t)P.lo_row * nq, acc);
+    }
+    if (NS > 1) cluster_sync();
+  }
+  // ------------------------------------------------------------------ teardown
+  __syncthreads();
+  if (*abort_flag) {
+    if (warp == 8 && lane == 0) {
+      *reinterpret_cast<volatile unsigned int*>(J.status + STATUS_ERROR) = 5u;  // STAIRS_ETIMEOUT
+      __threadfence_system();
+      const long long t0 = clock64();
+      const unsigned long long drain = lim > 2000000ull ? lim : 2000000ull;
+      for (int f = max(0, fills - 2 * NST); f < fills; ++f)      // fill f: chunk f / 2, K or V
+        while (!mbar_try(kv_full + (f & 1) * NST + (f >> 1) % NST, ((f >> 1) / NST) & 1)) {
+          if ((unsigned long long)(clock64() - t0) > drain) break;
+        }
+    }
+    __syncthreads();
+  }
+  if (warp == 9) { tc_fence_after(); tmem_dealloc(tmem_s, 256); }
 }
 
 // Embedding of the pass's rows (tok, pos, req written by k_rows): the residual stream, the first GEMM's

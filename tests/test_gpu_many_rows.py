@@ -76,3 +76,21 @@ def test_prefill_in_several_chunks_matches_one_chunk():
         got.append(lg.cpu())
         eng.close()
     assert float((got[0] - got[1]).abs().max()) < 5e-3
+
+
+@pytest.mark.parametrize("page", [32, 64, 128])
+@pytest.mark.parametrize("name", ["gqa_hd64", "mqa_hd128", "family_a"])
+def test_prefill_attention_over_many_chunks_matches_oracle(name, page):
+    # several K/V chunks and query blocks, a second pass over cached positions, every page size's copies
+    st = _stairs()
+    shape = SHAPES[name].replace(max_pos=1024)
+    tsrc, _ = sources(shape)
+    tgt, _ = gu.oracle_pair(tsrc)
+    eng = st.Stairs(tsrc, None, max_requests=1, max_seq_len=720, k_max=2, kv_page_tokens=page, prefill_chunk=400)
+    prompt = list(wl.zipf_tokens(701, shape.vocab, page))
+    eng.prefill(0, prompt)
+    tt, _, logits = eng.validate([0], [0], None, want_logits=True)
+    eng.sync()
+    ref = np.stack([so.forward_logits(tgt, prompt)])
+    gu.check_rows_against_oracle(logits.cpu().numpy(), tt.cpu().numpy()[0], ref, gu.LOGIT_TOL_BF16)
+    eng.close()
