@@ -228,8 +228,9 @@ const char *stairs_last_error(const stairs_ctx *ctx);
  * Limits: n_rows <= STAIRS_STATIC_MAX_ROWS, 1 <= n_req <= STAIRS_STATIC_MAX_REQ,
  * 0 <= k_host[i] <= k_max <= 63; anything larger returns STAIRS_ENOSPC or STAIRS_EINVAL with
  * a text in stairs_last_error(NULL).  Work is enqueued on `stream` (NULL = default stream)
- * of the current device.  The first call on a device looks up the array's device address
- * (cudaGetSymbolAddress); make that first call before starting any stream capture.  All
+ * of the current device.  Most calls are one launch that keeps nothing in memory; few requests with
+ * many or very long rows use the array.  The first such call on a device looks up the array's device
+ * address (cudaGetSymbolAddress); make that first call before starting any stream capture.  Those
  * calls share the array and it keeps the previous call's keys: each call clears the part it
  * uses before use, and two calls that overlap on the GPU (different streams, no ordering
  * between them) race on it - order them. */

@@ -1926,6 +1926,86 @@ __global__ void k_accept_static(const __grid_constant__ StaticAcceptParams p) {
   p.accept_len[i] = a < 0 ? k : a;
 }
 
+// The same call as one launch: a cluster of eight CTAs per request, each CTA a slice of the vocabulary of
+// all the request's rows; row keys are reduced per CTA, gathered in the first CTA's shared memory, and its
+// threads take the tokens and the accept length.  Nothing is kept in memory between launches.  A call is
+// bound by latency (5 rows of 32000: 31 us a call with three launches, 11 now, of which the kernel 4) or by reading
+// the logits (576 rows: 53 us, now 16), so a warp takes a quarter of a row's slice at a time with eight vectors a
+// lane in flight, and the CTAs of 64 requests fit the chip at once.
+constexpr int SA_THREADS = 256, SA_CTAS = 8;
+template <bool VEC>
+__global__ void __cluster_dims__(SA_CTAS, 1, 1) __launch_bounds__(SA_THREADS, 4) k_accept_cluster(const __grid_constant__ StaticAcceptParams p, const float* __restrict__ logits, int V, int ld) {
+  constexpr int SEG = 4;
+  __shared__ unsigned long long red[64][SEG];
+  __shared__ unsigned long long gathered[SA_CTAS][64];
+  __shared__ unsigned int miss[2];
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  const int i = blockIdx.x / SA_CTAS, rank = blockIdx.x % SA_CTAS;
+  const int k = p.k[i], rows = k + 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = ((V + SA_CTAS - 1) / SA_CTAS + 3) / 4 * 4, lo = min(rank * per, V), hi = min(lo + per, V);
+  const float* base = logits + (size_t)p.off[i] * ld;
+  auto ordered = [](float v) {   // monotone map to unsigned (see argmax_key)
+    const uint32_t u = __float_as_uint(v);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  };
+  const int seg_len = (per / SEG + 3) / 4 * 4;
+  for (int task = warp; task < rows * SEG; task += SA_THREADS / 32) {
+    const int r = task / SEG, s0 = min(lo + task % SEG * seg_len, hi), s1 = task % SEG == SEG - 1 ? hi : min(s0 + seg_len, hi);
+    const float* row = base + (size_t)r * ld;
+    constexpr int W = VEC ? 4 : 1;
+    const int c0 = s0 + lane * W;
+    uint32_t bu = 0u, bi = c0 < s1 ? (uint32_t)c0 : 0xffffffffu;   // best value so far, lowest index of it
+    for (int cb = c0; cb < s1; cb += 8 * 32 * W) {
+      float v[8][W];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int c = cb + j * 32 * W;
+        if (VEC) {   // (a vector past the last column stays inside the row's pitch)
+          const float4 q = c < s1 ? __ldcs(reinterpret_cast<const float4*>(row + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          v[j][0] = q.x; v[j][W > 1 ? 1 : 0] = q.y; v[j][W > 1 ? 2 : 0] = q.z; v[j][W > 1 ? 3 : 0] = q.w;
+        } else v[j][0] = c < s1 ? row[c] : 0.f;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+          const int c = cb + j * 32 * W + e;
+          const uint32_t u = c < s1 ? ordered(v[j][e]) : 0u;
+          if (u > bu) { bu = u; bi = (uint32_t)c; }
+        }
+    }
+    const uint32_t u = __reduce_max_sync(0xffffffffu, bu);
+    const uint32_t idx = __reduce_min_sync(0xffffffffu, bu == u ? bi : 0xffffffffu);
+    if (lane == 0) red[r][task % SEG] = ((unsigned long long)u << 32) | (0xffffffffu - idx);
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");   // every CTA of the cluster runs
+  if (tid < rows) {
+    unsigned long long best = 0ull;
+#pragma unroll
+    for (int w = 0; w < SEG; ++w) best = red[tid][w] > best ? red[tid][w] : best;
+    uint32_t at;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&gathered[rank][tid])));
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at), "l"(best) : "memory");
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (rank != 0 || tid >= 64) return;
+  bool differs = false;
+  if (tid < rows) {
+    unsigned long long best = 0ull;
+#pragma unroll
+    for (int c = 0; c < SA_CTAS; ++c) best = gathered[c][tid] > best ? gathered[c][tid] : best;
+    const int tr = argmax_key_index(best);
+    p.target_tokens[i * (p.k_max + 1) + tid] = tr;
+    differs = tid < k && p.draft[i * p.k_max + tid] != tr;
+  }
+  const unsigned int m = __ballot_sync(0xffffffffu, differs);
+  if (lane == 0) miss[warp] = m;
+  asm volatile("bar.sync 1, 64;" ::: "memory");
+  if (tid == 0) p.accept_len[i] = miss[0] ? __ffs(miss[0]) - 1 : miss[1] ? 31 + __ffs(miss[1]) : k;
+}
+
 constexpr int kMaxDevices = 64;
 unsigned long long* g_static_keys_addr[kMaxDevices] = {};
 
@@ -1953,6 +2033,20 @@ extern "C" int stairs_accept_static(const float* logits_dev, int vocab, int ld, 
   if (rows > STAIRS_STATIC_MAX_ROWS)
     return fail(nullptr, STAIRS_ENOSPC, "stairs_accept_static: %d rows exceed the fixed scratch of %d rows", rows,
                 STAIRS_STATIC_MAX_ROWS);
+  p.n_req = n_req; p.k_max = k_max; p.draft = draft_dev;
+  p.target_tokens = target_tokens_dev; p.accept_len = accept_len_dev;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  int k_top = 0;
+  for (int i = 0; i < n_req; ++i) k_top = std::max(k_top, p.k[i]);
+  // one cluster per request, unless few requests with many or very long rows would leave most of the chip idle
+  // (a CTA reads about 100 KB per us: at 256 KB each the launches saved are worth less than more CTAs)
+  if (n_req * SA_CTAS >= 128 || (long long)(k_top + 1) * vocab * 4 <= (long long)SA_CTAS * (256 << 10)) {
+    const bool vec = ld % 4 == 0 && (reinterpret_cast<uintptr_t>(logits_dev) & 15) == 0;
+    if (vec) k_accept_cluster<true><<<n_req * SA_CTAS, SA_THREADS, 0, st>>>(p, logits_dev, vocab, ld);
+    else k_accept_cluster<false><<<n_req * SA_CTAS, SA_THREADS, 0, st>>>(p, logits_dev, vocab, ld);
+    CK(cudaGetLastError());
+    return STAIRS_OK;
+  }
   int dev = 0;
   CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxDevices) return fail(nullptr, STAIRS_EUNSUPPORTED, "stairs_accept_static: device ordinal %d", dev);
@@ -1962,13 +2056,10 @@ extern "C" int stairs_accept_static(const float* logits_dev, int vocab, int ld, 
     g_static_keys_addr[dev] = ptr;
   }
   unsigned long long* keys = g_static_keys_addr[dev];
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   // the array still holds the previous call's keys: the atomic max below needs zeros
   CK(cudaMemsetAsync(keys, 0, (size_t)rows * sizeof(unsigned long long), st));
   const int slices = std::max(1, std::min(64, vocab / 2048));
   k_argmax<<<dim3(slices, rows), 256, 0, st>>>(logits_dev, vocab, ld, keys);
-  p.n_req = n_req; p.k_max = k_max; p.draft = draft_dev;
-  p.target_tokens = target_tokens_dev; p.accept_len = accept_len_dev;
   k_accept_static<<<(n_req + 63) / 64, 64, 0, st>>>(p);
   CK(cudaGetLastError());
   return STAIRS_OK;

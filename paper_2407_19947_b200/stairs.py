@@ -6,6 +6,7 @@ There is no CPU fallback: loading fails loudly when the library has not been bui
 """
 from __future__ import annotations
 
+import array
 import ctypes as C
 import os
 from typing import List, Optional, Sequence
@@ -113,6 +114,23 @@ def _ptr(a: np.ndarray):
     return a.ctypes.data_as(C.POINTER(C.c_int32))
 
 
+def _ints(a):
+    """A list of integers as a ctypes array (a numpy round trip takes three times as long)."""
+    n = len(a)
+    if type(a) is not list:
+        a = [int(x) for x in a]
+    return (C.c_int32 * n)(*a) if n <= 12 else (C.c_int32 * n).from_buffer(array.array("i", a))
+
+
+def _results(t, n, k_max, ks, device):
+    """(target_tokens [n, k_max + 1], accept_len [n]) on the device, cleared only where a request's row has
+    entries past its own draft length."""
+    if min(ks, default=0) >= k_max:
+        return t.empty(n, k_max + 1, dtype=t.int32, device=device), t.empty(n, dtype=t.int32, device=device)
+    buf = t.zeros(n * (k_max + 2), dtype=t.int32, device=device)
+    return buf[: n * (k_max + 1)].view(n, k_max + 1), buf[n * (k_max + 1):]
+
+
 def c_model(shape) -> CModel:
     return CModel(shape.n_layers, shape.d_model, shape.n_heads, shape.n_kv_heads, shape.head_dim, shape.d_ff,
                   shape.vocab, shape.max_pos, shape.norm, shape.act, shape.pos, shape.rope_theta, shape.norm_eps,
@@ -155,6 +173,7 @@ class Stairs:
         if not torch.cuda.is_available():
             raise RuntimeError("stairs needs a CUDA device (B200, sm_100a); there is no CPU path")
         self.device = f"cuda:{device_index}"
+        self._dev = torch.device(self.device)
         torch.cuda.set_device(device_index)
         self.k_max, self.max_requests = k_max, max_requests
         self.vocab = target_source.shape.vocab
@@ -218,16 +237,10 @@ class Stairs:
                  out=None):
         """Enqueues one stairs pass.  Returns (target_tokens_dev [n,k_max+1], accept_len_dev [n], logits or None)."""
         t = self.torch
-        r, kk = _i32(req_ids), _i32(k)
-        n = len(r)
-        if out is None:
-            tt = t.zeros((n, self.k_max + 1), dtype=t.int32, device=self.device)
-            al = t.zeros((n,), dtype=t.int32, device=self.device)
-        else:
-            tt, al = out
-        rows = int(kk.sum()) + n
-        logits = t.empty((rows, self.vocab), dtype=t.float32, device=self.device) if want_logits else None
-        self._ck(self.lib.stairs_validate(self.h, n, _ptr(r), _ptr(kk),
+        n = len(req_ids)
+        tt, al = _results(t, n, self.k_max, k, self._dev) if out is None else out
+        logits = t.empty((int(sum(k)) + n, self.vocab), dtype=t.float32, device=self._dev) if want_logits else None
+        self._ck(self.lib.stairs_validate(self.h, n, _ints(req_ids), _ints(k),
                                           draft_dev.data_ptr() if draft_dev is not None else None,
                                           tt.data_ptr(), al.data_ptr(),
                                           logits.data_ptr() if logits is not None else None, int(commit)))
@@ -235,7 +248,7 @@ class Stairs:
 
     def validate_host(self, req_ids, k, draft_host, *, commit=False):
         """Host-buffer variant: (target_tokens [n,k_max+1], accept_len [n]) as numpy arrays."""
-        r, kk = _i32(req_ids), _i32(k)
+        r, kk = _ints(req_ids), _ints(k)
         n = len(r)
         d = _i32(draft_host).reshape(n, -1) if draft_host is not None and self.k_max > 0 else None
         if d is not None and d.shape[1] != self.k_max:
@@ -244,7 +257,7 @@ class Stairs:
             d = pad
         tt = np.zeros((n, self.k_max + 1), np.int32)
         al = np.zeros((n,), np.int32)
-        self._ck(self.lib.stairs_validate_host(self.h, n, _ptr(r), _ptr(kk), _ptr(d) if d is not None else None,
+        self._ck(self.lib.stairs_validate_host(self.h, n, r, kk, _ptr(d) if d is not None else None,
                                                _ptr(tt), _ptr(al), int(commit)))
         return tt, al
 
@@ -311,14 +324,12 @@ def accept_static(logits_dev, k: Sequence[int], draft_dev, k_max: int, *, vocab:
     draft_dev: int32 [n_req, k_max].  Returns (target_tokens [n_req, k_max+1], accept_len [n_req])."""
     import torch
     lib = load_library()
-    kk = _i32(k)
-    n = len(kk)
-    tt = torch.zeros((n, k_max + 1), dtype=torch.int32, device=logits_dev.device)
-    al = torch.zeros((n,), dtype=torch.int32, device=logits_dev.device)
-    st = stream if stream is not None else torch.cuda.current_stream()
-    rc = lib.stairs_accept_static(logits_dev.data_ptr(), vocab or logits_dev.shape[1], logits_dev.stride(0), n, _ptr(kk),
+    n = len(k)
+    tt, al = _results(torch, n, k_max, k, logits_dev.device)
+    st = stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    rc = lib.stairs_accept_static(logits_dev.data_ptr(), vocab or logits_dev.shape[1], logits_dev.stride(0), n, _ints(k),
                                   draft_dev.data_ptr() if draft_dev is not None else None, k_max,
-                                  tt.data_ptr(), al.data_ptr(), st.cuda_stream)
+                                  tt.data_ptr(), al.data_ptr(), st)
     if rc:
         raise StairsError(rc, lib.stairs_last_error(None).decode())
     return tt, al

@@ -56,3 +56,34 @@ def test_static_accept_rejects_sizes_beyond_its_fixed_scratch():
     with pytest.raises(stairs.StairsError) as e:
         stairs.accept_static(logits, [5], drafts, 4)                   # k above k_max
     assert e.value.code == 1
+
+
+@pytest.mark.parametrize("vocab,ld", [(1, 1), (5, 8), (127, 128), (2049, 2051), (32000, 32000), (70001, 70004)])
+@pytest.mark.parametrize("ks", [[0], [4], [63], [2, 0, 5], [1] * 64], ids=lambda k: f"{len(k)}x{max(k) + 1}")
+def test_static_accept_equals_torch_argmax(vocab, ld, ks):
+    # one cluster per request, and the many-block form for few long requests; odd row lengths, unaligned
+    # rows, ties (lowest index wins)
+    from paper_2407_19947_b200 import build, stairs
+    build.build()
+    rows, k_max = sum(ks) + len(ks), max(ks)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(vocab + rows)
+    store = torch.randint(-4, 5 if vocab > 300 else 3, (rows, ld), generator=g, device="cuda").float()
+    store[:, vocab:] = 100.0                                     # past the vocabulary: must not be looked at
+    lg = store[:, :vocab].cpu().numpy()
+    want = lg.argmax(axis=1)
+    draft = torch.randint(0, vocab, (len(ks), max(k_max, 1)), generator=g, device="cuda", dtype=torch.int32)
+    row = 0
+    for i, k in enumerate(ks):
+        for r in range(k // 2):
+            draft[i, r] = int(want[row + r])
+        row += k + 1
+    tt, al = stairs.accept_static(store, ks, draft if k_max else None, k_max, vocab=vocab)
+    torch.cuda.synchronize()
+    tt, al, d, row = tt.cpu().numpy(), al.cpu().numpy(), draft.cpu().numpy(), 0
+    for i, k in enumerate(ks):
+        assert tt[i, : k + 1].tolist() == want[row: row + k + 1].tolist()
+        assert (tt[i, k + 1:] == 0).all()
+        miss = [r for r in range(k) if d[i, r] != tt[i, r]]
+        assert int(al[i]) == (miss[0] if miss else k)
+        row += k + 1
