@@ -19,6 +19,7 @@
 #include "gemm_tc.cuh"
 #include "kernels_basic.cuh"
 #include "megakernel.cuh"
+#include "small_f32.cuh"
 #include "wide.cuh"
 
 using namespace stairs;
@@ -59,12 +60,13 @@ struct DevModel {
   char* kpool = nullptr;  // [n_layers][pool_tokens][Hkv*hd] elements of the weight dtype
   char* vpool = nullptr;
   size_t kv_layer_bytes = 0;
+  const small::SmallLayer* small_layers = nullptr;   // device: per-layer pointers of the one-launch fp32 passes
 };
 
 struct Layout {
   size_t status, seq, n_seq, page_table, tok, pos, req, val_req, val_k, val_off, keys, x, h, qkv, q,
       o, ff, logits, draft_buf, tt_buf, al_buf, gemm_partial, gemm_counters, mk_partial, mk_partial_bytes, mk_bar, attn_part, prog_t, prog_d, mk_trace, mk_stats, rope_t, rope_d, aux_t, aux_d, w13_t, w13_d, kv_t_k, kv_t_v, kv_d_k, kv_d_v, total;
-  size_t kv_row, wide_rope, wide_stats;
+  size_t kv_row, wide_rope, wide_stats, small_t, small_d;
   int max_rows, logit_rows, max_pages, n_pages, t_box_max, attn_units, stat_tiles;
   size_t prog_slot_t, prog_slot_d, prog_maps_off_t, prog_maps_off_d;
   size_t kv_t_layer, kv_d_layer;
@@ -107,6 +109,7 @@ struct stairs_ctx {
   size_t io_draft = 0, io_tt = 0, io_al = 0;   // offsets in ints
   unsigned long long wait_limit = 0;
   bool use_mk = false;
+  int small_ctas = 0;                // cluster size of the small fp32 models' one-launch passes (0: not used)
   bool draft_shares_kv = false;      // early-exit assistant on the persistent kernel: it uses the main model's K/V pools
   unsigned long long bar_base = 0;   // grid-barrier arrivals consumed by earlier launches
   int kps_force = 0;                 // tuning: k-blocks per pipeline stage (0 = chosen per row box)
@@ -237,6 +240,8 @@ bool compute_layout(const stairs_config& c, Layout* L, const char** why) {
   L->draft_buf = take((size_t)c.max_requests * std::max(c.k_max, 1) * 4);
   L->tt_buf = take((size_t)c.max_requests * (c.k_max + 1) * 4);
   L->al_buf = take((size_t)c.max_requests * 4);
+  L->small_t = take(t.wdtype == 0 ? (size_t)t.n_layers * sizeof(small::SmallLayer) : 0);
+  L->small_d = take(t.wdtype == 0 && has_draft ? (size_t)d.n_layers * sizeof(small::SmallLayer) : 0);
   L->gemm_partial = take(t.wdtype == 1 ? (size_t)TC_GRID_MAX * 2 * L->t_box_max * tc::BM * 4 : 0);
   L->gemm_counters = take(t.wdtype == 1 ? (size_t)TC_COUNTERS * 4 : 0);
   // split-tile partial sums of the persistent kernel: two sets (alternate GEMM phases) of one slot per CTA;
@@ -1237,6 +1242,83 @@ int forward(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, int n_logi
   return forward_rows<bf16>(ctx, M, T, logit_first_row, n_logit_rows, logits_out);
 }
 
+// ---------------------------------------------------------------------------------------------
+// Small fp32 models: a pass in one launch (small_f32.cuh).
+// ---------------------------------------------------------------------------------------------
+// The cluster's 16 SMs stream weights at about a quarter of the chip's rate and save some 11 launches of 4 us per
+// layer: worth it up to about 32 MB of weights a layer.  Its attention gives one row and head to eight
+// warps, which long contexts would wait for.
+bool small_eligible(const stairs_ctx* ctx, const DevModel& M, int T, int n_req, int len) {
+  const stairs_model& m = M.m;
+  const size_t nq = (size_t)m.n_heads * m.head_dim, nkv = (size_t)m.n_kv_heads * m.head_dim;
+  const size_t layer = 4 * (size_t)m.d_model * (2 * nq + 2 * nkv + (size_t)m.d_ff * (m.act == 1 ? 3 : 2));
+  return ctx->small_ctas > 0 && M.small_layers && T <= small::S_ROWS && n_req <= small::S_MAX_REQ && m.n_layers >= 1 && m.n_layers <= small::S_MAX_LAYERS &&
+         m.head_dim <= small::S_MAX_HD && small::smem_bytes(m.d_model, (int)nq, m.d_ff) <= (size_t)tc::SMEM_LIMIT && layer <= (32u << 20) && len <= 2048;
+}
+
+small::SmallParams small_params(stairs_ctx* ctx, const DevModel& M) {
+  const stairs_model& m = M.m;
+  const Layout& L = ctx->lay;
+  char* ws = ctx->ws;
+  small::SmallParams p;
+  memset(&p, 0, sizeof p);
+  p.layers = M.small_layers; p.n_layers = m.n_layers;
+  p.d = m.d_model; p.Hq = m.n_heads; p.Hkv = m.n_kv_heads; p.hd = m.head_dim; p.F = m.d_ff; p.vocab = m.vocab;
+  p.norm_kind = m.norm; p.act = m.act; p.rope = m.pos; p.theta = m.rope_theta; p.eps = m.norm_eps;
+  p.tok_emb = (const float*)M.w.tok_emb; p.pos_emb = m.pos == 0 ? (const float*)M.w.pos_emb : nullptr;
+  p.fnw = (const float*)M.w.final_norm_w; p.fnb = m.norm == 0 ? (const float*)M.w.final_norm_b : nullptr; p.head = (const float*)M.w.lm_head;
+  p.steps = 1; p.k_max = ctx->cfg.k_max; p.status = ctx->status_dev; p.wait_limit = ctx->wait_limit;
+  p.seq = reinterpret_cast<int*>(ws + L.seq); p.n_seq = reinterpret_cast<int*>(ws + L.n_seq); p.max_seq_len = ctx->cfg.max_seq_len;
+  p.page_table = reinterpret_cast<int*>(ws + L.page_table); p.page_tokens = ctx->cfg.kv_page_tokens; p.max_pages = L.max_pages;
+  return p;
+}
+
+int launch_small(stairs_ctx* ctx, const DevModel& M, const small::SmallParams& p) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ctx->small_ctas); cfg.blockDim = dim3(small::S_THREADS); cfg.dynamicSmemBytes = small::smem_bytes(M.m.d_model, M.m.n_heads * M.m.head_dim, M.m.d_ff); cfg.stream = ctx->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = ctx->small_ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  ctx->launches++;
+  CK(cudaLaunchKernelEx(&cfg, small::k_small, p));
+  return STAIRS_OK;
+}
+
+// Uploads a model's per-layer pointers and finds the largest cluster that can run.
+int setup_small(stairs_ctx* ctx, DevModel& M, size_t off) {
+  std::vector<small::SmallLayer> v(M.m.n_layers);
+  for (int l = 0; l < M.m.n_layers; ++l) {
+    const stairs_layer_w& w = M.layers[l];
+    auto f = [](const void* q) { return (const float*)q; };
+    v[l] = {f(w.norm1_w), M.m.norm == 0 ? f(w.norm1_b) : nullptr, f(w.wq), f(w.wk), f(w.wv), f(w.wo), f(w.norm2_w), M.m.norm == 0 ? f(w.norm2_b) : nullptr,
+            f(w.w_gate_or_fc1), f(w.w_up), f(w.w_down_or_fc2), reinterpret_cast<float*>(M.kpool + (size_t)l * M.kv_layer_bytes),
+            reinterpret_cast<float*>(M.vpool + (size_t)l * M.kv_layer_bytes)};
+  }
+  if (v.empty()) return STAIRS_OK;
+  uintptr_t bits = (uintptr_t)M.w.tok_emb | (uintptr_t)M.w.pos_emb | (uintptr_t)M.w.final_norm_w | (uintptr_t)M.w.final_norm_b | (uintptr_t)M.w.lm_head;
+  for (const small::SmallLayer& w : v)
+    for (const float* q : {w.n1w, w.n1b, w.wq, w.wk, w.wv, w.wo, w.n2w, w.n2b, w.w1, w.w3, w.w2}) bits |= (uintptr_t)q;
+  if (bits & 15) return STAIRS_OK;   // (16-byte copies)
+  CK(cudaMemcpyAsync(ctx->ws + off, v.data(), v.size() * sizeof(small::SmallLayer), cudaMemcpyHostToDevice, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  M.small_layers = reinterpret_cast<const small::SmallLayer*>(ctx->ws + off);
+  if (ctx->small_ctas == 0) {
+    CK(cudaFuncSetAttribute(small::k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT));
+    CK(cudaFuncSetAttribute(small::k_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    for (int n = 16; n >= 4 && ctx->small_ctas == 0; n /= 2) {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(n); cfg.blockDim = dim3(small::S_THREADS); cfg.dynamicSmemBytes = tc::SMEM_LIMIT;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = n; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      cfg.attrs = at; cfg.numAttrs = 1;
+      int clusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&clusters, small::k_small, &cfg) == cudaSuccess && clusters >= 1) ctx->small_ctas = n;
+      else cudaGetLastError();
+    }
+  }
+  return STAIRS_OK;
+}
+
 RowParams base_rows(stairs_ctx* ctx) {
   RowParams p{};
   char* ws = ctx->ws;
@@ -1281,10 +1363,18 @@ int prefill_model(stairs_ctx* ctx, DevModel& M, int slot, int n_ctx) {
     return launch_forward_mk(ctx, M, n_ctx, 0, 0, c);
   }
   // longer: chunks of equal length
-  const bool wide = wide_eligible(ctx, M);
-  const int most = prefill_rows(ctx->cfg), n_chunks = (n_ctx + most - 1) / most, chunk = (n_ctx + n_chunks - 1) / n_chunks;
+  const bool wide = wide_eligible(ctx, M), tiny = small_eligible(ctx, M, 1, 1, n_ctx);
+  const int most = tiny ? std::min(prefill_rows(ctx->cfg), (int)small::S_ROWS) : prefill_rows(ctx->cfg);
+  const int n_chunks = (n_ctx + most - 1) / most, chunk = (n_ctx + n_chunks - 1) / n_chunks;
   for (int c0 = 0; c0 < n_ctx; c0 += chunk) {
     const int n = std::min(chunk, n_ctx - c0);
+    if (tiny) {
+      small::SmallParams sp = small_params(ctx, M);
+      sp.mode = ROWS_PREFILL; sp.slot = slot; sp.first = c0; sp.T = n;
+      const int rc = launch_small(ctx, M, sp);
+      if (rc) return rc;
+      continue;
+    }
     RowParams p = base_rows(ctx);
     p.mode = ROWS_PREFILL; p.slot = slot; p.first = c0; p.n_rows = n;
     int rc = launch_rows(ctx, p, n);
@@ -1409,6 +1499,15 @@ int stairs_init(const stairs_config* cfg, const stairs_weights* target, const st
       delete ctx;
       return rc;
     }
+    if (cfg->target.wdtype == 0 && cfg->gemm_impl == 0 && major >= 9) {
+      int rc = setup_small(ctx, ctx->target, L.small_t);
+      if (!rc && has_draft) rc = setup_small(ctx, ctx->draft, L.small_d);
+      if (rc) {
+        g_init_error = ctx->err;
+        stairs_destroy(ctx);
+        return rc;
+      }
+    }
     if (cfg->target.wdtype == 1 && cfg->gemm_impl != 1) {
       if (major != 10) {
         int rc = fail(nullptr, STAIRS_EUNSUPPORTED, "bf16 models need an sm_100 device (found compute capability %d.x)", major);
@@ -1518,6 +1617,11 @@ int stairs_draft(stairs_ctx* ctx, int req, int k, int32_t* draft_dev) {
     return fail(ctx, STAIRS_ENOSPC, "request %d: sequence would exceed max_seq_len", req);
   rc = ensure_pages(ctx, req, ctx->n_seq_ub[req] + k);
   if (rc) return rc;
+  if (small_eligible(ctx, ctx->draft, 2, 1, ctx->n_seq_ub[req] + k)) {
+    small::SmallParams sp = small_params(ctx, ctx->draft);
+    sp.mode = ROWS_DRAFT_FIRST; sp.slot = req; sp.steps = k; sp.head_rows = 1; sp.draft_out = draft_dev;
+    return launch_small(ctx, ctx->draft, sp);
+  }
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(ctx->ws + ctx->lay.keys);
   for (int j = 0; j < k; ++j) {
     RowParams p = base_rows(ctx);
@@ -1580,6 +1684,20 @@ int stairs_validate(stairs_ctx* ctx, int n_req, const int32_t* req_ids_host, con
       for (int i = 0; i < n_req; ++i) ctx->n_seq_ub[req_ids_host[i]] += k_host[i] + 1;
     return STAIRS_OK;
   }
+  int len_all = 0;
+  for (int i = 0; i < n_req; ++i) len_all = std::max(len_all, ctx->n_seq_ub[req_ids_host[i]] + k_host[i]);
+  if (small_eligible(ctx, ctx->target, T, n_req, len_all)) {
+    small::SmallParams sp = small_params(ctx, ctx->target);
+    sp.mode = ROWS_VALIDATE; sp.T = T; sp.n_req = n_req; sp.head_rows = 1; sp.draft = draft_dev;
+    for (int i = 0; i < n_req; ++i) { sp.val_req[i] = req_ids_host[i]; sp.val_k[i] = k_host[i]; sp.val_off[i] = off[i]; }
+    sp.logits = logits_dev_or_null; sp.target_tokens = target_tokens_dev; sp.accept_len = accept_len_dev; sp.commit = commit;
+    int rc = launch_small(ctx, ctx->target, sp);
+    if (rc) return rc;
+    if (ctx->profile) cudaEventRecord(ctx->call_end, ctx->stream);
+    if (commit)
+      for (int i = 0; i < n_req; ++i) ctx->n_seq_ub[req_ids_host[i]] += k_host[i] + 1;
+    return STAIRS_OK;
+  }
   CK(cudaMemcpyAsync(ws + L.val_req, req_ids_host, (size_t)n_req * 4, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ws + L.val_k, k_host, (size_t)n_req * 4, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ws + L.val_off, off.data(), (size_t)n_req * 4, cudaMemcpyHostToDevice, ctx->stream));
@@ -1591,9 +1709,9 @@ int stairs_validate(stairs_ctx* ctx, int n_req, const int32_t* req_ids_host, con
     wide::WideAttn a2{};
     a2.page_table = reinterpret_cast<const int*>(ws + L.page_table); a2.page_tokens = ctx->cfg.kv_page_tokens; a2.max_pages = L.max_pages;
     a2.val_req = p.val_req; a2.val_k = p.val_k; a2.val_off = p.val_off; a2.n_seq = p.n_seq;
-    int r_max = 0, len_max = 0;
-    for (int i = 0; i < n_req; ++i) { r_max = std::max(r_max, k_host[i] + 1); len_max = std::max(len_max, ctx->n_seq_ub[req_ids_host[i]] + k_host[i]); }
-    rc = forward_wide(ctx, ctx->target, T, T, logits_dev_or_null, a2, n_req, r_max, len_max);
+    int r_max = 0;
+    for (int i = 0; i < n_req; ++i) r_max = std::max(r_max, k_host[i] + 1);
+    rc = forward_wide(ctx, ctx->target, T, T, logits_dev_or_null, a2, n_req, r_max, len_all);
   } else if (!rc) {
     rc = forward(ctx, ctx->target, T, 0, T, logits_dev_or_null);
   }
