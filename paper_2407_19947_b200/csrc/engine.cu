@@ -578,10 +578,10 @@ MkPlan mk_plan(const stairs_ctx* ctx, const stairs_model& m, int t_box, int q_ro
   // copy path: two K/V chunk buffers where they are cheap (small heads) or needed (contexts so long
   // that a unit walks several chunks)
   pl.att_dbl = (hd <= 64 || (long long)ctx->cfg.max_seq_len * m.n_kv_heads / mk::ATT_CHUNK > 2ll * ctx->sm_count) ? 1 : 0;
-  pl.att_tma = (ctx->att_tma_off == 0 && (hd == 64 || hd == 128)) ? 1 : 0;
+  pl.att_tma = (ctx->att_tma_off == 0 && hd >= 64) ? 1 : 0;   // (below 64 a bulk copy would bring several heads)
   // tcgen05 attention: possible where the bulk-copy path is; used by the calls it pays for (tc_call, see
   // launch_forward_mk); tc_call < 0 plans for the mode that needs more shared memory
-  const bool tc_possible = pl.att_tma && ctx->att_tc_off == 0;
+  const bool tc_possible = pl.att_tma && hd % 64 == 0 && ctx->att_tc_off == 0;
   pl.att_tc = (tc_possible && tc_call != 0) ? 1 : 0;
   pl.att_qblk = pl.att_tc ? mk::ATT_QBLK_TC : mk::ATT_QBLK;
   pl.att_q_rows = pl.att_tc ? (q_rows_call > 0 ? std::min(q_rows_max, round8(q_rows_call)) : q_rows_max) : 0;
@@ -637,7 +637,7 @@ int build_program(stairs_ctx* ctx, DevModel& M, int t_box, int kps) {
   const int i_kv = i_head + 4;
   const int kv_box_rows = std::min(ctx->cfg.kv_page_tokens, mk::ATT_CHUNK);
   const long long pool_rows = (long long)L.n_pages * ctx->cfg.kv_page_tokens;
-  if (m.head_dim % 64 == 0)
+  if (m.head_dim >= 64)
     for (int l = 0; l < m.n_layers && ok; ++l)
       ok = ok && encode_kv_map(ctx, &maps[i_kv + 2 * l], M.kpool + (size_t)l * M.kv_layer_bytes, pool_rows, nkv, kv_box_rows) &&
            encode_kv_map(ctx, &maps[i_kv + 2 * l + 1], M.vpool + (size_t)l * M.kv_layer_bytes, pool_rows, nkv, kv_box_rows);
@@ -842,7 +842,7 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
   P.trace = (ctx->profile && &M == &ctx->target) ? reinterpret_cast<unsigned long long*>(ws + L.mk_trace) : nullptr;
   const int grid = std::min(ctx->sm_count, TC_GRID_MAX);
   void* args[] = {&P};
-  CK(cudaLaunchCooperativeKernel((const void*)mk::k_forward, dim3(grid), dim3(mk::MK_THREADS), args,
+  CK(cudaLaunchCooperativeKernel((const void*)mk::forward_fn(m, P.att_tma, P.att_tc, T), dim3(grid), dim3(mk::MK_THREADS), args,
                                  mk::smem_bytes(t_box, P.stages, m.head_dim, P.att_dbl, P.kps, P.att_tma, P.att_nbuf, P.att_q_rows), ctx->stream));
   ctx->bar_base += (unsigned long long)n_run * grid;
   ctx->launches++;
@@ -1540,7 +1540,11 @@ int stairs_init(const stairs_config* cfg, const stairs_weights* target, const st
       const int hkvm = has_draft ? std::max(cfg->target.n_kv_heads, cfg->draft.n_kv_heads) : cfg->target.n_kv_heads;
       const bool fits = mk::pick_stages(MK_MAX_ROWS, hdm, 1, 1) >= 3 && worst_chunks * hkvm / 64 <= 2 * std::min(ctx->sm_count, TC_GRID_MAX);
       if (coop && fits && cfg->gemm_impl == 0) {
-        e = cudaFuncSetAttribute(mk::k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
+        e = cudaSuccess;
+        for (int i = 0; i < 16 && e == cudaSuccess; ++i) {   // (every kernel the two models' calls may launch: also loads its code now)
+          const stairs_model& fm = i < 8 || !has_draft ? cfg->target : cfg->draft;
+          e = cudaFuncSetAttribute((const void*)mk::forward_fn(fm, i & 1, (i >> 1) & 1, i & 4 ? 1 : 64), cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
+        }
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_attn_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide::tc_att_smem<64>());
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_attn_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide::tc_att_smem<128>());

@@ -30,7 +30,7 @@
 //    tiled bulk copies (128-byte swizzle) through a ring of buffers; S = Q.K^T and O += P.V as
 //    tcgen05 MMAs (M = 128 queries, accumulators in TMEM) issued by the MMA warp one chunk ahead of
 //    the compute group's base-2 online softmax;
-//  - head sizes 64/128 otherwise: the same ring, contractions on fp16 mma.sync tiles, one warp per
+//  - head sizes of 64 and more otherwise: the same ring, contractions on fp16 mma.sync tiles, one warp per
 //    16-query block, softmax state in registers;
 //  - other head sizes: padded tiles staged by 16-byte asynchronous copies from the compute warps.
 // Unit boundaries depend only on the request's own committed length, never on the other requests.
@@ -110,7 +110,7 @@ struct Params {
   int stat_tiles;
   const float* rope_inv;
   int att_dbl;               // attention, copy path: two K/V chunk buffers, the next chunk's copies fly under the current chunk's MMAs
-  int att_tma;               // attention, TMA path (head sizes 64 and 128): a loader warp streams K/V chunks through att_nbuf buffers
+  int att_tma;               // attention, TMA path (head sizes from 64 on): a loader warp streams K/V chunks through att_nbuf buffers
   int att_nbuf;
   int kv_box_rows;           // rows of one K/V box: min(page_tokens, chunk)
   int att_tc;                // attention on tcgen05 (with att_tma): S = Q.K^T and O += P.V as M = 128 MMAs, accumulators in TMEM
@@ -140,13 +140,39 @@ constexpr int ATT_QBLK_TC = 128;                // ... on the tcgen05 path (the 
 constexpr int VT_LD = 132;                      // row pitch (floats) of the epilogue's 16 x 128 exchange tile
 constexpr int MK_XCH_BYTES = 16 * VT_LD * 4;     // the tile itself
 
+// What a launch knows at compile time.  Every phase runs its code once, so a phase's critical chain is bound by
+// instruction fetch (the kernel's text is far larger than the SM's instruction caches): a test that always goes the same
+// way, or an address computed from a run-time head size, costs what it adds to the text.  With the head size, the model
+// family, the attention path and "at most 16 rows" fixed, a validate call of 9 rows took 2728 us where the general code
+// took 2838 (7B), 1021 where it took 1134 (0.4B); 3B, 5 rows: 1959 and 2072.  HD 0, FAM 0, ATT -1 and ONE false are the general code.
+//   FAM 1: LayerNorm, GELU, learned positions; FAM 2: RMSNorm, SwiGLU, rotary positions
+//   ATT 0: bulk copies, contractions on mma.sync; 1: on tcgen05; 2: 16-byte copies
+template <int HD, int FAM, int ATT, bool ONE_CHUNK>
+struct Spec {
+  static constexpr bool ONE = ONE_CHUNK;
+  static __device__ __forceinline__ int hd(const Params& P) { return HD ? HD : P.hd; }
+  static __device__ __forceinline__ bool layer_norm(const Params& P) { return FAM ? FAM == 1 : P.norm_kind == 0; }
+  static __device__ __forceinline__ bool rope(const Params& P) { return FAM ? FAM == 2 : P.rope != 0; }
+  static __device__ __forceinline__ bool dual(const Phase& p) { return FAM != 1 && p.dual; }
+  static __device__ __forceinline__ bool swiglu(const Phase& p) { return FAM != 1 && p.epi == TC_SWIGLU; }
+  static __device__ __forceinline__ bool gelu(const Phase& p) { return FAM != 2 && p.epi == TC_GELU; }
+  static __device__ __forceinline__ bool store(const Phase& p) { return FAM != 1 && (HD == 0 || HD % 64 != 0) && p.epi == TC_STORE_F32; }
+  static __device__ __forceinline__ bool shifted(const Phase& p) { return FAM ? FAM == 1 : p.u != nullptr; }   // (LayerNorm: y = rstd (acc - mean u) + c)
+  static __device__ __forceinline__ bool tc(const Params& P) { return ATT < 0 ? P.att_tc != 0 : ATT == 1; }
+  static __device__ __forceinline__ bool tma(const Params& P) { return ATT < 0 ? P.att_tma != 0 : ATT != 2; }
+  static __device__ __forceinline__ int qblk(const Params& P) { return ATT < 0 ? P.att_qblk : ATT == 1 ? ATT_QBLK_TC : ATT_QBLK; }
+  static __device__ __forceinline__ bool prep(const Params& P) { return HD % 64 != 0 || HD == 0; }             // may the program hold PH_PREP phases?
+};
+
 struct AttnSmem {   // carved after the GEMM ring: Q block (bf16), K and V chunk tiles (bf16), merge buffer (fp32)
   static __host__ __device__ size_t k_pitch(int hd) { return (size_t)hd * 2 + 16; }
   static __host__ __device__ size_t q_bytes(int hd) { return (size_t)ATT_QBLK * k_pitch(hd); }
   static __host__ __device__ size_t kv_bytes(int hd) { return (size_t)ATT_CHUNK * k_pitch(hd); }
   static __host__ __device__ size_t merge_bytes(int hd) { return (size_t)16 * (hd + 4) * 4 + 64; }
-  // TMA path: a chunk buffer holds K then V, each as hd / 64 column halves of [CHUNK rows][128 bytes] with the 128-byte swizzle
-  static __host__ __device__ size_t kv_buf_bytes(int hd) { return (size_t)2 * ATT_CHUNK * hd * 2; }
+  // TMA path: a chunk buffer holds K then V, each as 64-column parts of [CHUNK rows][128 bytes] with the 128-byte swizzle (the
+  // last part of a head size that is no multiple of 64 brings columns of the next head, or zeros, that nothing reads)
+  static __host__ __device__ int parts(int hd) { return (hd + 63) / 64; }
+  static __host__ __device__ size_t kv_buf_bytes(int hd) { return (size_t)2 * ATT_CHUNK * parts(hd) * 128; }
   // copy path: Q block, then one or two padded K/V buffers; TMA path: nbuf chunk buffers (1024-byte aligned), then the Q block
   // tcgen05 path (tc_q_rows > 0): Q tile (hd / 64 halves of [q_rows][128 bytes]) and P tile ([q_rows][128 bytes]),
   // both swizzled, then the chunk buffers; an M = 128 MMA reads 128 rows from a tile's start, so at
@@ -558,8 +584,10 @@ __device__ __forceinline__ AttnReq attn_req(const Params& P, int i, int G) {
   a.n_chunks = (a.base + a.R + ATT_CHUNK - 1) / ATT_CHUNK;
   // chunks per unit: from the first row's position only (so it is the same for any draft length)
   const int c0 = (a.base + ATT_CHUNK) / ATT_CHUNK;
-  int cpu = 1;
-  while (cpu < 64 && P.Hkv * ((c0 + cpu - 1) / cpu) > G) cpu <<= 1;   // one unit per CTA where possible: a unit's fixed cost exceeds a chunk's
+  // One unit per CTA where possible (a unit's fixed cost exceeds a chunk's): G / Hkv ranges at most, ceil(c0 / ranges)
+  // chunks each.  (Rounded up to a power of two, 9 chunks x 32 heads on 148 CTAs were 4 a unit; now 3.)
+  const int ranges = max(1, G / P.Hkv);
+  const int cpu = min(64, (c0 + ranges - 1) / ranges);
   a.cpu = cpu;
   a.n_ranges = (a.n_chunks + cpu - 1) / cpu;
   a.n_qblk = (a.R * (P.Hq / P.Hkv) + P.att_qblk - 1) / P.att_qblk;
@@ -573,9 +601,10 @@ __device__ __forceinline__ AttnReq attn_req(const Params& P, int i, int G) {
 struct KvCons { int buf; uint32_t par; uint32_t sc; uint32_t o_par; };   // sc: chunks of the tcgen05 path so far (S / P buffer = sc & 1)
 
 // First chunk buffer of the TMA paths (1024-byte aligned; the tcgen05 path keeps its Q and P tiles in front of it).
+template <class S>
 __device__ __forceinline__ uint8_t* att_ring_base(const Params& P, uint8_t* att_smem) {
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(att_smem) + 1023) & ~(uintptr_t)1023);
-  return P.att_tc ? base + AttnSmem::tc_head_bytes(P.hd, P.att_q_rows) : base;
+  return S::tc(P) ? base + AttnSmem::tc_head_bytes(S::hd(P), P.att_q_rows) : base;
 }
 
 // One attention unit, executed by the 128 compute threads (4 warps), on the legacy tensor path
@@ -586,17 +615,17 @@ __device__ __forceinline__ uint8_t* att_ring_base(const Params& P, uint8_t* att_
 // each chunk's positions in two and merge once per unit.  The block's result is either final
 // (the unit saw every visible position) or parked for the merge at the end of the attention phase.
 //
-// K/V chunks of 64 positions reach shared memory in one of two ways.  TMA path (head sizes 64 and
-// 128): the loader warp streams them through a ring of buffers with tiled bulk copies (one box per
+// K/V chunks of 64 positions reach shared memory in one of two ways.  TMA path (head sizes from 64
+// on; size 80 came by the copy path before, 2.8 us a chunk): the loader warp streams them through a ring of buffers with tiled bulk copies (one box per
 // page slice and 64-column half, 128-byte swizzle) and this function only waits on the ring's
 // barriers - chunks of already cached positions are in flight before the phase even starts.
 // Copy path (other head sizes): the compute threads stage padded tiles with 16-byte asynchronous
 // copies, cache rows looked up once per chunk.
-template <bool TMA>
+template <class S, bool TMA>
 __device__ void attn_unit(const Params& P, const Phase& ph, const AttnReq& a, int kvh, int range, int qblk, int part_slot, int part_set,
                           uint8_t* att_smem, Ctl* ctl, int et, bool& ok, KvCons& kvc, const Waiter& W,
                           unsigned long long* tra) {
-  const int hd = P.hd, G = P.Hq / P.Hkv, nkv = P.Hkv * hd, nq = P.Hq * hd;
+  const int hd = S::hd(P), G = P.Hq / P.Hkv, nkv = P.Hkv * hd, nq = P.Hq * hd;
   const int lane = et & 31, w = et >> 5, g = lane >> 2, t4 = lane & 3;
   const int Q = a.R * G;
   const int q0 = qblk * ATT_QBLK, nQ = min(ATT_QBLK, Q - q0);
@@ -604,7 +633,7 @@ __device__ void attn_unit(const Params& P, const Phase& ph, const AttnReq& a, in
   const size_t kvb = AttnSmem::kv_bytes(hd);
   const size_t kvbuf = AttnSmem::kv_buf_bytes(hd);
   // TMA path: ring of chunk buffers (1024-byte aligned) then the Q block; copy path: Q block then padded buffers
-  uint8_t* ring = att_ring_base(P, att_smem);
+  uint8_t* ring = att_ring_base<S>(P, att_smem);
   uint8_t* qs = TMA ? ring + (size_t)P.att_nbuf * kvbuf : att_smem;   // [QBLK][pitch] fp16, rotated and pre-scaled
   uint8_t* kv0 = qs + AttnSmem::q_bytes(hd);                // copy path, buffer b: K [CHUNK][pitch] then V, at kv0 + b * 2 * kvb
   uint8_t* ks = kv0;                                        // the buffer being computed on
@@ -895,7 +924,7 @@ __device__ void attn_unit(const Params& P, const Phase& ph, const AttnReq& a, in
     for (int half_row = 0; half_row < 2; ++half_row) {
       const int ql = half_row ? ql_b : ql_a;
       if (ql < nQ) {
-        float* dst = P.attn_part + (size_t)part_set * P.attn_set_stride + ((size_t)part_slot * P.att_qblk + ql) * (hd + 4);
+        float* dst = P.attn_part + (size_t)part_set * P.attn_set_stride + ((size_t)part_slot * S::qblk(P) + ql) * (hd + 4);
 #pragma unroll
         for (int nd = 0; nd < 16; ++nd)
           if (nd < ntiles)
@@ -949,14 +978,15 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
 // When a running maximum moves, the warp rescales its rows of O in TMEM (load, multiply, store) after
 // the previous P.V has completed and before it releases the P tile.  Rows past the unit's queries run
 // along on zero queries.  This function is the compute group's side.
+template <class S>
 __device__ __noinline__ void attn_unit_tc(const Params& P, const Phase& ph, const AttnReq& a, int kvh, int range, int qblk, int part_slot, int part_set,
                                           uint8_t* att_smem, Ctl* ctl, int et, bool& ok, KvCons& kvc, const Waiter& W,
                                           uint32_t tmem_s, uint32_t tmem_o) {
-  const int hd = P.hd, G = P.Hq / P.Hkv, nq = P.Hq * hd, halves = hd / 64;
+  const int hd = S::hd(P), G = P.Hq / P.Hkv, nq = P.Hq * hd, halves = hd / 64;
   const int lane = et & 31, quad = ((et >> 5) + 2) & 3;       // compute warps are warps 2..5: TMEM lane quadrant = warp & 3
   const int ql = quad * 32 + lane;                             // this thread's query row (TMEM lane)
   const int Q = a.R * G;
-  const int q0 = qblk * P.att_qblk, nQ = min(P.att_qblk, Q - q0);
+  const int q0 = qblk * S::qblk(P), nQ = min(S::qblk(P), Q - q0);
   const int q_rows = P.att_q_rows;
   uint8_t* qs = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(att_smem) + 1023) & ~(uintptr_t)1023);   // halves x [q_rows][128 B]
   uint8_t* psm = qs + (size_t)halves * q_rows * 128;           // two P tiles of [q_rows][128 B]
@@ -1087,7 +1117,7 @@ __device__ __noinline__ void attn_unit_tc(const Params& P, const Phase& ph, cons
   const int q = q0 + (mine ? ql : 0);
   const float inv = a.n_ranges == 1 ? (l_run > 0.f ? 1.0f / l_run : 0.f) : 1.0f;
   bf16* orow = P.o + (size_t)(a.off + q / G) * P.Hq * hd + (size_t)(kvh * G + q % G) * hd;
-  float* prow = P.attn_part + (size_t)part_set * P.attn_set_stride + ((size_t)part_slot * P.att_qblk + (mine ? ql : 0)) * (hd + 4);
+  float* prow = P.attn_part + (size_t)part_set * P.attn_set_stride + ((size_t)part_slot * S::qblk(P) + (mine ? ql : 0)) * (hd + 4);
   for (int d0 = 0; d0 < hd; d0 += 16) {
     float ov[16];
     tmem_ld16(tmem_o + lane_sel + (uint32_t)d0, ov);
@@ -1113,9 +1143,10 @@ __device__ __noinline__ void attn_unit_tc(const Params& P, const Phase& ph, cons
 // signals the compute group, commits after each P.V hand the chunk buffer back to the loader and
 // publish the completion.  mc: this thread's running state across phases.
 struct AttIssue { int buf; uint32_t par; uint32_t sc; uint32_t q_par; };
+template <class S>
 __device__ __noinline__ bool attn_issue_tc(const Params& P, Ctl* ctl, uint8_t* att_smem, int cta, int G, const Waiter& W,
                                            uint32_t tmem_s, uint32_t tmem_o, AttIssue& mc) {
-  const int hd = P.hd, halves = hd / 64, q_rows = P.att_q_rows;
+  const int hd = S::hd(P), halves = hd / 64, q_rows = P.att_q_rows;
   uint8_t* qs = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(att_smem) + 1023) & ~(uintptr_t)1023);
   uint8_t* psm = qs + (size_t)halves * q_rows * 128;
   uint8_t* ring = psm + (size_t)2 * q_rows * 128;
@@ -1184,6 +1215,7 @@ __device__ __noinline__ bool attn_issue_tc(const Params& P, Ctl* ctl, uint8_t* a
 // ---------------------------------------------------------------------------------------------
 // The kernel
 // ---------------------------------------------------------------------------------------------
+template <class S>
 __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant__ Params P) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -1202,14 +1234,14 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
   uint32_t tmem_cols = 32;
   // two GEMM accumulators, each with hi-part and lo-part columns; tcgen05 attention adds S (one chunk) and O (head size)
   const uint32_t tmem_att = (uint32_t)(4 * P.t_box);
-  while ((int)tmem_cols < 4 * P.t_box + (P.att_tc ? 2 * ATT_CHUNK + P.hd : 0)) tmem_cols <<= 1;   // two S buffers, O
+  while ((int)tmem_cols < 4 * P.t_box + (S::tc(P) ? 2 * ATT_CHUNK + S::hd(P) : 0)) tmem_cols <<= 1;   // two S buffers, O
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(ctl->full + s, 1); mbar_init(ctl->empty + s, 1); }
     mbar_init(ctl->acc_full + 0, 1); mbar_init(ctl->acc_full + 1, 1);
     mbar_init(ctl->acc_empty + 0, 4); mbar_init(ctl->acc_empty + 1, 4);
     // a chunk buffer is handed back by the four compute warps (mma.sync path) or by one tcgen05.commit
-    for (int b = 0; b < MAX_KV_BUF; ++b) { mbar_init(ctl->kv_full + b, 1); mbar_init(ctl->kv_empty + b, P.att_tc ? 1 : 4); }
+    for (int b = 0; b < MAX_KV_BUF; ++b) { mbar_init(ctl->kv_full + b, 1); mbar_init(ctl->kv_empty + b, S::tc(P) ? 1 : 4); }
     mbar_init(ctl->s_full + 0, 1); mbar_init(ctl->s_full + 1, 1);
     mbar_init(ctl->p_full + 0, 4); mbar_init(ctl->p_full + 1, 4);
     mbar_init(&ctl->q_full, 4); mbar_init(&ctl->o_done, 1);
@@ -1302,14 +1334,14 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
       bool areq_seen = false;
       for (int ph = 0; ph < P.n_phases && ok; ++ph) {
         const Phase& p = P.phases[ph];
-        if (p.kind == PH_ATTN && P.att_tc) {
+        if (p.kind == PH_ATTN && S::tc(P)) {
           // attention contractions of this CTA's units (the compute group does the softmax in between)
           if (!areq_seen) {
             const long long t0 = clock64();
             while (!(areq_seen = ctl->areq_ready != 0)) { if (W.poll_abort(t0)) break; }
             if (!areq_seen) { ok = false; break; }
           }
-          ok = attn_issue_tc(P, ctl, att_smem, cta, G, W, tmem_base + tmem_att, tmem_base + tmem_att + 2 * ATT_CHUNK, att_mc);
+          ok = attn_issue_tc<S>(P, ctl, att_smem, cta, G, W, tmem_base + tmem_att, tmem_base + tmem_att + 2 * ATT_CHUNK, att_mc);
           continue;
         }
         if (p.kind != PH_GEMM) continue;
@@ -1370,7 +1402,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
     // 64-column half, page slice), each issued by its own lane.  Chunks that hold only positions
     // cached by earlier calls are fetched as soon as a buffer is free - also ahead of the phase;
     // a chunk with positions of this call waits for the grid barrier that publishes them.
-    if (P.att_tma) {
+    if (S::tma(P)) {
       bool ok = true;
       {
         bool seen = false;
@@ -1381,10 +1413,10 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
         ok = __shfl_sync(0xffffffffu, seen ? 1 : 0, 0) != 0;
         __syncwarp();
       }
-      const int hd = P.hd, halves = hd / 64, box_rows = P.kv_box_rows, slots = ATT_CHUNK / box_rows;
+      const int hd = S::hd(P), halves = AttnSmem::parts(hd), box_rows = P.kv_box_rows, slots = ATT_CHUNK / box_rows;
       const int n_boxes = 2 * halves * slots;
       const size_t kvbuf = AttnSmem::kv_buf_bytes(hd);
-      uint8_t* ring = att_ring_base(P, att_smem);
+      uint8_t* ring = att_ring_base<S>(P, att_smem);
       // this lane's box: which tensor (K, V), which 64-column half, which page slice of the chunk
       const int b_which = lane / (halves * slots), b_half = (lane % (halves * slots)) / slots, b_slot = lane % slots;
       int buf = 0; uint32_t par = 0;
@@ -1466,11 +1498,11 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
       if (et < PH_WORDS) ctl->phc[0][et] = __ldcg(reinterpret_cast<const uint32_t*>(P.phases) + et);
       const int n_req0 = P.mode == CALL_VALIDATE ? P.n_req : 1;
       if (et < n_req0 && et < 64) ctl->areq[et] = attn_req(P, et, G);
-      if (P.att_tma) {
+      if (S::tma(P)) {
         // the chunk buffers start out finite: a box that is never fetched (past the page table) must not feed NaNs to P.V
-        uint8_t* ring = att_ring_base(P, att_smem);
+        uint8_t* ring = att_ring_base<S>(P, att_smem);
         uint8_t* first = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(att_smem) + 1023) & ~(uintptr_t)1023);   // (the Q and P tiles too)
-        const int n16 = (int)((size_t)(ring - first) + (size_t)P.att_nbuf * AttnSmem::kv_buf_bytes(P.hd)) / 16;
+        const int n16 = (int)((size_t)(ring - first) + (size_t)P.att_nbuf * AttnSmem::kv_buf_bytes(S::hd(P))) / 16;
         for (int i = et; i < n16; i += 128) reinterpret_cast<uint4*>(first)[i] = make_uint4(0u, 0u, 0u, 0u);
         fence_proxy_async_smem();   // later bulk copies (async proxy) into these buffers
       }
@@ -1502,7 +1534,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
     int aph = 0;   // attention phases so far
     auto empty_own_states = [&](int set) {
       const int n_req_ = P.mode == CALL_VALIDATE ? P.n_req : 1;
-      const int Gq_ = P.Hq / P.Hkv, row_words = P.hd + 4;
+      const int Gq_ = P.Hq / P.Hkv, row_words = S::hd(P) + 4;
       int u0_ = 0;
       for (int i = 0; i < n_req_; ++i) {
         const AttnReq a = ctl->areq[i];
@@ -1510,9 +1542,9 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           const int first = (cta - u0_ % G + G) % G;
           for (int u = first; u < a.units; u += G) {
             const int qblk = u % a.n_qblk;
-            const int nQ = min(P.att_qblk, a.R * Gq_ - qblk * P.att_qblk);
+            const int nQ = min(S::qblk(P), a.R * Gq_ - qblk * S::qblk(P));
             if (u0_ + u >= P.attn_part_units) break;
-            float* st = P.attn_part + (size_t)set * P.attn_set_stride + (size_t)(u0_ + u) * P.att_qblk * row_words;
+            float* st = P.attn_part + (size_t)set * P.attn_set_stride + (size_t)(u0_ + u) * S::qblk(P) * row_words;
             for (int w4 = et; w4 < nQ * row_words / 4; w4 += 128)
               st_relaxed_u4(st + w4 * 4, make_uint4(PARTIAL_EMPTY, PARTIAL_EMPTY, PARTIAL_EMPTY, PARTIAL_EMPTY));
           }
@@ -1567,9 +1599,9 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
               break;
             }
             unsigned long long* tra_u = (MK_TRACE_PTR(P.trace) && et == 0 && u == first) ? MK_TRACE_PTR(P.trace) + (size_t)2 * P.n_phases * 8 + ((size_t)cta * P.n_phases + ph) * 8 : nullptr;
-            if (P.att_tc) attn_unit_tc(P, p, a, kvh, range, qblk, slot, aph & 1, att_smem, ctl, et, ok, kvc, W, tmem_base + tmem_att, tmem_base + tmem_att + 2 * ATT_CHUNK);
-            else if (P.att_tma) attn_unit<true>(P, p, a, kvh, range, qblk, slot, aph & 1, att_smem, ctl, et, ok, kvc, W, tra_u);
-            else attn_unit<false>(P, p, a, kvh, range, qblk, slot, aph & 1, att_smem, ctl, et, ok, kvc, W, tra_u);
+            if (S::tc(P)) attn_unit_tc<S>(P, p, a, kvh, range, qblk, slot, aph & 1, att_smem, ctl, et, ok, kvc, W, tmem_base + tmem_att, tmem_base + tmem_att + 2 * ATT_CHUNK);
+            else if (S::tma(P)) attn_unit<S, true>(P, p, a, kvh, range, qblk, slot, aph & 1, att_smem, ctl, et, ok, kvc, W, tra_u);
+            else attn_unit<S, false>(P, p, a, kvh, range, qblk, slot, aph & 1, att_smem, ctl, et, ok, kvc, W, tra_u);
           }
           u0 += a.units; g0 += P.Hkv * a.n_qblk;
         }
@@ -1579,7 +1611,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
         // from other CTAs' units of this same phase: a word reads PARTIAL_EMPTY until it has been
         // stored, and the warp repeats its loads (bounded) until none does.
         if (ok) {
-          const int hd = P.hd, Gq = P.Hq / P.Hkv;
+          const int hd = S::hd(P), Gq = P.Hq / P.Hkv;
           const float* set_base = P.attn_part + (size_t)(aph & 1) * P.attn_set_stride;
           int u0c = 0, item0 = 0;
           bool gave_up = false;
@@ -1599,10 +1631,10 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
               int it = ((cta * 4 + quad) - item0) % (G * 4);
               if (it < 0) it += G * 4;
               for (; it < items && !gave_up; it += G * 4) {
-                const int kvh = it / Q, q = it % Q, qblk = q / P.att_qblk, ql = q % P.att_qblk;
+                const int kvh = it / Q, q = it % Q, qblk = q / S::qblk(P), ql = q % S::qblk(P);
                 const int first_slot = u0c + (kvh * a.n_ranges) * a.n_qblk + qblk;
-                const size_t stride = (size_t)a.n_qblk * P.att_qblk * (hd + 4);
-                const float* base = set_base + ((size_t)first_slot * P.att_qblk + ql) * (hd + 4);
+                const size_t stride = (size_t)a.n_qblk * S::qblk(P) * (hd + 4);
+                const float* base = set_base + ((size_t)first_slot * S::qblk(P) + ql) * (hd + 4);
                 // (max, sum) of range lane, lane + 32, ...: one load round for up to 32 ranges, then
                 // the ranges' output vectors eight loads at a time; weights travel by shuffle and
                 // the accumulation stays in range order
@@ -1674,18 +1706,18 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           }
         }
         ++aph;
-      } else if (p.kind == PH_PREP) {
+      } else if (S::prep(P) && p.kind == PH_PREP) {
         // Models whose head size is neither 64 nor 128: a rotation pair (i, i + hd/2) need not sit in
         // one thread (or one tile) of the QKV epilogue, so that epilogue stores fp32 and this extra
         // phase rotates, converts and files q, k and v.  One item = one pair of one head of one row.
-        const int hd = P.hd, half = hd / 2, nq = P.Hq * hd, nkv = P.Hkv * hd, nqkv = nq + 2 * nkv, heads = P.Hq + 2 * P.Hkv;
+        const int hd = S::hd(P), half = hd / 2, nq = P.Hq * hd, nkv = P.Hkv * hd, nqkv = nq + 2 * nkv, heads = P.Hq + 2 * P.Hkv;
         const int items = P.T * heads * half;
         const float qscale = 1.4426950408889634f / sqrtf((float)hd);   // log2(e) / sqrt(hd): the softmax works in base 2
         for (int it = cta * 128 + et; it < items; it += G * 128) {
           const int i = it % half, hs = (it / half) % heads, t = it / (half * heads);
           const float* row = P.qkv + (size_t)t * nqkv + (size_t)hs * hd;   // q heads, then k heads, then v heads
           float x0 = __ldcg(row + i), x1 = __ldcg(row + i + half);
-          if (P.rope && hs < P.Hq + P.Hkv) {
+          if (S::rope(P) && hs < P.Hq + P.Hkv) {
             const float cs = __ldcg(P.rope_cs + (size_t)t * half + i), sn = __ldcg(P.rope_sn + (size_t)t * half + i);
             const float r0 = x0 * cs - x1 * sn, r1 = x1 * cs + x0 * sn;
             x0 = r0; x1 = r1;
@@ -1788,7 +1820,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
               for (int r = 0; r < 4; ++r) {
                 const int t = tb + 4 * r;
                 if (t < Tvalid) {
-                  if (P.norm_kind == 0) { ctl->mu[t] = s1[r]; ctl->rstd[t] = 1.0f / sqrtf(m2[r] / (float)P.d + P.eps); }
+                  if (S::layer_norm(P)) { ctl->mu[t] = s1[r]; ctl->rstd[t] = 1.0f / sqrtf(m2[r] / (float)P.d + P.eps); }
                   else { ctl->mu[t] = 0.f; ctl->rstd[t] = 1.0f / sqrtf((m2[r] + n[r] * s1[r] * s1[r]) / (float)P.d + P.eps); }
                 }
               }
@@ -1817,7 +1849,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           // first output column of the tile and how many of its columns exist (a tile never
           // straddles two sources)
           int n0, ncols, src_s = 0, src_col0 = 0;
-          if (p.dual) { n0 = tile * 64; ncols = min(64, p.N - n0); }
+          if (S::dual(p)) { n0 = tile * 64; ncols = min(64, p.N - n0); }
           else {
             int local = tile, col0 = 0, col1 = p.n_src > 1 ? p.src_col[1] : p.N;
             if (p.n_src > 1 && local >= p.src_tiles[0]) {
@@ -1844,8 +1876,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           auto rope_of = [&](int t, float4& c0, float4& s0, float4& c1, float4& s1) {
             // hd = 128: groups (0, 2) and (1, 3) pair up, at table columns cg*4 and 32 + cg*4;
             // hd = 64: groups (0, 1) and (2, 3), both at table column cg*4
-            const int hh = P.hd / 2;
-            const int i1 = P.hd == 128 ? 32 + cg * 4 : cg * 4;
+            const int hh = S::hd(P) / 2;
+            const int i1 = S::hd(P) == 128 ? 32 + cg * 4 : cg * 4;
             c0 = __ldcg(reinterpret_cast<const float4*>(P.rope_cs + (size_t)t * hh + cg * 4));
             s0 = __ldcg(reinterpret_cast<const float4*>(P.rope_sn + (size_t)t * hh + cg * 4));
             c1 = __ldcg(reinterpret_cast<const float4*>(P.rope_cs + (size_t)t * hh + i1));
@@ -1853,15 +1885,15 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           };
           if (finisher && p.qkv_prep && er < Tvalid) {
             if (src_s >= 1) kv_row0 = kv_row_of(er);
-            if (P.rope && src_s < 2) rope_of(er, rc0a, rs0a, rc0b, rs0b);
+            if (S::rope(P) && src_s < 2) rope_of(er, rc0a, rs0a, rc0b, rs0b);
           }
           if (finisher) {
-            const int mc = p.dual ? (m & 63) : m;
+            const int mc = S::dual(p) ? (m & 63) : m;
             const bool m_on = mc < ncols;
-            if (p.norm_in) {
-              const int ncol = (p.dual && m >= 64) ? p.N + n0 + mc : n0 + mc;
-              ctl->utile[m] = (p.u && m_on) ? p.u[ncol] : 0.f;
-              ctl->ctile[m] = (p.c && m_on) ? p.c[ncol] : 0.f;
+            if (p.norm_in && S::shifted(p)) {
+              const int ncol = (S::dual(p) && m >= 64) ? p.N + n0 + mc : n0 + mc;
+              ctl->utile[m] = (S::shifted(p) && m_on) ? p.u[ncol] : 0.f;
+              ctl->ctile[m] = (S::shifted(p) && m_on) ? p.c[ncol] : 0.f;
             }
             if (have_pre) {
 #pragma unroll
@@ -1885,7 +1917,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           if (!finisher) {
             if (tra) tra[4] = globaltimer_ns();
             float* mine = slot_of(pset, (unsigned)cta);
-            for (int c0 = 0; c0 < Tvalid; c0 += 16) {   // only rows that exist
+            for (int c0 = 0; c0 < (S::ONE ? 1 : Tvalid); c0 += 16) {   // only rows that exist
               float v[16];
               tmem_ld16(taddr + (uint32_t)c0, v);
               {
@@ -1906,7 +1938,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
             unsigned last_c = (unsigned)cta;   // CTAs cta + 1 .. last_c hold the tile's other segments
             if (!whole) while (last_c + 1 < ge32 && rb(last_c + 1) < (unsigned)tile_end) ++last_c;
             if (!whole) { pend_first = (unsigned)cta + 1u; pend_last = last_c; pend_set = pset; }   // (at most one split tile is finished per phase)
-            for (int c0 = 0; c0 < Tvalid; c0 += 16) {
+            for (int c0 = 0; c0 < (S::ONE ? 1 : Tvalid); c0 += 16) {
               {
                 float v[16];
                 tmem_ld16(taddr + (uint32_t)c0, v);
@@ -1916,7 +1948,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
 #pragma unroll
                   for (int j = 0; j < 16; ++j) v[j] += vl[j];
                 }
-                if (c0 + 16 >= Tvalid) {   // accumulator drained: the MMA warp may reuse it
+                if (S::ONE || c0 + 16 >= Tvalid) {   // accumulator drained: the MMA warp may reuse it
                   tc_fence_before();
                   if (lane == 0) mbar_arrive(ctl->acc_empty + buf);
                 }
@@ -1939,7 +1971,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
 #pragma unroll
                   for (int q = 0; q < 4; ++q) {
                     const int col = (cg + 8 * q) * 4;
-                    on[q] = row_on && (p.dual ? (col & 63) < ncols : col < ncols);
+                    on[q] = row_on && (S::dual(p) ? (col & 63) < ncols : col < ncols);
                     a[q] = on[q] ? *reinterpret_cast<const float4*>(vrow + col) : make_float4(0.f, 0.f, 0.f, 0.f);
                   }
                   if (!whole) {
@@ -2000,7 +2032,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
 #pragma unroll
                   for (int q = 0; q < 4; ++q)
                     if (on[q]) *reinterpret_cast<float4*>(vrow + (cg + 8 * q) * 4) = a[q];   // (this thread's own slots)
-                  if (add_res && c0 + 16 < Tvalid) {
+                  if (add_res && !S::ONE && c0 + 16 < Tvalid) {
                     // calls of more than 16 rows: the next chunk's old residual values are requested now,
                     // so that they do not add an L2 round trip to that chunk
                     const int tn = t + 16;
@@ -2017,10 +2049,12 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                 auto group = [&](int col) -> float4 {
                   float4 v = *reinterpret_cast<const float4*>(vrow + col);
                   if (p.norm_in) {
-                    const float4 u4 = *reinterpret_cast<const float4*>(ctl->utile + col);
-                    const float4 c4 = *reinterpret_cast<const float4*>(ctl->ctile + col);
-                    v.x = rs * (v.x - mu * u4.x) + c4.x; v.y = rs * (v.y - mu * u4.y) + c4.y;
-                    v.z = rs * (v.z - mu * u4.z) + c4.z; v.w = rs * (v.w - mu * u4.w) + c4.w;
+                    if (S::shifted(p)) {
+                      const float4 u4 = *reinterpret_cast<const float4*>(ctl->utile + col);
+                      const float4 c4 = *reinterpret_cast<const float4*>(ctl->ctile + col);
+                      v.x = rs * (v.x - mu * u4.x) + c4.x; v.y = rs * (v.y - mu * u4.y) + c4.y;
+                      v.z = rs * (v.z - mu * u4.z) + c4.z; v.w = rs * (v.w - mu * u4.w) + c4.w;
+                    } else { v.x *= rs; v.y *= rs; v.z *= rs; v.w *= rs; }
                   }
                   return v;
                 };
@@ -2057,7 +2091,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     for (int o = 1; o < 8; o <<= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
                     if (cg == 0 && row_on) P.stats[(size_t)t * P.stat_tiles + tile] = make_float4(mean, m2, cnt, 0.f);
                   }
-                } else if (p.epi == TC_SWIGLU) {
+                } else if (S::swiglu(p)) {
                   // gate columns (cg + 8 q) * 4 of the tile's first half, the matching up columns 64 further
 #pragma unroll 1
                   for (int q = 0; q < 2; ++q) {
@@ -2099,19 +2133,19 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                   // 64 (two heads: groups 0 and 1, 2 and 3) both columns of a pair belong to the same thread.
                   int kv_row = kv_row0;
                   float4 rca = rc0a, rcb = rc0b, rsa = rs0a, rsb = rs0b;
-                  if (c0 != 0 && row_on) {
+                  if (!S::ONE && c0 != 0 && row_on) {
                     if (src_s >= 1) kv_row = kv_row_of(t);
-                    if (P.rope && src_s < 2) rope_of(t, rca, rsa, rcb, rsb);
+                    if (S::rope(P) && src_s < 2) rope_of(t, rca, rsa, rcb, rsb);
                   }
-                  const float qscale = src_s == 0 ? 1.4426950408889634f / sqrtf((float)P.hd) : 1.0f;   // log2(e) / sqrt(hd): the softmax works in base 2
-                  const int nq_all = P.Hq * P.hd, nkv_all = P.Hkv * P.hd;
+                  const float qscale = src_s == 0 ? 1.4426950408889634f / sqrtf((float)S::hd(P)) : 1.0f;   // log2(e) / sqrt(hd): the softmax works in base 2
+                  const int nq_all = P.Hq * S::hd(P), nkv_all = P.Hkv * S::hd(P);
                   __half* dst = (src_s == 0 ? P.q16 + (size_t)t * nq_all
                                             : reinterpret_cast<__half*>(src_s == 1 ? p.kc : p.vc) + (size_t)kv_row * nkv_all) + (n0 - src_col0);
 #pragma unroll 1
                   for (int pi = 0; pi < 2; ++pi) {
-                    const int col_lo = (P.hd == 128 ? cg + 8 * pi : cg + 16 * pi) * 4, col_hi = col_lo + (P.hd == 128 ? 64 : 32);
+                    const int col_lo = (S::hd(P) == 128 ? cg + 8 * pi : cg + 16 * pi) * 4, col_hi = col_lo + (S::hd(P) == 128 ? 64 : 32);
                     float4 lo = group(col_lo), hi = group(col_hi);
-                    if (P.rope && src_s < 2) {
+                    if (S::rope(P) && src_s < 2) {
                       const float4 cs = pi ? rcb : rca, sn = pi ? rsb : rsa;
                       const float4 l = lo, h = hi;
                       lo = make_float4(l.x * cs.x - h.x * sn.x, l.y * cs.y - h.y * sn.y, l.z * cs.z - h.z * sn.z, l.w * cs.w - h.w * sn.w);
@@ -2129,7 +2163,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     if (row_on && col < ncols) {
                       const float4 v4 = group(col);
                       const size_t o = (size_t)t * p.ldo + n0 + col;
-                      if (p.epi == TC_STORE_F32) *reinterpret_cast<float4*>(out_f32 + o) = v4;
+                      if (S::store(p)) *reinterpret_cast<float4*>(out_f32 + o) = v4;
                       else store_split4(out_act, o, (size_t)P.lo_row * p.ldo, make_float4(gelu_erf(v4.x), gelu_erf(v4.y), gelu_erf(v4.z), gelu_erf(v4.w)));
                     }
                   }
@@ -2229,6 +2263,26 @@ inline int pick_stages(int t_box, int hd, int dbl, int kps, int tma = 0, int nbu
 }
 // k-blocks per stage: two while at least three stages still fit (small row boxes), else one
 inline int pick_kps(int t_box, int hd, int dbl) { return pick_stages(t_box, hd, dbl, 2) >= 3 ? 2 : 1; }
+
+// The kernel of a model and call: the compiled combinations are the families' usual head sizes.
+using ForwardFn = void (*)(const Params);
+template <int HD, int FAM>
+ForwardFn forward_of(bool tc, bool one) {
+  if constexpr (HD % 64 == 0) {
+    if (tc) return one ? k_forward<Spec<HD, FAM, 1, true>> : k_forward<Spec<HD, FAM, 1, false>>;
+  }
+  return one ? k_forward<Spec<HD, FAM, 0, true>> : k_forward<Spec<HD, FAM, 0, false>>;
+}
+inline ForwardFn forward_fn(const stairs_model& m, int att_tma, int att_tc, int T) {
+  const bool one = T <= 16, a = m.norm == 0 && m.act == 0 && m.pos == 0, b = m.norm == 1 && m.act == 1 && m.pos == 1;
+  if (att_tma) {
+    if (a && m.head_dim == 64) return forward_of<64, 1>(att_tc != 0, one);
+    if (b && m.head_dim == 64) return forward_of<64, 2>(att_tc != 0, one);
+    if (b && m.head_dim == 80) return forward_of<80, 2>(false, one);
+    if (b && m.head_dim == 128) return forward_of<128, 2>(att_tc != 0, one);
+  }
+  return k_forward<Spec<0, 0, -1, false>>;
+}
 
 }  // namespace mk
 }  // namespace stairs

@@ -1,0 +1,44 @@
+"""The compiled variants of the whole-pass kernel (head size, model family, attention path, at most 16 rows or more) against
+the oracle at the edges: 16 and 17 rows, positions around a 64-position chunk, smallest and largest page slices, and bitwise
+the same rows from a call on either side of the 16-row line."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2407_19947_b200 import workloads as wl
+from tests import gpu_util as gu
+from tests.test_gpu_parity import _stairs, small_a, small_b, sources
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = {"family_a": small_a(), "hd48": small_b(4, 2, 48, d=192, f=320), "hd64": small_b(8, 2, 64), "hd80": small_b(4, 4, 80, d=320, f=640),
+          "hd96": small_b(4, 2, 96, d=384, f=448), "hd128": small_b(4, 1, 128, d=512, f=832)}
+
+
+@pytest.mark.parametrize("page", [16, 128])
+@pytest.mark.parametrize("attention", [0, 2], ids=["register", "tcgen05"])
+@pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES.keys())
+def test_variant_matches_oracle_and_ignores_the_row_count(shape, attention, page):
+    st = _stairs()
+    tsrc, _ = sources(shape)
+    tgt, _ = gu.oracle_pair(tsrc)
+    lens = [63, 65, 300]
+    eng = st.Stairs(tsrc, None, max_requests=len(lens), max_seq_len=400, k_max=16, kv_page_tokens=page)
+    eng.debug_tune(3, attention)
+    prompts = [list(wl.zipf_tokens(n, shape.vocab, n)) for n in lens]
+    for i, p in enumerate(prompts):
+        eng.prefill(i, p)
+    drafts = np.random.default_rng(page).integers(0, shape.vocab, size=(3, 16)).astype(np.int32)
+    dd = torch.from_numpy(drafts).cuda()
+    _, _, two = eng.validate([0, 1], [7, 7], dd[:2].contiguous(), want_logits=True)       # 16 rows
+    _, _, three = eng.validate([0, 1, 2], [7, 7, 7], dd, want_logits=True)                # 24
+    tt, _, one = eng.validate([2], [16], dd[2:].contiguous(), want_logits=True)           # 17
+    eng.sync()
+    two, three, one, tt = two.cpu().numpy(), three.cpu().numpy(), one.cpu().numpy(), tt.cpu().numpy()
+    assert np.array_equal(two, three[:16])
+    for i in range(2):
+        ref, _ = gu.oracle_stair_logits(tgt, prompts[i], drafts[i][:7])
+        gu.check_rows_against_oracle(two[8 * i:8 * i + 8], ref.argmax(1), ref, gu.LOGIT_TOL_BF16)
+    ref, _ = gu.oracle_stair_logits(tgt, prompts[2], drafts[2])
+    gu.check_rows_against_oracle(one, tt[0][:17], ref, gu.LOGIT_TOL_BF16)
+    eng.close()
