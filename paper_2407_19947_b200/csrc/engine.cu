@@ -842,7 +842,7 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
   P.trace = (ctx->profile && &M == &ctx->target) ? reinterpret_cast<unsigned long long*>(ws + L.mk_trace) : nullptr;
   const int grid = std::min(ctx->sm_count, TC_GRID_MAX);
   void* args[] = {&P};
-  CK(cudaLaunchCooperativeKernel((const void*)mk::forward_fn(m, P.att_tma, P.att_tc, T), dim3(grid), dim3(mk::MK_THREADS), args,
+  CK(cudaLaunchCooperativeKernel(mk::forward_fn(m, P.att_tma, P.att_tc, T), dim3(grid), dim3(mk::MK_THREADS), args,
                                  mk::smem_bytes(t_box, P.stages, m.head_dim, P.att_dbl, P.kps, P.att_tma, P.att_nbuf, P.att_q_rows), ctx->stream));
   ctx->bar_base += (unsigned long long)n_run * grid;
   ctx->launches++;
@@ -1543,7 +1543,7 @@ int stairs_init(const stairs_config* cfg, const stairs_weights* target, const st
         e = cudaSuccess;
         for (int i = 0; i < 16 && e == cudaSuccess; ++i) {   // (every kernel the two models' calls may launch: also loads its code now)
           const stairs_model& fm = i < 8 || !has_draft ? cfg->target : cfg->draft;
-          e = cudaFuncSetAttribute((const void*)mk::forward_fn(fm, i & 1, (i >> 1) & 1, i & 4 ? 1 : 64), cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
+          e = cudaFuncSetAttribute(mk::forward_fn(fm, i & 1, (i >> 1) & 1, i & 4 ? 1 : 64), cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
         }
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_attn_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide::tc_att_smem<64>());

@@ -1,0 +1,15 @@
+// One compiled variant of the whole-pass kernel per object file: FWD_HD, FWD_FAM, FWD_ATT, FWD_ONE (see Spec) come from the
+// build, which compiles this file once for each: in parallel, and a variant's code does not depend on the others.
+#include "../../include/stairs.h"
+#include "megakernel.cuh"
+
+#define FWD_NAME3(a, b, c, d) forward_##a##_##b##_##c##_##d
+#define FWD_NAME2(a, b, c, d) FWD_NAME3(a, b, c, d)
+
+namespace stairs {
+namespace mk {
+const void* FWD_NAME2(FWD_HD, FWD_FAM, FWD_ATT, FWD_ONE)() {
+  return (const void*)k_forward<Spec<FWD_HD, FWD_FAM, FWD_ATT, FWD_ONE != 0>>;
+}
+}  // namespace mk
+}  // namespace stairs

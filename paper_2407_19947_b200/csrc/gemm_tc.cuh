@@ -172,7 +172,7 @@ __device__ __forceinline__ long long range_begin(long long total, int c, int g) 
 // ---------------------------------------------------------------------------------------------
 // The kernel
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(const __grid_constant__ GemmJob job) {
+static __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(const __grid_constant__ GemmJob job) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int stages = job.stages;

@@ -34,7 +34,7 @@ struct RowParams {
 // Stair-row construction (paper Section 3.3, Fig. 4): request i contributes rows r = 0..k_i;
 // row r ends with the last committed token (r = 0) or drafted token r-1, at position
 // n_seq-1+r.  The other modes build the rows of a prefill chunk or of an assistant step.
-__global__ void k_rows(RowParams p) {
+static __global__ void k_rows(RowParams p) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   if (tid < p.n_keys) p.keys[tid] = 0ull;
   auto clampv = [&](int t) { return t < 0 ? 0 : (t >= p.vocab ? p.vocab - 1 : t); };
@@ -232,7 +232,7 @@ k_attn_plain(const AT* __restrict__ q, const KT* __restrict__ kc, const KT* __re
 
 // Vocabulary-wide argmax of fp32 logits[T, V]: each block reduces a slice of one row to a
 // packed (value, inverted index) key and merges it with a 64-bit atomic max.
-__global__ void k_argmax(const float* __restrict__ logits, int V, int ld,
+static __global__ void k_argmax(const float* __restrict__ logits, int V, int ld,
                          unsigned long long* __restrict__ keys) {
   __shared__ unsigned long long red[32];
   const int t = blockIdx.y;
@@ -277,7 +277,7 @@ struct AcceptParams {
 // kept while drafted token r-1 equals the main model's token for row r-1; accept_len is the
 // number of kept rows after the first.  With commit, the kept drafts and the main model's
 // token for the last kept row are appended to the request's sequence.
-__global__ void k_accept(AcceptParams p) {
+static __global__ void k_accept(AcceptParams p) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= p.n_req) return;
   const int k = p.val_k[i], off = p.val_off[i], slot = p.val_req[i];
@@ -300,7 +300,7 @@ __global__ void k_accept(AcceptParams p) {
 }
 
 // Assistant step epilogue: the argmax of one row becomes drafted token j.
-__global__ void k_take_token(const unsigned long long* __restrict__ keys, int row, int* __restrict__ out, int j) {
+static __global__ void k_take_token(const unsigned long long* __restrict__ keys, int row, int* __restrict__ out, int j) {
   if (threadIdx.x == 0 && blockIdx.x == 0) out[j] = argmax_key_index(keys[row]);
 }
 

@@ -143,10 +143,10 @@ constexpr int MK_XCH_BYTES = 16 * VT_LD * 4;     // the tile itself
 // What a launch knows at compile time.  Every phase runs its code once, so a phase's critical chain is bound by
 // instruction fetch (the kernel's text is far larger than the SM's instruction caches): a test that always goes the same
 // way, or an address computed from a run-time head size, costs what it adds to the text.  With the head size, the model
-// family, the attention path and "at most 16 rows" fixed, a validate call of 9 rows took 2728 us where the general code
-// took 2838 (7B), 1021 where it took 1134 (0.4B); 3B, 5 rows: 1959 and 2072.  HD 0, FAM 0, ATT -1 and ONE false are the general code.
+// family, the attention path and "at most 16 rows" fixed, validate calls took: 7B, 9 rows 2770 us (general code 2860), 0.4B,
+// 9 rows 1012 (1128), 3B, 5 rows 1984 (2072), 7B of four layers, 4 x 16384 positions, 36 rows 1009 (1056).  HD 0, FAM 0, ATT 3 and ONE false are the general code.
 //   FAM 1: LayerNorm, GELU, learned positions; FAM 2: RMSNorm, SwiGLU, rotary positions
-//   ATT 0: bulk copies, contractions on mma.sync; 1: on tcgen05; 2: 16-byte copies
+//   ATT 0: bulk copies, contractions on mma.sync; 1: on tcgen05
 template <int HD, int FAM, int ATT, bool ONE_CHUNK>
 struct Spec {
   static constexpr bool ONE = ONE_CHUNK;
@@ -158,9 +158,9 @@ struct Spec {
   static __device__ __forceinline__ bool gelu(const Phase& p) { return FAM != 2 && p.epi == TC_GELU; }
   static __device__ __forceinline__ bool store(const Phase& p) { return FAM != 1 && (HD == 0 || HD % 64 != 0) && p.epi == TC_STORE_F32; }
   static __device__ __forceinline__ bool shifted(const Phase& p) { return FAM ? FAM == 1 : p.u != nullptr; }   // (LayerNorm: y = rstd (acc - mean u) + c)
-  static __device__ __forceinline__ bool tc(const Params& P) { return ATT < 0 ? P.att_tc != 0 : ATT == 1; }
-  static __device__ __forceinline__ bool tma(const Params& P) { return ATT < 0 ? P.att_tma != 0 : ATT != 2; }
-  static __device__ __forceinline__ int qblk(const Params& P) { return ATT < 0 ? P.att_qblk : ATT == 1 ? ATT_QBLK_TC : ATT_QBLK; }
+  static __device__ __forceinline__ bool tc(const Params& P) { return ATT == 3 ? P.att_tc != 0 : ATT == 1; }
+  static __device__ __forceinline__ bool tma(const Params& P) { return ATT == 3 ? P.att_tma != 0 : true; }
+  static __device__ __forceinline__ int qblk(const Params& P) { return ATT == 3 ? P.att_qblk : ATT == 1 ? ATT_QBLK_TC : ATT_QBLK; }
   static __device__ __forceinline__ bool prep(const Params& P) { return HD % 64 != 0 || HD == 0; }             // may the program hold PH_PREP phases?
 };
 
@@ -346,6 +346,7 @@ struct Ctl {
   uint32_t tmem_slot;
   volatile int abort_flag;
   volatile int bcast;
+  volatile int verdict[2];                              // of the compute group's threads, by phase parity
   float rstd[64], mu[64];       // per-row statistics of the current norm_in GEMM phase
   int rowbase[2][64];           // attention staging: cache row of each position of the chunk (per chunk buffer)
   AttnReq areq[64];             // per request, filled once per launch (a request has at least one row: <= 64)
@@ -532,7 +533,7 @@ __device__ __forceinline__ float group_sum(float v, float* red, int et) {
 
 // Row t of the residual stream from the embedding tables, the next GEMM's operand bf16(x * g)
 // and the row's statistics (one entry covering the whole row), by the 128 compute threads.
-__device__ void embed_row(const Params& P, int t, const RowInfo& r, const float* g, float* red, int et) {
+static __device__ void embed_row(const Params& P, int t, const RowInfo& r, const float* g, float* red, int et) {
   const int d = P.d;
   float* xr = P.x + (size_t)t * d;
   bf16* hr = P.h + (size_t)t * d;
@@ -1769,13 +1770,21 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
         float* out_f32 = (p.epi == TC_LMHEAD) ? P.logits : reinterpret_cast<float*>(p.out);
         bf16* out_act = reinterpret_cast<bf16*>(p.out);
         unsigned long long* keys = P.keys;
+        // LayerNorm: the per-column constants of the tile this CTA finishes first are requested before the wait for the
+        // statistics (they come from HBM, once a call; sources are whole tiles in this case): 0.4B, 9 rows 1012 -> 1002 us
+        float uq = 0.f, cq = 0.f;
+        int pre_tile = -1;
+        if (S::shifted(p) && p.norm_in && kb_begin < kb_end && p.n_tiles * BM == p.N) {
+          pre_tile = (kb_begin + p.kblocks - 1) / p.kblocks;
+          if (pre_tile < p.n_tiles) { uq = p.u[pre_tile * BM + m]; cq = p.c[pre_tile * BM + m]; }
+        }
         if (p.norm_in && kb_begin < kb_end) {
           // row statistics of the operand: merge the per-tile entries (published by the phase
           // that produced x) into mean and 1/std per row
           if (et == 0) ctl->bcast = W.wait_grid(bar_count, P.bar_base + (unsigned long long)ph * G) ? 1 : 0;
+          __syncwarp();
           epi_bar_sync();
-          ok = ctl->bcast != 0;
-          epi_bar_sync();
+          ok = ctl->bcast != 0;   // (written again in a later phase only, several barriers on)
           if (!ok) break;
           // One warp per row, four rows per warp at a time.  A lane holds the tile entries lane and
           // lane + 32 of each row (all loads of the four rows in flight together; at most 64 tiles,
@@ -1892,8 +1901,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
             const bool m_on = mc < ncols;
             if (p.norm_in && S::shifted(p)) {
               const int ncol = (S::dual(p) && m >= 64) ? p.N + n0 + mc : n0 + mc;
-              ctl->utile[m] = (S::shifted(p) && m_on) ? p.u[ncol] : 0.f;
-              ctl->ctile[m] = (S::shifted(p) && m_on) ? p.c[ncol] : 0.f;
+              ctl->utile[m] = tile == pre_tile ? uq : m_on ? p.u[ncol] : 0.f;
+              ctl->ctile[m] = tile == pre_tile ? cq : m_on ? p.c[ncol] : 0.f;
             }
             if (have_pre) {
 #pragma unroll
@@ -1907,8 +1916,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           }
           W.wait(ctl->acc_full + buf, (acc_bits >> buf) & 1u);
           __syncwarp();   // lanes may leave the wait an iteration apart; the barriers below want whole warps
-          ok = group_ok(ctl, et);   // (its barriers also publish the staged constants)
-          if (!ok) break;
+          epi_bar_sync();   // (publishes the staged constants; a wait that ran out is looked at once, at the end of the phase)
           if (tracing && first_seg) { tr[4] = globaltimer_ns(); first_seg = false; }
           acc_bits ^= 1u << buf;
           tc_fence_after();
@@ -2169,12 +2177,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                   }
                 }
               }
-              // one verdict for the 128 threads (a poll above may have run out in some of them; one that
-              // thread 0 misses here is seen at the next verdict or at the end of the kernel)
-              if (et == 0) ctl->bcast = ctl->abort_flag ? 0 : 1;
+              __syncwarp();
               epi_bar_sync();   // (the exchange tile is reused by the next chunk)
-              ok = ctl->bcast != 0;
-              if (!ok) break;
             }
             if (tra) tra[3] = globaltimer_ns();
           }
@@ -2204,15 +2208,18 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
       if (tracing && cta != 0) tr[6] = globaltimer_ns();
 #endif
       if (et < PH_WORDS) ctl->phc[(ph + 1) & 1][et] = next_word;   // (the barriers below publish it)
-      if (ph > 0 && p.kind == PH_GEMM && !gemm_worked) {
-        if (et == 0) ctl->bcast = W.wait_grid(bar_count, P.bar_base + (unsigned long long)ph * G) ? 1 : 0;
-        epi_bar_sync();
-        ok = ctl->bcast != 0;
-        epi_bar_sync();
-        if (!ok) break;
-      } else {
-        epi_bar_sync();
+      // One verdict for the compute group: a wait of this phase that ran out (some of its threads may have seen that and
+      // others not) ends the launch here.  Until then the threads go on in step on whatever they have; with the abort flag
+      // raised no later wait lasts.
+      if (et == 0) {
+        bool go = true;
+        if (ph > 0 && p.kind == PH_GEMM && !gemm_worked) go = W.wait_grid(bar_count, P.bar_base + (unsigned long long)ph * G);
+        ctl->verdict[ph & 1] = go && ctl->abort_flag == 0 ? 1 : 0;   // (two slots: one is written again only after everybody has read it)
       }
+      __syncwarp();
+      epi_bar_sync();
+      ok = ctl->verdict[ph & 1] != 0;
+      if (!ok) break;
 #ifdef STAIRS_TRACE
       if (tracing && cta != 0) tr[7] = globaltimer_ns();
 #endif
@@ -2264,24 +2271,24 @@ inline int pick_stages(int t_box, int hd, int dbl, int kps, int tma = 0, int nbu
 // k-blocks per stage: two while at least three stages still fit (small row boxes), else one
 inline int pick_kps(int t_box, int hd, int dbl) { return pick_stages(t_box, hd, dbl, 2) >= 3 ? 2 : 1; }
 
-// The kernel of a model and call: the compiled combinations are the families' usual head sizes.
-using ForwardFn = void (*)(const Params);
-template <int HD, int FAM>
-ForwardFn forward_of(bool tc, bool one) {
-  if constexpr (HD % 64 == 0) {
-    if (tc) return one ? k_forward<Spec<HD, FAM, 1, true>> : k_forward<Spec<HD, FAM, 1, false>>;
-  }
-  return one ? k_forward<Spec<HD, FAM, 0, true>> : k_forward<Spec<HD, FAM, 0, false>>;
-}
-inline ForwardFn forward_fn(const stairs_model& m, int att_tma, int att_tc, int T) {
-  const bool one = T <= 16, a = m.norm == 0 && m.act == 0 && m.pos == 0, b = m.norm == 1 && m.act == 1 && m.pos == 1;
-  if (att_tma) {
-    if (a && m.head_dim == 64) return forward_of<64, 1>(att_tc != 0, one);
-    if (b && m.head_dim == 64) return forward_of<64, 2>(att_tc != 0, one);
-    if (b && m.head_dim == 80) return forward_of<80, 2>(false, one);
-    if (b && m.head_dim == 128) return forward_of<128, 2>(att_tc != 0, one);
-  }
-  return k_forward<Spec<0, 0, -1, false>>;
+// The compiled variants (forward.cu, one object each): the families' usual head sizes, and the general code.
+#define STAIRS_FORWARD_VARIANTS(X)                                                    \
+  X(64, 1, 0, 0) X(64, 1, 0, 1) X(64, 1, 1, 0) X(64, 1, 1, 1)                         \
+  X(64, 2, 0, 0) X(64, 2, 0, 1) X(64, 2, 1, 0) X(64, 2, 1, 1)                         \
+  X(80, 2, 0, 0) X(80, 2, 0, 1)                                                       \
+  X(128, 2, 0, 0) X(128, 2, 0, 1) X(128, 2, 1, 0) X(128, 2, 1, 1)                     \
+  X(0, 0, 3, 0)
+#define STAIRS_FORWARD_DECLARE(hd, fam, att, one) const void* forward_##hd##_##fam##_##att##_##one();
+STAIRS_FORWARD_VARIANTS(STAIRS_FORWARD_DECLARE)
+
+// The kernel of a model and call.
+inline const void* forward_fn(const stairs_model& m, int att_tma, int att_tc, int T) {
+  const int fam = m.norm == 0 && m.act == 0 && m.pos == 0 ? 1 : m.norm == 1 && m.act == 1 && m.pos == 1 ? 2 : 0;
+  const int att = att_tc ? 1 : 0, one = T <= 16 ? 1 : 0;
+#define STAIRS_FORWARD_PICK(hd_, fam_, att_, one_) \
+  if (att_tma && m.head_dim == hd_ && fam == fam_ && att == att_ && one == one_) return forward_##hd_##_##fam_##_##att_##_##one_();
+  STAIRS_FORWARD_VARIANTS(STAIRS_FORWARD_PICK)
+  return forward_0_0_3_0();
 }
 
 }  // namespace mk
