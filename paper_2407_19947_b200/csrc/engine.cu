@@ -1273,15 +1273,34 @@ small::SmallParams small_params(stairs_ctx* ctx, const DevModel& M) {
   return p;
 }
 
-int launch_small(stairs_ctx* ctx, const DevModel& M, const small::SmallParams& p) {
+int launch_small(stairs_ctx* ctx, const DevModel& M, const small::SmallParams& p, int clusters = 1) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(ctx->small_ctas); cfg.blockDim = dim3(small::S_THREADS); cfg.dynamicSmemBytes = small::smem_bytes(M.m.d_model, M.m.n_heads * M.m.head_dim, M.m.d_ff); cfg.stream = ctx->stream;
+  cfg.gridDim = dim3(ctx->small_ctas * clusters); cfg.blockDim = dim3(small::S_THREADS); cfg.dynamicSmemBytes = small::smem_bytes(M.m.d_model, M.m.n_heads * M.m.head_dim, M.m.d_ff); cfg.stream = ctx->stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = ctx->small_ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = 1;
   ctx->launches++;
   CK(cudaLaunchKernelEx(&cfg, small::k_small, p));
   return STAIRS_OK;
+}
+
+// Deals a validate call's requests to clusters, in order, so that the busiest takes as few passes of eight rows as it can;
+// returns the number of clusters, 0 where that is too many passes (see S_MOST_PASSES).
+int small_deal(small::SmallParams& p, int n_req) {
+  for (int passes = 1; passes <= small::S_MOST_PASSES; ++passes) {
+    int n = 0, rows = 0;
+    bool fits = true;
+    for (int i = 0; i < n_req && fits; ++i) {
+      const int r = p.val_k[i] + 1, room = passes * small::S_BLOCK;
+      if (i == 0 || rows + r > room) {
+        fits = r <= room && n < small::S_MAX_CLUSTERS;
+        if (fits) { p.cl_req[n++] = i; rows = 0; }
+      }
+      rows += r;
+    }
+    if (fits) { p.cl_req[n] = n_req; return n; }
+  }
+  return 0;
 }
 
 // Uploads a model's per-layer pointers and finds the largest cluster that can run.
@@ -1363,8 +1382,8 @@ int prefill_model(stairs_ctx* ctx, DevModel& M, int slot, int n_ctx) {
     return launch_forward_mk(ctx, M, n_ctx, 0, 0, c);
   }
   // longer: chunks of equal length
-  const bool wide = wide_eligible(ctx, M), tiny = small_eligible(ctx, M, 1, 1, n_ctx);
-  const int most = tiny ? std::min(prefill_rows(ctx->cfg), (int)small::S_ROWS) : prefill_rows(ctx->cfg);
+  const bool wide = wide_eligible(ctx, M), tiny = n_ctx <= small::S_MOST_PASSES * small::S_BLOCK && small_eligible(ctx, M, 1, 1, n_ctx);
+  const int most = prefill_rows(ctx->cfg);
   const int n_chunks = (n_ctx + most - 1) / most, chunk = (n_ctx + n_chunks - 1) / n_chunks;
   for (int c0 = 0; c0 < n_ctx; c0 += chunk) {
     const int n = std::min(chunk, n_ctx - c0);
@@ -1695,12 +1714,14 @@ int stairs_validate(stairs_ctx* ctx, int n_req, const int32_t* req_ids_host, con
     sp.mode = ROWS_VALIDATE; sp.T = T; sp.n_req = n_req; sp.head_rows = 1; sp.draft = draft_dev;
     for (int i = 0; i < n_req; ++i) { sp.val_req[i] = req_ids_host[i]; sp.val_k[i] = k_host[i]; sp.val_off[i] = off[i]; }
     sp.logits = logits_dev_or_null; sp.target_tokens = target_tokens_dev; sp.accept_len = accept_len_dev; sp.commit = commit;
-    int rc = launch_small(ctx, ctx->target, sp);
-    if (rc) return rc;
-    if (ctx->profile) cudaEventRecord(ctx->call_end, ctx->stream);
-    if (commit)
-      for (int i = 0; i < n_req; ++i) ctx->n_seq_ub[req_ids_host[i]] += k_host[i] + 1;
-    return STAIRS_OK;
+    if (const int clusters = small_deal(sp, n_req)) {
+      int rc = launch_small(ctx, ctx->target, sp, clusters);
+      if (rc) return rc;
+      if (ctx->profile) cudaEventRecord(ctx->call_end, ctx->stream);
+      if (commit)
+        for (int i = 0; i < n_req; ++i) ctx->n_seq_ub[req_ids_host[i]] += k_host[i] + 1;
+      return STAIRS_OK;
+    }
   }
   CK(cudaMemcpyAsync(ws + L.val_req, req_ids_host, (size_t)n_req * 4, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ws + L.val_k, k_host, (size_t)n_req * 4, cudaMemcpyHostToDevice, ctx->stream));

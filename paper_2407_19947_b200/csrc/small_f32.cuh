@@ -18,7 +18,8 @@
 // Measured (four layers of width 256, 31-token prompt, 64 tokens generated): a validate pass of five rows 105 us (launch
 // by launch 220), the draft of four tokens 130 us (330), the whole call 7.24 ms -> 3.41 ms.  What is left is
 // latency: about 2.5 us for each of a layer's five steps (barrier and publication 1 us, the rest code that runs once).
-// Rows are taken eight at a time (a pass per block of rows: later rows only need earlier rows' K/V).
+// Rows are taken eight at a time (a pass per block of rows: later rows only need earlier rows' K/V); the requests of a
+// validate call are dealt to several clusters, which have nothing to do with one another.
 //
 // A warp owns whole features; its lanes stride the K dimension in 16-byte vectors and hold one sum per
 // (feature, row).  The order of the additions depends on K only, and a row's attention on its position
@@ -34,9 +35,14 @@ namespace stairs {
 namespace small {
 
 constexpr int S_WARPS = 8, S_THREADS = S_WARPS * 32;
-constexpr int S_ROWS = 64;           // rows of a call
 constexpr int S_BLOCK = 8;           // rows of a pass
+// Passes one launch pays for (four layers of width 256): one pass takes 107 us (5 rows) to 118 (8), two 207 to 232, three 320,
+// four 462; one launch per operation takes 270 us for 5 rows, 290 for 24 or 16 x 2, 315 for 64.  Prefills alike: two
+// passes 163 us against 229, three 250 against 245.
+constexpr int S_MOST_PASSES = 2;
 constexpr int S_MAX_HD = 128, S_MAX_REQ = 64, S_MAX_LAYERS = 32, S_MAX_CTAS = 16;
+constexpr int S_MAX_CLUSTERS = 8;    // clusters of a validate call, each with requests of its own
+constexpr int S_ROWS = S_MAX_CLUSTERS * S_MOST_PASSES * S_BLOCK;   // rows of a call
 constexpr int S_GROUP = 4;           // warps that share one (row, head) of the attention
 constexpr int S_RING = 16384;        // bytes of a warp's weight ring
 constexpr int S_SLOTS = 3;           // items a warp's ring holds at most
@@ -54,6 +60,7 @@ struct SmallParams {
   int mode;                          // RowMode; ROWS_DRAFT_FIRST: `steps` assistant steps
   int T, steps, n_req, slot, first, head_rows;   // head_rows 0: no logits (prefill)
   int val_req[S_MAX_REQ], val_k[S_MAX_REQ], val_off[S_MAX_REQ];
+  int cl_req[S_MAX_CLUSTERS + 1];    // validate: first request of every cluster, then n_req
   const int* draft; int* draft_out; int k_max;
   int* seq; int* n_seq; int max_seq_len;
   const int* page_table; int page_tokens, max_pages;
@@ -64,7 +71,7 @@ struct SmallParams {
 
 struct SmallSmem {
   int tok[S_BLOCK], pos[S_BLOCK], slot[S_BLOCK], kv[S_BLOCK];
-  int result[S_ROWS];                                    // argmax of every row of the call
+  int result[S_MOST_PASSES * S_BLOCK];                   // argmax of every row of the cluster
   unsigned long long keys[S_BLOCK][S_MAX_CTAS * S_WARPS];  // LM head: every warp's best of every row
   float part[S_WARPS][S_MAX_HD + 4];                     // attention: one warp's output, maximum and sum
   unsigned long long landed[S_WARPS][S_SLOTS];           // mbarriers of the weight rings
@@ -126,7 +133,13 @@ __global__ void __launch_bounds__(S_THREADS, 1) k_small(const __grid_constant__ 
   extern __shared__ __align__(16) uint8_t small_raw[];
   SmallSmem& S = *reinterpret_cast<SmallSmem*>(small_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int cta = blockIdx.x, NC = gridDim.x, gw = cta * S_WARPS + warp, NW = NC * S_WARPS;
+  int cta, NC;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(cta));
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(NC));
+  const int gw = cta * S_WARPS + warp, NW = NC * S_WARPS;
+  const bool validating = P.mode == ROWS_VALIDATE;
+  const int req0 = validating ? P.cl_req[blockIdx.x / NC] : 0, req1 = validating ? P.cl_req[blockIdx.x / NC + 1] : 0;   // this cluster's requests
+  const int off0 = validating ? P.val_off[req0] : 0;         // and first row
   const int nw_log = 31 - __clz(NW);         // (the cluster has 4, 8 or 16 CTAs)
   const int d = P.d, hd = P.hd, half = hd / 2, nq = P.Hq * hd, nkv = P.Hkv * hd, G = P.Hq / P.Hkv;
   float* ring = reinterpret_cast<float*>(small_raw + ((sizeof(SmallSmem) + 15) & ~(size_t)15)) + (size_t)warp * (S_RING / 4);
@@ -154,15 +167,15 @@ __global__ void __launch_bounds__(S_THREADS, 1) k_small(const __grid_constant__ 
   unsigned phases = 0, flying = 0;           // ring slots: parity of the next wait, copies not yet waited for
   int T = 0, rows = 0;                       // rows of this step, of this pass
   for (int step = 0; step < P.steps; ++step) {
-    T = P.mode == ROWS_DRAFT_FIRST ? (step == 0 ? 2 : 1) : P.T;
+    T = P.mode == ROWS_DRAFT_FIRST ? (step == 0 ? 2 : 1) : validating ? (req1 < P.n_req ? P.val_off[req1] : P.T) - off0 : P.T;
     for (int r0 = 0; r0 < T; r0 += S_BLOCK) {
       rows = min(S_BLOCK, T - r0);
       // ------------------------------------------------------------ rows of this pass
       if (tid < rows) {
-        const int tg = r0 + tid;
+        const int tg = off0 + r0 + tid;
         int token, pos, slot = P.slot;
         if (P.mode == ROWS_VALIDATE) {
-          int i = 0;
+          int i = req0;
           while (i + 1 < P.n_req && P.val_off[i + 1] <= tg) ++i;
           slot = P.val_req[i];
           const int base = P.n_seq[slot] - 1, r = tg - P.val_off[i];
@@ -438,7 +451,7 @@ __global__ void __launch_bounds__(S_THREADS, 1) k_small(const __grid_constant__ 
               if (on_row && n < P.vocab) {
                 const unsigned long long k = argmax_key(v, (uint32_t)n);
                 best = k > best ? k : best;
-                if (P.logits) P.logits[(size_t)(r0 + tl) * P.vocab + n] = v;
+                if (P.logits) P.logits[(size_t)(off0 + r0 + tl) * P.vocab + n] = v;
               }
               continue;
             }
@@ -522,8 +535,8 @@ __global__ void __launch_bounds__(S_THREADS, 1) k_small(const __grid_constant__ 
   }
   // ---------------------------------------------------------------- accept
   if (P.mode == ROWS_VALIDATE && cta == 0) {
-    for (int i = tid; i < P.n_req; i += S_THREADS) {
-      const int k = P.val_k[i], off = P.val_off[i], slot = P.val_req[i];
+    for (int i = req0 + tid; i < req1; i += S_THREADS) {
+      const int k = P.val_k[i], off = P.val_off[i] - off0, slot = P.val_req[i];
       int a = -1;
       for (int r = 0; r <= k; ++r) {
         const int tr = S.result[off + r];

@@ -58,3 +58,26 @@ def test_small_fp32_passes_match_oracle(shape):
                 assert torch.equal(alone, lg[row: row + ks[j] + 1])
             row += ks[j] + 1
     eng.close(); plain.close()
+
+
+@pytest.mark.parametrize("k,n_req,launches", [(0, 16, 1), (1, 16, 1), (7, 16, 1), (8, 8, 1), (15, 8, 1), (16, 1, None), (8, 9, None)])
+def test_requests_dealt_to_clusters_match_the_per_operation_kernels(k, n_req, launches):
+    # one and two passes a cluster, every cluster in use, one row or one request too many
+    st = _stairs()
+    shape = SHAPES["odd_widths"]
+    tsrc, _ = sources(shape, std=0.03)
+    got = []
+    for impl in (0, 1):
+        eng = st.Stairs(tsrc, None, max_requests=16, max_seq_len=128, k_max=16, kv_page_tokens=16, gemm_impl=impl)
+        for i in range(n_req):
+            eng.prefill(i, list(wl.zipf_tokens(3 + 5 * i, shape.vocab, i)))
+        drafts = torch.from_numpy(np.random.default_rng(k).integers(0, shape.vocab, size=(n_req, 16)).astype(np.int32)).cuda()
+        before = eng.launch_count()
+        tt, al, lg = eng.validate(list(range(n_req)), [k] * n_req, drafts, want_logits=True)
+        eng.sync()
+        if impl == 0:
+            assert (eng.launch_count() - before == 1) == (launches == 1)
+        got.append((tt.cpu(), al.cpu(), lg.cpu()))
+        eng.close()
+    assert torch.equal(got[0][0][:, : k + 1], got[1][0][:, : k + 1]) and torch.equal(got[0][1], got[1][1])
+    assert float((got[0][2] - got[1][2]).abs().max()) < 1e-4
