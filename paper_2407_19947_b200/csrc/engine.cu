@@ -756,7 +756,7 @@ struct MkCall {
   const int* draft = nullptr;
   int* target_tokens = nullptr; int* accept_len = nullptr; int commit = 0; int* draft_out = nullptr;
   float* logits = nullptr;
-  bool skip_head = false;   // prefill: stop after the last layer (no LM head, no accept)
+  bool skip_head = false;   // prefill: stop when the last layer's keys and values are filed
   const int* req_host = nullptr; // validate: slot, draft length and first row per request (travel as kernel parameters)
   const int* k_host = nullptr;
   const int* off_host = nullptr;
@@ -804,7 +804,9 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
   mk::Params P;
   memset(&P, 0, sizeof P);
   char* base = M.prog_base + (size_t)slot * M.prog_slot_bytes;
-  const int n_run = c.skip_head ? M.n_phases - 2 : M.n_phases;
+  // A prefill ends with the last layer's keys and values (filed by its QKV projection, or the phase after it): no attention,
+  // O projection, MLP, LM head or accept.
+  const int n_run = c.skip_head ? M.n_phases - 6 : M.n_phases;
   P.phases = reinterpret_cast<const mk::Phase*>(base); P.n_phases = n_run;
   P.maps = reinterpret_cast<const CUtensorMap*>(base + M.prog_maps_off);
   P.T = T; P.t_box = t_box;
