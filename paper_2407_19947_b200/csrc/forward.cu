@@ -1,5 +1,8 @@
 // One compiled variant of the whole-pass kernel per object file: FWD_HD, FWD_FAM, FWD_ATT, FWD_ONE (see Spec) come from the
 // build, which compiles this file once for each: in parallel, and a variant's code does not depend on the others.
+#if FWD_ATT == 0
+#define STAIRS_WAIT_SLOW __forceinline__
+#endif
 #include "../../include/stairs.h"
 #include "megakernel.cuh"
 

@@ -366,6 +366,13 @@ __device__ __forceinline__ bool group_ok(Ctl* ctl, int et) {
   return ctl->bcast != 0;
 }
 
+// Is an mbarrier wait's polling loop inlined?  In the variants whose attention runs on mma.sync a call spoils more registers of
+// the surrounding code than the loop is long: 7B, 9 rows 2770 -> 2682 us, 3B, 5 rows 1984 -> 1945, 0.4B even; the
+// tcgen05 ones get longer by 1 % (four layers of 7B, 4 x 16384 positions 1009 -> 1020).
+#ifndef STAIRS_WAIT_SLOW
+#define STAIRS_WAIT_SLOW __noinline__
+#endif
+
 struct Waiter {
   volatile int* abort_flag; const unsigned long long* gabort; unsigned long long limit;
   unsigned int* status;   // host-visible status words: [1] kind of the first wait that ran out, [2..5] where
@@ -380,11 +387,12 @@ struct Waiter {
     if ((unsigned long long)(clock64() - t0) > limit) { *abort_flag = 1; return true; }
     return false;
   }
-  // mbarrier wait (bounded).  The polling loops are kept out of line: they are inlined nowhere, so the
+  // mbarrier wait (bounded).  The polling loop of the variants with the tcgen05 attention (and of the general code), and the
+  // grid barrier's in all, are kept out of line: so the
   // many wait sites cost a test and a call each instead of a copy of the loop (the kernel's code has
   // to stay inside the instruction cache: every phase runs its code once, and code that misses runs
   // at a fraction of the warm issue rate).
-  __device__ __noinline__ bool wait_slow(uint64_t* bar, uint32_t parity) const {
+  __device__ STAIRS_WAIT_SLOW bool wait_slow(uint64_t* bar, uint32_t parity) const {
     const long long t0 = clock64();
     int spins = 0;
     while (true) {
