@@ -6,7 +6,6 @@ There is no CPU fallback: loading fails loudly when the library has not been bui
 """
 from __future__ import annotations
 
-import array
 import ctypes as C
 import os
 from typing import List, Optional, Sequence
@@ -115,11 +114,9 @@ def _ptr(a: np.ndarray):
 
 
 def _ints(a):
-    """A list of integers as a ctypes array (a numpy round trip takes three times as long)."""
-    n = len(a)
-    if type(a) is not list:
-        a = [int(x) for x in a]
-    return (C.c_int32 * n)(*a) if n <= 12 else (C.c_int32 * n).from_buffer(array.array("i", a))
+    """Integers as a ctypes array, accepted or refused as numpy does (ctypes itself would wrap what does not fit in
+    32 bits).  Passing the numpy array's pointer instead takes three times as long."""
+    return (C.c_int32 * len(a)).from_buffer_copy(_i32(a))
 
 
 def _results(t, n, k_max, ks, device):
@@ -237,10 +234,11 @@ class Stairs:
                  out=None):
         """Enqueues one stairs pass.  Returns (target_tokens_dev [n,k_max+1], accept_len_dev [n], logits or None)."""
         t = self.torch
-        n = len(req_ids)
-        tt, al = _results(t, n, self.k_max, k, self._dev) if out is None else out
-        logits = t.empty((int(sum(k)) + n, self.vocab), dtype=t.float32, device=self._dev) if want_logits else None
-        self._ck(self.lib.stairs_validate(self.h, n, _ints(req_ids), _ints(k),
+        r, kk = _ints(req_ids), _ints(k)
+        n = len(r)
+        tt, al = _results(t, n, self.k_max, kk, self._dev) if out is None else out
+        logits = t.empty((sum(kk) + n, self.vocab), dtype=t.float32, device=self._dev) if want_logits else None
+        self._ck(self.lib.stairs_validate(self.h, n, r, kk,
                                           draft_dev.data_ptr() if draft_dev is not None else None,
                                           tt.data_ptr(), al.data_ptr(),
                                           logits.data_ptr() if logits is not None else None, int(commit)))
@@ -324,10 +322,11 @@ def accept_static(logits_dev, k: Sequence[int], draft_dev, k_max: int, *, vocab:
     draft_dev: int32 [n_req, k_max].  Returns (target_tokens [n_req, k_max+1], accept_len [n_req])."""
     import torch
     lib = load_library()
-    n = len(k)
-    tt, al = _results(torch, n, k_max, k, logits_dev.device)
+    kk = _ints(k)
+    n = len(kk)
+    tt, al = _results(torch, n, k_max, kk, logits_dev.device)
     st = stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
-    rc = lib.stairs_accept_static(logits_dev.data_ptr(), vocab or logits_dev.shape[1], logits_dev.stride(0), n, _ints(k),
+    rc = lib.stairs_accept_static(logits_dev.data_ptr(), vocab or logits_dev.shape[1], logits_dev.stride(0), n, kk,
                                   draft_dev.data_ptr() if draft_dev is not None else None, k_max,
                                   tt.data_ptr(), al.data_ptr(), st)
     if rc:

@@ -4,6 +4,7 @@ import ctypes as C
 import os
 import re
 
+import numpy as np
 import pytest
 
 from paper_2407_19947_b200 import build as stairs_build
@@ -80,3 +81,19 @@ def test_null_context_is_an_error_not_a_crash(lib):
     assert lib.stairs_sync(None) == 1
     assert lib.stairs_destroy(None) == 1
     assert lib.stairs_launch_count(None) == 0
+
+
+@pytest.mark.parametrize("n", [1, 12, 13, 64])
+def test_request_ids_and_draft_lengths_convert_as_numpy_does(n):
+    # on either side of 32 bits; numbers that are whole, of any type and container
+    for edge in (2**31 - 1, -2**31):
+        assert list(st._ints([edge] * n)) == [edge] * n
+    for beyond in (2**31, -2**31 - 1, 2**32 + 1):
+        with pytest.raises(OverflowError):
+            st._ints([0] * (n - 1) + [beyond])
+    for whole in ([4.0] * n, (4,) * n, np.full(n, 4, np.int64), np.full(n, 4, np.int16), [np.int32(4)] * n):
+        assert list(st._ints(whole)) == [4] * n
+    for bad in ([None] * n, ["x"] * n):
+        with pytest.raises((TypeError, ValueError)):
+            st._ints(bad)
+    assert len(st._ints([])) == 0
