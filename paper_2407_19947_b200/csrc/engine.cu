@@ -880,7 +880,9 @@ WidePlan wide_plan(const stairs_ctx* ctx, int T, int K, const int* rows, int n_s
     const int x_box = m_tiles == 1 && cg == 1 ? (T + 15) / 16 * 16 : wide::WM;
     for (int tn = gran; tn <= 256; tn += gran) {
       if (tn < 32 || (cg == 2 && (tn % 32 || tn < 64))) continue;   // (either CTA of a pair holds half of the weight tile)
-      if (tn == 256 && gran == 16) continue;                        // (heads of 16: the QKV epilogue reads 8 columns past the tile)
+      // Heads of an odd number of 16-column groups: the QKV epilogue's last read of a tile ends 8 columns past it, and the
+      // second accumulator's columns end where the kernel's TMEM does.  (Only heads of 16 have widths without that room.)
+      if (epi_kind == wide::W_QKV && gran % 32 && wide::tmem_columns(tn) < 2 * tn + 16) continue;
       int n_tiles = 0;
       if (glu) n_tiles = (all_rows + tn - 1) / tn;
       else for (int s = 0; s < n_src; ++s) n_tiles += (rows[s] + tn - 1) / tn;

@@ -164,6 +164,13 @@ __device__ __forceinline__ float gelu_erfc(float v) {
   return 0.5f * v * (v < 0.f ? c : 2.0f - c);
 }
 
+// TMEM columns of two accumulators of TN columns (an allocation is a power of two of at least 32); the second one starts halfway
+__host__ __device__ inline int tmem_columns(int TN) {
+  int c = 32;
+  while (c < 2 * TN) c <<= 1;
+  return c;
+}
+
 // ---------------------------------------------------------------------------------------------
 // The GEMM
 // ---------------------------------------------------------------------------------------------
@@ -188,8 +195,7 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
   const int rank = CG == 2 ? (int)cluster_rank() : 0;
   const int cid = blockIdx.x / CG, G = gridDim.x / CG;               // this CTA (pair) among the CTAs (pairs)
   const int units = job.n_tiles * job.m_tiles * S;                   // one unit: a K range of one tile
-  uint32_t tmem_cols = 32;
-  while ((int)tmem_cols < 2 * TN) tmem_cols <<= 1;
+  const uint32_t tmem_cols = tmem_columns(TN);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }

@@ -12,7 +12,7 @@ from tests.test_gpu_parity import _stairs, small_a, small_b, sources
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = {"gqa_hd64": small_b(8, 2, 64), "mha_hd80": small_b(4, 4, 80, d=320, f=640), "mqa_hd128": small_b(4, 1, 128, d=512, f=832),
+SHAPES = {"gqa_hd16": small_b(8, 2, 16, d=128, f=192), "gqa_hd48": small_b(8, 4, 48, d=192, f=320), "gqa_hd64": small_b(8, 2, 64), "mha_hd80": small_b(4, 4, 80, d=320, f=640), "mqa_hd128": small_b(4, 1, 128, d=512, f=832),
           "hd96": small_b(4, 2, 96, d=384, f=448), "family_a": small_a()}
 
 
