@@ -976,7 +976,8 @@ int launch_wide_attn_ks(stairs_ctx* ctx, const wide::WideAttn& a, int n_req, int
     while (ns < 8 && blocks * ns * 2 <= 2ll * ctx->sm_count && chunks / (ns * 2) >= 2) ns *= 2;
     const size_t smem = wide::attn_smem(a.hd, NW, MT);
     auto kern = wide::k_wide_attn<KS, EXACT, NW, MT>;
-    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // (the kernel's largest head size, the same value whoever sets it: another thread's context may launch it with another head size)
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide::attn_smem(KS * 16, NW, MT)));
     ctx->launches++;
     CK(launch_chained(ctx->stream, kern, dim3(a.Hkv, n_req * p.n_qblk, ns), NW * 32, smem, dim3(1, 1, ns), p));
     return STAIRS_OK;

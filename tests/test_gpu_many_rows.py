@@ -94,3 +94,37 @@ def test_prefill_attention_over_many_chunks_matches_oracle(name, page):
     ref = np.stack([so.forward_logits(tgt, prompt)])
     gu.check_rows_against_oracle(logits.cpu().numpy(), tt.cpu().numpy()[0], ref, gu.LOGIT_TOL_BF16)
     eng.close()
+
+
+def test_contexts_of_two_threads_with_different_head_sizes():
+    # both head sizes run on one kernel, with different amounts of shared memory
+    import threading
+    st = _stairs()
+    errors = []
+
+    def work(hd, d):
+        try:
+            shape = small_b(4, 2, hd, layers=8, d=d, f=448)
+            tsrc, _ = sources(shape)
+            prompt = list(wl.zipf_tokens(131, shape.vocab, hd))
+            eng = st.Stairs(tsrc, None, max_requests=1, max_seq_len=200, k_max=2, kv_page_tokens=16, stream=torch.cuda.Stream())
+            want = None
+            start.wait(60)
+            for _ in range(400):
+                eng.prefill(0, prompt)
+                if want is None:
+                    want = eng.validate([0], [0], None, want_logits=True)     # (kept whole: the streams differ from torch's)
+            got = eng.validate([0], [0], None, want_logits=True)
+            eng.sync()
+            assert torch.equal(got[2], want[2])
+            eng.close()
+        except Exception as e:
+            errors.append(e)
+
+    start = threading.Barrier(2)
+    threads = [threading.Thread(target=work, args=a) for a in ((96, 384), (112, 448))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
