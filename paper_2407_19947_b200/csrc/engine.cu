@@ -2078,12 +2078,13 @@ __global__ void k_accept_static(const __grid_constant__ StaticAcceptParams p) {
 // all the request's rows; row keys are reduced per CTA, gathered in the first CTA's shared memory, and its
 // threads take the tokens and the accept length.  Nothing is kept in memory between launches.  A call is
 // bound by latency (5 rows of 32000: 31 us a call with three launches, 11 now, of which the kernel 4) or by reading
-// the logits (576 rows: 53 us, now 16), so a warp takes a quarter of a row's slice at a time with eight vectors a
-// lane in flight, and the CTAs of 64 requests fit the chip at once.
+// the logits (576 rows: 53 us, now 16), so a warp takes at most a quarter of a row's slice at a time with eight vectors a
+// lane in flight, and the CTAs of 64 requests fit the chip at once.  A slice is cut no finer than one such batch, though: a batch
+// takes its latency however few of its vectors exist (64 rows of 1000 in quarters: 28.8 us, in whole slices 10, three launches 14.4).
 constexpr int SA_THREADS = 256, SA_CTAS = 8;
-template <bool VEC>
+constexpr int sa_batch(bool vec) { return 8 * 32 * (vec ? 4 : 1); }   // columns of a warp's batch of loads
+template <bool VEC, int SEG>
 __global__ void __cluster_dims__(SA_CTAS, 1, 1) __launch_bounds__(SA_THREADS, 4) k_accept_cluster(const __grid_constant__ StaticAcceptParams p, const float* __restrict__ logits, int V, int ld) {
-  constexpr int SEG = 4;
   __shared__ unsigned long long red[64][SEG];
   __shared__ unsigned long long gathered[SA_CTAS][64];
   __shared__ unsigned int miss[2];
@@ -2190,8 +2191,10 @@ extern "C" int stairs_accept_static(const float* logits_dev, int vocab, int ld, 
   // (a CTA reads about 100 KB per us: at 256 KB each the launches saved are worth less than more CTAs)
   if (n_req * SA_CTAS >= 128 || (long long)(k_top + 1) * vocab * 4 <= (long long)SA_CTAS * (256 << 10)) {
     const bool vec = ld % 4 == 0 && (reinterpret_cast<uintptr_t>(logits_dev) & 15) == 0;
-    if (vec) k_accept_cluster<true><<<n_req * SA_CTAS, SA_THREADS, 0, st>>>(p, logits_dev, vocab, ld);
-    else k_accept_cluster<false><<<n_req * SA_CTAS, SA_THREADS, 0, st>>>(p, logits_dev, vocab, ld);
+    const int per = (vocab + SA_CTAS - 1) / SA_CTAS, batch = sa_batch(vec), seg = per <= batch ? 1 : per <= 2 * batch ? 2 : 4;
+    auto kern = vec ? (seg == 1 ? k_accept_cluster<true, 1> : seg == 2 ? k_accept_cluster<true, 2> : k_accept_cluster<true, 4>)
+                    : (seg == 1 ? k_accept_cluster<false, 1> : seg == 2 ? k_accept_cluster<false, 2> : k_accept_cluster<false, 4>);
+    kern<<<n_req * SA_CTAS, SA_THREADS, 0, st>>>(p, logits_dev, vocab, ld);
     CK(cudaGetLastError());
     return STAIRS_OK;
   }

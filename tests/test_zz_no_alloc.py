@@ -58,11 +58,11 @@ def test_static_accept_rejects_sizes_beyond_its_fixed_scratch():
     assert e.value.code == 1
 
 
-@pytest.mark.parametrize("vocab,ld", [(1, 1), (5, 8), (127, 128), (2049, 2051), (32000, 32000), (70001, 70004)])
+@pytest.mark.parametrize("vocab,ld", [(1, 1), (5, 8), (127, 128), (2049, 2051), (8192, 8192), (8193, 8196), (16384, 16384), (16385, 16388), (32000, 32000), (70001, 70004)])
 @pytest.mark.parametrize("ks", [[0], [4], [63], [2, 0, 5], [1] * 64], ids=lambda k: f"{len(k)}x{max(k) + 1}")
 def test_static_accept_equals_torch_argmax(vocab, ld, ks):
     # one cluster per request, and the many-block form for few long requests; odd row lengths, unaligned
-    # rows, ties (lowest index wins)
+    # rows, ties (lowest index wins), both sides of the lengths at which a slice is cut in two and in four
     from paper_2407_19947_b200 import build, stairs
     build.build()
     rows, k_max = sum(ks) + len(ks), max(ks)
