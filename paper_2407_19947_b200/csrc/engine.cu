@@ -109,7 +109,7 @@ struct stairs_ctx {
   size_t io_draft = 0, io_tt = 0, io_al = 0;   // offsets in ints
   unsigned long long wait_limit = 0;
   bool use_mk = false;
-  int small_ctas = 0;                // cluster size of the small fp32 models' one-launch passes (0: not used)
+  int small_fit[3] = {0, 0, 0};      // small fp32 models' one-launch passes: clusters of 16, 8 and 4 CTAs that run at once (0: none)
   bool draft_shares_kv = false;      // early-exit assistant on the persistent kernel: it uses the main model's K/V pools
   unsigned long long bar_base = 0;   // grid-barrier arrivals consumed by earlier launches
   int kps_force = 0;                 // tuning: k-blocks per pipeline stage (0 = chosen per row box)
@@ -1250,6 +1250,15 @@ int forward(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, int n_logi
 // ---------------------------------------------------------------------------------------------
 // Small fp32 models: a pass in one launch (small_f32.cuh).
 // ---------------------------------------------------------------------------------------------
+// CTAs per cluster of a launch of n clusters: the largest size of which so many run at once (a second wave would cost as much as
+// the first: of 16 CTAs, one per SM, seven clusters fit the chip; 8 requests x 16 rows of config 1 took 455 us in two waves, 285
+// in clusters of eight CTAs, 415 launched operation by operation).  0: none.
+int small_ctas(const stairs_ctx* ctx, int n) {
+  for (int i = 0; i < 3; ++i)
+    if (ctx->small_fit[i] >= n) return 16 >> i;
+  return 0;
+}
+
 // The cluster's 16 SMs stream weights at about a quarter of the chip's rate and save some 11 launches of 4 us per
 // layer: worth it up to about 32 MB of weights a layer.  Its attention gives one row and head to eight
 // warps, which long contexts would wait for.
@@ -1257,7 +1266,7 @@ bool small_eligible(const stairs_ctx* ctx, const DevModel& M, int T, int n_req, 
   const stairs_model& m = M.m;
   const size_t nq = (size_t)m.n_heads * m.head_dim, nkv = (size_t)m.n_kv_heads * m.head_dim;
   const size_t layer = 4 * (size_t)m.d_model * (2 * nq + 2 * nkv + (size_t)m.d_ff * (m.act == 1 ? 3 : 2));
-  return ctx->small_ctas > 0 && M.small_layers && T <= small::S_ROWS && n_req <= small::S_MAX_REQ && m.n_layers >= 1 && m.n_layers <= small::S_MAX_LAYERS &&
+  return small_ctas(ctx, 1) > 0 && M.small_layers && T <= small::S_ROWS && n_req <= small::S_MAX_REQ && m.n_layers >= 1 && m.n_layers <= small::S_MAX_LAYERS &&
          m.head_dim <= small::S_MAX_HD && small::smem_bytes(m.d_model, (int)nq, m.d_ff) <= (size_t)tc::SMEM_LIMIT && layer <= (32u << 20) && len <= 2048;
 }
 
@@ -1279,10 +1288,11 @@ small::SmallParams small_params(stairs_ctx* ctx, const DevModel& M) {
 }
 
 int launch_small(stairs_ctx* ctx, const DevModel& M, const small::SmallParams& p, int clusters = 1) {
+  const int ctas = small_ctas(ctx, clusters);
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(ctx->small_ctas * clusters); cfg.blockDim = dim3(small::S_THREADS); cfg.dynamicSmemBytes = small::smem_bytes(M.m.d_model, M.m.n_heads * M.m.head_dim, M.m.d_ff); cfg.stream = ctx->stream;
+  cfg.gridDim = dim3(ctas * clusters); cfg.blockDim = dim3(small::S_THREADS); cfg.dynamicSmemBytes = small::smem_bytes(M.m.d_model, M.m.n_heads * M.m.head_dim, M.m.d_ff); cfg.stream = ctx->stream;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = ctx->small_ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = 1;
   ctx->launches++;
   CK(cudaLaunchKernelEx(&cfg, small::k_small, p));
@@ -1308,7 +1318,7 @@ int small_deal(small::SmallParams& p, int n_req) {
   return 0;
 }
 
-// Uploads a model's per-layer pointers and finds the largest cluster that can run.
+// Uploads a model's per-layer pointers and finds how many clusters of each size run at once.
 int setup_small(stairs_ctx* ctx, DevModel& M, size_t off) {
   std::vector<small::SmallLayer> v(M.m.n_layers);
   for (int l = 0; l < M.m.n_layers; ++l) {
@@ -1326,18 +1336,16 @@ int setup_small(stairs_ctx* ctx, DevModel& M, size_t off) {
   CK(cudaMemcpyAsync(ctx->ws + off, v.data(), v.size() * sizeof(small::SmallLayer), cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   M.small_layers = reinterpret_cast<const small::SmallLayer*>(ctx->ws + off);
-  if (ctx->small_ctas == 0) {
+  if (small_ctas(ctx, 1) == 0) {
     CK(cudaFuncSetAttribute(small::k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT));
     CK(cudaFuncSetAttribute(small::k_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    for (int n = 16; n >= 4 && ctx->small_ctas == 0; n /= 2) {
+    for (int i = 0; i < 3; ++i) {
       cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3(n); cfg.blockDim = dim3(small::S_THREADS); cfg.dynamicSmemBytes = tc::SMEM_LIMIT;
+      cfg.gridDim = dim3(16 >> i); cfg.blockDim = dim3(small::S_THREADS); cfg.dynamicSmemBytes = tc::SMEM_LIMIT;
       cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = n; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = 16 >> i; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
       cfg.attrs = at; cfg.numAttrs = 1;
-      int clusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&clusters, small::k_small, &cfg) == cudaSuccess && clusters >= 1) ctx->small_ctas = n;
-      else cudaGetLastError();
+      if (cudaOccupancyMaxActiveClusters(&ctx->small_fit[i], small::k_small, &cfg) != cudaSuccess) { ctx->small_fit[i] = 0; cudaGetLastError(); }
     }
   }
   return STAIRS_OK;
@@ -1719,7 +1727,8 @@ int stairs_validate(stairs_ctx* ctx, int n_req, const int32_t* req_ids_host, con
     sp.mode = ROWS_VALIDATE; sp.T = T; sp.n_req = n_req; sp.head_rows = 1; sp.draft = draft_dev;
     for (int i = 0; i < n_req; ++i) { sp.val_req[i] = req_ids_host[i]; sp.val_k[i] = k_host[i]; sp.val_off[i] = off[i]; }
     sp.logits = logits_dev_or_null; sp.target_tokens = target_tokens_dev; sp.accept_len = accept_len_dev; sp.commit = commit;
-    if (const int clusters = small_deal(sp, n_req)) {
+    const int clusters = small_deal(sp, n_req);
+    if (clusters && small_ctas(ctx, clusters)) {
       int rc = launch_small(ctx, ctx->target, sp, clusters);
       if (rc) return rc;
       if (ctx->profile) cudaEventRecord(ctx->call_end, ctx->stream);

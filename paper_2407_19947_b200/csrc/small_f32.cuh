@@ -19,7 +19,7 @@
 // by launch 220), the draft of four tokens 130 us (330), the whole call 7.24 ms -> 3.41 ms.  What is left is
 // latency: about 2.5 us for each of a layer's five steps (barrier and publication 1 us, the rest code that runs once).
 // Rows are taken eight at a time (a pass per block of rows: later rows only need earlier rows' K/V); the requests of a
-// validate call are dealt to several clusters, which have nothing to do with one another.
+// validate call are dealt to several clusters, which have nothing to do with one another (8 CTAs each where not all of 16 would run at once).
 //
 // A warp owns whole features; its lanes stride the K dimension in 16-byte vectors and hold one sum per
 // (feature, row).  The order of the additions depends on K only, and a row's attention on its position

@@ -81,3 +81,23 @@ def test_requests_dealt_to_clusters_match_the_per_operation_kernels(k, n_req, la
         eng.close()
     assert torch.equal(got[0][0][:, : k + 1], got[1][0][:, : k + 1]) and torch.equal(got[0][1], got[1][1])
     assert float((got[0][2] - got[1][2]).abs().max()) < 1e-4
+
+
+@pytest.mark.parametrize("k", [4, 11])
+def test_rows_are_the_same_in_clusters_of_eight_and_sixteen_ctas(k):
+    # eight requests: eight clusters, which run at once only in the smaller size; one request: one cluster of 16
+    st = _stairs()
+    shape = SHAPES["gqa_rope"]
+    tsrc, _ = sources(shape, std=0.03)
+    eng = st.Stairs(tsrc, None, max_requests=8, max_seq_len=320, k_max=k, kv_page_tokens=16)
+    for i in range(8):
+        eng.prefill(i, list(wl.zipf_tokens(3 + 41 * i, shape.vocab, i)))
+    drafts = torch.from_numpy(np.random.default_rng(k).integers(0, shape.vocab, size=(8, k)).astype(np.int32)).cuda()
+    before = eng.launch_count()
+    tt, al, lg = eng.validate(list(range(8)), [k] * 8, drafts, want_logits=True)
+    assert eng.launch_count() - before == 1
+    for i in range(8):
+        tt1, al1, lg1 = eng.validate([i], [k], drafts[i:i + 1].contiguous(), want_logits=True)
+        assert torch.equal(lg1, lg[i * (k + 1):(i + 1) * (k + 1)]) and torch.equal(tt1[0], tt[i]) and torch.equal(al1[0], al[i])
+    eng.sync()
+    eng.close()
