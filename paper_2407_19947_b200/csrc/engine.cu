@@ -1259,15 +1259,36 @@ int small_ctas(const stairs_ctx* ctx, int n) {
   return 0;
 }
 
-// The cluster's 16 SMs stream weights at about a quarter of the chip's rate and save some 11 launches of 4 us per
-// layer: worth it up to about 32 MB of weights a layer.  Its attention gives one row and head to eight
-// warps, which long contexts would wait for.
+// What the cluster kernel can hold.  (A block of rows of one step has to fit the shared memory: a layer has 10 MB of weights at most.)
 bool small_eligible(const stairs_ctx* ctx, const DevModel& M, int T, int n_req, int len) {
   const stairs_model& m = M.m;
-  const size_t nq = (size_t)m.n_heads * m.head_dim, nkv = (size_t)m.n_kv_heads * m.head_dim;
-  const size_t layer = 4 * (size_t)m.d_model * (2 * nq + 2 * nkv + (size_t)m.d_ff * (m.act == 1 ? 3 : 2));
   return small_ctas(ctx, 1) > 0 && M.small_layers && T <= small::S_ROWS && n_req <= small::S_MAX_REQ && m.n_layers >= 1 && m.n_layers <= small::S_MAX_LAYERS &&
-         m.head_dim <= small::S_MAX_HD && small::smem_bytes(m.d_model, (int)nq, m.d_ff) <= (size_t)tc::SMEM_LIMIT && layer <= (32u << 20) && len <= 2048;
+         m.head_dim <= small::S_MAX_HD && small::smem_bytes(m.d_model, m.n_heads * m.head_dim, m.d_ff) <= (size_t)tc::SMEM_LIMIT && len <= 2048;
+}
+
+// Is a call quicker on the cluster kernel than launched operation by operation?  T rows in all, `rows` of them in the busiest
+// cluster, `len` positions in the longest context.  Both estimates (us) are fitted to 954 measured calls of eleven models (one to
+// eight layers of width 128 to 512, head sizes 32 to 128, vocabularies of 500 to 128256, 1 to 16 rows a request, contexts of 16
+// to 2000).  A pass of eight rows takes its steps, in which most of the layers' weights are hidden, the LM head at the cluster's rate
+// of about half a TB/s, and its rounds of attention; the launches take 4.2 us each, the weights, products that grow
+// with the rows, and attention of one block a row and head.  Always taking the cluster was up to twice as slow (one row of four
+// layers of 256 with 128256 tokens: 372 us against 249; 9 rows with 32000 tokens: 306 against 207); this choice misses the better
+// side by more than 3 % in five of the 954, by 9 % at most.
+bool small_pays(const stairs_ctx* ctx, const DevModel& M, int ctas, int rows, int T, int len, bool head) {
+  const stairs_model& m = M.m;
+  const double nq = (double)m.n_heads * m.head_dim, nkv = (double)m.n_kv_heads * m.head_dim, L = m.n_layers;
+  const double layers_mb = 4e-6 * m.d_model * L * (2 * nq + 2 * nkv + (double)m.d_ff * (m.act == 1 ? 3 : 2)), head_mb = head ? 4e-6 * m.d_model * m.vocab : 0.0;
+  double one = 0;
+  for (int r0 = 0; r0 < rows; r0 += small::S_BLOCK) {
+    const int r = std::min(small::S_BLOCK, rows - r0), groups = ctas * (small::S_WARPS / small::S_GROUP);
+    const int rounds = (r * m.n_heads + groups - 1) / groups, chunks = (len + small::S_GROUP * 32 - 1) / (small::S_GROUP * 32);
+    one += 3.9 * (5 * L + (head ? 1 : -4)) + (layers_mb * (r <= 2 ? 0.39 : 1.3) + head_mb * (r <= 2 ? 1.6 : r <= 5 ? 1.9 : 2.4)) * 16 / ctas +
+           L * rounds * chunks * (m.head_dim <= 64 ? 2.9 : 6.4);
+  }
+  const double blocks = (double)T * m.n_heads / (2.0 * ctx->sm_count);
+  const double ops = 4.2 * (11 * L + 5) + 1.5 * layers_mb + 0.081 * head_mb + 0.079 * T * (layers_mb + head_mb) +
+                     L * len * (0.045 + 0.0006 * m.head_dim) * (1.1 + 0.37 * std::max(0.0, blocks - 1.0));
+  return one <= ops;
 }
 
 small::SmallParams small_params(stairs_ctx* ctx, const DevModel& M) {
@@ -1300,11 +1321,12 @@ int launch_small(stairs_ctx* ctx, const DevModel& M, const small::SmallParams& p
 }
 
 // Deals a validate call's requests to clusters, in order, so that the busiest takes as few passes of eight rows as it can;
-// returns the number of clusters, 0 where that is too many passes (see S_MOST_PASSES).
-int small_deal(small::SmallParams& p, int n_req) {
+// returns the number of clusters (0: more than S_MOST_PASSES passes), and the rows of the busiest in *most.
+int small_deal(small::SmallParams& p, int n_req, int* most) {
   for (int passes = 1; passes <= small::S_MOST_PASSES; ++passes) {
     int n = 0, rows = 0;
     bool fits = true;
+    *most = 0;
     for (int i = 0; i < n_req && fits; ++i) {
       const int r = p.val_k[i] + 1, room = passes * small::S_BLOCK;
       if (i == 0 || rows + r > room) {
@@ -1312,6 +1334,7 @@ int small_deal(small::SmallParams& p, int n_req) {
         if (fits) { p.cl_req[n++] = i; rows = 0; }
       }
       rows += r;
+      *most = std::max(*most, rows);
     }
     if (fits) { p.cl_req[n] = n_req; return n; }
   }
@@ -1395,7 +1418,8 @@ int prefill_model(stairs_ctx* ctx, DevModel& M, int slot, int n_ctx) {
     return launch_forward_mk(ctx, M, n_ctx, 0, 0, c);
   }
   // longer: chunks of equal length
-  const bool wide = wide_eligible(ctx, M), tiny = n_ctx <= small::S_MOST_PASSES * small::S_BLOCK && small_eligible(ctx, M, 1, 1, n_ctx);
+  const bool wide = wide_eligible(ctx, M), tiny = n_ctx <= small::S_MOST_PASSES * small::S_BLOCK && small_eligible(ctx, M, 1, 1, n_ctx) &&
+                                                 small_pays(ctx, M, small_ctas(ctx, 1), n_ctx, n_ctx, n_ctx, false);
   const int most = prefill_rows(ctx->cfg);
   const int n_chunks = (n_ctx + most - 1) / most, chunk = (n_ctx + n_chunks - 1) / n_chunks;
   for (int c0 = 0; c0 < n_ctx; c0 += chunk) {
@@ -1653,7 +1677,7 @@ int stairs_draft(stairs_ctx* ctx, int req, int k, int32_t* draft_dev) {
     return fail(ctx, STAIRS_ENOSPC, "request %d: sequence would exceed max_seq_len", req);
   rc = ensure_pages(ctx, req, ctx->n_seq_ub[req] + k);
   if (rc) return rc;
-  if (small_eligible(ctx, ctx->draft, 2, 1, ctx->n_seq_ub[req] + k)) {
+  if (small_eligible(ctx, ctx->draft, 2, 1, ctx->n_seq_ub[req] + k) && small_pays(ctx, ctx->draft, small_ctas(ctx, 1), 1, 1, ctx->n_seq_ub[req] + k, true)) {
     small::SmallParams sp = small_params(ctx, ctx->draft);
     sp.mode = ROWS_DRAFT_FIRST; sp.slot = req; sp.steps = k; sp.head_rows = 1; sp.draft_out = draft_dev;
     return launch_small(ctx, ctx->draft, sp);
@@ -1727,8 +1751,9 @@ int stairs_validate(stairs_ctx* ctx, int n_req, const int32_t* req_ids_host, con
     sp.mode = ROWS_VALIDATE; sp.T = T; sp.n_req = n_req; sp.head_rows = 1; sp.draft = draft_dev;
     for (int i = 0; i < n_req; ++i) { sp.val_req[i] = req_ids_host[i]; sp.val_k[i] = k_host[i]; sp.val_off[i] = off[i]; }
     sp.logits = logits_dev_or_null; sp.target_tokens = target_tokens_dev; sp.accept_len = accept_len_dev; sp.commit = commit;
-    const int clusters = small_deal(sp, n_req);
-    if (clusters && small_ctas(ctx, clusters)) {
+    int most = 0;
+    const int clusters = small_deal(sp, n_req, &most), ctas = clusters ? small_ctas(ctx, clusters) : 0;
+    if (ctas && small_pays(ctx, ctx->target, ctas, most, T, len_all, true)) {
       int rc = launch_small(ctx, ctx->target, sp, clusters);
       if (rc) return rc;
       if (ctx->profile) cudaEventRecord(ctx->call_end, ctx->stream);

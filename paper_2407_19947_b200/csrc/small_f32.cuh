@@ -36,9 +36,7 @@ namespace small {
 
 constexpr int S_WARPS = 8, S_THREADS = S_WARPS * 32;
 constexpr int S_BLOCK = 8;           // rows of a pass
-// Passes one launch pays for (four layers of width 256): one pass takes 107 us (5 rows) to 118 (8), two 207 to 232, three 320,
-// four 462; one launch per operation takes 270 us for 5 rows, 290 for 24 or 16 x 2, 315 for 64.  Prefills alike: two
-// passes 163 us against 229, three 250 against 245.
+// Most passes of a launch; whether a call's are quicker than one launch per operation is small_pays' to say.
 constexpr int S_MOST_PASSES = 2;
 constexpr int S_MAX_HD = 128, S_MAX_REQ = 64, S_MAX_LAYERS = 32, S_MAX_CTAS = 16;
 constexpr int S_MAX_CLUSTERS = 8;    // clusters of a validate call, each with requests of its own

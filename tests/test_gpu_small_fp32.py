@@ -101,3 +101,26 @@ def test_rows_are_the_same_in_clusters_of_eight_and_sixteen_ctas(k):
         assert torch.equal(lg1, lg[i * (k + 1):(i + 1) * (k + 1)]) and torch.equal(tt1[0], tt[i]) and torch.equal(al1[0], al[i])
     eng.sync()
     eng.close()
+
+
+@pytest.mark.parametrize("vocab,launches", [(512, 1), (128256, None)])
+def test_a_large_vocabulary_is_left_to_the_per_operation_kernels(vocab, launches):
+    # one cluster reads the LM head at a fraction of the chip's rate; the results are the per-operation kernels' either way
+    st = _stairs()
+    shape = wl.family_a(1, 128, 2, 256, vocab, 128, F32)
+    tsrc, dsrc = sources(shape, std=0.03)
+    got = []
+    for impl in (0, 1):
+        eng = st.Stairs(tsrc, dsrc, max_requests=1, max_seq_len=64, k_max=8, kv_page_tokens=16, gemm_impl=impl)
+        eng.prefill(0, list(wl.zipf_tokens(20, shape.vocab, 1)))
+        before = eng.launch_count()
+        draft = eng.draft(0, 4)
+        mid = eng.launch_count()
+        tt, al, lg = eng.validate([0], [8], draft, want_logits=True)
+        if impl == 0:
+            assert (mid - before == 1) == (launches == 1) and (eng.launch_count() - mid == 1) == (launches == 1)
+        eng.sync()
+        got.append((draft.cpu(), tt.cpu(), al.cpu(), lg.cpu()))
+        eng.close()
+    assert all(torch.equal(a, b) for a, b in zip(got[0][:3], got[1][:3]))
+    assert float((got[0][3] - got[1][3]).abs().max()) < 1e-4
