@@ -1,9 +1,12 @@
 """Passes over many rows (prefill of more than 64 positions, validate calls of more than 64 rows): logits
 against the oracle within the bf16 bar, at the edges of the row tiles, for both tile forms (one CTA, CTA
 pair), whole and split K ranges, all attention forms and head sizes."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
+from scipy.special import erfc
 
 from oracle import stairs_oracle as so
 from paper_2407_19947_b200 import workloads as wl
@@ -128,3 +131,55 @@ def test_contexts_of_two_threads_with_different_head_sizes():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+class _OneInputPerFeature(wl.WeightSource):
+    """Attention adds nothing to the residual stream; every MLP feature sees one element of it, so its value is known to a few
+    roundings."""
+
+    def _draw_numpy(self, layer, name):
+        a = super()._draw_numpy(layer, name)
+        if name == "wo":
+            a[:] = 0.0
+        elif name == "w_gate_or_fc1":
+            f = np.arange(a.shape[0])
+            a[:] = 0.0
+            a[f, f % a.shape[1]] = np.linspace(-3.5, 3.5, a.shape[0])
+        return a
+
+
+def test_gelu_of_many_row_calls_matches_64_bits():
+    # the MLP activation itself, as stored (bf16 hi + lo: 2^-17), for arguments of both signs and all sizes that occur: the exact
+    # GELU by erfc, which keeps its relative precision where 1 + erf cancels
+    st = _stairs()
+    shape = small_a(layers=1, f=1024)
+    src = _OneInputPerFeature(shape, 11, "numpy", norm_jitter=0.1, std=0.03)
+    eng = st.Stairs(src, None, max_requests=14, max_seq_len=32, k_max=4, kv_page_tokens=16)
+    prompts = [list(wl.zipf_tokens(3 + i, shape.vocab, i)) for i in range(14)]
+    for i, p in enumerate(prompts):
+        eng.prefill(i, p)
+    drafts = np.random.default_rng(2).integers(0, shape.vocab, size=(14, 4)).astype(np.int32)
+    eng.validate(list(range(14)), [4] * 14, torch.from_numpy(drafts).cuda())          # 70 rows
+    ptr, nbytes = C.c_void_p(), C.c_size_t()
+    eng._ck(eng.lib.stairs_debug_buffer(eng.h, 4, C.byref(ptr), C.byref(nbytes)))
+    rows = nbytes.value // (4 * shape.d_ff)
+    got = eng.debug_buffer(4, torch.bfloat16, rows * shape.d_ff * 2).view(2, rows, shape.d_ff)[:, :70].double().sum(0).cpu().numpy()
+    eng.close()
+    w = lambda layer, name: so.widen(src.host_array(layer, name)).astype(np.float64)
+    tok = np.concatenate([[p[-1], *d] for p, d in zip(prompts, drafts)])
+    pos = np.concatenate([len(p) - 1 + np.arange(5) for p in prompts])
+    x = w(-1, "tok_emb")[tok] + w(-1, "pos_emb")[pos]
+    mean = x.mean(1, keepdims=True)
+    xc = (x - mean) / np.sqrt(((x - mean) ** 2).mean(1, keepdims=True) + shape.norm_eps)
+    h = xc * w(0, "norm2_w")
+    v = h @ w(0, "w_gate_or_fc1").T + (w(0, "norm2_b") @ w(0, "w_gate_or_fc1").T)
+    want = 0.5 * v * erfc(-v / np.sqrt(2))
+    assert v.min() < -8 and v.max() > 8
+    # the argument: the operand's hi + lo (2^-17), 1/std, mean and products (ten roundings of 2^-24), all relative to its terms; the
+    # function: 8e-6 at most; the result: 2^-17.  d gelu / dv is at most (|v| + 1) |gelu / v| + 1 where v < 0, 1.13 elsewhere.
+    term = np.abs(h) @ np.abs(w(0, "w_gate_or_fc1")).T + np.abs(v) + np.abs(mean / x.std(1, keepdims=True)) * np.abs(w(0, "w_gate_or_fc1") @ w(0, "norm2_w"))
+    slope = np.abs(0.5 * erfc(-v / np.sqrt(2)) + v * np.exp(-v * v / 2) / np.sqrt(2 * np.pi))
+    bound = np.abs(want) * (2.0 ** -17 + 8e-6) + 1.05 * slope * term * (2.0 ** -17 + 10 * 2.0 ** -24)
+    seen = np.abs(want) > 1e-30                                      # (below, the lo part leaves bf16's range)
+    assert np.all(np.abs(got - want)[seen] <= bound[seen])
+    assert np.count_nonzero(seen & (v < -5)) > 100
