@@ -851,6 +851,17 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
   return STAIRS_OK;
 }
 
+// Events around a GEMM launch of a validate call, while profiling is on.
+struct GemmTimer {
+  stairs_ctx* c;
+  bool on;
+  explicit GemmTimer(stairs_ctx* ctx)
+      : c(ctx), on(ctx->profile && ctx->in_validate && ctx->ev_used + 2 <= (int)ctx->ev.size()) {
+    if (on) cudaEventRecord(c->ev[c->ev_used++], c->stream);
+  }
+  ~GemmTimer() { if (on) cudaEventRecord(c->ev[c->ev_used++], c->stream); }
+};
+
 // ---------------------------------------------------------------------------------------------
 // Many-row passes (wide.cuh): tile plan per GEMM, launches chained with programmatic dependent launch.
 // ---------------------------------------------------------------------------------------------
@@ -959,6 +970,7 @@ int launch_wide_gemm(stairs_ctx* ctx, wide::WideJob& job, const void* x, int K, 
   const int grid = std::min(slots, job.n_tiles * job.m_tiles * pl.splits) * pl.cg;
   const size_t smem = wide::gemm_smem(job.x_box, pl.tn, pl.cg, job.stages);
   ctx->launches++;
+  GemmTimer tm(ctx);
   CK(launch_chained(ctx->stream, pl.cg == 2 ? wide::k_wide_gemm<2> : wide::k_wide_gemm<1>, dim3(grid), wide::WTHREADS, smem, dim3(pl.cg, 1, 1), job));
   return STAIRS_OK;
 }
@@ -1113,16 +1125,6 @@ int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* l
 // ---------------------------------------------------------------------------------------------
 // One forward pass over T rows (tok/pos/req already built on the device).
 // ---------------------------------------------------------------------------------------------
-struct GemmTimer {
-  stairs_ctx* c;
-  bool on;
-  explicit GemmTimer(stairs_ctx* ctx)
-      : c(ctx), on(ctx->profile && ctx->in_validate && ctx->ev_used + 2 <= (int)ctx->ev.size()) {
-    if (on) cudaEventRecord(c->ev[c->ev_used++], c->stream);
-  }
-  ~GemmTimer() { if (on) cudaEventRecord(c->ev[c->ev_used++], c->stream); }
-};
-
 template <typename WT>
 int forward_rows(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, int n_logit_rows, float* logits_out) {
   const stairs_model& m = M.m;

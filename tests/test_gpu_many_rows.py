@@ -183,3 +183,19 @@ def test_gelu_of_many_row_calls_matches_64_bits():
     seen = np.abs(want) > 1e-30                                      # (below, the lo part leaves bf16's range)
     assert np.all(np.abs(got - want)[seen] <= bound[seen])
     assert np.count_nonzero(seen & (v < -5)) > 100
+
+
+def test_profile_times_every_gemm_of_a_many_row_call():
+    st = _stairs()
+    shape = small_b(8, 2, 64)
+    tsrc, _ = sources(shape)
+    eng = st.Stairs(tsrc, None, max_requests=2, max_seq_len=128, k_max=39, kv_page_tokens=16)
+    for i in range(2):
+        eng.prefill(i, list(wl.zipf_tokens(20 + i, shape.vocab, i)))
+    drafts = torch.zeros((2, 39), dtype=torch.int32, device="cuda")
+    eng.profile(True)
+    eng.validate([0, 1], [39, 39], drafts)
+    gemm_ms, launches, call_ms = eng.profile_read()
+    eng.profile(False)
+    assert launches == 4 * shape.n_layers + 1 and 0 < gemm_ms < call_ms     # QKV, O, gate + up, down; the LM head
+    eng.close()
