@@ -960,7 +960,7 @@ int launch_wide_gemm(stairs_ctx* ctx, wide::WideJob& job, const void* x, int K, 
   const CUtensorMap* xm = wide_map(ctx, x, L.max_rows, K, job.x_box, 2);
   if (!xm) return fail(ctx, STAIRS_ECUDA, "cuTensorMapEncodeTiled failed for an activation buffer");
   job.x_map = *xm;
-  if (job.n_tiles * job.m_tiles > TC_COUNTERS) return fail(ctx, STAIRS_EUNSUPPORTED, "too many tiles for the split bookkeeping");
+  if (pl.splits > 1 && (long long)job.n_tiles * job.m_tiles > TC_COUNTERS) return fail(ctx, STAIRS_EUNSUPPORTED, "too many tiles for the split bookkeeping");
   job.stages = wide::gemm_stages(job.x_box, pl.tn, pl.cg);
   job.lo_row = L.max_rows;
   job.partial = reinterpret_cast<float*>(ctx->ws + L.gemm_partial);

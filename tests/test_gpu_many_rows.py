@@ -199,3 +199,21 @@ def test_profile_times_every_gemm_of_a_many_row_call():
     eng.profile(False)
     assert launches == 4 * shape.n_layers + 1 and 0 < gemm_ms < call_ms     # QKV, O, gate + up, down; the LM head
     eng.close()
+
+
+def test_prefill_pass_of_more_tiles_than_split_counters():
+    # 72000 rows x 61440 gate and up columns in one pass: 67680 tiles (whole ones need no counter); against passes of 2048 rows
+    st = _stairs()
+    shape = small_b(1, 1, 64, layers=2, d=64, f=30720, v=512)
+    tsrc, _ = sources(shape)
+    prompt = list(wl.zipf_tokens(72001, shape.vocab, 3))
+    got = []
+    for chunk in (72000, 0):
+        eng = st.Stairs(tsrc, None, max_requests=1, max_seq_len=72008, k_max=2, kv_page_tokens=128, prefill_chunk=chunk)
+        eng.prefill(0, prompt)
+        _, _, lg = eng.validate([0], [0], None, want_logits=True)
+        eng.sync()
+        got.append(lg.cpu())
+        eng.close()
+        del eng
+    assert torch.isfinite(got[0]).all() and float((got[0] - got[1]).abs().max()) < 5e-3
