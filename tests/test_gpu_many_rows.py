@@ -217,3 +217,41 @@ def test_prefill_pass_of_more_tiles_than_split_counters():
         eng.close()
         del eng
     assert torch.isfinite(got[0]).all() and float((got[0] - got[1]).abs().max()) < 5e-3
+
+
+# Distances between the two bf16 paths (2-norm over the logits' 2-norm).  Both take operands as bf16 hi + lo (2^-17) and K and V as
+# fp16, so they differ by the order of fp32 sums and by what that flips in an operand's last bit: 1.5e-5 to 8.7e-5 measured.  The same
+# passes emulated in numpy with the lo part of just one operand (norm 1, attention, norm 2, MLP or final norm) left out are off by at
+# least 4.7e-4 where the rows themselves went through them, and by 1.6e-4 where only the cached positions did.
+ROWS_BAR, PREFIX_BAR = 2.5e-4, 1.2e-4
+
+
+def _distance(a, b):
+    return float((a.double() - b.double()).norm() / b.double().norm())
+
+
+@pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES.keys())
+def test_many_row_passes_agree_with_small_ones(shape):
+    st = _stairs()
+    tsrc, _ = sources(shape)
+    eng = st.Stairs(tsrc, None, max_requests=26, max_seq_len=400, k_max=4, kv_page_tokens=16)
+    # 65 positions prefilled in one many-row pass, against 64 by the persistent kernel and the last as a row of the call
+    prompt = list(wl.zipf_tokens(66, shape.vocab, 5))
+    eng.prefill(0, prompt)
+    eng.prefill(1, prompt[:65])
+    _, _, a = eng.validate([0], [0], None, want_logits=True)
+    nxt = torch.tensor([[prompt[65], 0, 0, 0]], dtype=torch.int32, device="cuda")
+    _, _, b = eng.validate([1], [1], nxt, want_logits=True)
+    eng.sync()
+    assert _distance(a[0], b[1]) < PREFIX_BAR
+    # 65 rows (one tile) and 130 (two, or a pair) against calls of 5 rows
+    for i in range(26):
+        eng.prefill(i, list(wl.zipf_tokens(20 + 3 * i, shape.vocab, 60 + i))[:64])
+    drafts = torch.from_numpy(np.random.default_rng(1).integers(0, shape.vocab, size=(26, 4)).astype(np.int32)).cuda()
+    alone = torch.cat([eng.validate([i], [4], drafts[i:i + 1].contiguous(), want_logits=True)[2] for i in range(26)])
+    for cg, n in ((0, 13), (1, 26), (2, 26)):
+        eng.debug_tune(4, cg)
+        _, _, many = eng.validate(list(range(n)), [4] * n, drafts[:n].contiguous(), want_logits=True)
+        eng.sync()
+        assert _distance(many, alone[: 5 * n]) < ROWS_BAR
+    eng.close()
