@@ -367,8 +367,8 @@ __device__ __forceinline__ bool group_ok(Ctl* ctl, int et) {
 }
 
 // Is an mbarrier wait's polling loop inlined?  In the variants whose attention runs on mma.sync a call spoils more registers of
-// the surrounding code than the loop is long: 7B, 9 rows 2770 -> 2682 us, 3B, 5 rows 1984 -> 1945, 0.4B even; the
-// tcgen05 ones get longer by 1 % (four layers of 7B, 4 x 16384 positions 1009 -> 1020).
+// the surrounding code than the loop is long: 7B, 9 rows 2745 -> 2681 us, 3B, 5 rows 1983 -> 1943, draft of 4 tokens by two 7B layers
+// 905 -> 886, 0.4B even (1003, 1005); the tcgen05 ones get longer by 1 % (four layers of 7B, 4 x 16384 positions 1012 -> 1019).
 #ifndef STAIRS_WAIT_SLOW
 #define STAIRS_WAIT_SLOW __noinline__
 #endif
