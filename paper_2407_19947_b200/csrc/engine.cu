@@ -870,7 +870,8 @@ struct WidePlan { int cg, tn, splits; };
 // Tile shape of one GEMM over T rows: pairs of CTAs (256 rows) or single CTAs (128 rows), tile width a
 // multiple of `gran` (whole heads for the QKV projection), K cut in up to 8 ranges where few tiles would leave
 // the chip idle.  The estimate is fitted to measured sweeps of every form over 72 to 2048 rows at the
-// configs' widths (its choice is 3 % from the best one on average): about 4.5 us per launch; a k-block
+// configs' widths (its choice is 3 % from the best one on average; six other models of width 512 to 5120: never more than 3 % behind
+// one form for all their GEMMs up to 1024 rows, 8 to 11 % behind pairs at 1500 and 2048 rows of width 3072 and 5120): about 4.5 us per launch; a k-block
 // costs the slowest of its MMAs (hi and lo part; 810 cycles at least: issue and commit), the SM's loads (95 GB/s)
 // and the L2's (10 TB/s over the active SMs); whole waves of units, weights from HBM once; the last
 // tile's epilogue is exposed; split tiles add the round trip of their parked sums, pairs their handshakes.
