@@ -114,9 +114,17 @@ def _ptr(a: np.ndarray):
 
 
 def _ints(a):
-    """Integers as a ctypes array, accepted or refused as numpy does (ctypes itself would wrap what does not fit in
-    32 bits).  Passing the numpy array's pointer instead takes three times as long."""
-    return (C.c_int32 * len(a)).from_buffer_copy(_i32(a))
+    """Integers as a ctypes array, accepted or refused as numpy does.  Short lists go to ctypes directly, which takes half the
+    time, and count if they come back as they were (ctypes wraps what does not fit in 32 bits)."""
+    n = len(a)
+    if n <= 4 and type(a) is list:
+        try:
+            r = (C.c_int32 * n)(*a)
+            if r[:] == a:
+                return r
+        except TypeError:   # not integers
+            pass
+    return (C.c_int32 * n).from_buffer_copy(_i32(a))
 
 
 def _results(t, n, k_max, ks, device):
@@ -236,8 +244,8 @@ class Stairs:
         t = self.torch
         r, kk = _ints(req_ids), _ints(k)
         n = len(r)
-        tt, al = _results(t, n, self.k_max, kk, self._dev) if out is None else out
-        logits = t.empty((sum(kk) + n, self.vocab), dtype=t.float32, device=self._dev) if want_logits else None
+        tt, al = _results(t, n, self.k_max, kk[:], self._dev) if out is None else out
+        logits = t.empty((sum(kk[:]) + n, self.vocab), dtype=t.float32, device=self._dev) if want_logits else None
         self._ck(self.lib.stairs_validate(self.h, n, r, kk,
                                           draft_dev.data_ptr() if draft_dev is not None else None,
                                           tt.data_ptr(), al.data_ptr(),
@@ -324,7 +332,7 @@ def accept_static(logits_dev, k: Sequence[int], draft_dev, k_max: int, *, vocab:
     lib = load_library()
     kk = _ints(k)
     n = len(kk)
-    tt, al = _results(torch, n, k_max, kk, logits_dev.device)
+    tt, al = _results(torch, n, k_max, kk[:], logits_dev.device)
     st = stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     rc = lib.stairs_accept_static(logits_dev.data_ptr(), vocab or logits_dev.shape[1], logits_dev.stride(0), n, kk,
                                   draft_dev.data_ptr() if draft_dev is not None else None, k_max,

@@ -83,12 +83,12 @@ def test_null_context_is_an_error_not_a_crash(lib):
     assert lib.stairs_launch_count(None) == 0
 
 
-@pytest.mark.parametrize("n", [1, 12, 13, 64])
+@pytest.mark.parametrize("n", [1, 4, 5, 64])
 def test_request_ids_and_draft_lengths_convert_as_numpy_does(n):
     # on either side of 32 bits; numbers that are whole, of any type and container
     for edge in (2**31 - 1, -2**31):
         assert list(st._ints([edge] * n)) == [edge] * n
-    for beyond in (2**31, -2**31 - 1, 2**32 + 1):
+    for beyond in (2**31, -2**31 - 1, 2**32 + 1, 2**70):
         with pytest.raises(OverflowError):
             st._ints([0] * (n - 1) + [beyond])
     for whole in ([4.0] * n, (4,) * n, np.full(n, 4, np.int64), np.full(n, 4, np.int16), [np.int32(4)] * n):
