@@ -19,6 +19,7 @@
 #include "gemm_tc.cuh"
 #include "kernels_basic.cuh"
 #include "megakernel.cuh"
+#include "mid.cuh"
 #include "small_f32.cuh"
 #include "wide.cuh"
 
@@ -116,6 +117,8 @@ struct stairs_ctx {
   int att_nbuf_force = 0;            // tuning: K/V chunk buffers of the attention phases (0 = chosen from the context length)
   int att_tc_force = 0;              // tuning: 1 = tcgen05 attention for every call it can serve
   int att_tc_off = 0;                // tuning: 1 = attention contractions on mma.sync even where the tcgen05 path applies
+  int mid_force = 0;                 // tuning: pairs per cluster of those (0 = planned)
+  int mid_fit[mid::MAX_C + 1] = {};  // passes of 65 to 128 rows: clusters of so many CTA pairs that run at once
   int wide_cg_force = 0, wide_split_force = 0;   // tuning: CTAs per tile and K ranges of the many-row GEMMs (0 = planned)
   int att_tma_off = 0;               // tuning: 1 = stage K/V with 16-byte copies from the compute warps even where bulk copies apply
 };
@@ -360,11 +363,11 @@ bool encode_map3(stairs_ctx* ctx, CUtensorMap* out, const void* ptr, long long r
   return r == CUDA_SUCCESS;
 }
 
-// [2 parts][rows][K] view of a hi + lo operand; box = 64 k-elements x box_rows rows of both parts.
-bool encode_map_parts(stairs_ctx* ctx, CUtensorMap* out, const void* ptr, long long rows, long long K, int box_rows) {
+// [2 parts][rows][K] view of a hi + lo operand; box = 64 k-elements x box_rows rows of both parts or of one.
+bool encode_map_parts(stairs_ctx* ctx, CUtensorMap* out, const void* ptr, long long rows, long long K, int box_rows, int box_parts) {
   cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, 2};
   cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)(rows * K) * 2};
-  cuuint32_t box[3] = {(cuuint32_t)tc::BK, (cuuint32_t)box_rows, 2};
+  cuuint32_t box[3] = {(cuuint32_t)tc::BK, (cuuint32_t)box_rows, (cuuint32_t)box_parts};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = ctx->encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -869,7 +872,7 @@ struct WidePlan { int cg, tn, splits; };
 
 // Tile shape of one GEMM over T rows: pairs of CTAs (256 rows) or single CTAs (128 rows), tile width a
 // multiple of `gran` (whole heads for the QKV projection), K cut in up to 8 ranges where few tiles would leave
-// the chip idle.  The estimate is fitted to measured sweeps of every form over 72 to 2048 rows at the
+// the chip idle.  The estimate is fitted to measured sweeps of every form over 72 to 2048 rows (up to 128 rows mid.cuh is quicker) at the
 // configs' widths (its choice is 3 % from the best one on average; six other models of width 512 to 5120: never more than 3 % behind
 // one form for all their GEMMs up to 1024 rows, 8 to 11 % behind pairs at 1500 and 2048 rows of width 3072 and 5120): about 4.5 us per launch; a k-block
 // costs the slowest of its MMAs (hi and lo part; 810 cycles at least: issue and commit), the SM's loads (95 GB/s)
@@ -886,10 +889,8 @@ WidePlan wide_plan(const stairs_ctx* ctx, int T, int K, const int* rows, int n_s
   WidePlan best{1, gran, 1};
   double best_us = 1e30;
   for (int cg = 1; cg <= 2; ++cg) {
-    if (cg == 2 && T <= wide::WM) continue;
-    if (ctx->wide_cg_force && cg != ctx->wide_cg_force && T > wide::WM) continue;
+    if (ctx->wide_cg_force && cg != ctx->wide_cg_force) continue;
     const int m_tiles = (T + wide::WM * cg - 1) / (wide::WM * cg);
-    const int x_box = m_tiles == 1 && cg == 1 ? (T + 15) / 16 * 16 : wide::WM;
     for (int tn = gran; tn <= 256; tn += gran) {
       if (tn < 32 || (cg == 2 && (tn % 32 || tn < 64))) continue;   // (either CTA of a pair holds half of the weight tile)
       // Heads of an odd number of 16-column groups: the QKV epilogue's last read of a tile ends 8 columns past it, and the
@@ -903,7 +904,7 @@ WidePlan wide_plan(const stairs_ctx* ctx, int T, int K, const int* rows, int n_s
         if (ctx->wide_split_force && cg == 1 && sp != std::min(ctx->wide_split_force, max_splits)) continue;
         if (sp > 1 && (cg == 2 || units > sms || kblocks < sp || (size_t)units * tn * wide::WM * 4 > partial_bytes)) continue;
         const double waves = std::ceil((double)units / (sms / cg)), active = std::min<double>((double)units * cg, sms);
-        const double mma = std::max(4.5 * tn, 810.0) / 1.8e3, load = (2.0 * x_box + tn / cg) * 128.0 / std::min(95e3, 10e6 / active);
+        const double mma = std::max(4.5 * tn, 810.0) / 1.8e3, load = (2.0 * wide::WM + tn / cg) * 128.0 / std::min(95e3, 10e6 / active);
         const double unit = std::ceil((double)kblocks / sp) * std::max(mma, load), epi = 0.03 * tn;
         const double us = 4.5 + std::max(waves * unit, w_bytes / 6.5e6) + epi + (waves - 1) * std::max(0.0, epi - unit) +
                           (sp > 1 ? 2.0 + split_us * tn * sp : 0.0) + (cg == 2 ? 1.5 + 0.006 * tn : 0.0);
@@ -928,13 +929,14 @@ cudaError_t launch_chained(cudaStream_t st, void (*kern)(A...), dim3 grid, int t
 // Weight matrices of one many-row GEMM: up to three sources that share the operand.
 struct WideW { const void* ptr[3]; int rows[3]; int n_src; };
 
-// parts 2: an activation operand, `rows` hi rows and as many lo rows behind them, one box of both
+// parts 2 or ONE_PART: an activation operand, `rows` hi rows and as many lo rows behind them; one box of both, or of one of them
+constexpr int ONE_PART = -1;
 const CUtensorMap* wide_map(stairs_ctx* ctx, const void* ptr, long long rows, int K, int box, int parts = 1) {
-  auto key = std::make_tuple(ptr, K, box);
+  auto key = std::make_tuple(ptr, K, parts == ONE_PART ? -box : box);
   auto it = ctx->wide_maps.find(key);
   if (it == ctx->wide_maps.end()) {
     CUtensorMap mp;
-    if (!(parts == 2 ? encode_map_parts(ctx, &mp, ptr, rows, K, box) : encode_map(ctx, &mp, ptr, rows, K, box))) return nullptr;
+    if (!(parts != 1 ? encode_map_parts(ctx, &mp, ptr, rows, K, box, parts == ONE_PART ? 1 : 2) : encode_map(ctx, &mp, ptr, rows, K, box))) return nullptr;
     it = ctx->wide_maps.emplace(key, mp).first;
   }
   return &it->second;
@@ -947,7 +949,6 @@ int launch_wide_gemm(stairs_ctx* ctx, wide::WideJob& job, const void* x, int K, 
   job.TN = pl.tn; job.splits = pl.splits;
   job.kblocks = (K + tc::BK - 1) / tc::BK;
   job.m_tiles = (job.T + wide::WM * pl.cg - 1) / (wide::WM * pl.cg);
-  job.x_box = job.m_tiles == 1 && pl.cg == 1 ? (job.T + 15) / 16 * 16 : wide::WM;
   job.n_src = w.n_src; job.n_tiles = 0;
   for (int s = 0; s < 3; ++s) {
     const int i = s < w.n_src ? s : 0;
@@ -958,22 +959,93 @@ int launch_wide_gemm(stairs_ctx* ctx, wide::WideJob& job, const void* x, int K, 
     if (s < w.n_src) job.n_tiles += job.src_tiles[s];
   }
   if (glu) { job.n_src = 1; job.n_tiles = job.src_tiles[0] = (2 * w.rows[0] + pl.tn - 1) / pl.tn; }
-  const CUtensorMap* xm = wide_map(ctx, x, L.max_rows, K, job.x_box, 2);
+  const CUtensorMap* xm = wide_map(ctx, x, L.max_rows, K, wide::WM, 2);
   if (!xm) return fail(ctx, STAIRS_ECUDA, "cuTensorMapEncodeTiled failed for an activation buffer");
   job.x_map = *xm;
   if (pl.splits > 1 && (long long)job.n_tiles * job.m_tiles > TC_COUNTERS) return fail(ctx, STAIRS_EUNSUPPORTED, "too many tiles for the split bookkeeping");
-  job.stages = wide::gemm_stages(job.x_box, pl.tn, pl.cg);
+  job.stages = wide::gemm_stages(pl.tn, pl.cg);
   job.lo_row = L.max_rows;
   job.partial = reinterpret_cast<float*>(ctx->ws + L.gemm_partial);
   job.counters = reinterpret_cast<int*>(ctx->ws + L.gemm_counters);
   job.status = ctx->status_dev; job.wait_limit = ctx->wait_limit;
   const int slots = std::min(ctx->sm_count, TC_GRID_MAX) / pl.cg;
   const int grid = std::min(slots, job.n_tiles * job.m_tiles * pl.splits) * pl.cg;
-  const size_t smem = wide::gemm_smem(job.x_box, pl.tn, pl.cg, job.stages);
+  const size_t smem = wide::gemm_smem(pl.tn, pl.cg, job.stages);
   ctx->launches++;
   GemmTimer tm(ctx);
   CK(launch_chained(ctx->stream, pl.cg == 2 ? wide::k_wide_gemm<2> : wide::k_wide_gemm<1>, dim3(grid), wide::WTHREADS, smem, dim3(pl.cg, 1, 1), job));
   return STAIRS_OK;
+}
+
+// Pairs per cluster of a GEMM over 65 to 128 rows (mid.cuh): whole rounds of tile pairs over the clusters that run at once, a k-block
+// at the SM's load rate (all weights at the copy rate), the exchange of the sums.
+int mid_cluster(const stairs_ctx* ctx, int n_tiles, int kblocks, int TN, int x_box) {
+  int best = 1;
+  double best_us = 1e30;
+  const int pairs = (n_tiles + 1) / 2;
+  for (int c = 1; c <= mid::MAX_C; ++c) {
+    if (ctx->mid_force && c != std::min(ctx->mid_force, kblocks)) continue;
+    const int fit = ctx->mid_fit[c];
+    if (fit <= 0 || c > kblocks) continue;
+    const int clusters = std::min(fit, pairs), rounds = (pairs + clusters - 1) / clusters;
+    const double kb = std::max((TN + x_box) * 128.0 / 100e3, TN * 256.0 * clusters * c / 6.3e6);
+    const double chain = ((kblocks + c - 1) / c) * kb, epi = (c > 1 ? 3.0 : 1.0) + 0.03 * x_box / c;
+    const double us = chain + (rounds - 1) * std::max(chain, epi) + epi;
+    if (us < best_us - 1e-9) { best_us = us; best = c; }
+  }
+  return best;
+}
+
+// One GEMM of a pass over at most 128 rows.  gran: weight rows that stay in one tile (heads of the QKV projection).  w: as for
+// launch_wide_gemm, but the gate and up matrices interleaved (64 rows of each per tile) as one source.
+template <int EPI>
+int launch_mid_gemm(stairs_ctx* ctx, wide::WideJob& job, const void* x, int K, const WideW& w, int gran) {
+  const Layout& L = ctx->lay;
+  job.TN = mid::M_MAX_ROWS / gran * gran;
+  job.x_box = (job.T + 15) / 16 * 16;
+  job.kblocks = (K + tc::BK - 1) / tc::BK;
+  job.n_src = w.n_src; job.n_tiles = 0; job.m_tiles = 1;
+  for (int s = 0; s < w.n_src; ++s) {
+    const CUtensorMap* m = wide_map(ctx, w.ptr[s], w.rows[s], K, job.TN);
+    if (!m) return fail(ctx, STAIRS_ECUDA, "cuTensorMapEncodeTiled failed for a weight matrix");
+    job.w_map[s] = *m;
+    job.src_tiles[s] = (w.rows[s] + job.TN - 1) / job.TN; job.src_rows[s] = w.rows[s];
+    job.n_tiles += job.src_tiles[s];
+  }
+  const CUtensorMap* xm = wide_map(ctx, x, L.max_rows, K, job.x_box, ONE_PART);
+  if (!xm) return fail(ctx, STAIRS_ECUDA, "cuTensorMapEncodeTiled failed for an activation buffer");
+  job.x_map = *xm;
+  job.splits = mid_cluster(ctx, job.n_tiles, job.kblocks, job.TN, job.x_box);
+  job.lo_row = L.max_rows;
+  job.status = ctx->status_dev; job.wait_limit = ctx->wait_limit;
+  const int grid = std::min(ctx->mid_fit[job.splits], (job.n_tiles + 1) / 2) * 2 * job.splits;
+  const bool alone = mid::one_round(job, grid);
+  job.stages = mid::gemm_stages(job.x_box, job.TN, alone);
+  ctx->launches++;
+  GemmTimer tm(ctx);
+  CK(launch_chained(ctx->stream, job.splits > 1 ? mid::k_mid_gemm<EPI, true> : mid::k_mid_gemm<EPI, false>, dim3(grid), wide::WTHREADS,
+                    mid::gemm_smem(job.x_box, job.TN, job.stages, alone), dim3(2 * job.splits, 1, 1), job));
+  return STAIRS_OK;
+}
+
+// Shared-memory limits of the kernels above and how many of their clusters run at once.
+cudaError_t setup_mid(stairs_ctx* ctx) {
+  cudaError_t e = cudaSuccess;
+  auto limit = [&](auto kern) { if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT); };
+  limit(mid::k_mid_gemm<wide::W_ADD, false>); limit(mid::k_mid_gemm<wide::W_ADD, true>);
+  limit(mid::k_mid_gemm<wide::W_GELU, false>); limit(mid::k_mid_gemm<wide::W_GELU, true>);
+  limit(mid::k_mid_gemm<wide::W_SWIGLU, false>); limit(mid::k_mid_gemm<wide::W_SWIGLU, true>);
+  limit(mid::k_mid_gemm<wide::W_QKV, false>); limit(mid::k_mid_gemm<wide::W_QKV, true>);
+  limit(mid::k_mid_gemm<wide::W_LMHEAD, false>); limit(mid::k_mid_gemm<wide::W_LMHEAD, true>);
+  for (int c = 1; c <= mid::MAX_C && e == cudaSuccess; ++c) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(2 * c); cfg.blockDim = dim3(wide::WTHREADS); cfg.dynamicSmemBytes = tc::SMEM_LIMIT;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = 2 * c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&ctx->mid_fit[c], mid::k_mid_gemm<wide::W_ADD, true>, &cfg);
+  }
+  return e;
 }
 
 template <int KS, bool EXACT>
@@ -1062,6 +1134,7 @@ int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* l
   float* sn = cs + (size_t)L.max_rows * half;
   float4* stats = reinterpret_cast<float4*>(ws + L.wide_stats);
   const bool ln = m.norm == 0;
+  const bool few = T <= mid::M_MAX_ROWS;   // one row tile: weights on the MMA's M side
   const size_t f_aux = (size_t)F * (m.act == 1 ? 2 : 1), aux_layer = ((size_t)nqkv + f_aux) * 2;
   CK(launch_chained(ctx->stream, wide::k_wide_embed, dim3(T), 256, (size_t)0, dim3(1, 1, 1), (const bf16*)M.w.tok_emb, (const bf16*)M.w.pos_emb,
                     (const int*)(ws + L.tok), (const int*)(ws + L.pos), (const int*)(ws + L.req), (const int*)(ws + L.page_table), (int)ctx->cfg.kv_page_tokens,
@@ -1079,8 +1152,9 @@ int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* l
   auto residual = [&](const void* w, const void* in, int K, const void* g) -> int {
     wide::WideJob j = job0(wide::W_ADD, false);
     j.N = d; j.ldo = d; j.out_f32 = x; j.out_act = h; j.next_g = (const float*)g; j.stats_out = stats;
-    const int rc = launch_wide_gemm(ctx, j, in, K, WideW{{w}, {d}, 1}, 32, 8);
-    stat_tiles = 2 * j.n_tiles;
+    const WideW one{{w}, {d}, 1};
+    const int rc = few ? launch_mid_gemm<wide::W_ADD>(ctx, j, in, K, one, mid::M_MAX_ROWS) : launch_wide_gemm(ctx, j, in, K, one, 32, 8);
+    stat_tiles = few ? j.n_tiles : 2 * j.n_tiles;
     return rc;
   };
   int rc = STAIRS_OK;
@@ -1099,7 +1173,7 @@ int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* l
       const WideW all{{w.wq, w.wk, w.wv}, {nq, nkv, nkv}, 3}, kv{{w.wk, w.wv}, {nkv, nkv}, 2};
       const int off[4] = {0, nq, nq + nkv, 0};
       for (int s = 0; s < 3; ++s) j.u_off[s] = off[s + j.src0];
-      rc = launch_wide_gemm(ctx, j, h, d, last_kv ? kv : all, hd, 8);
+      rc = few ? launch_mid_gemm<wide::W_QKV>(ctx, j, h, d, last_kv ? kv : all, hd) : launch_wide_gemm(ctx, j, h, d, last_kv ? kv : all, hd, 8);
     }
     if (rc || last_kv) break;
     wide::WideAttn a = at;
@@ -1111,8 +1185,11 @@ int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* l
       wide::WideJob j = job0(m.act == 1 ? wide::W_SWIGLU : wide::W_GELU, true);
       j.N = F; j.ldo = F; j.out_act = ff;
       if (ln) { j.u = M.ln_aux + (size_t)l * aux_layer + 2 * (size_t)nqkv; j.c = j.u + f_aux; j.u_last = (int)f_aux - 1; }
-      rc = m.act == 1 ? launch_wide_gemm(ctx, j, h, d, WideW{{w.w_gate_or_fc1, w.w_up}, {F, F}, 2}, 32, 4)
-                      : launch_wide_gemm(ctx, j, h, d, WideW{{w.w_gate_or_fc1}, {F}, 1}, 32, 4);
+      const WideW fc1{{w.w_gate_or_fc1}, {F}, 1};
+      if (m.act == 1)
+        rc = few ? launch_mid_gemm<wide::W_SWIGLU>(ctx, j, h, d, WideW{{M.w13_ptr[l]}, {(F + 63) / 64 * 128}, 1}, mid::M_MAX_ROWS)
+                 : launch_wide_gemm(ctx, j, h, d, WideW{{w.w_gate_or_fc1, w.w_up}, {F, F}, 2}, 32, 4);
+      else rc = few ? launch_mid_gemm<wide::W_GELU>(ctx, j, h, d, fc1, mid::M_MAX_ROWS) : launch_wide_gemm(ctx, j, h, d, fc1, 32, 4);
     }
     if (!rc) rc = residual(w.w_down_or_fc2, ff, F, l + 1 < m.n_layers ? M.layers[l + 1].norm1_w : M.w.final_norm_w);
   }
@@ -1120,7 +1197,8 @@ int forward_wide(stairs_ctx* ctx, DevModel& M, int T, int n_logit_rows, float* l
   wide::WideJob j = job0(wide::W_LMHEAD, true);
   j.N = m.vocab; j.ldo = m.vocab; j.out_f32 = logits; j.keys = reinterpret_cast<unsigned long long*>(ws + L.keys);
   if (ln) { j.u = M.ln_aux + (size_t)m.n_layers * aux_layer; j.c = j.u + m.vocab; j.u_last = m.vocab - 1; }
-  return launch_wide_gemm(ctx, j, h, d, WideW{{M.w.lm_head}, {m.vocab}, 1}, 32, 1);
+  const WideW head{{M.w.lm_head}, {m.vocab}, 1};
+  return few ? launch_mid_gemm<wide::W_LMHEAD>(ctx, j, h, d, head, mid::M_MAX_ROWS) : launch_wide_gemm(ctx, j, h, d, head, 32, 1);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1608,6 +1686,7 @@ int stairs_init(const stairs_config* cfg, const stairs_weights* target, const st
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_attn_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide::tc_att_smem<64>());
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_attn_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide::tc_att_smem<128>());
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_gemm<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
+        if (e == cudaSuccess) e = setup_mid(ctx);
         if (e == cudaSuccess) {
           ctx->use_mk = true;
           ctx->target.prog_base = ctx->ws + L.prog_t; ctx->target.prog_slot_bytes = L.prog_slot_t; ctx->target.prog_maps_off = L.prog_maps_off_t;
@@ -2044,6 +2123,10 @@ int stairs_debug_tune(stairs_ctx* ctx, int what, long long value) {
     case 5:
       if (value != 0 && value != 1 && value != 2 && value != 4 && value != 8) return fail(ctx, STAIRS_EINVAL, "K ranges must be 0 (planned), 1, 2, 4 or 8");
       ctx->wide_split_force = (int)value;
+      return STAIRS_OK;
+    case 6:
+      if (value < 0 || value > mid::MAX_C) return fail(ctx, STAIRS_EINVAL, "CTA pairs per tile must be 0 (planned) .. %d", mid::MAX_C);
+      ctx->mid_force = (int)value;
       return STAIRS_OK;
     default: return fail(ctx, STAIRS_EINVAL, "unknown tuning knob %d", what);
   }

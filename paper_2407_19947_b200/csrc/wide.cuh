@@ -1,4 +1,4 @@
-// Passes over many rows (prefill chunks, serving batches of more than 64 stair rows): one launch per
+// Passes over many rows (prefill chunks, serving batches of more than 128 stair rows; up to 128 the GEMMs are mid.cuh's): one launch per
 // GEMM and per attention layer, everything a layer needs besides the contractions folded into their
 // epilogues.  The persistent kernel streams all weights once per 64 rows, so it is HBM-bound however
 // long the prompt is; here a tile holds 128 or 256 rows and the weights are read once per pass.
@@ -45,11 +45,11 @@ constexpr int ST_BYTES = EPI_WARPS * (32 * ST_LD + 64) * 4;   // (and 64 folded-
 enum WEpi { W_ADD = 0, W_GELU = 1, W_SWIGLU = 2, W_QKV = 3, W_LMHEAD = 4 };
 
 struct WideJob {
-  CUtensorMap x_map;        // [2 parts][lo_row rows][K]; box 64 x x_box x 2
+  CUtensorMap x_map;        // [2 parts][lo_row rows][K]; box 64 x 128 x 2 (mid.cuh: 64 x x_box x 1)
   CUtensorMap w_map[3];     // box 64 x TN / CG rows; SwiGLU: gate and up matrix, box 64 x TN / 2 rows
   int n_src, src_tiles[3], src_rows[3];
   int src0;                 // W_QKV: first source present (0: q, k, v; 1: k and v only)
-  int x_box;
+  int x_box;                // mid.cuh: rows of the activation box
   int T, TN, n_tiles, m_tiles, kblocks, splits, stages;
   int lo_row;               // rows between the hi and the lo part of every bf16 operand
   int epi;
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int TN = job.TN, TNc = TN / CG, stages = job.stages, S = job.splits;
-  const int a_bytes = job.x_box * BK * 2;                            // one part of the activation tile
+  constexpr int a_bytes = WM * BK * 2;                               // one part of the activation tile
   const int stage_bytes = 2 * a_bytes + TNc * BK * 2;
   uint8_t* tail = smem + (size_t)stages * stage_bytes;
   float* stile = reinterpret_cast<float*>(tail);                     // [EPI_WARPS][32][ST_LD]
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
     // (they depend on nothing: fetched while the predecessor still runs)
     if (lane == 0) {
       const uint64_t pol_w = policy_evict_first();
-      const uint32_t tx = (uint32_t)(CG * (2 * job.x_box * BK * 2 + TNc * BK * 2));   // both parts, both CTAs
+      const uint32_t tx = (uint32_t)(CG * stage_bytes);   // both parts, both CTAs
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
       for (int u = cid; u < units && ok; u += G) {
@@ -674,15 +674,13 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
   if (warp == 1) { tc_fence_after(); w_dealloc<CG>(tmem_base, tmem_cols); }
 }
 
-// x_box: rows of the activation box (a single row tile only fetches its own rows; the MMAs of the last stage
-// still read 128 from the lo part's start, so the tail behind the stages has to be as long)
-inline size_t gemm_smem(int x_box, int TN, int CG, int stages) {
-  const size_t stage = 2 * (size_t)x_box * BK * 2 + (size_t)(TN / CG) * BK * 2;
+inline size_t gemm_smem(int TN, int CG, int stages) {
+  const size_t stage = 2 * (size_t)WM * BK * 2 + (size_t)(TN / CG) * BK * 2;
   return 1024 + stages * stage + ST_BYTES + (2 * W_MAX_STAGES + 4) * 8 + 64;
 }
-inline int gemm_stages(int x_box, int TN, int CG) {
+inline int gemm_stages(int TN, int CG) {
   int s = W_MAX_STAGES;
-  while (s > 2 && gemm_smem(x_box, TN, CG, s) > (size_t)SMEM_LIMIT) --s;
+  while (s > 2 && gemm_smem(TN, CG, s) > (size_t)SMEM_LIMIT) --s;
   return s;
 }
 
@@ -729,13 +727,14 @@ inline size_t attn_smem(int hd, int nw, int mt) {
 // One block: MT blocks of 16 queries (query q of a request = row q / G, head q % G of the kv head) times
 // NW / MT position slices of every 64-position chunk, one warp each, on mma.sync m16n8k16 with the online
 // softmax in registers (base 2).  <8, 8> serves prefill chunks (128 queries share a chunk's copies);
-// <4, 1..4> requests with few query rows, whose warps split the positions instead.  Long contexts of few
+// <4, 1..4> requests with few query rows, whose warps split the positions instead, three or four blocks to an SM (16 requests x 32
+// heads of 80 are 512 blocks: with 141 registers a thread, three to an SM, the last 68 were a second wave; with 128, 3.5 us less a layer).  Long contexts of few
 // blocks are cut over a cluster of up to 8 CTAs (grid z); slices and ranges are merged at the end through
 // (distributed) shared memory in a fixed order.  Chunks are staged by 16-byte asynchronous copies, the
 // next one under the current one's MMAs.
 // EXACT: hd == 16 * KS (loops without guards).
 template <int KS, bool EXACT, int NW, int MT>
-__global__ void __launch_bounds__(NW * 32, (KS <= 5 && NW == 8) ? 2 : 1) k_wide_attn(const __grid_constant__ WideAttn P) {
+__global__ void __launch_bounds__(NW * 32, NW == 8 ? (KS <= 5 ? 2 : 1) : (KS <= 5 ? 4 : 3)) k_wide_attn(const __grid_constant__ WideAttn P) {
   extern __shared__ __align__(16) uint8_t asm_raw[];
   constexpr int NP = NW / MT, SL = WCH / NP;       // position slices, positions per slice
   constexpr int RND = SL < 32 ? SL : 32;           // positions per softmax round
@@ -747,7 +746,8 @@ __global__ void __launch_bounds__(NW * 32, (KS <= 5 && NW == 8) ? 2 : 1) k_wide_
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, g = lane >> 2, t4 = lane & 3;
   const int NS = gridDim.z, zr = blockIdx.z;
   if (tid == 0) pdl_launch();
-  pdl_wait();
+  // (requests, page table and cached positions are older than this pass: read, and the first chunks' copies started, while the
+  // predecessor still runs; the queries and this call's own positions are its work)
   int slot, base, R, off;
   const int i_req = blockIdx.y / P.n_qblk, kvh = blockIdx.x;
   int qblk = blockIdx.y % P.n_qblk;
@@ -755,7 +755,7 @@ __global__ void __launch_bounds__(NW * 32, (KS <= 5 && NW == 8) ? 2 : 1) k_wide_
     slot = P.val_req[i_req]; R = P.val_k[i_req] + 1; off = P.val_off[i_req]; base = P.n_seq[slot] - 1;
   } else { slot = P.slot; R = P.rows; off = 0; base = P.first; qblk = P.n_qblk - 1 - qblk; }   // (the longest blocks first)
   const int Q = R * G, q0 = qblk * MT * 16;
-  if (q0 >= Q) return;                              // (uniform over the cluster)
+  if (q0 >= Q) { pdl_wait(); return; }              // (uniform over the cluster)
   const int mt = w % MT, part = w / MT;
   const int nQ = min(MT * 16, Q - q0);
   const int last_pos = base + (q0 + nQ - 1) / G;    // last position any query of the block sees
@@ -788,10 +788,24 @@ __global__ void __launch_bounds__(NW * 32, (KS <= 5 && NW == 8) ? 2 : 1) k_wide_
     mk::cp_async_commit();
   };
 
-  // this warp's queries: MMA A fragments straight from memory
   const int ql_a = mt * 16 + g, ql_b = ql_a + 8;
   const bool on_a = ql_a < nQ, on_b = ql_b < nQ;
   const int qa = q0 + (on_a ? ql_a : 0), qb = q0 + (on_b ? ql_b : 0);
+  const int last_a = on_a ? base + qa / G : -1, last_b = on_b ? base + qb / G : -1;
+  const int warp_first = base + (q0 + mt * 16) / G;                                       // first query's last visible position
+  const int warp_last = mt * 16 < nQ ? base + (q0 + min(mt * 16 + 15, nQ - 1)) / G : -1;  // (-1: no queries)
+  float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
+  float o[2 * KS][4];
+#pragma unroll
+  for (int nd = 0; nd < 2 * KS; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = 0.f;
+
+  if (c_begin < c_end) { look_up(c_begin); if (c_begin + 1 < c_end) look_up(c_begin + 1); }
+  __syncthreads();
+  const bool early = c_begin < c_end && (c_begin + 1) * WCH <= base;   // (the chunk holds cached positions only)
+  if (early) stage(c_begin, 0);
+  pdl_wait();
+  if (c_begin < c_end && !early) stage(c_begin, 0);
+  // this warp's queries: MMA A fragments straight from memory
   uint32_t qf[KS][4];
   {
     const __half* pa = P.q16 + (size_t)(off + qa / G) * nq + (size_t)(kvh * G + qa % G) * hd + t4 * 2;
@@ -806,17 +820,6 @@ __global__ void __launch_bounds__(NW * 32, (KS <= 5 && NW == 8) ? 2 : 1) k_wide_
       } else { qf[kk][0] = qf[kk][1] = qf[kk][2] = qf[kk][3] = 0u; }
     }
   }
-  const int last_a = on_a ? base + qa / G : -1, last_b = on_b ? base + qb / G : -1;
-  const int warp_first = base + (q0 + mt * 16) / G;                                       // first query's last visible position
-  const int warp_last = mt * 16 < nQ ? base + (q0 + min(mt * 16 + 15, nQ - 1)) / G : -1;  // (-1: no queries)
-  float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
-  float o[2 * KS][4];
-#pragma unroll
-  for (int nd = 0; nd < 2 * KS; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = 0.f;
-
-  if (c_begin < c_end) { look_up(c_begin); if (c_begin + 1 < c_end) look_up(c_begin + 1); }
-  __syncthreads();
-  if (c_begin < c_end) stage(c_begin, 0);
   int cur = 0;
   for (int c = c_begin; c < c_end; ++c, cur ^= 1) {
     if (c + 1 < c_end) {

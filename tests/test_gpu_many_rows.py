@@ -255,3 +255,25 @@ def test_many_row_passes_agree_with_small_ones(shape):
         eng.sync()
         assert _distance(many, alone[: 5 * n]) < ROWS_BAR
     eng.close()
+
+
+@pytest.mark.parametrize("pairs", [0, 1, 2, 3, 4])
+@pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES.keys())
+def test_calls_of_one_row_tile_at_every_cluster_size(shape, pairs):
+    # the GEMMs of 65 to 128 rows: rows that end before, at and behind a 16-row box, shares of the rows that are no multiples of
+    # anything, K cut over one to four pairs of CTAs, tiles of whole heads, an odd number of tiles
+    st = _stairs()
+    tsrc, _ = sources(shape)
+    eng = st.Stairs(tsrc, None, max_requests=26, max_seq_len=128, k_max=4, kv_page_tokens=16)
+    for i in range(26):
+        eng.prefill(i, list(wl.zipf_tokens(20 + 3 * (i % 15), shape.vocab, 60 + i)))
+    drafts = torch.from_numpy(np.random.default_rng(1).integers(0, shape.vocab, size=(26, 4)).astype(np.int32)).cuda()
+    alone = [eng.validate([i], [4], drafts[i:i + 1].contiguous(), want_logits=True)[2] for i in range(26)]
+    eng.debug_tune(6, pairs)
+    for rows in (65, 81, 96, 97, 127, 128):
+        ks = [4] * (rows // 5) + ([rows % 5 - 1] if rows % 5 else [])
+        n = len(ks)
+        _, _, many = eng.validate(list(range(n)), ks, drafts[:n].contiguous(), want_logits=True)
+        eng.sync()
+        assert _distance(many, torch.cat([alone[i][: k + 1] for i, k in enumerate(ks)])) < ROWS_BAR
+    eng.close()
