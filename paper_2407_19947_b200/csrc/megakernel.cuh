@@ -1786,64 +1786,40 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           pre_tile = (kb_begin + p.kblocks - 1) / p.kblocks;
           if (pre_tile < p.n_tiles) { uq = p.u[pre_tile * BM + m]; cq = p.c[pre_tile * BM + m]; }
         }
-        if (p.norm_in && kb_begin < kb_end) {
-          // row statistics of the operand: merge the per-tile entries (published by the phase
-          // that produced x) into mean and 1/std per row
-          if (et == 0) ctl->bcast = W.wait_grid(bar_count, P.bar_base + (unsigned long long)ph * G) ? 1 : 0;
+        // Row statistics of the operand (published by the phase that produced x): merged into mean and 1/std per row, eight lanes per
+        // row as in the epilogue, and only by CTAs that finish a tile in this phase.  (A first form, by all CTAs, a warp per
+        // row, held up the partial sums of those that only park them, and its longer text slowed the MMA warp's first stage, which is
+        // fetched at the same time: 0.4B, 9 rows 993 -> 915 us.  Merging them between parking and finishing: 3B, 5 rows 1 % slower.)
+        if (p.norm_in && (kb_begin + p.kblocks - 1) / p.kblocks * p.kblocks < kb_end) {
+          if (lane == 0) W.wait_grid(bar_count, P.bar_base + (unsigned long long)ph * G);   // (one that ran out is looked at once, at the end of the phase)
           __syncwarp();
-          epi_bar_sync();
-          ok = ctl->bcast != 0;   // (written again in a later phase only, several barriers on)
-          if (!ok) break;
-          // One warp per row, four rows per warp at a time.  A lane holds the tile entries lane and
-          // lane + 32 of each row (all loads of the four rows in flight together; at most 64 tiles,
-          // d <= 8192).  The merged mean is the count-weighted mean of the tiles' means, and the
-          // merged M2 the sum of the tiles' M2 plus count * (tile mean - mean)^2: two warp sums
-          // of non-negative or well-scaled terms, identical on every lane.
-          for (int tb = quad; tb < Tvalid; tb += 16) {
-            float4 sv[4][2];
+          for (int t = et >> 3; t < (S::ONE ? 16 : (Tvalid + 15) & ~15); t += 16) {
+            const float4* sr = P.stats + (size_t)min(t, Tvalid - 1) * P.stat_tiles;
+            const int sub = et & 7;
+            // this lane's tiles, sums shifted by its first tile's mean; then count-weighted mean and M2 over the eight lanes
+            float n = 0.f, s1 = 0.f, s2 = 0.f, m0 = 0.f;
+#pragma unroll 1
+            for (int i0 = sub; i0 < P.stat_tiles; i0 += 32) {
+              float4 e[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              const int t = tb + 4 * r;
+              for (int i = 0; i < 4; ++i) e[i] = i0 + 8 * i < P.stat_tiles ? __ldcg(sr + i0 + 8 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+              if (i0 == sub) m0 = e[0].x;
 #pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const int tl = lane + 32 * e;
-                sv[r][e] = (t < Tvalid && tl < P.stat_tiles) ? __ldcg(P.stats + (size_t)t * P.stat_tiles + tl) : make_float4(0.f, 0.f, 0.f, 0.f);
-              }
+              for (int i = 0; i < 4; ++i) { const float d0 = e[i].x - m0, nd = e[i].z * d0; n += e[i].z; s1 += nd; s2 += e[i].y + nd * d0; }
             }
-            float n[4], s1[4], m2[4];
+            const float dm = s1 / fmaxf(n, 1.f), mean_l = m0 + dm, m2_l = fmaxf(s2 - s1 * dm, 0.f);
+            float n_all = n, w = n * mean_l;
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              n[r] = sv[r][0].z + sv[r][1].z;
-              s1[r] = sv[r][0].z * sv[r][0].x + sv[r][1].z * sv[r][1].x;
-            }
+            for (int o = 1; o < 8; o <<= 1) { n_all += __shfl_xor_sync(0xffffffffu, n_all, o); w += __shfl_xor_sync(0xffffffffu, w, o); }
+            const float mean = w / fmaxf(n_all, 1.f);
+            float m2 = m2_l + n * (mean_l - mean) * (mean_l - mean);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-              for (int r = 0; r < 4; ++r) { n[r] += __shfl_xor_sync(0xffffffffu, n[r], o); s1[r] += __shfl_xor_sync(0xffffffffu, s1[r], o); }
-            }
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              s1[r] = s1[r] / fmaxf(n[r], 1.f);   // the row's mean
-              const float d0 = sv[r][0].x - s1[r], d1 = sv[r][1].x - s1[r];
-              m2[r] = (sv[r][0].y + sv[r][0].z * d0 * d0) + (sv[r][1].y + sv[r][1].z * d1 * d1);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-              for (int r = 0; r < 4; ++r) m2[r] += __shfl_xor_sync(0xffffffffu, m2[r], o);
-            }
-            if (lane == 0) {
-#pragma unroll
-              for (int r = 0; r < 4; ++r) {
-                const int t = tb + 4 * r;
-                if (t < Tvalid) {
-                  if (S::layer_norm(P)) { ctl->mu[t] = s1[r]; ctl->rstd[t] = 1.0f / sqrtf(m2[r] / (float)P.d + P.eps); }
-                  else { ctl->mu[t] = 0.f; ctl->rstd[t] = 1.0f / sqrtf((m2[r] + n[r] * s1[r] * s1[r]) / (float)P.d + P.eps); }
-                }
-              }
+            for (int o = 1; o < 8; o <<= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+            if (sub == 0 && t < Tvalid) {
+              ctl->mu[t] = S::layer_norm(P) ? mean : 0.f;
+              ctl->rstd[t] = 1.0f / sqrtf((S::layer_norm(P) ? m2 : m2 + n_all * mean * mean) / (float)P.d + P.eps);
             }
           }
-          epi_bar_sync();
         }
         if (tracing) tr[3] = globaltimer_ns();
         bool first_seg = true;
@@ -1935,13 +1911,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
             float* mine = slot_of(pset, (unsigned)cta);
             for (int c0 = 0; c0 < (S::ONE ? 1 : Tvalid); c0 += 16) {   // only rows that exist
               float v[16];
-              tmem_ld16(taddr + (uint32_t)c0, v);
-              {
-                float vl[16];
-                tmem_ld16(taddr + (uint32_t)(P.t_box + c0), vl);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] += vl[j];
-              }
+              tmem_ld16_sum(taddr + (uint32_t)c0, taddr + (uint32_t)(P.t_box + c0), v);
               const int jn = min(16, Tvalid - c0);
 #pragma unroll
               for (int j = 0; j < 16; ++j) if (j < jn) st_relaxed_f32(mine + (size_t)(c0 + j) * BM + m, v[j]);
@@ -1957,13 +1927,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
             for (int c0 = 0; c0 < (S::ONE ? 1 : Tvalid); c0 += 16) {
               {
                 float v[16];
-                tmem_ld16(taddr + (uint32_t)c0, v);
-                {
-                  float vl[16];
-                  tmem_ld16(taddr + (uint32_t)(P.t_box + c0), vl);
-#pragma unroll
-                  for (int j = 0; j < 16; ++j) v[j] += vl[j];
-                }
+                tmem_ld16_sum(taddr + (uint32_t)c0, taddr + (uint32_t)(P.t_box + c0), v);
                 if (S::ONE || c0 + 16 >= Tvalid) {   // accumulator drained: the MMA warp may reuse it
                   tc_fence_before();
                   if (lane == 0) mbar_arrive(ctl->acc_empty + buf);
@@ -1971,8 +1935,6 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
 #pragma unroll
                 for (int j = 0; j < 16; ++j) vt[j * VT_LD + m] = v[j];
               }
-              epi_bar_sync();   // the exchange tile is complete
-              if (tra && !whole && c0 == 0) tra[1] = globaltimer_ns();
               {
                 // Each phase runs this code once per tile, so its instruction fetch is what it costs:
                 // the loads that must be in flight together are unrolled, everything per column group
@@ -1981,15 +1943,16 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                 const bool row_on = t < Tvalid;
                 float* vrow = vt + er * VT_LD;
                 const bool add_res = p.epi == TC_ADD_F32;
+                epi_bar_sync();   // the exchange tile is complete
+                if (tra && !whole && c0 == 0) tra[1] = globaltimer_ns();
+                float a0x = 0.f;             // (the row's value in this thread's first column)
                 if (!whole || add_res) {
                   float4 a[4];
                   bool on[4];
 #pragma unroll
-                  for (int q = 0; q < 4; ++q) {
-                    const int col = (cg + 8 * q) * 4;
-                    on[q] = row_on && (S::dual(p) ? (col & 63) < ncols : col < ncols);
-                    a[q] = on[q] ? *reinterpret_cast<const float4*>(vrow + col) : make_float4(0.f, 0.f, 0.f, 0.f);
-                  }
+                  for (int q = 0; q < 4; ++q) on[q] = row_on && (S::dual(p) ? (((cg + 8 * q) * 4) & 63) < ncols : (cg + 8 * q) * 4 < ncols);
+#pragma unroll
+                  for (int q = 0; q < 4; ++q) a[q] = on[q] ? *reinterpret_cast<const float4*>(vrow + (cg + 8 * q) * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
                   if (!whole) {
                     // The other segments' partial sums, six segments' loads in flight together, added in k
                     // order.  A slot element reads PARTIAL_EMPTY until its producer has stored the sum: when
@@ -2048,6 +2011,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
 #pragma unroll
                   for (int q = 0; q < 4; ++q)
                     if (on[q]) *reinterpret_cast<float4*>(vrow + (cg + 8 * q) * 4) = a[q];   // (this thread's own slots)
+                  a0x = a[0].x;
                   if (add_res && !S::ONE && c0 + 16 < Tvalid) {
                     // calls of more than 16 rows: the next chunk's old residual values are requested now,
                     // so that they do not add an L2 round trip to that chunk
@@ -2076,9 +2040,11 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                 };
                 if (add_res) {
                   // with a following normalised GEMM: its operand bf16(x * gain) and this tile's row
-                  // statistics (count, mean, centred sum of squares; two passes over the row's 128 values)
+                  // statistics (count, mean, centred sum of squares)
                   if (p.next_g) {
-                    float cnt = 0.f, sum = 0.f;
+                    // (sums shifted by the row's first value of the tile, in one pass)
+                    const float sh = __shfl_sync(0xffffffffu, a0x, lane & 24);
+                    float s1 = 0.f, s2 = 0.f;
 #pragma unroll 1
                     for (int q = 0; q < 4; ++q) {
                       const int col = (cg + 8 * q) * 4;
@@ -2086,26 +2052,17 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                         const float4 x4 = *reinterpret_cast<const float4*>(vrow + col);
                         const float4 g4 = *reinterpret_cast<const float4*>(ctl->gtile + col);
                         store_split4(P.h, (size_t)t * p.ldo + n0 + col, (size_t)P.lo_row * p.ldo, make_float4(x4.x * g4.x, x4.y * g4.y, x4.z * g4.z, x4.w * g4.w));
-                        cnt += 4.f; sum += (x4.x + x4.y) + (x4.z + x4.w);
+                        const float d0 = x4.x - sh, d1 = x4.y - sh, d2 = x4.z - sh, d3 = x4.w - sh;
+                        s1 += (d0 + d1) + (d2 + d3); s2 += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
                       }
                     }
-                    if (tra) { asm volatile("" ::"f"(sum), "f"(cnt)); tra[7] = globaltimer_ns(); }
+                    if (tra) { asm volatile("" ::"f"(s1), "f"(s2)); tra[7] = globaltimer_ns(); }
 #pragma unroll
-                    for (int o = 1; o < 8; o <<= 1) { cnt += __shfl_xor_sync(0xffffffffu, cnt, o); sum += __shfl_xor_sync(0xffffffffu, sum, o); }
-                    const float mean = cnt > 0.f ? sum / cnt : 0.f;
-                    float m2 = 0.f;
-#pragma unroll 1
-                    for (int q = 0; q < 4; ++q) {
-                      const int col = (cg + 8 * q) * 4;
-                      if (row_on && col < ncols) {
-                        const float4 x4 = *reinterpret_cast<const float4*>(vrow + col);
-                        const float d0 = x4.x - mean, d1 = x4.y - mean, d2 = x4.z - mean, d3 = x4.w - mean;
-                        m2 += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
-                      }
+                    for (int o = 1; o < 8; o <<= 1) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }
+                    if (cg == 0 && row_on) {
+                      const float cnt = (float)ncols, dm = s1 / cnt;
+                      P.stats[(size_t)t * P.stat_tiles + tile] = make_float4(sh + dm, fmaxf(s2 - s1 * dm, 0.f), cnt, 0.f);
                     }
-#pragma unroll
-                    for (int o = 1; o < 8; o <<= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
-                    if (cg == 0 && row_on) P.stats[(size_t)t * P.stat_tiles + tile] = make_float4(mean, m2, cnt, 0.f);
                   }
                 } else if (S::swiglu(p)) {
                   // gate columns (cg + 8 q) * 4 of the tile's first half, the matching up columns 64 further
