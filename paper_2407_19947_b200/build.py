@@ -14,9 +14,9 @@ import tempfile
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB_PATH = os.path.join(HERE, "libstairs_b200.so")
-# variants of the whole-pass kernel (head size, model family, attention path, at most 16 rows), one object each
-FORWARD = ([(64, 1, a, o) for a in (0, 1) for o in (0, 1)] + [(64, 2, a, o) for a in (0, 1) for o in (0, 1)] +
-           [(80, 2, 0, o) for o in (0, 1)] + [(128, 2, a, o) for a in (0, 1) for o in (0, 1)] + [(0, 0, 3, 0)])
+# variants of the whole-pass kernel (head size, model family, attention path, at most 16 rows, shared rows), one object each
+FORWARD = [v + (s,) for s in (0, 1) for v in ([(64, 1, a, o) for a in (0, 1) for o in (0, 1)] + [(64, 2, a, o) for a in (0, 1) for o in (0, 1)] +
+           [(80, 2, 0, o) for o in (0, 1)] + [(128, 2, a, o) for a in (0, 1) for o in (0, 1)] + [(0, 0, 3, 0)])]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", "-Xptxas", "-v"]
 
@@ -41,8 +41,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Compiles csrc/*.cu into libstairs_b200.so (skipped when up to date).  Returns the path."""
     if not force and not _stale():
         return LIB_PATH
-    jobs = [("engine.cu", [])] + [("forward.cu", ["-DFWD_HD=%d" % hd, "-DFWD_FAM=%d" % fam, "-DFWD_ATT=%d" % att, "-DFWD_ONE=%d" % one])
-                                  for hd, fam, att, one in FORWARD]
+    jobs = [("engine.cu", [])] + [("forward.cu", ["-DFWD_HD=%d" % hd, "-DFWD_FAM=%d" % fam, "-DFWD_ATT=%d" % att, "-DFWD_ONE=%d" % one, "-DFWD_SHARE=%d" % share])
+                                  for hd, fam, att, one, share in FORWARD]
     log = ""
     failed = False
     with tempfile.TemporaryDirectory() as tmp:

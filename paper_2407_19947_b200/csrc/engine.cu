@@ -117,6 +117,7 @@ struct stairs_ctx {
   int att_nbuf_force = 0;            // tuning: K/V chunk buffers of the attention phases (0 = chosen from the context length)
   int att_tc_force = 0;              // tuning: 1 = tcgen05 attention for every call it can serve
   int att_tc_off = 0;                // tuning: 1 = attention contractions on mma.sync even where the tcgen05 path applies
+  int share_force = 0;               // tuning: split tiles of the persistent kernel finished by one CTA (1) or all of theirs (2); 0 = chosen per call
   int mid_force = 0;                 // tuning: pairs per cluster of those (0 = planned)
   int mid_fit[mid::MAX_C + 1] = {};  // passes of 65 to 128 rows: clusters of so many CTA pairs that run at once
   int wide_cg_force = 0, wide_split_force = 0;   // tuning: CTAs per tile and K ranges of the many-row GEMMs (0 = planned)
@@ -247,9 +248,9 @@ bool compute_layout(const stairs_config& c, Layout* L, const char** why) {
   L->small_d = take(t.wdtype == 0 && has_draft ? (size_t)d.n_layers * sizeof(small::SmallLayer) : 0);
   L->gemm_partial = take(t.wdtype == 1 ? (size_t)TC_GRID_MAX * 2 * L->t_box_max * tc::BM * 4 : 0);
   L->gemm_counters = take(t.wdtype == 1 ? (size_t)TC_COUNTERS * 4 : 0);
-  // split-tile partial sums of the persistent kernel: two sets (alternate GEMM phases) of one slot per CTA;
+  // split-tile partial sums of the persistent kernel: two sets (alternate GEMM phases) of two slots per CTA;
   // every element holds the "empty" pattern between uses
-  L->mk_partial_bytes = t.wdtype == 1 ? (size_t)2 * TC_GRID_MAX * MK_MAX_ROWS * tc::BM * 4 : 0;
+  L->mk_partial_bytes = t.wdtype == 1 ? (size_t)2 * TC_GRID_MAX * 2 * MK_MAX_ROWS * tc::BM * 4 : 0;
   L->mk_partial = take(L->mk_partial_bytes);
   {
     // persistent-kernel scratch: attention unit states and the per-(model, row box) programs
@@ -611,6 +612,44 @@ MkPlan mk_plan(const stairs_ctx* ctx, const stairs_model& m, int t_box, int q_ro
 }
 
 
+// How many CTAs to cut a GEMM of the persistent kernel over: more CTAs stream faster, but every tile is then finished from more
+// partial tiles.  Model: stream time at ~44 GB/s per SM plus ~1.6 us per batch of four partials.  (Must not depend on the row
+// box: see RANGE_UNIT_KB.)
+int gemm_ctas(const stairs_ctx* ctx, int tiles, int K) {
+  const int grid = std::min(ctx->sm_count, TC_GRID_MAX);
+  const double bytes = (double)tiles * ((K + tc::BK - 1) / tc::BK) * tc::A_STAGE_BYTES;
+  double best = 1e30; int best_ge = grid;
+  for (int s2 = 1; s2 <= 64; s2 *= 2) {
+    const int ge = std::min(grid, tiles * s2);
+    const double seg = (double)ge / tiles + (ge % tiles ? 1.0 : 0.0);
+    const double t_us = bytes / (ge * 44.0e3) + (seg > 1.0 ? std::ceil(seg / 4.0) * 1.6 + 2.0 : 0.0);
+    if (t_us < best - 1e-9) { best = t_us; best_ge = ge; }
+    if (ge == grid) break;
+  }
+  return best_ge;
+}
+
+// Do the CTAs of a split tile share its rows in this call, or does one finish them all (both give the same bits)?  Shared, a
+// phase ends about 1.2 us after its sums are parked where no warp has more than one row, and 1.9 us later for every further row
+// of a warp; finished by one CTA, about 2.5 us per 16 rows.
+int share_rows(const stairs_ctx* ctx, const stairs_model& m, int T) {
+  if (ctx->share_force) return ctx->share_force - 1;
+  double shared = 0, one = 0;
+  auto gemm = [&](int tiles, int K) {
+    const int units = tiles * (((K + tc::BK - 1) / tc::BK + mk::RANGE_UNIT_KB - 1) / mk::RANGE_UNIT_KB), ge = std::min(gemm_ctas(ctx, tiles, K), units);
+    const int seg = ge / tiles;   // CTAs per tile at least; a CTA has parts of two tiles unless they divide evenly
+    const int rows = seg >= 1 && ge > tiles ? (ge % tiles ? 2 : 1) * ((T + seg - 1) / seg) : T;
+    shared += 1.2 + 1.9 * ((rows + 3) / 4 - 1);
+    one += 2.5 * ((T + 15) / 16);
+  };
+  const int nq = m.n_heads * m.head_dim, nkv = m.n_kv_heads * m.head_dim;
+  gemm((nq + tc::BM - 1) / tc::BM + 2 * ((nkv + tc::BM - 1) / tc::BM), m.d_model);
+  gemm((m.d_model + tc::BM - 1) / tc::BM, nq);
+  gemm(m.act == 1 ? (m.d_ff + 63) / 64 : (m.d_ff + tc::BM - 1) / tc::BM, m.d_model);
+  gemm((m.d_model + tc::BM - 1) / tc::BM, m.d_ff);
+  return shared < one ? 1 : 0;
+}
+
 int build_program(stairs_ctx* ctx, DevModel& M, int t_box, int kps) {
   const stairs_model& m = M.m;
   const Layout& L = ctx->lay;
@@ -663,22 +702,7 @@ int build_program(stairs_ctx* ctx, DevModel& M, int t_box, int kps) {
       p.N = col;
     }
     p.n_tiles = tiles; p.epi = epi; p.out = out; p.ldo = ldo;
-    {
-      // How many CTAs to cut this GEMM over: more CTAs stream faster, but every tile is then
-      // finished from more partial tiles, which the finisher reads four at a time.  Model:
-      // stream time at ~44 GB/s per SM plus ~1.6 us per batch of four partials.
-      const int grid = std::min(ctx->sm_count, TC_GRID_MAX);
-      const double bytes = (double)tiles * ((K + tc::BK - 1) / tc::BK) * tc::A_STAGE_BYTES;   // (must not depend on the row box: see RANGE_UNIT_KB)
-      double best = 1e30; int best_ge = grid;
-      for (int s2 = 1; s2 <= 64; s2 *= 2) {
-        const int ge = std::min(grid, tiles * s2);
-        const double seg = (double)ge / tiles + (ge % tiles ? 1.0 : 0.0);
-        const double t_us = bytes / (ge * 44.0e3) + (seg > 1.0 ? std::ceil(seg / 4.0) * 1.6 + 2.0 : 0.0);
-        if (t_us < best - 1e-9) { best = t_us; best_ge = ge; }
-        if (ge == grid) break;
-      }
-      p.ge_max = best_ge;
-    }
+    p.ge_max = gemm_ctas(ctx, tiles, K);
     ph.push_back(p);
     return ph.back();
   };
@@ -847,7 +871,7 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
   P.trace = (ctx->profile && &M == &ctx->target) ? reinterpret_cast<unsigned long long*>(ws + L.mk_trace) : nullptr;
   const int grid = std::min(ctx->sm_count, TC_GRID_MAX);
   void* args[] = {&P};
-  CK(cudaLaunchCooperativeKernel(mk::forward_fn(m, P.att_tma, P.att_tc, T), dim3(grid), dim3(mk::MK_THREADS), args,
+  CK(cudaLaunchCooperativeKernel(mk::forward_fn(m, P.att_tma, P.att_tc, T, share_rows(ctx, m, T)), dim3(grid), dim3(mk::MK_THREADS), args,
                                  mk::smem_bytes(t_box, P.stages, m.head_dim, P.att_dbl, P.kps, P.att_tma, P.att_nbuf, P.att_q_rows), ctx->stream));
   ctx->bar_base += (unsigned long long)n_run * grid;
   ctx->launches++;
@@ -1678,9 +1702,9 @@ int stairs_init(const stairs_config* cfg, const stairs_weights* target, const st
       const bool fits = mk::pick_stages(MK_MAX_ROWS, hdm, 1, 1) >= 3 && worst_chunks * hkvm / 64 <= 2 * std::min(ctx->sm_count, TC_GRID_MAX);
       if (coop && fits && cfg->gemm_impl == 0) {
         e = cudaSuccess;
-        for (int i = 0; i < 16 && e == cudaSuccess; ++i) {   // (every kernel the two models' calls may launch: also loads its code now)
-          const stairs_model& fm = i < 8 || !has_draft ? cfg->target : cfg->draft;
-          e = cudaFuncSetAttribute(mk::forward_fn(fm, i & 1, (i >> 1) & 1, i & 4 ? 1 : 64), cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
+        for (int i = 0; i < 32 && e == cudaSuccess; ++i) {   // (every kernel the two models' calls may launch: also loads its code now)
+          const stairs_model& fm = i < 16 || !has_draft ? cfg->target : cfg->draft;
+          e = cudaFuncSetAttribute(mk::forward_fn(fm, i & 1, (i >> 1) & 1, i & 4 ? 1 : 64, (i >> 3) & 1), cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
         }
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(wide::k_wide_attn_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide::tc_att_smem<64>());
@@ -2127,6 +2151,10 @@ int stairs_debug_tune(stairs_ctx* ctx, int what, long long value) {
     case 6:
       if (value < 0 || value > mid::MAX_C) return fail(ctx, STAIRS_EINVAL, "CTA pairs per tile must be 0 (planned) .. %d", mid::MAX_C);
       ctx->mid_force = (int)value;
+      return STAIRS_OK;
+    case 7:
+      if (value < 0 || value > 2) return fail(ctx, STAIRS_EINVAL, "split tiles must be 0 (planned), 1 (one CTA) or 2 (shared rows)");
+      ctx->share_force = (int)value;
       return STAIRS_OK;
     default: return fail(ctx, STAIRS_EINVAL, "unknown tuning knob %d", what);
   }

@@ -17,9 +17,9 @@
 // 3-D bulk tensor copy per operand and freed by ONE commit (issue costs, not bandwidth, bound the
 // single-thread roles).  GEMM work is cut into contiguous ranges per CTA, in units of two k-blocks
 // whatever the stage depth, so results do not depend on the call's row count; a tile cut over
-// several CTAs is finished by the CTA that owns its first k-block, which adds the other CTAs' parked
-// partial tiles in k order; no flags: a parked word reads as an "empty" pattern until it has been
-// stored, and the finisher polls the words it needs.  Normalisation is folded into the GEMMs (operand
+// several CTAs is finished by the CTA that owns its first k-block, or by all of them with a share of the rows each
+// (compiled separately: the kernel is bound by instruction fetch), from partial tiles parked by the others and added
+// in k order; no flags: a parked word reads as an "empty" pattern until it has been stored, and the finisher polls the words it needs.  Normalisation is folded into the GEMMs (operand
 // x * gain, epilogue rescales by the row's 1/std from per-tile statistics).
 //
 // Attention (staircase mask over the paged cache): a unit is (request, kv head, range of 64-position
@@ -145,10 +145,13 @@ constexpr int MK_XCH_BYTES = 16 * VT_LD * 4;     // the tile itself
 // way, or an address computed from a run-time head size, costs what it adds to the text.  With the head size, the model
 // family, the attention path and "at most 16 rows" fixed, validate calls took: 7B, 9 rows 2770 us (general code 2860), 0.4B,
 // 9 rows 1012 (1128), 3B, 5 rows 1984 (2072), 7B of four layers, 4 x 16384 positions, 36 rows 1009 (1056).  HD 0, FAM 0, ATT 3 and ONE false are the general code.
+// With a way of finishing split tiles per kernel: 0.4B, 9 rows 928 -> 848 us (shared rows; both ways in one kernel 864), draft of 4 tokens 891 -> 880.
 //   FAM 1: LayerNorm, GELU, learned positions; FAM 2: RMSNorm, SwiGLU, rotary positions
 //   ATT 0: bulk copies, contractions on mma.sync; 1: on tcgen05
-template <int HD, int FAM, int ATT, bool ONE_CHUNK>
+//   SHARE: split tiles are finished by all their CTAs, a share of the rows each (few rows or few tiles; see share_rows in engine.cu), or by one
+template <int HD, int FAM, int ATT, bool ONE_CHUNK, bool SHARE_ROWS>
 struct Spec {
+  static constexpr bool SHARE = SHARE_ROWS;
   static constexpr bool ONE = ONE_CHUNK;
   static __device__ __forceinline__ int hd(const Params& P) { return HD ? HD : P.hd; }
   static __device__ __forceinline__ bool layer_norm(const Params& P) { return FAM ? FAM == 1 : P.norm_kind == 0; }
@@ -315,6 +318,19 @@ __device__ __forceinline__ void store_split4(bf16* base, size_t idx, size_t lo_o
       make_uint2(pack_bf16x2(v.x - __low2float(h01), v.y - __high2float(h01)), pack_bf16x2(v.z - __low2float(h23), v.w - __high2float(h23)));
 }
 
+// Roundings that two compiled forms of the epilogue have to share: contractions are spelt out.
+__device__ __forceinline__ float normed(float v, float mu, float rs, float u, float c) { return __fmaf_rn(rs, __fmaf_rn(-mu, u, v), c); }
+__device__ __forceinline__ float rotated(float a, float b, float cs, float sn) { return __fmaf_rn(b, sn, __fmul_rn(a, cs)); }
+__device__ __forceinline__ float square_sum(float a, float b, float c, float d) { return __fadd_rn(__fmaf_rn(b, b, __fmul_rn(a, a)), __fmaf_rn(d, d, __fmul_rn(c, c))); }
+// (mean, M2, count) of n values from their sums shifted by sh
+__device__ __forceinline__ float4 tile_stats(float sh, float s1, float s2, int n) {
+  const float dm = s1 / (float)n;
+  return make_float4(__fadd_rn(sh, dm), fmaxf(__fmaf_rn(-s1, dm, s2), 0.f), (float)n, 0.f);
+}
+__device__ __forceinline__ float row_rstd(bool layer_norm, float m2, float n, float mean, int d, float eps) {
+  return 1.0f / sqrtf(__fadd_rn((layer_norm ? m2 : __fmaf_rn(__fmul_rn(n, mean), mean, m2)) / (float)d, eps));
+}
+
 // Sums 32 per-lane values across the warp, all at once: on return lane l holds the warp-wide
 // total of a[l].  Each halving step exchanges the half a lane does not keep (31 shuffles in five
 // dependent steps, instead of 32 separate five-step reductions).
@@ -342,6 +358,7 @@ struct Ctl {
   // tcgen05 attention: S of a chunk is in TMEM (two S buffers) / the chunk's P tile is written and O rescaled
   // (two P tiles; one arrival per compute warp) / the unit's Q tile is staged / a P.V has completed
   uint64_t s_full[2], p_full[2], q_full, o_done;
+  uint64_t in_ready;            // the inputs of the CTA's next GEMM phase are published (seen by the producer)
   volatile int areq_ready;                              // the requests' attention geometry below is filled in
   uint32_t tmem_slot;
   volatile int abort_flag;
@@ -352,6 +369,7 @@ struct Ctl {
   AttnReq areq[64];             // per request, filled once per launch (a request has at least one row: <= 64)
   alignas(16) uint32_t phc[2][(sizeof(Phase) + 3) / 4];   // this and the next phase's descriptor (global memory is a
                                                           // long round trip with the L1 carved down to almost nothing)
+  int kv_row[64];               // cache row of each row's position, filled once per launch
   alignas(16) float gtile[128]; // next operand's gain for the current tile's columns
   alignas(16) float utile[128]; // folded-normalisation constants u[n], c[n] of the tile's columns
   alignas(16) float ctile[128];
@@ -1253,7 +1271,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
     for (int b = 0; b < MAX_KV_BUF; ++b) { mbar_init(ctl->kv_full + b, 1); mbar_init(ctl->kv_empty + b, S::tc(P) ? 1 : 4); }
     mbar_init(ctl->s_full + 0, 1); mbar_init(ctl->s_full + 1, 1);
     mbar_init(ctl->p_full + 0, 4); mbar_init(ctl->p_full + 1, 4);
-    mbar_init(&ctl->q_full, 4); mbar_init(&ctl->o_done, 1);
+    mbar_init(&ctl->q_full, 4); mbar_init(&ctl->o_done, 1); mbar_init(&ctl->in_ready, 1);
     ctl->abort_flag = 0; ctl->bcast = 0; ctl->areq_ready = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1278,6 +1296,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
       uint32_t a_par = 0;
       unsigned int a_count = 0, b_count = 0, idle = 0;
       int ready_ph = -1;   // phases <= ready_ph have their inputs published
+      int told_ph = -1;
       unsigned long long poll_val = 0; bool poll_pending = false;
       int traced_ph = -1;
       long long t_idle = clock64();
@@ -1306,6 +1325,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
             if (B.ph > ready_ph) { poll_val = ld_acquire_u64(bar_count); poll_pending = true; }
           }
           if (B.ph <= ready_ph) {
+            if (B.ph != told_ph) { told_ph = B.ph; mbar_arrive(&ctl->in_ready); }   // (the epilogue warps read statistics and residuals)
             uint8_t* b_dst = smem + (size_t)b_stage * stage_bytes + a_stage_bytes;
             tma_load_3d(b_dst, P.maps + B.x_map, 0, 0, B.kk * kps, ctl->full + b_stage, pol_x);   // hi and lo rows in one box
             if (MK_TRACE_PTR(P.trace) && cta == 0 && B.ph != traced_ph) { traced_ph = B.ph; MK_TRACE_PTR(P.trace)[(size_t)B.ph * 8 + 7] = globaltimer_ns(); }
@@ -1507,6 +1527,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
       if (et < PH_WORDS) ctl->phc[0][et] = __ldcg(reinterpret_cast<const uint32_t*>(P.phases) + et);
       const int n_req0 = P.mode == CALL_VALIDATE ? P.n_req : 1;
       if (et < n_req0 && et < 64) ctl->areq[et] = attn_req(P, et, G);
+      if (et < P.T) ctl->kv_row[et] = cache_row_of(P, et);
       if (S::tma(P)) {
         // the chunk buffers start out finite: a box that is never fetched (past the page table) must not feed NaNs to P.V
         uint8_t* ring = att_ring_base<S>(P, att_smem);
@@ -1519,22 +1540,23 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
       if (et == 0) { __threadfence_block(); ctl->areq_ready = 1; }
     }
     KvCons kvc{0, 0u, 0u, 0u};
-    // Split-tile partial sums: two sets of slots, used by alternate GEMM phases; the slots a finisher
-    // has read are emptied again one GEMM phase later (or at the end of the kernel), while it waits
-    // for that phase's accumulator - off the chain that ends a phase, and before the set's next use.
+    // Split-tile partial sums: two sets of slots (two per CTA: of a tile that began in an earlier CTA's range, and of one that goes on
+    // in a later one's), used by alternate GEMM phases; what a CTA has read it empties one GEMM phase later (or at the
+    // end of the kernel), while it waits for that phase's accumulator - off the chain that ends a phase, and before the set's next use.
+    struct Split { unsigned c0, n; int tile, r0, r1; };   // CTAs c0 .. c0 + n - 1; this CTA's rows
     int gph = 0;                               // GEMM phases so far
-    unsigned pend_first = 1u, pend_last = 0u;  // slots (CTAs) read and not yet emptied
-    int pend_set = 0;
-    auto slot_of = [&](int set, unsigned c) { return P.partial + ((size_t)set * G + c) * P.t_box * BM; };
-    auto empty_pending = [&]() {
-      const int er_ = et >> 3, cg_ = et & 7;
-      for (unsigned c = pend_first; c <= pend_last; ++c)
-        for (int t = er_; t < P.T; t += 16) {
-          float* row = slot_of(pend_set, c) + (size_t)t * BM;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) st_relaxed_u4(row + (cg_ + 8 * q) * 4, make_uint4(PARTIAL_EMPTY, PARTIAL_EMPTY, PARTIAL_EMPTY, PARTIAL_EMPTY));
-        }
-      pend_first = 1u; pend_last = 0u;
+    Split ea{0u, 0u, 0, 0, 0}, eb{0u, 0u, 0, 0, 0};       // read in the last GEMM phase and not yet emptied
+    uint32_t in_par = 0;
+    auto slot_of = [&](int set, unsigned c, bool head) { return P.partial + (((size_t)set * G + c) * 2 + (head ? 1 : 0)) * P.t_box * BM; };
+    auto empty_pending = [&](int set) {
+#pragma unroll 1
+      for (int k = 0; k < (S::SHARE ? 2 : 1); ++k) {
+        const Split q = k ? eb : ea;
+        for (unsigned c = 0; c < q.n; ++c)
+          for (int r = q.r0 + (et >> 5); r < q.r1; r += 4)
+            st_relaxed_u4(slot_of(set, q.c0 + c, S::SHARE && c == 0) + (size_t)r * BM + lane * 4, make_uint4(PARTIAL_EMPTY, PARTIAL_EMPTY, PARTIAL_EMPTY, PARTIAL_EMPTY));
+      }
+      ea.n = eb.n = 0u;
     };
     // Parked attention states: two sets, used by alternate attention phases.  The states are merged
     // inside the attention phase itself (each warp polls the words it needs: no grid barrier in
@@ -1768,16 +1790,280 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
         }
       } else {
         // ---------------------------------------------------------------- GEMM epilogue
-        empty_pending();
         const int pset = gph & 1;
+        empty_pending(pset ^ 1);
         const KRange kr = phase_range(p.n_tiles, p.upt, p.kblocks, RANGE_UNIT_KB / kps, cta, G, p.ge_max);
-        const int kb_begin = kr.begin, kb_end = kr.end;
-        const int Ge = kr.ge;
-        gemm_worked = kb_begin < kb_end;
-        const int Tvalid = P.T;
+        const int kb_end = kr.end, T = P.T;
+        gemm_worked = kr.begin < kb_end;
         float* out_f32 = (p.epi == TC_LMHEAD) ? P.logits : reinterpret_cast<float*>(p.out);
         bf16* out_act = reinterpret_cast<bf16*>(p.out);
+        Split sa{0u, 0u, 0, 0, 0}, sb{0u, 0u, 0, 0, 0};   // what this CTA reads of split tiles
+        int kb = kr.begin;
+        // (both ways below give bit for bit the same: sums in k order, statistics in the same tree of additions)
+        if constexpr (S::SHARE) {
+        // Every CTA of a split tile finishes an equal share of the call's rows; a warp finishes a row at a time, four columns to a lane.
+        // Each phase runs this code once or twice, so what it costs is its instruction fetch: one copy serves rows of split
+        // and of whole tiles, and what does not depend on the sums (geometry, residuals, constants) is done before the
+        // accumulator is waited for.
+        // The tiles this CTA shares with others: one that began before its range, one that goes on behind it; whole tiles in between.
+        const int w = et >> 5, col = lane * 4, tb = S::ONE ? 16 : P.t_box;
+        unsigned long long* tra = (MK_TRACE_PTR(P.trace) && et == 0) ? MK_TRACE_PTR(P.trace) + (size_t)2 * P.n_phases * 8 + ((size_t)cta * P.n_phases + ph) * 8 : nullptr;
+        int wt = 0, wt_end = 0;
+        if (gemm_worked) {
+          const int tf = kb / p.kblocks, tl = (kb_end - 1) / p.kblocks;
+          const bool cut_a = kb != tf * p.kblocks, cut_b = kb_end != (tl + 1) * p.kblocks && (tl != tf || !cut_a);
+          wt = cut_a ? tf + 1 : tf; wt_end = cut_b ? tl : tl + 1;
+          const unsigned units = (unsigned)(p.n_tiles * p.upt), ge = (unsigned)kr.ge;
+#pragma unroll 1
+          for (int k = 0; k < 2; ++k) {
+            if (!(k ? cut_b : cut_a)) continue;
+            // the CTAs whose ranges hold the tile's first and its last unit (unit u is CTA ((u + 1) ge - 1) / units's)
+            Split q;
+            q.tile = k ? tl : tf;
+            q.c0 = (((unsigned)q.tile * p.upt + 1u) * ge - 1u) / units;
+            q.n = ((unsigned)(q.tile + 1) * p.upt * ge - 1u) / units - q.c0 + 1u;
+            q.r0 = (int)((unsigned)T * ((unsigned)cta - q.c0) / q.n); q.r1 = (int)((unsigned)T * ((unsigned)cta - q.c0 + 1u) / q.n);
+            if (k) sb = q; else sa = q;
+          }
+          W.wait(&ctl->in_ready, in_par);   // inputs are published (a wait that ran out is looked at once, at the end of the phase)
+          in_par ^= 1u;
+          __syncwarp();
+        }
+        if (tracing) tr[3] = globaltimer_ns();
+        bool first_seg = true;
+        int cw = 0;                                      // rows of whole tile wt finished so far
+        auto wait_acc = [&]() {
+          W.wait(ctl->acc_full + buf, (acc_bits >> buf) & 1u);
+          __syncwarp();   // lanes may leave the wait an iteration apart
+          if (tracing && first_seg) { tr[4] = globaltimer_ns(); first_seg = false; }
+          acc_bits ^= 1u << buf;
+          tc_fence_after();
+        };
+        while (gemm_worked) {
+
+          // the next rows to finish: 16 of a whole tile, or in the end this CTA's shares of the split ones (the tile that goes on behind
+          // the range first: its other CTAs are done with it by then)
+          const bool whole = wt < wt_end;
+          const int nb = sb.r1 - sb.r0, jobs = whole ? min(16, T - cw) : nb + sa.r1 - sa.r0;
+          bool parked = false;
+#pragma unroll 1
+          for (int j = w; j < jobs || !parked; j += 4) {
+            int row = 0, tile = 0, n0 = 0, ncols = 0, src = 0, dcol = 0;
+            unsigned c0 = 0, cn = 0;
+            float4 k1 = make_float4(0.f, 0.f, 0.f, 0.f), k2 = k1, cs = k1, sn = k1;   // residual and gain, or LayerNorm's u and c; rotation
+            float4 st0 = k1, st1 = k1;                   // statistics of this row's tiles lane, lane + 32
+            bool on = false;
+            if (j < jobs) {
+              const Split q = j < nb ? sb : sa;
+              row = whole ? cw + j : q.r0 + (j < nb ? j : j - nb);
+              tile = whole ? wt : q.tile; c0 = q.c0; cn = q.n;
+              // first output column of the tile and how many of its columns exist (a tile never straddles two sources)
+              if (S::dual(p)) { n0 = tile * 64; ncols = min(64, p.N - n0); on = (col & 63) < ncols; }
+              else {
+                int src_col = 0, local = tile, col1 = p.n_src > 1 ? p.src_col[1] : p.N;
+                if (p.n_src > 1 && local >= p.src_tiles[0]) {
+                  local -= p.src_tiles[0]; src = 1; src_col = p.src_col[1]; col1 = p.n_src > 2 ? p.src_col[2] : p.N;
+                  if (p.n_src > 2 && local >= p.src_tiles[1]) { local -= p.src_tiles[1]; src = 2; src_col = p.src_col[2]; col1 = p.N; }
+                }
+                dcol = local * BM; n0 = src_col + dcol; ncols = min(BM, col1 - n0); on = col < ncols;
+              }
+              if (p.norm_in) {
+                const float4* sr = P.stats + (size_t)row * P.stat_tiles;
+                if (lane < P.stat_tiles) st0 = __ldcg(sr + lane);
+                if (lane + 32 < P.stat_tiles) st1 = __ldcg(sr + lane + 32);
+              }
+              if (p.epi == TC_ADD_F32) {
+                if (on) k1 = __ldcg(reinterpret_cast<const float4*>(out_f32 + (size_t)row * p.ldo + n0 + col));
+                if (on && p.next_g) k2 = __ldg(reinterpret_cast<const float4*>(p.next_g + n0 + col));
+              } else if (S::shifted(p)) {
+                const int n = S::dual(p) && col >= 64 ? p.N + n0 + col - 64 : n0 + col;
+                if (p.epi == TC_LMHEAD) {   // (a vocabulary need not be a multiple of four)
+                  float* u = reinterpret_cast<float*>(&k1);
+                  float* c = reinterpret_cast<float*>(&k2);
+#pragma unroll
+                  for (int e = 0; e < 4; ++e) if (col + e < ncols) { u[e] = __ldg(p.u + n + e); c[e] = __ldg(p.c + n + e); }
+                } else if (on) { k1 = __ldg(reinterpret_cast<const float4*>(p.u + n)); k2 = __ldg(reinterpret_cast<const float4*>(p.c + n)); }
+              }
+              if (p.qkv_prep && S::rope(P) && src < 2 && on) {
+                const int i4 = lane % (S::hd(P) / 8) * 4;
+                cs = __ldcg(reinterpret_cast<const float4*>(P.rope_cs + (size_t)row * (S::hd(P) / 2) + i4));
+                sn = __ldcg(reinterpret_cast<const float4*>(P.rope_sn + (size_t)row * (S::hd(P) / 2) + i4));
+              }
+            }
+            if (!parked) {
+              parked = true;
+              // parks the partial sums of the segments before these rows
+              while (kb < (whole ? wt * p.kblocks : kb_end)) {
+                const int tile_k = kb / p.kblocks * p.kblocks;
+                wait_acc();
+                if (tra) tra[4] = globaltimer_ns();
+                const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * 2 * tb);
+                float* mine = slot_of(pset, (unsigned)cta, kb == tile_k);
+                for (int r0 = 0; r0 < (S::ONE ? 1 : T); r0 += 16) {   // only rows that exist
+                  float v[16];
+                  tmem_ld16_sum(taddr + (uint32_t)r0, taddr + (uint32_t)(tb + r0), v);
+                  const int jn = min(16, T - r0);
+#pragma unroll
+                  for (int i = 0; i < 16; ++i) if (i < jn) st_relaxed_f32(mine + (size_t)(r0 + i) * BM + m, v[i]);
+                }
+                // (no flag and no fence: the readers poll the values themselves)
+                tc_fence_before();
+                if (lane == 0) mbar_arrive(ctl->acc_empty + buf);
+                if (tra) tra[5] = globaltimer_ns();
+                buf ^= 1; kb = min(tile_k + p.kblocks, kb_end);
+              }
+              if (whole) {   // 16 rows of a whole tile, through the exchange tile
+                if (cw == 0) wait_acc();
+                const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * 2 * tb);
+                float v[16];
+                tmem_ld16_sum(taddr + (uint32_t)cw, taddr + (uint32_t)(tb + cw), v);
+                if (S::ONE || cw + 16 >= T) {   // accumulator drained: the MMA warp may reuse it
+                  tc_fence_before();
+                  if (lane == 0) mbar_arrive(ctl->acc_empty + buf);
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i) vt[i * VT_LD + m] = v[i];
+                epi_bar_sync();   // the exchange tile is complete
+              }
+            }
+            if (j >= jobs) break;
+            float mu = 0.f, rs = 1.f;
+            if (p.norm_in) {   // (also what passes the time until the other CTAs' sums can be seen)
+              // (count-weighted mean, then M2, over the tiles)
+              float n = st0.z + st1.z, wm = __fmaf_rn(st1.z, st1.x, __fmul_rn(st0.z, st0.x));
+#pragma unroll
+              for (int o = 8; o != 8 * 8; o = o == 16 ? 1 : o == 4 ? 64 : 2 * o) { n += __shfl_xor_sync(0xffffffffu, n, o); wm += __shfl_xor_sync(0xffffffffu, wm, o); }   // (8, 16, 1, 2, 4)
+              const float mean = wm / fmaxf(n, 1.f), d0 = st0.x - mean, d1 = st1.x - mean;
+              float m2 = __fadd_rn(__fmaf_rn(__fmul_rn(st0.z, d0), d0, st0.y), __fmaf_rn(__fmul_rn(st1.z, d1), d1, st1.y));
+#pragma unroll
+              for (int o = 8; o != 8 * 8; o = o == 16 ? 1 : o == 4 ? 64 : 2 * o) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+              mu = S::layer_norm(P) ? mean : 0.f;
+              rs = row_rstd(S::layer_norm(P), m2, n, mean, P.d, P.eps);
+            }
+            if (tra) tra[1] = globaltimer_ns();
+            float4 v;
+            if (whole) v = *reinterpret_cast<const float4*>(vt + j * VT_LD + col);
+            else {
+              v = make_float4(0.f, 0.f, 0.f, 0.f);
+              const size_t step = (size_t)2 * tb * BM;
+              const float* part = slot_of(pset, c0, false) + (size_t)row * BM + (on ? col : 0);   // (segment 0 is in its CTA's second slot)
+              uint4 s[8];
+              // The segments' partial sums, eight in flight together, added in k order.  A slot element reads PARTIAL_EMPTY until its
+              // producer has stored the sum: then the loads are repeated, from the second time on after one word of every
+              // segment has been waited for (little traffic while others still stream weights).  All waits are bounded.
+#pragma unroll 1
+              for (unsigned c = 0; c < cn; c += 8) {
+                int tries = 0;
+                long long t0 = 0;
+                while (true) {
+                  uint32_t mx = 0u;
+                  {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) if (c + u < cn) s[u] = ld_relaxed_u4(part + (c + u) * step + (u == 0 && c == 0 ? step / 2 : 0));
+                  }
+#pragma unroll
+                  for (int u = 0; u < 8; ++u) if (c + u < cn) mx = max(max(mx, max(s[u].x, s[u].y)), max(s[u].z, s[u].w));
+                  if (!__any_sync(0xffffffffu, mx == PARTIAL_EMPTY) || tries == 99) break;
+                  if (++tries == 1) continue;
+                  if (tries == 2) t0 = clock64();
+                  while (true) {   // one word of every segment
+                    const unsigned u = c + lane;
+                    const uint4 x = lane < 8 && u < cn ? ld_relaxed_u4(slot_of(pset, c0 + u, u == 0) + (size_t)row * BM) : make_uint4(0u, 0u, 0u, 0u);
+                    if (!__any_sync(0xffffffffu, x.x == PARTIAL_EMPTY)) break;
+                    bool quit = false;
+                    if (lane == 0) quit = W.poll_abort(t0);
+                    if (__any_sync(0xffffffffu, quit)) { if (lane == 0) W.note(3u, (unsigned)ph, (unsigned)cta, cn, (unsigned)tile); tries = 99; break; }
+                    __nanosleep(32);
+                  }
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                  if (c + u < cn) { v.x += __uint_as_float(s[u].x); v.y += __uint_as_float(s[u].y); v.z += __uint_as_float(s[u].z); v.w += __uint_as_float(s[u].w); }
+              }
+              if (tra) tra[2] = globaltimer_ns();
+            }
+            if (p.norm_in) {
+              // the folded normalisation: y = rstd_t * (acc - mean_t * u[n]) + c[n]
+              if (S::shifted(p)) {
+                v.x = normed(v.x, mu, rs, k1.x, k2.x); v.y = normed(v.y, mu, rs, k1.y, k2.y);
+                v.z = normed(v.z, mu, rs, k1.z, k2.z); v.w = normed(v.w, mu, rs, k1.w, k2.w);
+              } else { v.x *= rs; v.y *= rs; v.z *= rs; v.w *= rs; }
+            }
+            if (p.epi == TC_ADD_F32) {
+              // residual update (such a GEMM has no folded normalisation); with a following normalised GEMM its operand
+              // bf16(x * gain) and this tile's row statistics (count, mean, centred sum of squares; shifted by the row's first value)
+              v = make_float4(k1.x + v.x, k1.y + v.y, k1.z + v.z, k1.w + v.w);
+              if (on) {
+                *reinterpret_cast<float4*>(out_f32 + (size_t)row * p.ldo + n0 + col) = v;
+                if (p.next_g) store_split4(P.h, (size_t)row * p.ldo + n0 + col, (size_t)P.lo_row * p.ldo, make_float4(v.x * k2.x, v.y * k2.y, v.z * k2.z, v.w * k2.w));
+              }
+              if (p.next_g) {
+                const float sh = __shfl_sync(0xffffffffu, v.x, 0), d0 = v.x - sh, d1 = v.y - sh, d2 = v.z - sh, d3 = v.w - sh;
+                float s1 = on ? (d0 + d1) + (d2 + d3) : 0.f, s2 = on ? square_sum(d0, d1, d2, d3) : 0.f;
+#pragma unroll
+                for (int o = 8; o != 8 * 8; o = o == 16 ? 1 : o == 4 ? 64 : 2 * o) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }   // (8, 16, 1, 2, 4)
+                if (lane == 0) P.stats[(size_t)row * P.stat_tiles + tile] = tile_stats(sh, s1, s2, ncols);
+              }
+            } else if (S::swiglu(p)) {
+              // gate columns in lanes 0 to 15, the matching up columns in 16 to 31: each of a pair takes two of the four
+              const bool up = lane >= 16;
+              const float r0 = __shfl_xor_sync(0xffffffffu, up ? v.x : v.z, 16), r1 = __shfl_xor_sync(0xffffffffu, up ? v.y : v.w, 16);
+              const float g0 = up ? r0 : v.x, g1 = up ? r1 : v.y, y0 = silu_f(g0) * (up ? v.z : r0), y1 = silu_f(g1) * (up ? v.w : r1);
+              if (on) {
+                bf16* o = out_act + (size_t)row * p.ldo + n0 + (col & 63) + (up ? 2 : 0);
+                const __nv_bfloat162 h = __floats2bfloat162_rn(y0, y1);
+                *reinterpret_cast<__nv_bfloat162*>(o) = h;
+                *reinterpret_cast<uint32_t*>(o + (size_t)P.lo_row * p.ldo) = pack_bf16x2(y0 - __low2float(h), y1 - __high2float(h));
+              }
+            } else if (p.epi == TC_LMHEAD) {
+              // logits (optional) and the row's running argmax; the vocabulary need not be a multiple of 4
+              const float e4[4] = {v.x, v.y, v.z, v.w};
+              unsigned long long key = 0ull;
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                if (col + e < ncols) {
+                  if (out_f32) out_f32[(size_t)row * p.ldo + n0 + col + e] = e4[e];
+                  const unsigned long long k = argmax_key(e4[e], (uint32_t)(n0 + col + e));
+                  key = k > key ? k : key;
+                }
+#pragma unroll
+              for (int o = 16; o >= 1; o >>= 1) {
+                const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
+                key = other > key ? other : key;
+              }
+              if (lane == 0 && key) atomicMax(P.keys + row, key);
+            } else if (p.qkv_prep) {
+              // q: rotate, scale by 1/sqrt(hd), fp16, to the query buffer; k: rotate, fp16, to its row of the cache; v: fp16
+              // to the cache.  The rotation pairs column i with i + hd/2 of a head, hd/8 lanes away (head size 64 or 128).
+              const int hd = S::hd(P);
+              if (S::rope(P) && src < 2) {
+                const bool lower = lane % (hd / 4) < hd / 8;
+                const int other = lower ? lane + hd / 8 : lane - hd / 8;
+                float4 o = make_float4(__shfl_sync(0xffffffffu, v.x, other), __shfl_sync(0xffffffffu, v.y, other),
+                                       __shfl_sync(0xffffffffu, v.z, other), __shfl_sync(0xffffffffu, v.w, other));
+                if (lower) o = make_float4(-o.x, -o.y, -o.z, -o.w);
+                v = make_float4(rotated(v.x, o.x, cs.x, sn.x), rotated(v.y, o.y, cs.y, sn.y), rotated(v.z, o.z, cs.z, sn.z), rotated(v.w, o.w, cs.w, sn.w));
+              }
+              const float qs = src == 0 ? 1.4426950408889634f / sqrtf((float)hd) : 1.0f;   // log2(e) / sqrt(hd): the softmax works in base 2
+              __half* dst = (src == 0 ? P.q16 + (size_t)row * (P.Hq * hd)
+                                      : reinterpret_cast<__half*>(src == 1 ? p.kc : p.vc) + (size_t)ctl->kv_row[row] * (P.Hkv * hd)) + dcol;
+              if (on) *reinterpret_cast<uint2*>(dst + col) = make_uint2(pack_f16x2(v.x * qs, v.y * qs), pack_f16x2(v.z * qs, v.w * qs));
+            } else if (on) {
+              if (S::store(p)) *reinterpret_cast<float4*>(out_f32 + (size_t)row * p.ldo + n0 + col) = v;
+              else store_split4(out_act, (size_t)row * p.ldo + n0 + col, (size_t)P.lo_row * p.ldo, make_float4(gelu_erf(v.x), gelu_erf(v.y), gelu_erf(v.z), gelu_erf(v.w)));
+            }
+          }
+          __syncwarp();
+          if (!whole) break;
+          epi_bar_sync();   // (the exchange tile is reused)
+          cw += 16;
+          if (cw >= T) { cw = 0; buf ^= 1; ++wt; kb = wt * p.kblocks; }
+        }
+        if (tra) tra[3] = globaltimer_ns();
+        } else {
+        // The CTA that owns a tile's first k-block finishes the tile, 16 rows at a time.
         unsigned long long* keys = P.keys;
+        const int kb_begin = kr.begin, Tvalid = T;
         // LayerNorm: the per-column constants of the tile this CTA finishes first are requested before the wait for the
         // statistics (they come from HBM, once a call; sources are whole tiles in this case): 0.4B, 9 rows 1012 -> 1002 us
         float uq = 0.f, cq = 0.f;
@@ -1786,49 +2072,56 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           pre_tile = (kb_begin + p.kblocks - 1) / p.kblocks;
           if (pre_tile < p.n_tiles) { uq = p.u[pre_tile * BM + m]; cq = p.c[pre_tile * BM + m]; }
         }
-        // Row statistics of the operand (published by the phase that produced x): merged into mean and 1/std per row, eight lanes per
-        // row as in the epilogue, and only by CTAs that finish a tile in this phase.  (A first form, by all CTAs, a warp per
-        // row, held up the partial sums of those that only park them, and its longer text slowed the MMA warp's first stage, which is
-        // fetched at the same time: 0.4B, 9 rows 993 -> 915 us.  Merging them between parking and finishing: 3B, 5 rows 1 % slower.)
-        if (p.norm_in && (kb_begin + p.kblocks - 1) / p.kblocks * p.kblocks < kb_end) {
-          if (lane == 0) W.wait_grid(bar_count, P.bar_base + (unsigned long long)ph * G);   // (one that ran out is looked at once, at the end of the phase)
+        if (gemm_worked) {
+          W.wait(&ctl->in_ready, in_par);   // inputs are published (a wait that ran out is looked at once, at the end of the phase)
+          in_par ^= 1u;
           __syncwarp();
+        }
+        // Row statistics of the operand (published by the phase that produced x): count-weighted mean, then M2, over the tiles, eight
+        // lanes per row as in the epilogue, and only by CTAs that finish a tile in this phase.  (A first form, by all CTAs, a warp
+        // per row, held up the partial sums of those that only park them, and its longer text slowed the MMA warp's first stage, which
+        // is fetched at the same time: 0.4B, 9 rows 993 -> 915 us.  Merging them between parking and finishing: 3B, 5 rows 1 % slower.)
+        if (p.norm_in && (kb_begin + p.kblocks - 1) / p.kblocks * p.kblocks < kb_end) {
           for (int t = et >> 3; t < (S::ONE ? 16 : (Tvalid + 15) & ~15); t += 16) {
             const float4* sr = P.stats + (size_t)min(t, Tvalid - 1) * P.stat_tiles;
             const int sub = et & 7;
-            // this lane's tiles, sums shifted by its first tile's mean; then count-weighted mean and M2 over the eight lanes
-            float n = 0.f, s1 = 0.f, s2 = 0.f, m0 = 0.f;
-#pragma unroll 1
-            for (int i0 = sub; i0 < P.stat_tiles; i0 += 32) {
-              float4 e[4];
+            float4 e[8];   // tiles sub + 8 i
 #pragma unroll
-              for (int i = 0; i < 4; ++i) e[i] = i0 + 8 * i < P.stat_tiles ? __ldcg(sr + i0 + 8 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
-              if (i0 == sub) m0 = e[0].x;
+            for (int i = 0; i < 4; ++i) e[i] = sub + 8 * i < P.stat_tiles ? __ldcg(sr + sub + 8 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-              for (int i = 0; i < 4; ++i) { const float d0 = e[i].x - m0, nd = e[i].z * d0; n += e[i].z; s1 += nd; s2 += e[i].y + nd * d0; }
+            for (int i = 4; i < 8; ++i) e[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (P.stat_tiles > 32) {
+#pragma unroll
+              for (int i = 4; i < 8; ++i) if (sub + 8 * i < P.stat_tiles) e[i] = __ldcg(sr + sub + 8 * i);
             }
-            const float dm = s1 / fmaxf(n, 1.f), mean_l = m0 + dm, m2_l = fmaxf(s2 - s1 * dm, 0.f);
-            float n_all = n, w = n * mean_l;
+            float nn[4], ww[4];
 #pragma unroll
-            for (int o = 1; o < 8; o <<= 1) { n_all += __shfl_xor_sync(0xffffffffu, n_all, o); w += __shfl_xor_sync(0xffffffffu, w, o); }
-            const float mean = w / fmaxf(n_all, 1.f);
-            float m2 = m2_l + n * (mean_l - mean) * (mean_l - mean);
+            for (int i = 0; i < 4; ++i) { nn[i] = e[i].z + e[i + 4].z; ww[i] = __fmaf_rn(e[i + 4].z, e[i + 4].x, __fmul_rn(e[i].z, e[i].x)); }
+            float n = (nn[0] + nn[1]) + (nn[2] + nn[3]), wm = (ww[0] + ww[1]) + (ww[2] + ww[3]);
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) { n += __shfl_xor_sync(0xffffffffu, n, o); wm += __shfl_xor_sync(0xffffffffu, wm, o); }
+            const float mean = wm / fmaxf(n, 1.f);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float d0 = e[i].x - mean, d1 = e[i + 4].x - mean;
+              ww[i] = __fadd_rn(__fmaf_rn(__fmul_rn(e[i].z, d0), d0, e[i].y), __fmaf_rn(__fmul_rn(e[i + 4].z, d1), d1, e[i + 4].y));
+            }
+            float m2 = (ww[0] + ww[1]) + (ww[2] + ww[3]);
 #pragma unroll
             for (int o = 1; o < 8; o <<= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
             if (sub == 0 && t < Tvalid) {
               ctl->mu[t] = S::layer_norm(P) ? mean : 0.f;
-              ctl->rstd[t] = 1.0f / sqrtf((S::layer_norm(P) ? m2 : m2 + n_all * mean * mean) / (float)P.d + P.eps);
+              ctl->rstd[t] = row_rstd(S::layer_norm(P), m2, n, mean, P.d, P.eps);
             }
           }
         }
         if (tracing) tr[3] = globaltimer_ns();
         bool first_seg = true;
-        int kb = kb_begin;
-        const unsigned tot32 = (unsigned)(p.n_tiles * p.upt), ge32 = (unsigned)Ge;
+        const unsigned tot32 = (unsigned)(p.n_tiles * p.upt), ge32 = (unsigned)kr.ge;
         // first stage of CTA c's range (units * Ge < 2^32, checked on the host)
         auto rb = [&](unsigned c) { return (unsigned)unit_to_stage((tot32 * c) / ge32, p.upt, p.kblocks, RANGE_UNIT_KB / kps); };
         const int er = et >> 3, cg = et & 7;
-        while (kb < kb_end && ok) {
+        while (kb < kb_end) {
           const int tile = kb / p.kblocks, kk0 = kb - tile * p.kblocks;
           const int tile_first = tile * p.kblocks, tile_end = tile_first + p.kblocks;
           const int seg_end = tile_end < kb_end ? tile_end : kb_end;
@@ -1865,7 +2158,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           // table entries of its column groups (q and k tiles), for the first chunk
           int kv_row0 = 0;
           float4 rc0a, rc0b, rs0a, rs0b;
-          auto kv_row_of = [&](int t) { return cache_row_of(P, t); };
+          auto kv_row_of = [&](int t) { return ctl->kv_row[t]; };
           auto rope_of = [&](int t, float4& c0, float4& s0, float4& c1, float4& s1) {
             // hd = 128: groups (0, 2) and (1, 3) pair up, at table columns cg*4 and 32 + cg*4;
             // hd = 64: groups (0, 1) and (2, 3), both at table column cg*4
@@ -1908,7 +2201,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           unsigned long long* tra = (MK_TRACE_PTR(P.trace) && et == 0 && !whole) ? MK_TRACE_PTR(P.trace) + (size_t)2 * P.n_phases * 8 + ((size_t)cta * P.n_phases + ph) * 8 : nullptr;
           if (!finisher) {
             if (tra) tra[4] = globaltimer_ns();
-            float* mine = slot_of(pset, (unsigned)cta);
+            float* mine = slot_of(pset, (unsigned)cta, false);
             for (int c0 = 0; c0 < (S::ONE ? 1 : Tvalid); c0 += 16) {   // only rows that exist
               float v[16];
               tmem_ld16_sum(taddr + (uint32_t)c0, taddr + (uint32_t)(P.t_box + c0), v);
@@ -1923,7 +2216,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           } else {
             unsigned last_c = (unsigned)cta;   // CTAs cta + 1 .. last_c hold the tile's other segments
             if (!whole) while (last_c + 1 < ge32 && rb(last_c + 1) < (unsigned)tile_end) ++last_c;
-            if (!whole) { pend_first = (unsigned)cta + 1u; pend_last = last_c; pend_set = pset; }   // (at most one split tile is finished per phase)
+            if (!whole) sa = Split{(unsigned)cta + 1u, last_c - (unsigned)cta, tile, 0, Tvalid};   // (at most one split tile is finished per phase)
             for (int c0 = 0; c0 < (S::ONE ? 1 : Tvalid); c0 += 16) {
               {
                 float v[16];
@@ -1960,14 +2253,14 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     // stream weights) and then looks at all of them again.  All waits are bounded.
                     for (unsigned c = (unsigned)cta + 1; c <= last_c; c += 6) {
                       uint4 tmp[6][4];
-                      const float* probe = slot_of(pset, min(c + 5, last_c)) + (size_t)(row_on ? t : 0) * BM + cg * 4;
+                      const float* probe = slot_of(pset, min(c + 5, last_c), false) + (size_t)(row_on ? t : 0) * BM + cg * 4;
                       long long t0 = 0;
                       bool timing = false, give_up = false;
                       while (true) {
                         uint32_t mx = 0u;
 #pragma unroll
                         for (int u = 0; u < 6; ++u) {
-                          const float* part = slot_of(pset, min(c + u, last_c)) + (size_t)(row_on ? t : 0) * BM;
+                          const float* part = slot_of(pset, min(c + u, last_c), false) + (size_t)(row_on ? t : 0) * BM;
 #pragma unroll
                           for (int q = 0; q < 4; ++q) {
                             tmp[u][q] = (on[q] && c + u <= last_c) ? ld_relaxed_u4(part + (cg + 8 * q) * 4) : make_uint4(0u, 0u, 0u, 0u);
@@ -2032,8 +2325,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     if (S::shifted(p)) {
                       const float4 u4 = *reinterpret_cast<const float4*>(ctl->utile + col);
                       const float4 c4 = *reinterpret_cast<const float4*>(ctl->ctile + col);
-                      v.x = rs * (v.x - mu * u4.x) + c4.x; v.y = rs * (v.y - mu * u4.y) + c4.y;
-                      v.z = rs * (v.z - mu * u4.z) + c4.z; v.w = rs * (v.w - mu * u4.w) + c4.w;
+                      v.x = normed(v.x, mu, rs, u4.x, c4.x); v.y = normed(v.y, mu, rs, u4.y, c4.y);
+                      v.z = normed(v.z, mu, rs, u4.z, c4.z); v.w = normed(v.w, mu, rs, u4.w, c4.w);
                     } else { v.x *= rs; v.y *= rs; v.z *= rs; v.w *= rs; }
                   }
                   return v;
@@ -2044,7 +2337,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                   if (p.next_g) {
                     // (sums shifted by the row's first value of the tile, in one pass)
                     const float sh = __shfl_sync(0xffffffffu, a0x, lane & 24);
-                    float s1 = 0.f, s2 = 0.f;
+                    float s1 = 0.f, s2 = 0.f, h1 = 0.f, h2 = 0.f;   // (groups 0 and 1, groups 2 and 3)
 #pragma unroll 1
                     for (int q = 0; q < 4; ++q) {
                       const int col = (cg + 8 * q) * 4;
@@ -2053,16 +2346,15 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                         const float4 g4 = *reinterpret_cast<const float4*>(ctl->gtile + col);
                         store_split4(P.h, (size_t)t * p.ldo + n0 + col, (size_t)P.lo_row * p.ldo, make_float4(x4.x * g4.x, x4.y * g4.y, x4.z * g4.z, x4.w * g4.w));
                         const float d0 = x4.x - sh, d1 = x4.y - sh, d2 = x4.z - sh, d3 = x4.w - sh;
-                        s1 += (d0 + d1) + (d2 + d3); s2 += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+                        s1 += (d0 + d1) + (d2 + d3); s2 += square_sum(d0, d1, d2, d3);
                       }
+                      if (q == 1) { h1 = s1; h2 = s2; s1 = s2 = 0.f; }
                     }
+                    s1 += h1; s2 += h2;
                     if (tra) { asm volatile("" ::"f"(s1), "f"(s2)); tra[7] = globaltimer_ns(); }
 #pragma unroll
                     for (int o = 1; o < 8; o <<= 1) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }
-                    if (cg == 0 && row_on) {
-                      const float cnt = (float)ncols, dm = s1 / cnt;
-                      P.stats[(size_t)t * P.stat_tiles + tile] = make_float4(sh + dm, fmaxf(s2 - s1 * dm, 0.f), cnt, 0.f);
-                    }
+                    if (cg == 0 && row_on) P.stats[(size_t)t * P.stat_tiles + tile] = tile_stats(sh, s1, s2, ncols);
                   }
                 } else if (S::swiglu(p)) {
                   // gate columns (cg + 8 q) * 4 of the tile's first half, the matching up columns 64 further
@@ -2121,8 +2413,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     if (S::rope(P) && src_s < 2) {
                       const float4 cs = pi ? rcb : rca, sn = pi ? rsb : rsa;
                       const float4 l = lo, h = hi;
-                      lo = make_float4(l.x * cs.x - h.x * sn.x, l.y * cs.y - h.y * sn.y, l.z * cs.z - h.z * sn.z, l.w * cs.w - h.w * sn.w);
-                      hi = make_float4(h.x * cs.x + l.x * sn.x, h.y * cs.y + l.y * sn.y, h.z * cs.z + l.z * sn.z, h.w * cs.w + l.w * sn.w);
+                      lo = make_float4(rotated(l.x, -h.x, cs.x, sn.x), rotated(l.y, -h.y, cs.y, sn.y), rotated(l.z, -h.z, cs.z, sn.z), rotated(l.w, -h.w, cs.w, sn.w));
+                      hi = make_float4(rotated(h.x, l.x, cs.x, sn.x), rotated(h.y, l.y, cs.y, sn.y), rotated(h.z, l.z, cs.z, sn.z), rotated(h.w, l.w, cs.w, sn.w));
                     }
                     if (row_on && col_lo < ncols)
                       *reinterpret_cast<uint2*>(dst + col_lo) = make_uint2(pack_f16x2(lo.x * qscale, lo.y * qscale), pack_f16x2(lo.z * qscale, lo.w * qscale));
@@ -2147,10 +2439,11 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
             }
             if (tra) tra[3] = globaltimer_ns();
           }
-          if (!ok) break;
           buf ^= 1;
           kb = seg_end;
         }
+        }
+        ea = sa; eb = sb;
       }
       if (!ok) break;
       if (tracing) tr[1] = globaltimer_ns();
@@ -2193,7 +2486,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
       waited = false;
       if (p.kind == PH_GEMM) ++gph;
     }
-    if (ok) { empty_pending(); if (aph > 0) empty_own_states((aph - 1) & 1); }   // (after an abort the host empties every slot)
+    if (ok) { empty_pending((gph & 1) ^ 1); if (aph > 0) empty_own_states((aph - 1) & 1); }   // (after an abort the host empties every slot)
   }
 
   // ================================================================== teardown
@@ -2237,23 +2530,24 @@ inline int pick_stages(int t_box, int hd, int dbl, int kps, int tma = 0, int nbu
 inline int pick_kps(int t_box, int hd, int dbl) { return pick_stages(t_box, hd, dbl, 2) >= 3 ? 2 : 1; }
 
 // The compiled variants (forward.cu, one object each): the families' usual head sizes, and the general code.
-#define STAIRS_FORWARD_VARIANTS(X)                                                    \
-  X(64, 1, 0, 0) X(64, 1, 0, 1) X(64, 1, 1, 0) X(64, 1, 1, 1)                         \
-  X(64, 2, 0, 0) X(64, 2, 0, 1) X(64, 2, 1, 0) X(64, 2, 1, 1)                         \
-  X(80, 2, 0, 0) X(80, 2, 0, 1)                                                       \
-  X(128, 2, 0, 0) X(128, 2, 0, 1) X(128, 2, 1, 0) X(128, 2, 1, 1)                     \
-  X(0, 0, 3, 0)
-#define STAIRS_FORWARD_DECLARE(hd, fam, att, one) const void* forward_##hd##_##fam##_##att##_##one();
+#define STAIRS_FORWARD_BOTH(X, hd, fam, att, one) X(hd, fam, att, one, 0) X(hd, fam, att, one, 1)
+#define STAIRS_FORWARD_VARIANTS(X)                                                                                                             \
+  STAIRS_FORWARD_BOTH(X, 64, 1, 0, 0) STAIRS_FORWARD_BOTH(X, 64, 1, 0, 1) STAIRS_FORWARD_BOTH(X, 64, 1, 1, 0) STAIRS_FORWARD_BOTH(X, 64, 1, 1, 1) \
+  STAIRS_FORWARD_BOTH(X, 64, 2, 0, 0) STAIRS_FORWARD_BOTH(X, 64, 2, 0, 1) STAIRS_FORWARD_BOTH(X, 64, 2, 1, 0) STAIRS_FORWARD_BOTH(X, 64, 2, 1, 1) \
+  STAIRS_FORWARD_BOTH(X, 80, 2, 0, 0) STAIRS_FORWARD_BOTH(X, 80, 2, 0, 1)                                                                          \
+  STAIRS_FORWARD_BOTH(X, 128, 2, 0, 0) STAIRS_FORWARD_BOTH(X, 128, 2, 0, 1) STAIRS_FORWARD_BOTH(X, 128, 2, 1, 0) STAIRS_FORWARD_BOTH(X, 128, 2, 1, 1) \
+  STAIRS_FORWARD_BOTH(X, 0, 0, 3, 0)
+#define STAIRS_FORWARD_DECLARE(hd, fam, att, one, share) const void* forward_##hd##_##fam##_##att##_##one##_##share();
 STAIRS_FORWARD_VARIANTS(STAIRS_FORWARD_DECLARE)
 
 // The kernel of a model and call.
-inline const void* forward_fn(const stairs_model& m, int att_tma, int att_tc, int T) {
+inline const void* forward_fn(const stairs_model& m, int att_tma, int att_tc, int T, int share) {
   const int fam = m.norm == 0 && m.act == 0 && m.pos == 0 ? 1 : m.norm == 1 && m.act == 1 && m.pos == 1 ? 2 : 0;
   const int att = att_tc ? 1 : 0, one = T <= 16 ? 1 : 0;
-#define STAIRS_FORWARD_PICK(hd_, fam_, att_, one_) \
-  if (att_tma && m.head_dim == hd_ && fam == fam_ && att == att_ && one == one_) return forward_##hd_##_##fam_##_##att_##_##one_();
+#define STAIRS_FORWARD_PICK(hd_, fam_, att_, one_, share_) \
+  if (att_tma && m.head_dim == hd_ && fam == fam_ && att == att_ && one == one_ && share == share_) return forward_##hd_##_##fam_##_##att_##_##one_##_##share_();
   STAIRS_FORWARD_VARIANTS(STAIRS_FORWARD_PICK)
-  return forward_0_0_3_0();
+  return share ? forward_0_0_3_0_1() : forward_0_0_3_0_0();
 }
 
 }  // namespace mk

@@ -42,3 +42,34 @@ def test_variant_matches_oracle_and_ignores_the_row_count(shape, attention, page
     ref, _ = gu.oracle_stair_logits(tgt, prompts[2], drafts[2])
     gu.check_rows_against_oracle(one, tt[0][:17], ref, gu.LOGIT_TOL_BF16)
     eng.close()
+
+@pytest.mark.parametrize("wide_d", [False, True], ids=["", "33_tiles"])
+@pytest.mark.parametrize("attention", [1, 2], ids=["register", "tcgen05"])
+@pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES.keys())
+def test_both_ways_of_finishing_split_tiles_give_the_same_bits(shape, attention, wide_d):
+    # rows that are fewer than a tile's CTAs, one to several a warp, in one and in several 16-row chunks; vocabularies of whole and of
+    # cut tiles; row statistics over more than 32 column tiles
+    st = _stairs()
+    shape = shape.replace(vocab=2044, n_layers=2)
+    if wide_d:
+        if shape.d_model % 128:
+            pytest.skip("one width is enough")
+        shape = shape.replace(d_model=33 * 128)
+    tsrc, _ = sources(shape)
+    eng = st.Stairs(tsrc, None, max_requests=4, max_seq_len=200, k_max=15, kv_page_tokens=16)
+    eng.debug_tune(3, attention)
+    for i in range(4):
+        eng.prefill(i, list(wl.zipf_tokens(100 + i, shape.vocab, i)))
+    drafts = torch.from_numpy(np.random.default_rng(5).integers(0, shape.vocab, size=(4, 15)).astype(np.int32)).cuda()
+    for ks in ([0], [4], [8], [15], [7, 9], [15, 15, 15, 15]):
+        got = []
+        for way in (1, 2):
+            eng.debug_tune(7, way)
+            tt, al, lg = eng.validate(list(range(len(ks))), ks, drafts[:len(ks)].contiguous(), want_logits=True)
+            eng.sync()
+            got.append((tt.clone(), al.clone(), lg.clone()))
+        for a, b in zip(*got):
+            assert torch.equal(a, b)
+        for which in (7, 8):   # every word of the parked sums and states is empty again
+            assert bool((eng.debug_buffer(which, torch.int32, 1 << 16) == -1).all())
+    eng.close()
