@@ -485,11 +485,13 @@ struct WCursor {
   }
 };
 
-// Asks L2 for one weight tile ahead of the shared-memory ring (no shared memory, no barrier involved).
 __device__ __forceinline__ void tma_load_2d_nohint(void* dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
       ::"r"(smem_u32(dst)), "l"(map), "r"(c0), "r"(c1), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int c0, int c1) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(map), "r"(c0), "r"(c1) : "memory");
 }
 // Tiled 3-D load global -> shared.  The operand matrices [rows, K] are described to TMA as
 // [K / 64][rows][64]: a box of (64, rows of the tile, kps) lands as kps consecutive K-major slabs
@@ -1489,6 +1491,13 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                 tma_load_2d_nohint(dst, b_which ? vmap : kmap, kvh * hd + b_half * 64, row, ctl->kv_full + buf);
               }
               __syncwarp();
+              // Units of a few chunks with fewer buffers: the later chunks, where they hold cached positions only, are asked of L2 when the
+              // first one is fetched (3B, 5 rows after 512: three chunks a unit, one buffer; a chunk then took 1.9 us, mostly its way from HBM).
+              if (!S::tc(P) && c == c_begin && my_box)
+                for (int c2 = c + P.att_nbuf; c2 < min(c_end, c + 4); ++c2) {
+                  const int p2 = c2 * ATT_CHUNK + b_slot * box_rows;
+                  if ((c2 + 1) * ATT_CHUNK <= a.base) tma_prefetch_2d(b_which ? vmap : kmap, kvh * hd + b_half * 64, __ldcg(pt + p2 / P.page_tokens) * P.page_tokens + p2 % P.page_tokens);
+                }
               used |= 1u << buf;
               last_par = (last_par & ~(1u << buf)) | (par << buf);
               if (++buf == P.att_nbuf) { buf = 0; par ^= 1u; }
@@ -1637,12 +1646,16 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           u0 += a.units; g0 += P.Hkv * a.n_qblk;
         }
         // Requests whose positions were split over several units: merge the parked states of every
-        // (kv head, query) in position order.  One warp per item; each lane owns 4 consecutive
-        // elements of head_dim, so every partial is one 16-byte load per lane.  The states come
+        // (kv head, query).  One warp per item, or on the mma.sync path, where items are few, per 64 columns of one (head sizes 64 and
+        // 128: half a warp per range, up to twenty ranges in one round trip instead of eight: 7B, 9 rows, 18 ranges 0.6 % of a call,
+        // 0.4B, 9 rows, nine ranges 1.4 %; four layers of 7B with 144 query rows a head 1 % slower so); each lane
+        // owns 4 consecutive elements of head_dim, so every partial is one 16-byte load per lane.  The states come
         // from other CTAs' units of this same phase: a word reads PARTIAL_EMPTY until it has been
         // stored, and the warp repeats its loads (bounded) until none does.
         if (ok) {
           const int hd = S::hd(P), Gq = P.Hq / P.Hkv;
+          const bool pairs = hd % 64 == 0 && !S::tc(P);
+          const int halves = pairs ? hd / 64 : 1, sub = pairs ? lane >> 4 : 0, per = pairs ? 2 : 1;   // parts of an item; ranges per load
           const float* set_base = P.attn_part + (size_t)(aph & 1) * P.attn_set_stride;
           int u0c = 0, item0 = 0;
           bool gave_up = false;
@@ -1658,18 +1671,18 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           for (int i = 0; i < n_req; ++i) {
             const AttnReq a = ctl->areq[i];
             if (a.n_ranges > 1) {
-              const int Q = a.R * Gq, items = P.Hkv * Q;
+              const int Q = a.R * Gq, items = P.Hkv * Q * halves;
               int it = ((cta * 4 + quad) - item0) % (G * 4);
               if (it < 0) it += G * 4;
               for (; it < items && !gave_up; it += G * 4) {
-                const int kvh = it / Q, q = it % Q, qblk = q / S::qblk(P), ql = q % S::qblk(P);
+                const int it1 = it / halves, kvh = it1 / Q, q = it1 % Q, qblk = q / S::qblk(P), ql = q % S::qblk(P);
                 const int first_slot = u0c + (kvh * a.n_ranges) * a.n_qblk + qblk;
                 const size_t stride = (size_t)a.n_qblk * S::qblk(P) * (hd + 4);
                 const float* base = set_base + ((size_t)first_slot * S::qblk(P) + ql) * (hd + 4);
                 // (max, sum) of range lane, lane + 32, ...: one load round for up to 32 ranges, then
-                // the ranges' output vectors eight loads at a time; weights travel by shuffle and
-                // the accumulation stays in range order
-                const int nr = a.n_ranges, dd = lane * 4;
+                // the ranges' output vectors five or ten loads at a time; weights travel by shuffle and
+                // the accumulation is in range order (of even and odd ranges)
+                const int nr = a.n_ranges, dd = per == 2 ? (it % halves) * 64 + (lane & 15) * 4 : lane * 4;
                 long long t0 = 0;
                 bool timing = false;
                 auto state_of = [&](int r, float& mu, float& lu) {   // all lanes call it together
@@ -1700,28 +1713,45 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                   const float wgt = mu == -INFINITY ? 0.f : fast_exp2(mu - M);   // 0 for lanes past the last range (maxima are base-2 exponents)
                   L += lu * wgt;
                   const int nb = min(32, nr - rb);
-                  for (int g0 = 0; g0 < nb && !gave_up; g0 += 8) {
-                    uint4 v[8];
+                  for (int g0 = 0; g0 < nb && !gave_up; g0 += (hd % 64 == 0 ? 10 * per : 5)) {
+                    uint4 v[10];
+                    const float* at = base + (size_t)(rb + g0 + sub) * stride + dd;
+                    const bool more = hd % 64 == 0 && nb - g0 > 5 * per;
+                    auto load = [&](int u) { v[u] = (g0 + u * per + sub < nb && dd < hd) ? ld_relaxed_u4(at + (size_t)(u * per) * stride) : make_uint4(0u, 0u, 0u, 0u); };
+                    auto add = [&](int u) {
+                      const float wu = __shfl_sync(0xffffffffu, wgt, (g0 + u * per + sub) & 31);
+                      acc.x += __uint_as_float(v[u].x) * wu; acc.y += __uint_as_float(v[u].y) * wu;
+                      acc.z += __uint_as_float(v[u].z) * wu; acc.w += __uint_as_float(v[u].w) * wu;
+                    };
                     while (true) {
                       uint32_t mx = 0u;
 #pragma unroll
-                      for (int u = 0; u < 8; ++u) {
-                        v[u] = (g0 + u < nb && dd < hd) ? ld_relaxed_u4(base + (size_t)(rb + g0 + u) * stride + dd) : make_uint4(0u, 0u, 0u, 0u);
-                        mx = max(max(mx, max(v[u].x, v[u].y)), max(v[u].z, v[u].w));
+                      for (int u = 0; u < 5; ++u) load(u);
+                      if (more) {
+#pragma unroll
+                        for (int u = 5; u < 10; ++u) load(u);
+#pragma unroll
+                        for (int u = 5; u < 10; ++u) mx = max(max(mx, max(v[u].x, v[u].y)), max(v[u].z, v[u].w));
                       }
+#pragma unroll
+                      for (int u = 0; u < 5; ++u) mx = max(max(mx, max(v[u].x, v[u].y)), max(v[u].z, v[u].w));
                       if (!__any_sync(0xffffffffu, mx == PARTIAL_EMPTY)) break;
                       if (backoff(t0, timing)) { gave_up = true; break; }
                     }
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                      const float wu = __shfl_sync(0xffffffffu, wgt, (g0 + u) & 31);
-                      acc.x += __uint_as_float(v[u].x) * wu; acc.y += __uint_as_float(v[u].y) * wu;
-                      acc.z += __uint_as_float(v[u].z) * wu; acc.w += __uint_as_float(v[u].w) * wu;
+                    for (int u = 0; u < 5; ++u) add(u);
+                    if (more) {
+#pragma unroll
+                      for (int u = 5; u < 10; ++u) add(u);
                     }
                   }
                 }
+                if (per == 2) {
+                  acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
+                  acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 16); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 16);
+                }
                 L = warp_sum(L);
-                if (dd < hd) {
+                if (dd < hd && (per == 1 || sub == 0)) {
                   bf16* orow = P.o + (size_t)(a.off + q / Gq) * P.Hq * hd + (size_t)(kvh * Gq + q % Gq) * hd + dd;
                   const float inv = 1.0f / L;
                   const __nv_bfloat162 h01 = __floats2bfloat162_rn(acc.x * inv, acc.y * inv), h23 = __floats2bfloat162_rn(acc.z * inv, acc.w * inv);
