@@ -40,7 +40,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 constexpr int MK_MAX_ROWS = 64;          // rows per call the persistent kernel handles
 constexpr int MK_TBOX_SLOTS = MK_MAX_ROWS / 16;
-constexpr int MK_PROG_SLOTS = MK_TBOX_SLOTS * 2;   // one program per (row box, k-blocks per stage)
+constexpr int MK_PROG_SLOTS = MK_TBOX_SLOTS * 4;   // one program per (row box, k-blocks per stage, rotation phase or not)
 
 struct DevModel {
   float* rope_inv = nullptr;     // device: theta^(-2i/hd), i < hd/2
@@ -51,7 +51,7 @@ struct DevModel {
   bool prog_built[MK_PROG_SLOTS] = {};
   char* prog_base = nullptr;     // device: per t_box slot, phases followed by tensor maps
   size_t prog_slot_bytes = 0, prog_maps_off = 0;
-  int n_phases = 0;
+  int n_phases[MK_PROG_SLOTS] = {};
   std::vector<LayerMaps> maps;   // tensor maps of the bf16 weight matrices (tensor-core path)
   CUtensorMap head_map{};
   stairs_model m{};
@@ -629,6 +629,15 @@ int gemm_ctas(const stairs_ctx* ctx, int tiles, int K) {
   return best_ge;
 }
 
+// Rotation by the QKV projection's epilogue where tiles cut heads (see Phase::cross): every tile has to be parked, so no CTA's range
+// may hold more than one.
+bool cross_possible(const stairs_ctx* ctx, const stairs_model& m) {
+  if (m.pos == 0 || m.head_dim == 64 || m.head_dim == 128) return false;
+  const int nq = m.n_heads * m.head_dim, nkv = m.n_kv_heads * m.head_dim, tiles = (nq + tc::BM - 1) / tc::BM + 2 * ((nkv + tc::BM - 1) / tc::BM);
+  const int units = tiles * (((m.d_model + tc::BK - 1) / tc::BK + mk::RANGE_UNIT_KB - 1) / mk::RANGE_UNIT_KB);
+  return tiles < std::min(gemm_ctas(ctx, tiles, m.d_model), units);
+}
+
 // Do the CTAs of a split tile share its rows in this call, or does one finish them all (both give the same bits)?  Shared, a
 // phase ends about 1.2 us after its sums are parked where no warp has more than one row, and 1.9 us later for every further row
 // of a warp; finished by one CTA, about 2.5 us per 16 rows.
@@ -647,13 +656,16 @@ int share_rows(const stairs_ctx* ctx, const stairs_model& m, int T) {
   gemm((m.d_model + tc::BM - 1) / tc::BM, nq);
   gemm(m.act == 1 ? (m.d_ff + 63) / 64 : (m.d_ff + tc::BM - 1) / tc::BM, m.d_model);
   gemm((m.d_model + tc::BM - 1) / tc::BM, m.d_ff);
+  if (cross_possible(ctx, m)) one += 3.0;   // (the rotation's phase)
   return shared < one ? 1 : 0;
 }
 
-int build_program(stairs_ctx* ctx, DevModel& M, int t_box, int kps) {
+int program_slot(int t_box, int kps, int cross) { return ((t_box / 16 - 1) * 2 + (kps - 1)) * 2 + cross; }
+
+int build_program(stairs_ctx* ctx, DevModel& M, int t_box, int kps, int cross) {
   const stairs_model& m = M.m;
   const Layout& L = ctx->lay;
-  const int slot = (t_box / 16 - 1) * 2 + (kps - 1);
+  const int slot = program_slot(t_box, kps, cross);
   const int d = m.d_model, nq = m.n_heads * m.head_dim, nkv = m.n_kv_heads * m.head_dim, nqkv = nq + 2 * nkv, F = m.d_ff;
   char* ws = ctx->ws;
   std::vector<CUtensorMap> maps((size_t)9 * m.n_layers + 4);
@@ -729,13 +741,14 @@ int build_program(stairs_ctx* ctx, DevModel& M, int t_box, int kps) {
     const stairs_layer_w& w = M.layers[l];
     const int b = 7 * l;
     const int r3[3] = {nq, nkv, nkv};
-    const bool in_epilogue = m.pos == 0 || m.head_dim == 64 || m.head_dim == 128;
+    const bool in_epilogue = m.pos == 0 || m.head_dim == 64 || m.head_dim == 128 || cross;
     {
       mk::Phase& p = gemm(l, b + 0, b + 1, b + 2, 3, r3, false, i_h, d, tc::TC_STORE_F32, ws + L.qkv, nqkv);
       p.norm_in = 1; p.u = aux_ptr(l, 0); p.c = aux_ptr(l, 1);
       // q to the query buffer, k and v (fp16) to this layer's cache rows: in the epilogue where a
-      // rotation pair sits in one thread (head size 64 or 128, or no rotation), else in a phase of its own
+      // rotation pair sits in one tile (head size 64 or 128, or no rotation) or can be had from two, else in a phase of its own
       p.qkv_prep = in_epilogue ? 1 : 0;
+      p.cross = cross;
       p.kc = M.kpool + (size_t)l * M.kv_layer_bytes; p.vc = M.vpool + (size_t)l * M.kv_layer_bytes;
     }
     if (!in_epilogue) simple(mk::PH_PREP, l, nullptr, M.kpool + (size_t)l * M.kv_layer_bytes, M.vpool + (size_t)l * M.kv_layer_bytes);
@@ -767,7 +780,7 @@ int build_program(stairs_ctx* ctx, DevModel& M, int t_box, int kps) {
   for (const mk::Phase& p : ph)
     if (p.kind == mk::PH_GEMM && (p.n_tiles > TC_COUNTERS || (long long)p.n_tiles * p.kblocks * TC_GRID_MAX >= (1ll << 32)))
       return fail(ctx, STAIRS_EUNSUPPORTED, "too many tiles for the split bookkeeping");
-  M.n_phases = (int)ph.size();
+  M.n_phases[slot] = (int)ph.size();
   char* base = M.prog_base + (size_t)slot * M.prog_slot_bytes;
   if (ph.size() * sizeof(mk::Phase) > M.prog_maps_off || M.prog_maps_off + maps.size() * sizeof(CUtensorMap) > M.prog_slot_bytes)
     return fail(ctx, STAIRS_ENOSPC, "program area too small");
@@ -823,9 +836,10 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
       return fail(ctx, STAIRS_ENOSPC, "attention scratch holds %lld units, this call may need %lld", units_avail, need);
   }
   const MkPlan pl = mk_plan(ctx, m, t_box, q_rows_call, tc_call);
-  const int slot = (t_box / 16 - 1) * 2 + (pl.kps - 1);
+  const int share = share_rows(ctx, m, T), cross = share && cross_possible(ctx, m) ? 1 : 0;
+  const int slot = program_slot(t_box, pl.kps, cross);
   if (!M.prog_built[slot]) {
-    int rc = build_program(ctx, M, t_box, pl.kps);
+    int rc = build_program(ctx, M, t_box, pl.kps, cross);
     if (rc) return rc;
   }
   mk::Params P;
@@ -833,7 +847,7 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
   char* base = M.prog_base + (size_t)slot * M.prog_slot_bytes;
   // A prefill ends with the last layer's keys and values (filed by its QKV projection, or the phase after it): no attention,
   // O projection, MLP, LM head or accept.
-  const int n_run = c.skip_head ? M.n_phases - 6 : M.n_phases;
+  const int n_run = c.skip_head ? M.n_phases[slot] - 6 : M.n_phases[slot];
   P.phases = reinterpret_cast<const mk::Phase*>(base); P.n_phases = n_run;
   P.maps = reinterpret_cast<const CUtensorMap*>(base + M.prog_maps_off);
   P.T = T; P.t_box = t_box;
@@ -871,7 +885,7 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
   P.trace = (ctx->profile && &M == &ctx->target) ? reinterpret_cast<unsigned long long*>(ws + L.mk_trace) : nullptr;
   const int grid = std::min(ctx->sm_count, TC_GRID_MAX);
   void* args[] = {&P};
-  CK(cudaLaunchCooperativeKernel(mk::forward_fn(m, P.att_tma, P.att_tc, T, share_rows(ctx, m, T)), dim3(grid), dim3(mk::MK_THREADS), args,
+  CK(cudaLaunchCooperativeKernel(mk::forward_fn(m, P.att_tma, P.att_tc, T, share), dim3(grid), dim3(mk::MK_THREADS), args,
                                  mk::smem_bytes(t_box, P.stages, m.head_dim, P.att_dbl, P.kps, P.att_tma, P.att_nbuf, P.att_q_rows), ctx->stream));
   ctx->bar_base += (unsigned long long)n_run * grid;
   ctx->launches++;

@@ -76,6 +76,7 @@ struct Phase {
   int ge_max;                // CTAs this GEMM is cut over (0 = all): few tiles are not worth a wide split
   int norm_in;
   int qkv_prep;              // QKV projection: the epilogue rotates, converts and files q, k, v (see epilogue)
+  int cross;                 // ... of heads that are cut by tiles: a rotation's partner columns may be a neighbouring tile's (shared rows only)
   const float* u; const float* c;
   const float* next_g;
   // PH_EMBED
@@ -164,6 +165,8 @@ struct Spec {
   static __device__ __forceinline__ bool tc(const Params& P) { return ATT == 3 ? P.att_tc != 0 : ATT == 1; }
   static __device__ __forceinline__ bool tma(const Params& P) { return ATT == 3 ? P.att_tma != 0 : true; }
   static __device__ __forceinline__ int qblk(const Params& P) { return ATT == 3 ? P.att_qblk : ATT == 1 ? ATT_QBLK_TC : ATT_QBLK; }
+  static __device__ __forceinline__ constexpr bool may_cross() { return SHARE && FAM != 1 && (HD == 0 || HD % 64 != 0); }
+  static __device__ __forceinline__ bool cross(const Phase& p) { return may_cross() && p.cross; }
   static __device__ __forceinline__ bool prep(const Params& P) { return HD % 64 != 0 || HD == 0; }             // may the program hold PH_PREP phases?
 };
 
@@ -1780,7 +1783,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           float x0 = __ldcg(row + i), x1 = __ldcg(row + i + half);
           if (S::rope(P) && hs < P.Hq + P.Hkv) {
             const float cs = __ldcg(P.rope_cs + (size_t)t * half + i), sn = __ldcg(P.rope_sn + (size_t)t * half + i);
-            const float r0 = x0 * cs - x1 * sn, r1 = x1 * cs + x0 * sn;
+            const float r0 = rotated(x0, -x1, cs, sn), r1 = rotated(x1, x0, cs, sn);
             x0 = r0; x1 = r1;
           }
           if (hs < P.Hq) {
@@ -1841,7 +1844,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
         int wt = 0, wt_end = 0;
         if (gemm_worked) {
           const int tf = kb / p.kblocks, tl = (kb_end - 1) / p.kblocks;
-          const bool cut_a = kb != tf * p.kblocks, cut_b = kb_end != (tl + 1) * p.kblocks && (tl != tf || !cut_a);
+          // (with partners in neighbouring tiles every tile is parked, also one that is a CTA's whole range; none is longer then)
+          const bool cut_a = kb != tf * p.kblocks, cut_b = (kb_end != (tl + 1) * p.kblocks || S::cross(p)) && (tl != tf || !cut_a);
           wt = cut_a ? tf + 1 : tf; wt_end = cut_b ? tl : tl + 1;
           const unsigned units = (unsigned)(p.n_tiles * p.upt), ge = (unsigned)kr.ge;
 #pragma unroll 1
@@ -1882,7 +1886,10 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
             unsigned c0 = 0, cn = 0;
             float4 k1 = make_float4(0.f, 0.f, 0.f, 0.f), k2 = k1, cs = k1, sn = k1;   // residual and gain, or LayerNorm's u and c; rotation
             float4 st0 = k1, st1 = k1;                   // statistics of this row's tiles lane, lane + 32
-            bool on = false;
+            bool on = false, plow = false;
+            unsigned pc0 = 0, pcn = 0;                   // rotation partner in another place: its tile's CTAs, its column there
+            int pcol = 0, tab = 0;
+            float4 pu, pv;
             if (j < jobs) {
               const Split q = j < nb ? sb : sa;
               row = whole ? cw + j : q.r0 + (j < nb ? j : j - nb);
@@ -1914,8 +1921,18 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                   for (int e = 0; e < 4; ++e) if (col + e < ncols) { u[e] = __ldg(p.u + n + e); c[e] = __ldg(p.c + n + e); }
                 } else if (on) { k1 = __ldg(reinterpret_cast<const float4*>(p.u + n)); k2 = __ldg(reinterpret_cast<const float4*>(p.c + n)); }
               }
+              if (S::cross(p) && src < 2) {
+                // the columns half a head away: their tile's slots
+                const int hd = S::hd(P), gc = dcol + col, lower = gc % hd < hd / 2, pc = lower ? gc + hd / 2 : gc - hd / 2;
+                const unsigned units = (unsigned)(p.n_tiles * p.upt), ge = (unsigned)kr.ge, pt = (unsigned)(tile + pc / BM - dcol / BM);
+                pc0 = ((pt * p.upt + 1u) * ge - 1u) / units;
+                pcn = on ? ((pt + 1u) * p.upt * ge - 1u) / units - pc0 + 1u : 0u;
+                pcol = pc % BM; plow = lower != 0;
+                tab = gc % (hd / 2);
+                if (S::shifted(p) && on) { pu = __ldg(reinterpret_cast<const float4*>(p.u + n0 - dcol + pc)); pv = __ldg(reinterpret_cast<const float4*>(p.c + n0 - dcol + pc)); }
+              }
               if (p.qkv_prep && S::rope(P) && src < 2 && on) {
-                const int i4 = lane % (S::hd(P) / 8) * 4;
+                const int i4 = S::cross(p) ? tab : lane % (S::hd(P) / 8) * 4;
                 cs = __ldcg(reinterpret_cast<const float4*>(P.rope_cs + (size_t)row * (S::hd(P) / 2) + i4));
                 sn = __ldcg(reinterpret_cast<const float4*>(P.rope_sn + (size_t)row * (S::hd(P) / 2) + i4));
               }
@@ -1971,11 +1988,18 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
               rs = row_rstd(S::layer_norm(P), m2, n, mean, P.d, P.eps);
             }
             if (tra) tra[1] = globaltimer_ns();
-            float4 v;
+            float4 v, ov;
             if (whole) v = *reinterpret_cast<const float4*>(vt + j * VT_LD + col);
             else {
               v = make_float4(0.f, 0.f, 0.f, 0.f);
               const size_t step = (size_t)2 * tb * BM;
+              const bool other = S::cross(p) && S::rope(P) && src < 2;
+              const float* opart = slot_of(pset, pc0, false) + (size_t)row * BM + pcol;
+              uint4 os[4];   // the partner's first four segments, requested ahead of this column's
+              if (other) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) if (u < pcn) os[u] = ld_relaxed_u4(opart + u * step + (u == 0 ? step / 2 : 0));
+              }
               const float* part = slot_of(pset, c0, false) + (size_t)row * BM + (on ? col : 0);   // (segment 0 is in its CTA's second slot)
               uint4 s[8];
               // The segments' partial sums, eight in flight together, added in k order.  A slot element reads PARTIAL_EMPTY until its
@@ -2009,6 +2033,34 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
                   if (c + u < cn) { v.x += __uint_as_float(s[u].x); v.y += __uint_as_float(s[u].y); v.z += __uint_as_float(s[u].z); v.w += __uint_as_float(s[u].w); }
+              }
+              if (other) {
+                // the partner's sums, four segments at a time (its tile's CTAs differ between lanes), and its folded normalisation
+                ov = make_float4(0.f, 0.f, 0.f, 0.f);
+                long long t0 = 0;
+#pragma unroll 1
+                for (unsigned c = 0; __any_sync(0xffffffffu, c < pcn);) {
+                  uint32_t mx = 0u;
+#pragma unroll
+                  for (int u = 0; u < 4; ++u) if (c + u < pcn) mx = max(max(mx, max(os[u].x, os[u].y)), max(os[u].z, os[u].w));
+                  bool quit = false;
+                  if (__any_sync(0xffffffffu, mx == PARTIAL_EMPTY)) {
+                    if (t0 == 0) t0 = clock64();
+                    if (lane == 0) quit = W.poll_abort(t0);
+                    quit = __any_sync(0xffffffffu, quit);
+                    if (quit && lane == 0) W.note(3u, (unsigned)ph, (unsigned)cta, pcn, (unsigned)tile);
+                  } else {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                      if (c + u < pcn) { ov.x += __uint_as_float(os[u].x); ov.y += __uint_as_float(os[u].y); ov.z += __uint_as_float(os[u].z); ov.w += __uint_as_float(os[u].w); }
+                    c += 4;
+                  }
+                  if (quit) break;
+#pragma unroll
+                  for (int u = 0; u < 4; ++u) if (c + u < pcn) os[u] = ld_relaxed_u4(opart + (c + u) * step + (c + u == 0 ? step / 2 : 0));
+                }
+                if (S::shifted(p)) { ov.x = normed(ov.x, mu, rs, pu.x, pv.x); ov.y = normed(ov.y, mu, rs, pu.y, pv.y); ov.z = normed(ov.z, mu, rs, pu.z, pv.z); ov.w = normed(ov.w, mu, rs, pu.w, pv.w); }
+                else { ov.x *= rs; ov.y *= rs; ov.z *= rs; ov.w *= rs; }
               }
               if (tra) tra[2] = globaltimer_ns();
             }
@@ -2064,13 +2116,15 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
               if (lane == 0 && key) atomicMax(P.keys + row, key);
             } else if (p.qkv_prep) {
               // q: rotate, scale by 1/sqrt(hd), fp16, to the query buffer; k: rotate, fp16, to its row of the cache; v: fp16
-              // to the cache.  The rotation pairs column i with i + hd/2 of a head, hd/8 lanes away (head size 64 or 128).
+              // to the cache.  The rotation pairs column i with i + hd/2 of a head: hd/8 lanes away (head size 64 or 128), or, of heads
+              // that tiles cut, summed beside this column's (a phase of its own for it took 3.0 us a layer: 3B, 5 rows 1903 us, so 1875).
               const int hd = S::hd(P);
               if (S::rope(P) && src < 2) {
-                const bool lower = lane % (hd / 4) < hd / 8;
+                const bool lower = S::cross(p) ? plow : lane % (hd / 4) < hd / 8;
                 const int other = lower ? lane + hd / 8 : lane - hd / 8;
-                float4 o = make_float4(__shfl_sync(0xffffffffu, v.x, other), __shfl_sync(0xffffffffu, v.y, other),
-                                       __shfl_sync(0xffffffffu, v.z, other), __shfl_sync(0xffffffffu, v.w, other));
+                float4 o = ov;
+                if (!S::cross(p)) o = make_float4(__shfl_sync(0xffffffffu, v.x, other), __shfl_sync(0xffffffffu, v.y, other),
+                                                  __shfl_sync(0xffffffffu, v.z, other), __shfl_sync(0xffffffffu, v.w, other));
                 if (lower) o = make_float4(-o.x, -o.y, -o.z, -o.w);
                 v = make_float4(rotated(v.x, o.x, cs.x, sn.x), rotated(v.y, o.y, cs.y, sn.y), rotated(v.z, o.z, cs.z, sn.z), rotated(v.w, o.w, cs.w, sn.w));
               }
@@ -2515,6 +2569,13 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
       if (tracing) tr[2] = globaltimer_ns();
       waited = false;
       if (p.kind == PH_GEMM) ++gph;
+    }
+    if (ok && S::may_cross() && P.mode == CALL_PREFILL) {
+      // such a pass ends with a QKV projection, whose parked sums neighbouring tiles' CTAs read too: they are all done with them
+      if (et == 0) ctl->bcast = W.wait_grid(bar_count, P.bar_base + (unsigned long long)P.n_phases * G) ? 1 : 0;
+      __syncwarp();
+      epi_bar_sync();
+      ok = ctl->bcast != 0;
     }
     if (ok) { empty_pending((gph & 1) ^ 1); if (aph > 0) empty_own_states((aph - 1) & 1); }   // (after an abort the host empties every slot)
   }
