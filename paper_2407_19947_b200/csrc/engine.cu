@@ -613,21 +613,23 @@ MkPlan mk_plan(const stairs_ctx* ctx, const stairs_model& m, int t_box, int q_ro
 
 
 // How many CTAs to cut a GEMM of the persistent kernel over: more CTAs stream faster, but every tile is then finished from more
-// partial tiles.  Model: stream time at ~44 GB/s per SM plus ~1.6 us per batch of four partials.  (Must not depend on the row
-// box: see RANGE_UNIT_KB.)
+// partial tiles.  Model: the longest range's units (two k-blocks) at ~44 GB/s per SM; 1.4 us and 1.6 us per batch of eight partials
+// where tiles are split, 0.7 us more where CTAs do not divide evenly among tiles (a CTA then has parts of two).  (Must not depend on
+// the row box: see RANGE_UNIT_KB.)
 int gemm_ctas(const stairs_ctx* ctx, int tiles, int K) {
-  const int grid = std::min(ctx->sm_count, TC_GRID_MAX);
-  const double bytes = (double)tiles * ((K + tc::BK - 1) / tc::BK) * tc::A_STAGE_BYTES;
+  const int grid = std::min(ctx->sm_count, TC_GRID_MAX), units = tiles * (((K + tc::BK - 1) / tc::BK + mk::RANGE_UNIT_KB - 1) / mk::RANGE_UNIT_KB);
   double best = 1e30; int best_ge = grid;
-  for (int s2 = 1; s2 <= 64; s2 *= 2) {
+  for (int s2 = 1; s2 <= 64; ++s2) {
     const int ge = std::min(grid, tiles * s2);
     const double seg = (double)ge / tiles + (ge % tiles ? 1.0 : 0.0);
-    const double t_us = bytes / (ge * 44.0e3) + (seg > 1.0 ? std::ceil(seg / 4.0) * 1.6 + 2.0 : 0.0);
+    const double t_us = ((units + ge - 1) / ge) * (mk::RANGE_UNIT_KB * tc::A_STAGE_BYTES / 44.0e3) + (seg > 1.0 ? std::ceil(seg / 8.0) * 1.6 + 1.4 + (ge % tiles ? 0.7 : 0.0) : 0.0);
     if (t_us < best - 1e-9) { best = t_us; best_ge = ge; }
     if (ge == grid) break;
   }
   return best_ge;
 }
+
+int program_slot(int t_box, int kps, int cross) { return ((t_box / 16 - 1) * 2 + (kps - 1)) * 2 + cross; }
 
 // Rotation by the QKV projection's epilogue where tiles cut heads (see Phase::cross): every tile has to be parked, so no CTA's range
 // may hold more than one.
@@ -638,29 +640,27 @@ bool cross_possible(const stairs_ctx* ctx, const stairs_model& m) {
   return tiles < std::min(gemm_ctas(ctx, tiles, m.d_model), units);
 }
 
-// Do the CTAs of a split tile share its rows in this call, or does one finish them all (both give the same bits)?  Shared, a
-// phase ends about 1.2 us after its sums are parked where no warp has more than one row, and 1.9 us later for every further row
-// of a warp; finished by one CTA, about 2.5 us per 16 rows.
+// Do the CTAs of a split tile share its rows in this call, or does one finish them all (both give the same bits)?  The difference
+// per layer (us), fitted to both forms of three models at 1 to 64 rows: shared, a GEMM phase ends 1.25 us sooner where ranges are
+// short (0.5 where they stream for long, and the slowest CTA counts), 1.2 later for every further row of a warp (3.0 where tiles
+// are more than CTAs: whole ones come on top), and finished by one CTA 1.7 later for every further 16 rows.  0.4B: shared up to 64 rows,
+// 0.82 of the other form at 64; 3B: up to 4, 0.97; 7B: up to 4, 0.98 (nine rows, shared: 1.06).
 int share_rows(const stairs_ctx* ctx, const stairs_model& m, int T) {
   if (ctx->share_force) return ctx->share_force - 1;
-  double shared = 0, one = 0;
+  double later = cross_possible(ctx, m) ? -1.0 : 0.0;   // (the rotation's phase is saved, the projection's gets longer)
   auto gemm = [&](int tiles, int K) {
     const int units = tiles * (((K + tc::BK - 1) / tc::BK + mk::RANGE_UNIT_KB - 1) / mk::RANGE_UNIT_KB), ge = std::min(gemm_ctas(ctx, tiles, K), units);
     const int seg = ge / tiles;   // CTAs per tile at least; a CTA has parts of two tiles unless they divide evenly
-    const int rows = seg >= 1 && ge > tiles ? (ge % tiles ? 2 : 1) * ((T + seg - 1) / seg) : T;
-    shared += 1.2 + 1.9 * ((rows + 3) / 4 - 1);
-    one += 2.5 * ((T + 15) / 16);
+    const int rows = ge > tiles ? (ge % tiles ? 2 : 1) * ((T + seg - 1) / seg) : (T * tiles + ge - 1) / ge, rounds = (rows + 3) / 4;
+    later += (units <= 4 * ge ? -1.25 : -0.5) + (tiles >= ge ? 3.0 : 1.2) * (rounds - 1) - 1.7 * ((T + 15) / 16 - 1);
   };
   const int nq = m.n_heads * m.head_dim, nkv = m.n_kv_heads * m.head_dim;
   gemm((nq + tc::BM - 1) / tc::BM + 2 * ((nkv + tc::BM - 1) / tc::BM), m.d_model);
   gemm((m.d_model + tc::BM - 1) / tc::BM, nq);
   gemm(m.act == 1 ? (m.d_ff + 63) / 64 : (m.d_ff + tc::BM - 1) / tc::BM, m.d_model);
   gemm((m.d_model + tc::BM - 1) / tc::BM, m.d_ff);
-  if (cross_possible(ctx, m)) one += 3.0;   // (the rotation's phase)
-  return shared < one ? 1 : 0;
+  return later < 0 ? 1 : 0;
 }
-
-int program_slot(int t_box, int kps, int cross) { return ((t_box / 16 - 1) * 2 + (kps - 1)) * 2 + cross; }
 
 int build_program(stairs_ctx* ctx, DevModel& M, int t_box, int kps, int cross) {
   const stairs_model& m = M.m;

@@ -1649,15 +1649,15 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           u0 += a.units; g0 += P.Hkv * a.n_qblk;
         }
         // Requests whose positions were split over several units: merge the parked states of every
-        // (kv head, query).  One warp per item, or on the mma.sync path, where items are few, per 64 columns of one (head sizes 64 and
-        // 128: half a warp per range, up to twenty ranges in one round trip instead of eight: 7B, 9 rows, 18 ranges 0.6 % of a call,
+        // (kv head, query).  One warp per item, or, where items are few, per 64 columns of one (head sizes 64 and
+        // 128, mma.sync path: half a warp per range, up to twenty ranges in one round trip instead of eight: 7B, 9 rows, 18 ranges 0.6 % of a call,
         // 0.4B, 9 rows, nine ranges 1.4 %; four layers of 7B with 144 query rows a head 1 % slower so); each lane
         // owns 4 consecutive elements of head_dim, so every partial is one 16-byte load per lane.  The states come
         // from other CTAs' units of this same phase: a word reads PARTIAL_EMPTY until it has been
         // stored, and the warp repeats its loads (bounded) until none does.
         if (ok) {
           const int hd = S::hd(P), Gq = P.Hq / P.Hkv;
-          const bool pairs = hd % 64 == 0 && !S::tc(P);
+          const bool pairs = hd % 64 == 0 && !S::tc(P) && (hd == 64 || P.Hq * P.T <= 2 * G);   // (all halves of items at once)
           const int halves = pairs ? hd / 64 : 1, sub = pairs ? lane >> 4 : 0, per = pairs ? 2 : 1;   // parts of an item; ranges per load
           const float* set_base = P.attn_part + (size_t)(aph & 1) * P.attn_set_stride;
           int u0c = 0, item0 = 0;
@@ -1709,7 +1709,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                 }
                 M = warp_max(M);
                 float L = 0.f;
-                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), odd = acc;
                 for (int rb = 0; rb < nr && !gave_up; rb += 32) {
                   float mu = m0, lu = l0;
                   if (rb != 0) state_of(rb + lane, mu, lu);
@@ -1723,8 +1723,9 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     auto load = [&](int u) { v[u] = (g0 + u * per + sub < nb && dd < hd) ? ld_relaxed_u4(at + (size_t)(u * per) * stride) : make_uint4(0u, 0u, 0u, 0u); };
                     auto add = [&](int u) {
                       const float wu = __shfl_sync(0xffffffffu, wgt, (g0 + u * per + sub) & 31);
-                      acc.x += __uint_as_float(v[u].x) * wu; acc.y += __uint_as_float(v[u].y) * wu;
-                      acc.z += __uint_as_float(v[u].z) * wu; acc.w += __uint_as_float(v[u].w) * wu;
+                      float4& to = hd % 64 == 0 && per == 1 && (u & 1) ? odd : acc;   // (even and odd ranges apart, as where two share a load: the same bits)
+                      to.x += __uint_as_float(v[u].x) * wu; to.y += __uint_as_float(v[u].y) * wu;
+                      to.z += __uint_as_float(v[u].z) * wu; to.w += __uint_as_float(v[u].w) * wu;
                     };
                     while (true) {
                       uint32_t mx = 0u;
@@ -1749,6 +1750,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     }
                   }
                 }
+                if (hd % 64 == 0 && per == 1) { acc.x += odd.x; acc.y += odd.y; acc.z += odd.z; acc.w += odd.w; }
                 if (per == 2) {
                   acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
                   acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 16); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 16);
