@@ -1027,7 +1027,7 @@ int mid_cluster(const stairs_ctx* ctx, int n_tiles, int kblocks, int TN, int x_b
     if (fit <= 0 || c > kblocks) continue;
     const int clusters = std::min(fit, pairs), rounds = (pairs + clusters - 1) / clusters;
     const double kb = std::max((TN + x_box) * 128.0 / 100e3, TN * 256.0 * clusters * c / 6.3e6);
-    const double chain = ((kblocks + c - 1) / c) * kb, epi = (c > 1 ? 3.0 : 1.0) + 0.03 * x_box / c;
+    const double chain = ((kblocks + c - 1) / c) * kb, epi = (c > 1 ? 5.0 : 1.0) + 0.03 * x_box / c;
     const double us = chain + (rounds - 1) * std::max(chain, epi) + epi;
     if (us < best_us - 1e-9) { best_us = us; best = c; }
   }
