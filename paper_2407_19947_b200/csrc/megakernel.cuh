@@ -2213,7 +2213,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           const int seg_end = tile_end < kb_end ? tile_end : kb_end;
           // The CTA that owns a tile's first k-block finishes the tile; a CTA whose segment starts
           // inside a tile (always the first segment of its range, so at most one per phase) parks
-          // the partial sums in its slot and raises its flag.  The finisher's segment is the
+          // the partial sums in its slot.  The finisher's segment is the
           // last thing its range holds, so it reaches the tile when the others are done or
           // nearly so, and it adds their partials to its own in k order - a fixed order: results
           // do not depend on timing.
