@@ -87,3 +87,44 @@ def test_static_accept_equals_torch_argmax(vocab, ld, ks):
         miss = [r for r in range(k) if d[i, r] != tt[i, r]]
         assert int(al[i]) == (miss[0] if miss else k)
         row += k + 1
+
+
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("n_req", [39, 40, 64])      # on both sides of the calls that are started behind the previous kernel
+def test_static_accept_waits_for_the_kernels_before_it(n_req, captured):
+    # the logits and drafts of every call are written by kernels right before it, and its results read right behind it
+    from paper_2407_19947_b200 import build, stairs
+    build.build()
+    vocab, k, calls = 16500, 3, 12
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n_req)
+    src = torch.randn((calls, n_req * (k + 1), vocab), generator=g, device="cuda")
+    want = src.argmax(dim=2).view(calls, n_req, k + 1).to(torch.int32)
+    logits, draft = torch.empty_like(src[0]), torch.zeros((n_req, k), dtype=torch.int32, device="cuda")
+    got_t, got_a = torch.zeros_like(want), torch.zeros((calls, n_req), dtype=torch.int32, device="cuda")
+
+    def one(i, stream=None):
+        logits.copy_(src[i])
+        draft.copy_(want[i, :, :k])
+        draft[:, i % k] += 1                          # the first mismatch of every request
+        tt, al = stairs.accept_static(logits, [k] * n_req, draft, k, stream=stream)
+        got_t[i].copy_(tt)
+        got_a[i].copy_(al)
+
+    one(0)
+    torch.cuda.synchronize()
+    if captured:
+        graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=side):
+            for i in range(calls):
+                one(i, side)
+        for _ in range(3):
+            got_t.zero_()
+            got_a.zero_()
+            graph.replay()
+    else:
+        for i in range(calls):
+            one(i)
+    torch.cuda.synchronize()
+    assert torch.equal(got_t, want)
+    assert torch.equal(got_a, (torch.arange(calls, device="cuda", dtype=torch.int32) % k).view(-1, 1).expand(calls, n_req))
