@@ -1649,16 +1649,16 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           u0 += a.units; g0 += P.Hkv * a.n_qblk;
         }
         // Requests whose positions were split over several units: merge the parked states of every
-        // (kv head, query).  One warp per item, or, where items are few, per 64 columns of one (head sizes 64 and
-        // 128, mma.sync path: half a warp per range, up to twenty ranges in one round trip instead of eight: 7B, 9 rows, 18 ranges 0.6 % of a call,
-        // 0.4B, 9 rows, nine ranges 1.4 %; four layers of 7B with 144 query rows a head 1 % slower so); each lane
+        // (kv head, query), one warp per item; at head size 64 (mma.sync path) half a warp takes a range, up to twenty ranges in one round
+        // trip (0.4B, 9 rows, nine ranges: 1.4 % of a call).  Heads of 128 by halves of an item, chosen at run time, made the kernel's
+        // text longer: 16 layers of 7B, 2 x 6 rows after 300 1356 us so and 1349 now, 6 rows after 100 1330 and 1322.  Each lane
         // owns 4 consecutive elements of head_dim, so every partial is one 16-byte load per lane.  The states come
         // from other CTAs' units of this same phase: a word reads PARTIAL_EMPTY until it has been
         // stored, and the warp repeats its loads (bounded) until none does.
         if (ok) {
           const int hd = S::hd(P), Gq = P.Hq / P.Hkv;
-          const bool pairs = hd % 64 == 0 && !S::tc(P) && (hd == 64 || P.Hq * P.T <= 2 * G);   // (all halves of items at once)
-          const int halves = pairs ? hd / 64 : 1, sub = pairs ? lane >> 4 : 0, per = pairs ? 2 : 1;   // parts of an item; ranges per load
+          const bool pairs = hd == 64 && !S::tc(P);
+          const int sub = pairs ? lane >> 4 : 0, per = pairs ? 2 : 1;   // ranges per load
           const float* set_base = P.attn_part + (size_t)(aph & 1) * P.attn_set_stride;
           int u0c = 0, item0 = 0;
           bool gave_up = false;
@@ -1674,18 +1674,18 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           for (int i = 0; i < n_req; ++i) {
             const AttnReq a = ctl->areq[i];
             if (a.n_ranges > 1) {
-              const int Q = a.R * Gq, items = P.Hkv * Q * halves;
+              const int Q = a.R * Gq, items = P.Hkv * Q;
               int it = ((cta * 4 + quad) - item0) % (G * 4);
               if (it < 0) it += G * 4;
               for (; it < items && !gave_up; it += G * 4) {
-                const int it1 = it / halves, kvh = it1 / Q, q = it1 % Q, qblk = q / S::qblk(P), ql = q % S::qblk(P);
+                const int kvh = it / Q, q = it % Q, qblk = q / S::qblk(P), ql = q % S::qblk(P);
                 const int first_slot = u0c + (kvh * a.n_ranges) * a.n_qblk + qblk;
                 const size_t stride = (size_t)a.n_qblk * S::qblk(P) * (hd + 4);
                 const float* base = set_base + ((size_t)first_slot * S::qblk(P) + ql) * (hd + 4);
                 // (max, sum) of range lane, lane + 32, ...: one load round for up to 32 ranges, then
                 // the ranges' output vectors five or ten loads at a time; weights travel by shuffle and
                 // the accumulation is in range order (of even and odd ranges)
-                const int nr = a.n_ranges, dd = per == 2 ? (it % halves) * 64 + (lane & 15) * 4 : lane * 4;
+                const int nr = a.n_ranges, dd = per == 2 ? (lane & 15) * 4 : lane * 4;
                 long long t0 = 0;
                 bool timing = false;
                 auto state_of = [&](int r, float& mu, float& lu) {   // all lanes call it together
@@ -1723,7 +1723,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     auto load = [&](int u) { v[u] = (g0 + u * per + sub < nb && dd < hd) ? ld_relaxed_u4(at + (size_t)(u * per) * stride) : make_uint4(0u, 0u, 0u, 0u); };
                     auto add = [&](int u) {
                       const float wu = __shfl_sync(0xffffffffu, wgt, (g0 + u * per + sub) & 31);
-                      float4& to = hd % 64 == 0 && per == 1 && (u & 1) ? odd : acc;   // (even and odd ranges apart, as where two share a load: the same bits)
+                      float4& to = hd == 64 && per == 1 && (u & 1) ? odd : acc;   // (even and odd ranges apart, as where two share a load: the same bits)
                       to.x += __uint_as_float(v[u].x) * wu; to.y += __uint_as_float(v[u].y) * wu;
                       to.z += __uint_as_float(v[u].z) * wu; to.w += __uint_as_float(v[u].w) * wu;
                     };
@@ -1750,7 +1750,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     }
                   }
                 }
-                if (hd % 64 == 0 && per == 1) { acc.x += odd.x; acc.y += odd.y; acc.z += odd.z; acc.w += odd.w; }
+                if (hd == 64 && per == 1) { acc.x += odd.x; acc.y += odd.y; acc.z += odd.z; acc.w += odd.w; }
                 if (per == 2) {
                   acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
                   acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 16); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 16);
