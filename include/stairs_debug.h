@@ -24,7 +24,9 @@ int stairs_profile_read(stairs_ctx *ctx, float *gemm_ms, int32_t *gemm_launches,
  * 3 attention output o, 4 MLP activation ff, 5 argmax keys u64, 6 per-phase timestamps of the
  * persistent kernel, u64 ns [2 CTAs][phases][8 stamps: start, work done, arrived, prologue done, first tile ready, first MMA, last MMA, first activation load], written while
  * profiling is on; 7 the persistent kernel's split-tile partial-sum slots and 8 its parked attention
- * states, both u32 words that all read 0xffffffff ("empty") between calls). */
+ * states, both u32 words that all read 0xffffffff ("empty") between calls; row statistics of x, float4 (mean, centred sum of
+ * squares, count, -) per row and part of the row: 9 the persistent kernel's [64 rows][128-column tiles], 10 the many-row passes'
+ * [rows][parts], as many parts as the last GEMM's tiles made). */
 int stairs_debug_buffer(stairs_ctx *ctx, int which, void **ptr_dev, size_t *bytes);
 
 /* Tuning knobs of the persistent kernel, for sweeps.  what 0: 64-element k-blocks per pipeline

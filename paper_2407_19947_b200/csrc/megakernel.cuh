@@ -325,10 +325,21 @@ __device__ __forceinline__ void store_split4(bf16* base, size_t idx, size_t lo_o
 __device__ __forceinline__ float normed(float v, float mu, float rs, float u, float c) { return __fmaf_rn(rs, __fmaf_rn(-mu, u, v), c); }
 __device__ __forceinline__ float rotated(float a, float b, float cs, float sn) { return __fmaf_rn(b, sn, __fmul_rn(a, cs)); }
 __device__ __forceinline__ float square_sum(float a, float b, float c, float d) { return __fadd_rn(__fmaf_rn(b, b, __fmul_rn(a, a)), __fmaf_rn(d, d, __fmul_rn(c, c))); }
-// (mean, M2, count) of n values from their sums shifted by sh
-__device__ __forceinline__ float4 tile_stats(float sh, float s1, float s2, int n) {
-  const float dm = s1 / (float)n;
-  return make_float4(__fadd_rn(sh, dm), fmaxf(__fmaf_rn(-s1, dm, s2), 0.f), (float)n, 0.f);
+// Mean and centred sum of squares of a tile's part of a row, four values at a time and then pair by pair (Chan, Golub and LeVeque's
+// formula for equal counts, the same bits from either side; half: half of one side's count).  Sums shifted by one of the values, in
+// one pass, lose up to seven bits where that value is an outlier channel's (largest relative error of a sum of squares 5e-5, this one
+// 4e-7) and want a division: 0.4B, 9 rows 831 us, this one 819.  The mean first and the squares in a second pass over the lanes: 843.
+struct Moments { float mean, m2; };
+__device__ __forceinline__ Moments moments4(float4 v) {
+  const float m = 0.25f * ((v.x + v.y) + (v.z + v.w));
+  return Moments{m, square_sum(v.x - m, v.y - m, v.z - m, v.w - m)};
+}
+__device__ __forceinline__ Moments merged(Moments a, Moments b, float half) {
+  const float d = b.mean - a.mean;
+  return Moments{0.5f * (a.mean + b.mean), __fmaf_rn(__fmul_rn(d, d), half, __fadd_rn(a.m2, b.m2))};
+}
+__device__ __forceinline__ Moments merged_lanes(Moments a, int o, float half) {
+  return merged(a, Moments{__shfl_xor_sync(0xffffffffu, a.mean, o), __shfl_xor_sync(0xffffffffu, a.m2, o)}, half);
 }
 __device__ __forceinline__ float row_rstd(bool layer_norm, float m2, float n, float mean, int d, float eps) {
   return 1.0f / sqrtf(__fadd_rn((layer_norm ? m2 : __fmaf_rn(__fmul_rn(n, mean), mean, m2)) / (float)d, eps));
@@ -2075,18 +2086,21 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
             }
             if (p.epi == TC_ADD_F32) {
               // residual update (such a GEMM has no folded normalisation); with a following normalised GEMM its operand
-              // bf16(x * gain) and this tile's row statistics (count, mean, centred sum of squares; shifted by the row's first value)
+              // bf16(x * gain) and this tile's row statistics (count, mean, centred sum of squares)
               v = make_float4(k1.x + v.x, k1.y + v.y, k1.z + v.z, k1.w + v.w);
               if (on) {
                 *reinterpret_cast<float4*>(out_f32 + (size_t)row * p.ldo + n0 + col) = v;
                 if (p.next_g) store_split4(P.h, (size_t)row * p.ldo + n0 + col, (size_t)P.lo_row * p.ldo, make_float4(v.x * k2.x, v.y * k2.y, v.z * k2.z, v.w * k2.w));
               }
               if (p.next_g) {
-                const float sh = __shfl_sync(0xffffffffu, v.x, 0), d0 = v.x - sh, d1 = v.y - sh, d2 = v.z - sh, d3 = v.w - sh;
-                float s1 = on ? (d0 + d1) + (d2 + d3) : 0.f, s2 = on ? square_sum(d0, d1, d2, d3) : 0.f;
+                // (a tile of 64 columns, the last one of some widths: lanes 16 to 31 have none)
+                const float n = ncols > 64 ? 8.f : 4.f;
+                Moments r = merged_lanes(moments4(v), 8, 2.f);
+                const Moments all = merged_lanes(r, 16, 4.f);
+                if (ncols > 64) r = all;
 #pragma unroll
-                for (int o = 8; o != 8 * 8; o = o == 16 ? 1 : o == 4 ? 64 : 2 * o) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }   // (8, 16, 1, 2, 4)
-                if (lane == 0) P.stats[(size_t)row * P.stat_tiles + tile] = tile_stats(sh, s1, s2, ncols);
+                for (int o = 1; o < 8; o <<= 1) r = merged_lanes(r, o, n * (float)o);
+                if (lane == 0) P.stats[(size_t)row * P.stat_tiles + tile] = make_float4(r.mean, r.m2, (float)ncols, 0.f);
               }
             } else if (S::swiglu(p)) {
               // gate columns in lanes 0 to 15, the matching up columns in 16 to 31: each of a pair takes two of the four
@@ -2324,7 +2338,6 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                 const bool add_res = p.epi == TC_ADD_F32;
                 epi_bar_sync();   // the exchange tile is complete
                 if (tra && !whole && c0 == 0) tra[1] = globaltimer_ns();
-                float a0x = 0.f;             // (the row's value in this thread's first column)
                 if (!whole || add_res) {
                   float4 a[4];
                   bool on[4];
@@ -2390,7 +2403,6 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
 #pragma unroll
                   for (int q = 0; q < 4; ++q)
                     if (on[q]) *reinterpret_cast<float4*>(vrow + (cg + 8 * q) * 4) = a[q];   // (this thread's own slots)
-                  a0x = a[0].x;
                   if (add_res && !S::ONE && c0 + 16 < Tvalid) {
                     // calls of more than 16 rows: the next chunk's old residual values are requested now,
                     // so that they do not add an L2 round trip to that chunk
@@ -2421,26 +2433,29 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                   // with a following normalised GEMM: its operand bf16(x * gain) and this tile's row
                   // statistics (count, mean, centred sum of squares)
                   if (p.next_g) {
-                    // (sums shifted by the row's first value of the tile, in one pass)
-                    const float sh = __shfl_sync(0xffffffffu, a0x, lane & 24);
-                    float s1 = 0.f, s2 = 0.f, h1 = 0.f, h2 = 0.f;   // (groups 0 and 1, groups 2 and 3)
+                    Moments r{0.f, 0.f}, low = r;   // of a pair of groups; of the first pair
 #pragma unroll 1
-                    for (int q = 0; q < 4; ++q) {
-                      const int col = (cg + 8 * q) * 4;
-                      if (row_on && col < ncols) {
-                        const float4 x4 = *reinterpret_cast<const float4*>(vrow + col);
-                        const float4 g4 = *reinterpret_cast<const float4*>(ctl->gtile + col);
-                        store_split4(P.h, (size_t)t * p.ldo + n0 + col, (size_t)P.lo_row * p.ldo, make_float4(x4.x * g4.x, x4.y * g4.y, x4.z * g4.z, x4.w * g4.w));
-                        const float d0 = x4.x - sh, d1 = x4.y - sh, d2 = x4.z - sh, d3 = x4.w - sh;
-                        s1 += (d0 + d1) + (d2 + d3); s2 += square_sum(d0, d1, d2, d3);
-                      }
-                      if (q == 1) { h1 = s1; h2 = s2; s1 = s2 = 0.f; }
-                    }
-                    s1 += h1; s2 += h2;
-                    if (tra) { asm volatile("" ::"f"(s1), "f"(s2)); tra[7] = globaltimer_ns(); }
+                    for (int h = 0; h < 2; ++h) {
+                      low = r;
+                      if (row_on && h * 64 < ncols) {
+                        Moments part[2];
 #pragma unroll
-                    for (int o = 1; o < 8; o <<= 1) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }
-                    if (cg == 0 && row_on) P.stats[(size_t)t * P.stat_tiles + tile] = tile_stats(sh, s1, s2, ncols);
+                        for (int e = 0; e < 2; ++e) {
+                          const int col = (cg + 8 * (2 * h + e)) * 4;
+                          const float4 x4 = *reinterpret_cast<const float4*>(vrow + col);
+                          const float4 g4 = *reinterpret_cast<const float4*>(ctl->gtile + col);
+                          store_split4(P.h, (size_t)t * p.ldo + n0 + col, (size_t)P.lo_row * p.ldo, make_float4(x4.x * g4.x, x4.y * g4.y, x4.z * g4.z, x4.w * g4.w));
+                          part[e] = moments4(x4);
+                        }
+                        r = merged(part[0], part[1], 2.f);
+                      }
+                    }
+                    if (ncols > 64) r = merged(low, r, 4.f);
+                    const float n = ncols > 64 ? 8.f : 4.f;
+                    if (tra) { asm volatile("" ::"f"(r.mean), "f"(r.m2)); tra[7] = globaltimer_ns(); }
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1) r = merged_lanes(r, o, n * (float)o);
+                    if (cg == 0 && row_on) P.stats[(size_t)t * P.stat_tiles + tile] = make_float4(r.mean, r.m2, (float)ncols, 0.f);
                   }
                 } else if (S::swiglu(p)) {
                   // gate columns (cg + 8 q) * 4 of the tile's first half, the matching up columns 64 further
