@@ -498,11 +498,12 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
       };
       if (finish) {
         if (job.epi == W_ADD) {
-          // residual update, the next GEMM's operand bf16(x * gain), and this warp's row statistics of the
-          // tile (shifted sums: the shift is the row's first value)
-          float s1[4], s2[4], sh[4];
+          // residual update, the next GEMM's operand bf16(x * gain), and this warp's row statistics of the tile: mean and centred sum of
+          // squares of four values a lane and chunk, merged pair by pair (Chan, Golub and LeVeque's formula).  Sums shifted by one of the
+          // row's values, in one pass, lose up to seven bits where that value is an outlier channel's.
+          float mean[4], m2[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) { s1[i] = s2[i] = sh[i] = 0.f; }
+          for (int i = 0; i < 4; ++i) mean[i] = m2[i] = 0.f;
           const int nch = (min(TN, job.N - col0) / ECH - hw + 1) / 2;   // this warp's chunks
           for (int k0 = 0; k0 < nch; k0 += 4) {
 #pragma unroll
@@ -513,6 +514,7 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
                 acc(c0, v);
                 to_tile(v);
                 const float4 g4 = job.next_g ? __ldg(reinterpret_cast<const float4*>(job.next_g + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float share = 1.0f / (float)(k0 + j + 1), weight = 4.0f * (float)(k0 + j) * share;   // (4 values after 4 (k0 + j))
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                   const int r = row0 + 8 * i + tr;
@@ -523,10 +525,10 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
                     if (job.next_g)
                       store_split4(job.out_act, (size_t)r * job.ldo + col, (size_t)job.lo_row * job.ldo, make_float4(x4.x * g4.x, x4.y * g4.y, x4.z * g4.z, x4.w * g4.w));
                   }
-                  if (k0 + j == 0) sh[i] = __shfl_sync(0xffffffffu, x4.x, lane & 28);
-                  const float d0 = x4.x - sh[i], d1 = x4.y - sh[i], d2 = x4.z - sh[i], d3 = x4.w - sh[i];
-                  s1[i] += (d0 + d1) + (d2 + d3);
-                  s2[i] += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+                  const float m = 0.25f * ((x4.x + x4.y) + (x4.z + x4.w)), dm = m - mean[i];
+                  const float d0 = x4.x - m, d1 = x4.y - m, d2 = x4.z - m, d3 = x4.w - m;
+                  m2[i] += ((d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3)) + dm * dm * weight;
+                  mean[i] += dm * share;
                 }
                 load_x(xq[j], col_of(k0 + j + 4));
               }
@@ -537,10 +539,13 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
 #pragma unroll
-              for (int o = 1; o < 4; o <<= 1) { s1[i] += __shfl_xor_sync(0xffffffffu, s1[i], o); s2[i] += __shfl_xor_sync(0xffffffffu, s2[i], o); }
+              for (int o = 1; o < 4; o <<= 1) {   // (as many values on either side: cnt / 4, then cnt / 2)
+                const float m = __shfl_xor_sync(0xffffffffu, mean[i], o), q = __shfl_xor_sync(0xffffffffu, m2[i], o), dm = m - mean[i];
+                m2[i] = (m2[i] + q) + dm * dm * (0.125f * (float)o * cnt);
+                mean[i] = 0.5f * (mean[i] + m);
+              }
               const int r = row0 + 8 * i + tr;
-              const float m = s1[i] / fmaxf(cnt, 1.f);
-              if ((lane & 3) == 0 && r < job.T) job.stats_out[(size_t)r * (2 * job.n_tiles) + 2 * nt + hw] = make_float4(sh[i] + m, fmaxf(s2[i] - s1[i] * m, 0.f), cnt, 0.f);
+              if ((lane & 3) == 0 && r < job.T) job.stats_out[(size_t)r * (2 * job.n_tiles) + 2 * nt + hw] = make_float4(mean[i], m2[i], cnt, 0.f);
             }
           }
         } else if (job.epi == W_GELU) {

@@ -35,7 +35,8 @@ def _parts(eng, which, rows, stride, d):
 
 # (requests of five rows, tuning knobs, roundings of a sum of squares on its way, as counted below)
 FORMS = {"one_cta": (1, {7: 1}, 28), "shared": (1, {7: 2}, 28), "one_cta_40_rows": (8, {7: 1}, 28), "shared_40_rows": (8, {7: 2}, 28),
-         "80_rows": (16, {}, 28), "80_rows_split": (16, {6: 3}, 28)}
+         "80_rows": (16, {}, 28), "80_rows_split": (16, {6: 3}, 28),
+         "130_rows": (26, {4: 1, 5: 1}, 64), "130_rows_split": (26, {4: 1, 5: 4}, 64), "130_rows_pair": (26, {4: 2}, 64)}
 
 
 @pytest.mark.parametrize("form", FORMS.values(), ids=FORMS.keys())
