@@ -2248,13 +2248,15 @@ __global__ void k_accept_static(const __grid_constant__ StaticAcceptParams p) {
 constexpr int SA_THREADS = 256, SA_CTAS = 8;
 constexpr int sa_batch(bool vec) { return 8 * 32 * (vec ? 4 : 1); }   // columns of a warp's batch of loads
 template <bool VEC, int SEG>
-__global__ void __cluster_dims__(SA_CTAS, 1, 1) __launch_bounds__(SA_THREADS, 4) k_accept_cluster(const __grid_constant__ StaticAcceptParams p, const float* __restrict__ logits, int V, int ld) {
+__global__ void __cluster_dims__(SA_CTAS, 1, 1) __launch_bounds__(SA_THREADS, 4) k_accept_cluster(const __grid_constant__ StaticAcceptParams p, const float* logits, int V, int ld) {
   __shared__ unsigned long long red[64][SEG];
   __shared__ unsigned long long gathered[SA_CTAS][64];
   __shared__ unsigned int miss[2];
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   wide::pdl_launch();
-  wide::pdl_wait();   // (nothing is read or written before: large calls are started while the stream's previous kernel ends)
+  // Nothing is read or written before this: large calls are started while the stream's previous kernel, which may write the logits and
+  // drafts, ends.  (For the same reason no pointer is declared restrict, and the logits are read by streaming loads, never by the read-only path.)
+  wide::pdl_wait();
   const int i = blockIdx.x / SA_CTAS, rank = blockIdx.x % SA_CTAS;
   const int k = p.k[i], rows = k + 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int per = ((V + SA_CTAS - 1) / SA_CTAS + 3) / 4 * 4, lo = min(rank * per, V), hi = min(lo + per, V);
@@ -2278,7 +2280,7 @@ __global__ void __cluster_dims__(SA_CTAS, 1, 1) __launch_bounds__(SA_THREADS, 4)
         if (VEC) {   // (a vector past the last column stays inside the row's pitch)
           const float4 q = c < s1 ? __ldcs(reinterpret_cast<const float4*>(row + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
           v[j][0] = q.x; v[j][W > 1 ? 1 : 0] = q.y; v[j][W > 1 ? 2 : 0] = q.z; v[j][W > 1 ? 3 : 0] = q.w;
-        } else v[j][0] = c < s1 ? row[c] : 0.f;
+        } else v[j][0] = c < s1 ? __ldcs(row + c) : 0.f;
       }
 #pragma unroll
       for (int j = 0; j < 8; ++j)

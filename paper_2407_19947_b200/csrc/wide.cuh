@@ -1308,8 +1308,9 @@ __global__ void __launch_bounds__(TC_ATT_THREADS, 2) k_wide_attn_tc(const __grid
 
 // Embedding of the pass's rows (tok, pos, req written by k_rows): the residual stream, the first GEMM's
 // operand bf16(x * gain) hi + lo, the row's statistics, its rotation table and its cache row.  One block per row.
-__global__ void __launch_bounds__(256) k_wide_embed(const bf16* __restrict__ tok_emb, const bf16* __restrict__ pos_emb, const int* __restrict__ tok,
-                                                    const int* __restrict__ pos, const int* __restrict__ req, const int* __restrict__ page_table,
+// (What the stream's previous kernel may still write when this one starts is not declared restrict: the loads stay behind the wait.)
+__global__ void __launch_bounds__(256) k_wide_embed(const bf16* __restrict__ tok_emb, const bf16* __restrict__ pos_emb, const int* tok,
+                                                    const int* pos, const int* req, const int* page_table,
                                                     int page_tokens, int max_pages, const float* __restrict__ g, float* __restrict__ x, bf16* __restrict__ h,
                                                     int lo_row, int d, float4* __restrict__ stats, const float* __restrict__ rope_inv, int half,
                                                     float* __restrict__ rope_cs, float* __restrict__ rope_sn, int* __restrict__ kv_row) {

@@ -91,15 +91,17 @@ def test_static_accept_equals_torch_argmax(vocab, ld, ks):
 
 @pytest.mark.parametrize("captured", [False, True])
 @pytest.mark.parametrize("n_req", [39, 40, 64])      # on both sides of the calls that are started behind the previous kernel
-def test_static_accept_waits_for_the_kernels_before_it(n_req, captured):
-    # the logits and drafts of every call are written by kernels right before it, and its results read right behind it
+@pytest.mark.parametrize("ld", [16500, 16501], ids=["vectors", "scalars"])
+def test_static_accept_waits_for_the_kernels_before_it(ld, n_req, captured):
+    # the logits and drafts of every call are written by kernels right before it, and its results read right behind it; rows on
+    # 16-byte boundaries (whole vectors are loaded) and others
     from paper_2407_19947_b200 import build, stairs
     build.build()
     vocab, k, calls = 16500, 3, 12
     g = torch.Generator(device="cuda")
     g.manual_seed(n_req)
-    src = torch.randn((calls, n_req * (k + 1), vocab), generator=g, device="cuda")
-    want = src.argmax(dim=2).view(calls, n_req, k + 1).to(torch.int32)
+    src = torch.randn((calls, n_req * (k + 1), ld), generator=g, device="cuda")
+    want = src[:, :, :vocab].argmax(dim=2).view(calls, n_req, k + 1).to(torch.int32)
     logits, draft = torch.empty_like(src[0]), torch.zeros((n_req, k), dtype=torch.int32, device="cuda")
     got_t, got_a = torch.zeros_like(want), torch.zeros((calls, n_req), dtype=torch.int32, device="cuda")
 
@@ -107,7 +109,7 @@ def test_static_accept_waits_for_the_kernels_before_it(n_req, captured):
         logits.copy_(src[i])
         draft.copy_(want[i, :, :k])
         draft[:, i % k] += 1                          # the first mismatch of every request
-        tt, al = stairs.accept_static(logits, [k] * n_req, draft, k, stream=stream)
+        tt, al = stairs.accept_static(logits, [k] * n_req, draft, k, stream=stream, vocab=vocab)
         got_t[i].copy_(tt)
         got_a[i].copy_(al)
 
