@@ -37,7 +37,8 @@ int stairs_debug_buffer(stairs_ctx *ctx, int which, void **ptr_dev, size_t *byte
  * call it can serve (0: chosen per call); what 4: CTAs per tile of the many-row GEMMs (0 = planned, 1 or
  * 2), what 5: K ranges per tile of those on single CTAs (0 = planned, 1, 2, 4 or 8), what 6: CTA
  * pairs that share a tile of the GEMMs of 65 to 128 rows (0 = planned, 1 to 4), what 7: split tiles of
- * the persistent kernel finished by one CTA (1) or by all of theirs, a share of the rows each (2; 0 = chosen per call).  Takes effect with the next call. */
+ * the persistent kernel finished by one CTA (1) or by all of theirs, a share of the rows each (2; 0 = chosen per call), what 8:
+ * the bound of device-side waits in cycles (0 = the default).  Takes effect with the next call. */
 int stairs_debug_tune(stairs_ctx *ctx, int what, long long value);
 
 #ifdef __cplusplus

@@ -32,6 +32,7 @@ thread_local std::string g_init_error;
 struct LayerMaps { CUtensorMap wq, wk, wv, wo, w1, w3, w2; };
 
 constexpr int TC_GRID_MAX = 160;        // scratch is sized for at most this many CTAs
+constexpr unsigned long long kWaitLimit = 2000000000ull;   // cycles a device-side wait may take (about a second)
 constexpr int TC_COUNTERS = 1 << 16;    // tiles per GEMM the split bookkeeping can hold
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1655,7 +1656,7 @@ int stairs_init(const stairs_config* cfg, const stairs_weights* target, const st
     int major = 0;
     cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cfg->device);
     cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, cfg->device);
-    ctx->wait_limit = cfg->wait_limit_cycles ? cfg->wait_limit_cycles : 2000000000ull;
+    ctx->wait_limit = cfg->wait_limit_cycles ? cfg->wait_limit_cycles : kWaitLimit;
     e = cudaHostAlloc(reinterpret_cast<void**>(&ctx->status_host), STATUS_WORDS * 4, cudaHostAllocMapped);
     if (e == cudaSuccess) {
       memset(ctx->status_host, 0, STATUS_WORDS * 4);
@@ -2171,6 +2172,10 @@ int stairs_debug_tune(stairs_ctx* ctx, int what, long long value) {
     case 7:
       if (value < 0 || value > 2) return fail(ctx, STAIRS_EINVAL, "split tiles must be 0 (planned), 1 (one CTA) or 2 (shared rows)");
       ctx->share_force = (int)value;
+      return STAIRS_OK;
+    case 8:
+      if (value < 0) return fail(ctx, STAIRS_EINVAL, "the bound of a wait must be 0 (the default) or a number of cycles");
+      ctx->wait_limit = value ? (unsigned long long)value : kWaitLimit;
       return STAIRS_OK;
     default: return fail(ctx, STAIRS_EINVAL, "unknown tuning knob %d", what);
   }

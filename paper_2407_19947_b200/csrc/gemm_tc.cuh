@@ -96,6 +96,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// After an abort, by one thread before the CTA gives up its shared memory and TMEM: what no wait of the teardown sees (MMAs and commits
+// issued before it, also to the other CTA of a pair; a copy into a stage that was only half requested) is over within a
+// millisecond, a thousand times what it takes.
+__device__ __forceinline__ void settle(long long t0) {
+  while (clock64() - t0 < 2000000) __nanosleep(1000);
+}
+
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar,
                                             uint64_t policy) {
   asm volatile(
@@ -447,6 +454,7 @@ static __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc(const __grid_cons
           if ((unsigned long long)(clock64() - t0) > job.wait_limit) break;
         }
       }
+      settle(t0);
     }
     __syncthreads();
   }

@@ -2619,6 +2619,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
           if ((unsigned long long)(clock64() - t0) > drain_limit) break;
         }
       }
+      settle(t0);
     }
     __syncthreads();
   }

@@ -471,6 +471,7 @@ __global__ void __launch_bounds__(wide::WTHREADS, 1) k_mid_gemm(const __grid_con
           if ((unsigned long long)(clock64() - t0) > lim) break;
         }
       }
+      settle(t0);
     }
     __syncthreads();
   }

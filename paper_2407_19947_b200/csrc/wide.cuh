@@ -672,6 +672,7 @@ __global__ void __launch_bounds__(WTHREADS, 1) k_wide_gemm(const __grid_constant
           if ((unsigned long long)(clock64() - t0) > lim) break;
         }
       }
+      settle(t0);
     }
     __syncthreads();
   }
@@ -1300,6 +1301,7 @@ __global__ void __launch_bounds__(TC_ATT_THREADS, 2) k_wide_attn_tc(const __grid
         while (!mbar_try(kv_full + (f & 1) * NST + (f >> 1) % NST, ((f >> 1) / NST) & 1)) {
           if ((unsigned long long)(clock64() - t0) > drain) break;
         }
+      settle(t0);
     }
     __syncthreads();
   }

@@ -257,6 +257,32 @@ def test_many_row_passes_agree_with_small_ones(shape):
     eng.close()
 
 
+@pytest.mark.parametrize("pairs", [1, 3])
+def test_expired_wait_of_a_call_of_one_row_tile_is_reported(pairs):
+    # Of the kernels of a call of 70 rows only its GEMMs have bounded waits.  With a bound of about a microsecond they run out: every
+    # launch must end by itself, the next sync report STAIRS_ETIMEOUT (5), and the same call with the default bound work afterwards.
+    st = _stairs()
+    shape = small_b()
+    tsrc, _ = sources(shape)
+    drafts = torch.from_numpy(np.random.default_rng(1).integers(0, shape.vocab, size=(14, 4)).astype(np.int32)).cuda()
+    eng = st.Stairs(tsrc, None, max_requests=14, max_seq_len=64, k_max=4, kv_page_tokens=16)
+    eng.debug_tune(6, pairs)
+    for i in range(14):
+        eng.prefill(i, list(wl.zipf_tokens(20 + i, shape.vocab, i)))
+    alone = torch.cat([eng.validate([i], [4], drafts[i:i + 1].contiguous(), want_logits=True)[2] for i in range(14)])
+    eng.sync()
+    eng.debug_tune(8, 2000)
+    with pytest.raises(st.StairsError) as e:
+        eng.validate(list(range(14)), [4] * 14, drafts)
+        eng.sync()
+    assert e.value.code == 5
+    eng.debug_tune(8, 0)
+    _, _, many = eng.validate(list(range(14)), [4] * 14, drafts, want_logits=True)
+    eng.sync()
+    assert _distance(many, alone) < ROWS_BAR
+    eng.close()
+
+
 @pytest.mark.parametrize("pairs", [0, 1, 2, 3, 4])
 @pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES.keys())
 def test_calls_of_one_row_tile_at_every_cluster_size(shape, pairs):
