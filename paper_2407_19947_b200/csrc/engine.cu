@@ -840,8 +840,15 @@ int launch_forward_mk(stairs_ctx* ctx, DevModel& M, int T, int logit_first_row, 
   const int share = share_rows(ctx, m, T), cross = share && cross_possible(ctx, m) ? 1 : 0;
   const int slot = program_slot(t_box, pl.kps, cross);
   if (!M.prog_built[slot]) {
-    int rc = build_program(ctx, M, t_box, pl.kps, cross);
-    if (rc) return rc;
+    // Both forms of the program, if calls of this row box take both: building one waits for the stream, which a later call (a draft
+    // length that follows the acceptance) is not to do.
+    bool other = false;
+    for (int t = t_box - 15; t <= t_box; ++t) other = other || (share_rows(ctx, m, t) && cross_possible(ctx, m)) != (cross != 0);
+    for (int c = 0; c <= 1; ++c)
+      if (c == cross || other) {
+        int rc = build_program(ctx, M, t_box, pl.kps, c);
+        if (rc) return rc;
+      }
   }
   mk::Params P;
   memset(&P, 0, sizeof P);

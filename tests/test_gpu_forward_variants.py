@@ -43,6 +43,26 @@ def test_variant_matches_oracle_and_ignores_the_row_count(shape, attention, page
     gu.check_rows_against_oracle(one, tt[0][:17], ref, gu.LOGIT_TOL_BF16)
     eng.close()
 
+
+def test_calls_of_a_row_box_wait_for_the_stream_once():
+    # a model whose calls of few and of more rows take different programs (heads of 80): 16 rows first, then every smaller number while
+    # the stream is busy
+    st = _stairs()
+    shape = wl.workload(3).target.replace(n_layers=1, vocab=2048)
+    src = wl.WeightSource(shape, 1, "torch-cuda")
+    eng = st.Stairs(src, None, max_requests=1, max_seq_len=64, k_max=15, kv_page_tokens=16)
+    eng.prefill(0, list(wl.zipf_tokens(20, shape.vocab, 1)))
+    draft = torch.zeros((1, 15), dtype=torch.int32, device="cuda")
+    kept = [eng.validate([0], [15], draft)]
+    eng.sync()
+    torch.cuda._sleep(400_000_000)
+    busy = torch.cuda.Event()
+    busy.record()
+    kept += [eng.validate([0], [k], draft) for k in range(15)]
+    assert not busy.query()
+    eng.close()
+
+
 @pytest.mark.parametrize("wide_d", [False, True], ids=["", "33_tiles"])
 @pytest.mark.parametrize("attention", [1, 2], ids=["register", "tcgen05"])
 @pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES.keys())
