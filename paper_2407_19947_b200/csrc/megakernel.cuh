@@ -1661,8 +1661,9 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
         }
         // Requests whose positions were split over several units: merge the parked states of every
         // (kv head, query), one warp per item; at head size 64 (mma.sync path) half a warp takes a range, up to twenty ranges in one round
-        // trip (0.4B, 9 rows, nine ranges: 1.4 % of a call).  Heads of 128 by halves of an item, chosen at run time, made the kernel's
-        // text longer: 16 layers of 7B, 2 x 6 rows after 300 1356 us so and 1349 now, 6 rows after 100 1330 and 1322.  Each lane
+        // trip (0.4B, 9 rows, nine ranges: 1.4 % of a call).  Heads of 128: what counts is the text.  By halves of an item, chosen at run
+        // time, 16 layers of 7B, 2 x 6 rows after 300 took 1356 us, with a choice of five and ten loads 1343, with eight 1329;
+        // 9 rows after 1024 1379 and 1370, 6 rows after 100 1310 and 1294, 27 rows after 300 1609 and 1589.  Each lane
         // owns 4 consecutive elements of head_dim, so every partial is one 16-byte load per lane.  The states come
         // from other CTAs' units of this same phase: a word reads PARTIAL_EMPTY until it has been
         // stored, and the warp repeats its loads (bounded) until none does.
@@ -1694,8 +1695,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                 const size_t stride = (size_t)a.n_qblk * S::qblk(P) * (hd + 4);
                 const float* base = set_base + ((size_t)first_slot * S::qblk(P) + ql) * (hd + 4);
                 // (max, sum) of range lane, lane + 32, ...: one load round for up to 32 ranges, then
-                // the ranges' output vectors five or ten loads at a time; weights travel by shuffle and
-                // the accumulation is in range order (of even and odd ranges)
+                // the ranges' output vectors, eight at a time (head size 128), or five, and up to ten where there are more (64), or five;
+                // weights travel by shuffle and the accumulation is in range order (of even and odd ranges)
                 const int nr = a.n_ranges, dd = per == 2 ? (lane & 15) * 4 : lane * 4;
                 long long t0 = 0;
                 bool timing = false;
@@ -1727,10 +1728,10 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                   const float wgt = mu == -INFINITY ? 0.f : fast_exp2(mu - M);   // 0 for lanes past the last range (maxima are base-2 exponents)
                   L += lu * wgt;
                   const int nb = min(32, nr - rb);
-                  for (int g0 = 0; g0 < nb && !gave_up; g0 += (hd % 64 == 0 ? 10 * per : 5)) {
+                  for (int g0 = 0; g0 < nb && !gave_up; g0 += (hd == 128 ? 8 : hd == 64 ? 10 * per : 5)) {
                     uint4 v[10];
                     const float* at = base + (size_t)(rb + g0 + sub) * stride + dd;
-                    const bool more = hd % 64 == 0 && nb - g0 > 5 * per;
+                    const bool eight = hd == 128, more = hd == 64 && nb - g0 > 5 * per;
                     auto load = [&](int u) { v[u] = (g0 + u * per + sub < nb && dd < hd) ? ld_relaxed_u4(at + (size_t)(u * per) * stride) : make_uint4(0u, 0u, 0u, 0u); };
                     auto add = [&](int u) {
                       const float wu = __shfl_sync(0xffffffffu, wgt, (g0 + u * per + sub) & 31);
@@ -1742,6 +1743,12 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                       uint32_t mx = 0u;
 #pragma unroll
                       for (int u = 0; u < 5; ++u) load(u);
+                      if (eight) {
+#pragma unroll
+                        for (int u = 5; u < 8; ++u) load(u);
+#pragma unroll
+                        for (int u = 5; u < 8; ++u) mx = max(max(mx, max(v[u].x, v[u].y)), max(v[u].z, v[u].w));
+                      }
                       if (more) {
 #pragma unroll
                         for (int u = 5; u < 10; ++u) load(u);
@@ -1755,6 +1762,10 @@ __global__ void __launch_bounds__(MK_THREADS, 1) k_forward(const __grid_constant
                     }
 #pragma unroll
                     for (int u = 0; u < 5; ++u) add(u);
+                    if (eight) {
+#pragma unroll
+                      for (int u = 5; u < 8; ++u) add(u);
+                    }
                     if (more) {
 #pragma unroll
                       for (int u = 5; u < 10; ++u) add(u);
