@@ -641,26 +641,30 @@ bool cross_possible(const stairs_ctx* ctx, const stairs_model& m) {
   return tiles < std::min(gemm_ctas(ctx, tiles, m.d_model), units);
 }
 
-// Do the CTAs of a split tile share its rows in this call, or does one finish them all (both give the same bits)?  The difference
-// per layer (us), fitted to both forms of three models at 1 to 64 rows: shared, a GEMM phase ends 1.25 us sooner where ranges are
-// short (0.5 where they stream for long, and the slowest CTA counts), 1.2 later for every further row of a warp (3.0 where tiles
-// are more than CTAs: whole ones come on top), and finished by one CTA 1.7 later for every further 16 rows.  0.4B: shared up to 64 rows,
-// 0.82 of the other form at 64; 3B: up to 4, 0.97; 7B: up to 4, 0.98 (nine rows, shared: 1.06).
+// Do the CTAs of a split tile share its rows in this call, or does one finish them all (both give the same bits)?  What sharing adds to
+// a call (us): a GEMM phase ends 1.4 sooner where ranges are short, 0.5 where they stream for long and the slowest CTA counts (0.2 with
+// the rotation of cut heads in it, which saves a phase), 0.8 later for every further row of a warp (1.9 where tiles are as many as CTAs or more);
+// finished by one CTA it ends 1.2 later for every further 16 rows and 0.6 later where there are more than 16 at all.  The LM head, with
+// tiles for all CTAs, is 1 and 4 for every further row of a warp later when shared.
+// Fitted to both forms of fourteen models (width 512 to 5120, both families, heads of 64 to 128, two depths) at 1 to 64 rows after 200 and
+// 800 positions, 896 pairs: 0.04 % behind the better form on average, 3.3 % at most.  An earlier fit to three models: 0.25 % and 11.6 %.
+// 0.4B: shared up to 64 rows, 0.79 of the other form at 64; 3B: up to 6, 0.98 (7 rows 1.02); 7B: up to 4, 0.98 (5 rows 1.01, nine 1.06).
 int share_rows(const stairs_ctx* ctx, const stairs_model& m, int T) {
   if (ctx->share_force) return ctx->share_force - 1;
-  double later = cross_possible(ctx, m) ? -1.0 : 0.0;   // (the rotation's phase is saved, the projection's gets longer)
-  auto gemm = [&](int tiles, int K) {
+  double layer = 0.0;
+  auto gemm = [&](int tiles, int K, bool cross) {
     const int units = tiles * (((K + tc::BK - 1) / tc::BK + mk::RANGE_UNIT_KB - 1) / mk::RANGE_UNIT_KB), ge = std::min(gemm_ctas(ctx, tiles, K), units);
-    const int seg = ge / tiles;   // CTAs per tile at least; a CTA has parts of two tiles unless they divide evenly
-    const int rows = ge > tiles ? (ge % tiles ? 2 : 1) * ((T + seg - 1) / seg) : (T * tiles + ge - 1) / ge, rounds = (rows + 3) / 4;
-    later += (units <= 4 * ge ? -1.25 : -0.5) + (tiles >= ge ? 3.0 : 1.2) * (rounds - 1) - 1.7 * ((T + 15) / 16 - 1);
+    // rows a CTA finishes when its last MMA is done: its share of a tile, of two unless CTAs divide evenly among tiles; a whole tile's, or
+    // those of the two it has parts of
+    const int seg = ge / tiles, rows = ge > tiles ? (ge % tiles ? 2 : 1) * ((T + seg - 1) / seg) : T;
+    layer += (cross ? -0.2 : units <= 4 * ge ? -1.4 : -0.5) + (tiles >= ge ? 1.9 : 0.8) * ((rows + 3) / 4 - 1) - 1.2 * ((T + 15) / 16 - 1) - (T > 16 ? 0.6 : 0.0);
   };
   const int nq = m.n_heads * m.head_dim, nkv = m.n_kv_heads * m.head_dim;
-  gemm((nq + tc::BM - 1) / tc::BM + 2 * ((nkv + tc::BM - 1) / tc::BM), m.d_model);
-  gemm((m.d_model + tc::BM - 1) / tc::BM, nq);
-  gemm(m.act == 1 ? (m.d_ff + 63) / 64 : (m.d_ff + tc::BM - 1) / tc::BM, m.d_model);
-  gemm((m.d_model + tc::BM - 1) / tc::BM, m.d_ff);
-  return later < 0 ? 1 : 0;
+  gemm((nq + tc::BM - 1) / tc::BM + 2 * ((nkv + tc::BM - 1) / tc::BM), m.d_model, cross_possible(ctx, m));
+  gemm((m.d_model + tc::BM - 1) / tc::BM, nq, false);
+  gemm(m.act == 1 ? (m.d_ff + 63) / 64 : (m.d_ff + tc::BM - 1) / tc::BM, m.d_model, false);
+  gemm((m.d_model + tc::BM - 1) / tc::BM, m.d_ff, false);
+  return m.n_layers * layer + 1.0 + 4.0 * ((T + 3) / 4 - 1) < 0.0 ? 1 : 0;
 }
 
 int build_program(stairs_ctx* ctx, DevModel& M, int t_box, int kps, int cross) {
