@@ -617,6 +617,8 @@ MkPlan mk_plan(const stairs_ctx* ctx, const stairs_model& m, int t_box, int q_ro
 // partial tiles.  Model: the longest range's units (two k-blocks) at ~44 GB/s per SM; 1.4 us and 1.6 us per batch of eight partials
 // where tiles are split, 0.7 us more where CTAs do not divide evenly among tiles (a CTA then has parts of two).  (Must not depend on
 // the row box: see RANGE_UNIT_KB.)
+// Against the estimate before, on fourteen models (width 512 to 5120, 1 to 64 rows), with the ways of finishing tiles: none slower by
+// more than 1.3 % (width 512, 16 rows), most 2 to 20 % quicker.
 int gemm_ctas(const stairs_ctx* ctx, int tiles, int K) {
   const int grid = std::min(ctx->sm_count, TC_GRID_MAX), units = tiles * (((K + tc::BK - 1) / tc::BK + mk::RANGE_UNIT_KB - 1) / mk::RANGE_UNIT_KB);
   double best = 1e30; int best_ge = grid;
@@ -1029,6 +1031,9 @@ int launch_wide_gemm(stairs_ctx* ctx, wide::WideJob& job, const void* x, int K, 
 
 // Pairs per cluster of a GEMM over 65 to 128 rows (mid.cuh): whole rounds of tile pairs over the clusters that run at once, a k-block
 // at the SM's load rate (all weights at the copy rate), the exchange of the sums.
+// Fitted at the configs' widths (0.4B, 3B, 7B: never more than 1.5 % behind the best count for all GEMMs of a pass); on eleven other models of
+// width 512 to 5120 at 66 to 128 rows 22 to 42 % quicker than the kernels before (width 512: 2 to 19 %), but up to 20 % behind three pairs for
+// all at width 512, 9 % at width 768, 7 % at width 5120 with heads of 80.
 int mid_cluster(const stairs_ctx* ctx, int n_tiles, int kblocks, int TN, int x_box) {
   int best = 1;
   double best_us = 1e30;
