@@ -2263,7 +2263,7 @@ __global__ void k_accept_static(const __grid_constant__ StaticAcceptParams p) {
 // all the request's rows; row keys are reduced per CTA, gathered in the first CTA's shared memory, and its
 // threads take the tokens and the accept length.  Nothing is kept in memory between launches.  A call is
 // bound by latency (5 rows of 32000: 31 us a call with three launches, 11 now, of which the kernel 4) or by reading
-// the logits (576 rows: 53 us, now 15.6), so a warp takes at most a quarter of a row's slice at a time with eight vectors a
+// the logits (576 rows: 53 us, now 17.1, or 15.6 with its start behind the call before), so a warp takes at most a quarter of a row's slice at a time with eight vectors a
 // lane in flight, and the CTAs of 64 requests fit the chip at once.  A slice is cut no finer than one such batch, though: a batch
 // takes its latency however few of its vectors exist (64 rows of 1000 in quarters: 28.8 us, in whole slices 10, three launches 14.4).
 constexpr int SA_THREADS = 256, SA_CTAS = 8;
@@ -2383,8 +2383,9 @@ extern "C" int stairs_accept_static(const float* logits_dev, int vocab, int ld, 
     const int per = (vocab + SA_CTAS - 1) / SA_CTAS, batch = sa_batch(vec), seg = per <= batch ? 1 : per <= 2 * batch ? 2 : 4;
     auto kern = vec ? (seg == 1 ? k_accept_cluster<true, 1> : seg == 2 ? k_accept_cluster<true, 2> : k_accept_cluster<true, 4>)
                     : (seg == 1 ? k_accept_cluster<false, 1> : seg == 2 ? k_accept_cluster<false, 2> : k_accept_cluster<false, 4>);
-    // Calls of many logits and at least 320 CTAs: their start is hidden behind the stream's previous kernel (576 rows of 32128: 17.1 ->
-    // 15.6 us; 40 x 4 rows of 20000 13.3 -> 12.7).  Small calls are bound by the host, which pays for the attribute; of fewer CTAs
+    // Calls of many logits and at least 320 CTAs: their start is hidden behind the stream's previous kernel where that still runs when the
+    // call arrives (calls one behind another, 576 rows of 32128: 17.1 -> 15.6 us; 40 x 4 rows of 20000 13.3 -> 12.7; reading the logits is
+    // no quicker, and a call on an idle stream, waited for, takes 38.4 either way).  Small calls are bound by the host, which pays for the attribute; of fewer CTAs
     // the second call's share SMs that the first one's still hold (16 x 16 rows of 32128: 16.0 -> 19.8).
     if ((long long)rows * vocab >= (2 << 20) && n_req * SA_CTAS >= 320) {
       cudaLaunchConfig_t cfg{};
